@@ -18,28 +18,41 @@
 // (L, M, C, D: the exact sums of orders 2..5) into an FP32 double-float
 // (hi, lo), every term through an error-free TwoSum.  Y = hi + lo in FP64.
 //
-// MMA form: one chain of same-shape MMAs per K tile.  A stage holds the four A
-// slices and the X slices stacked as seven 64-row blocks [0 0 0 x1 x2 x3 x4]
-// (three zero blocks written once).  A slice s times the 256 rows starting at
-// block 4 - s is [0 ... x1 .. x(5-s)], so its N = 256 product lands, column
-// block j, in the accumulator of order j + 2 for every s: all sixteen MMAs of
-// a 32-wide K tile (4 slices x 2 K steps) have the same accumulator and shape
-// and are ordered by the tensor pipe without waits.  The zero blocks cost 6 of
-// 16 products' worth of tensor work; the MMAs are large enough (128 x 256 x 16)
-// that one thread's issue keeps the pipe fed.
+// MMA form: a stage holds the four A slices and the X slices stacked as five
+// 64-row blocks [0 x1 x2 x3 x4] (the zero block written once).  A pair of
+// neighbouring blocks times an A slice s is an N = 128 product that lands in two
+// neighbouring orders: x1 x2 and x3 x4 for slice 1, 0 x1 and x2 x3 for slice 2,
+// x1 x2 for slice 3, 0 x1 for slice 4 give the ten products of orders 2..5 in six
+// MMAs per 16 K values (twelve per tile), all of one shape and in two accumulator
+// halves, so that they are ordered by the tensor pipe without waits.
 //
-// Block: 128 rows of op(A) x 64 columns of X, eighteen warps:
-//   warp 17 (one lane): TMA loads of the FP32 tiles of A (128 x 32) into four
-//     raw stages;
-//   warps 0-7: move a raw tile to registers (releasing the stage), scale and
-//     cut the slices into one of two operand stages (K-major, 64-byte swizzle);
-//     one lane loads the pre-cut X slices by TMA.  An entry that does not fit
-//     its recorded row scale (the operator changed after the scales were taken)
-//     aborts the block, whose outputs are then NaN;
-//   warp 8: allocates 512 TMEM columns (two windows x four orders x 64
-//     columns); one lane issues the MMAs;
-//   warps 9-16: drain once per window (two warps per TMEM lane quarter, 32
+// What bounds it and what was measured (dense A^T X, N = 32768, 60 columns, every
+// tile active, the pre-cut of X included): 2.40 -> 1.74 ms; per 32-wide tile and
+// block 2430 -> ~1600 cycles, of which the twelve MMAs take 768, the FP32 pipe ~640
+// (cuts and drain) and shared memory ~1400 (operands read by the MMAs, slices
+// written, raw tile and X copied in).  A clock of every role showed where the rest
+// went: the tile search in each role (TileIter now), 256 arrivals a barrier (one per
+// warp now), one X-copying thread that searched three tiles ahead, and one cutter
+// group whose cycle (two waits, loads, cuts, the proxy fence: ~2000 cycles, mostly
+// latency) the MMAs waited for (three groups now, one per stage).  Eight N = 256
+// products a tile over three zero blocks (the earlier form) cost 1024 cycles of MMAs
+// and 8 KB more a stage; a fourth raw buffer measured the same as three.
+//
+// Block: 128 rows of op(A) x 64 columns of X, 32 warps:
+//   warp 0: allocates 512 TMEM columns (two windows x four orders x 64 columns);
+//     one elected lane issues the MMAs;
+//   warp 1 (one lane): TMA loads of the FP32 tiles of A (128 x 32), one raw buffer
+//     per cutter group;
+//   warp 2 (one lane): bulk copies of the pre-cut X slices;
+//   warps 4-15, three groups: move a raw tile to registers (releasing its buffer),
+//     scale, and cut the slices into the group's operand stage (K-major, 64-byte
+//     swizzle).  An entry that does not fit its recorded row scale (the operator
+//     changed after the scales were taken) aborts the block, whose outputs are
+//     then NaN;
+//   warps 16-31: drain once per window (four warps per TMEM lane quarter, 16
 //     columns each) and write Y.
+// Every waiter on an mbarrier here waits for each of its phases in turn: a parity
+// says nothing about a phase further away.
 // All-zero K tiles of X are skipped; the four X slices of an active tile are
 // always loaded (a zero slice contributes zeros).  Every mbarrier wait is bounded
 // (the pipeline waits by the limit the host sets, hm_set_wait_limit); on timeout
@@ -61,16 +74,21 @@ constexpr int TM = 128, TN = 64, TK = 32;  // TK: the K extent of a stage
 constexpr int NSL = 4;                  // slices of A and of X
 constexpr int A_SLICE = TM * TK * 2;    // 8 KB: 128 rows x 64 bytes
 constexpr int XB = TN * TK * 2;         // 4 KB: one X slice, 64 rows x 64 bytes
-constexpr int XZ = 3;                   // zero blocks before x1
-constexpr int X_BYTES = (XZ + NSL) * XB;                 // 28 KB
-constexpr int STAGE_BYTES = NSL * A_SLICE + X_BYTES;     // 60 KB
+constexpr int XZ = 1;                   // zero blocks before x1
+constexpr int X_BYTES = (XZ + NSL) * XB;                 // 20 KB
+constexpr int STAGE_BYTES = NSL * A_SLICE + X_BYTES;     // 52 KB
 constexpr int SSTAGES = 3;
 constexpr int RAW_BYTES = TM * TK * 4;  // 16 KB
-constexpr int RSTAGES = 2;
-constexpr int RAW_REGION = RSTAGES * RAW_BYTES;          // 32 KB
-constexpr int LAYOUT_BYTES = RAW_REGION + SSTAGES * STAGE_BYTES;  // 212 KB
-constexpr int NCONV = 256, NDRAIN = 256, NTHREADS = 608;
-constexpr int W_MMA = 8, W_DRAIN0 = 9, W_TMA = 17, W_XTMA = 18;
+constexpr int RSTAGES = SSTAGES;  // one raw tile per cutter group
+constexpr int RAW_REGION = RSTAGES * RAW_BYTES;          // 48 KB
+constexpr int LAYOUT_BYTES = RAW_REGION + SSTAGES * STAGE_BYTES;  // 204 KB
+// Warps: 0 MMA, 1 TMA of A, 2 copies of X, 3 idle; then three groups of four
+// cutter warps (group g cuts the tiles of stage g), then sixteen drain warps.
+constexpr int GT = 128, NG = SSTAGES;    // threads of a group, groups
+constexpr int NDRAIN = 512, NTHREADS = 128 + NG * GT + NDRAIN;
+constexpr int W_MMA = 0, W_TMA = 1, W_XTMA = 2, W_CUT0 = 4, W_DRAIN0 = W_CUT0 + NG * GT / 32;
+constexpr int DC = TN * TM / NDRAIN;     // columns of a drain thread: 16
+static_assert(NTHREADS <= 1024, "one block");
 constexpr uint32_t TMEM_COLS = 512;  // 2 buffers x 4 orders x 64 columns
 constexpr int WIN_ROWS = 256;        // K values per exact accumulation window
 constexpr int WIN_TILES = WIN_ROWS / TK;
@@ -108,32 +126,71 @@ __device__ __forceinline__ int exp_above(float x) {
   return e;
 }
 
-// Round to the nearest integer, ties to even, for |x| < 2^22: adding 1.5 * 2^23
-// lands in [2^23, 2^24), where the FP32 spacing is 1, so the add rounds x and
-// the subtraction is exact.  Two adds on the FMA pipe instead of one rounding
-// instruction on the slower conversion pipe; the compiler does not reassociate
-// the pair (no fast-math).
-__device__ __forceinline__ float round_int(float x) {
-  return (x + 12582912.f) - 12582912.f;
+// Two FP32 values as one operand of the packed FP32 instructions: one issue slot
+// for two lanes' worth of adds, at the scalar instructions' FP32 rate.  The
+// cutter and drain warps share four schedulers with the MMA-issuing warp, so
+// the issue slots are what they save (both results round as the scalar forms).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float x, float y) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& x, float& y) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(v));
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+// a - b as b * (-1) + a: one rounding, the same one, in one instruction (the
+// packed add takes no negated operand: negating by xor costs two more)
+__device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(b), "l"(0xbf800000bf800000ull), "l"(a));
+  return r;
+}
+// the largest magnitude of three, NaN if one is (the range check of the cutters)
+__device__ __forceinline__ float max_abs(float a, float b, float c) {
+  float r;
+  asm("max.NaN.abs.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
-// Cut v (|v| < 128, a multiple of 2^-24 of the scale) into four 8-bit integers
-// (the digits of v rounded to a multiple of 2^-24, each in [-128, 128]).
-__device__ __forceinline__ void cut4(float v, float& s1, float& s2, float& s3, float& s4) {
-  s1 = round_int(v);
-  float r = (v - s1) * 256.f;
-  s2 = round_int(r);
-  r = (r - s2) * 256.f;
-  s3 = round_int(r);
-  r = (r - s3) * 256.f;
-  s4 = round_int(r);
+// Cut v (|v| < 128) into four digits, digit t a multiple of 2^(-8 (t - 1)) with at
+// most eight significant bits: v rounded to a multiple of 2^-24.  Each digit is
+// rounded (ties to even) by adding 1.5 * 2^(23 - 8 (t - 1)), which lands where
+// the FP32 spacing is the digit's unit, and taking the constant off again
+// (exact); two adds on the FMA pipe instead of an instruction of the slower
+// conversion pipe.  The digits keep their scale 2^(-8 (t - 1)): the X slices carry
+// theirs too, so every product of order d = s + t has the weight 2^(-8 (d - 2)) in
+// its accumulator and the drain needs no factor per order.  The compiler does not
+// reassociate the adds (no fast-math).
+__device__ __forceinline__ void cut4(f32x2 v, f32x2& s1, f32x2& s2, f32x2& s3, f32x2& s4) {
+  constexpr float C1 = 12582912.f, C2 = 49152.f, C3 = 192.f, C4 = 0.75f;
+  const f32x2 c1 = pack2(C1, C1), c2 = pack2(C2, C2), c3 = pack2(C3, C3), c4 = pack2(C4, C4);
+  const f32x2 m1 = pack2(-C1, -C1), m2 = pack2(-C2, -C2), m3 = pack2(-C3, -C3),
+              m4 = pack2(-C4, -C4);
+  s1 = add2(add2(v, c1), m1);
+  v = sub2(v, s1);
+  s2 = add2(add2(v, c2), m2);
+  v = sub2(v, s2);
+  s3 = add2(add2(v, c3), m3);
+  v = sub2(v, s3);
+  s4 = add2(add2(v, c4), m4);
 }
 
-// Two digits as a BF16 pair (lo in the low half).  A digit is an integer of at
-// most 8 significant bits, so its FP32 pattern ends in 16 zero bits and its BF16
-// pattern is the FP32 pattern's upper half: one byte permute, no rounding.
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
+// Two digits as a BF16 pair (the first in the low half).  A digit has at most 8
+// significant bits, so its FP32 pattern ends in 16 zero bits and its BF16 pattern
+// is the FP32 pattern's upper half: one byte permute, no rounding.
+__device__ __forceinline__ uint32_t pack_bf16(f32x2 d) {
+  return __byte_perm((uint32_t)d, (uint32_t)(d >> 32), 0x7632);
 }
 
 // Exponents of A per row and window of 256 columns: e_row[i * nw + w] = e with
@@ -214,7 +271,7 @@ __global__ __launch_bounds__(256) void k_split_x64(const double* __restrict__ X,
         const int rr = t * TN + c, kk = (int)(row % TK);
         const int64_t tile = (int64_t)ct * (kpad / TK) + row / TK;
         Xs[(tile * (NSL * TN) + rr) * TK + ((((kk >> 3) ^ ((rr >> 1) & 3))) << 3) + (kk & 7)] =
-            __float2bfloat16_rn((float)st);
+            __float2bfloat16_rn(pow2f(-8 * t) * (float)st);
       }
     }
   }
@@ -229,20 +286,39 @@ __global__ __launch_bounds__(256) void k_split_x64(const double* __restrict__ X,
   }
 }
 
-// Named barrier 1 of the 256 cutter threads (warps 0-7), and its AND-reduction
-// form: the generating cutters (GEN) stage table windows in shared memory and
-// must leave their loop together.
-__device__ __forceinline__ void cutters_sync() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
-__device__ __forceinline__ bool cutters_all(bool v) {
+// Named barrier 1 + g of the 128 threads of cutter group g, and its AND-reduction
+// form: the generating cutters (GEN) stage their group's table windows in shared
+// memory and must leave their loop together.
+__device__ __forceinline__ void group_sync(int g) {
+  asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory");
+}
+__device__ __forceinline__ bool group_all(int g, bool v) {
   uint32_t r;
   asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, 1, 256, p;\n\t"
+      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 p, %1, 0;\n\tbar.red.and.pred q, %2, 128, p;\n\t"
       "selp.u32 %0, 1, 0, q;\n\t}\n"
       : "=r"(r)
-      : "r"((uint32_t)v)
+      : "r"((uint32_t)v), "r"(g + 1)
       : "memory");
   return r != 0;
 }
+// Walk over a block's active K tiles: the bits of the current word stay in a
+// register, so a step is a handful of instructions (a search from shared memory at
+// every step took each role 150-450 cycles a tile).
+struct TileIter {
+  const uint32_t* bits;
+  int nwords, end, wd;
+  uint32_t b;
+  __device__ __forceinline__ int next() {  // the next active tile, `end` past the last
+    while (!b) {
+      if (++wd >= nwords) { wd = nwords; return end; }
+      b = bits[wd];
+    }
+    const int kt = (wd << 5) + __ffs((int)b) - 1;
+    b &= b - 1u;
+    return kt;
+  }
+};
 
 // GEN = 1: the operator is the matrix-free log kernel of the ellipse (see
 // launch_gemm_esg_gen): the cutters generate each tile's entries from two
@@ -255,8 +331,9 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_esg(
     const int* __restrict__ e_rows, double* __restrict__ Y, int64_t ldy, int* __restrict__ err,
     long long poll_limit, const float* __restrict__ tabS, const float* __restrict__ tabP) {
   extern __shared__ unsigned char smem_raw[];
+  // st_full: one arrival per cutter warp (not per thread) and the X copy's bytes
   __shared__ __align__(8) uint64_t raw_full[RSTAGES], raw_empty[RSTAGES], st_full[SSTAGES],
-      x_full[SSTAGES], st_empty[SSTAGES], acc_full[2], acc_empty[2], bar_final;
+      st_empty[SSTAGES], acc_full[2], acc_empty[2], bar_final;
   __shared__ uint32_t tmem_base_slot;
   __shared__ volatile int abort_flag;
   __shared__ int win_lo, win_hi;  // this block's share of the windows (split over K)
@@ -279,16 +356,15 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_esg(
     abort_flag = 0;
     for (int i = 0; i < RSTAGES; ++i) {
       mbar_init(smem_u32(&raw_full[i]), 1);
-      mbar_init(smem_u32(&raw_empty[i]), NCONV);
+      mbar_init(smem_u32(&raw_empty[i]), GT / 32);
     }
     for (int i = 0; i < SSTAGES; ++i) {
-      mbar_init(smem_u32(&st_full[i]), NCONV);
-      mbar_init(smem_u32(&x_full[i]), 1);
+      mbar_init(smem_u32(&st_full[i]), GT / 32 + 1);
       mbar_init(smem_u32(&st_empty[i]), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&acc_full[b]), 1);
-      mbar_init(smem_u32(&acc_empty[b]), NDRAIN);
+      mbar_init(smem_u32(&acc_empty[b]), NDRAIN / 32);
     }
     mbar_init(smem_u32(&bar_final), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -364,378 +440,437 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_esg(
     act_bits[wd] = b;
   }
   __syncthreads();
-  auto active = [&](int kt) -> int { return (act_bits[kt >> 5] >> (kt & 31)) & 1; };
-  // the first active K tile at or after `from` (nkt if none)
   const int nwords = (nkt + 31) / 32;
-  auto next_active = [&](int from) -> int {
-    int wd = from >> 5;
-    if (wd >= nwords) return nkt;
-    uint32_t b = act_bits[wd] & (~0u << (from & 31));
-    while (!b) {
-      if (++wd >= nwords) return nkt;
-      b = act_bits[wd];
-    }
-    return (wd << 5) + __ffs(b) - 1;
+  const auto tiles = [&]() { return TileIter{act_bits, nwords, nkt, -1, 0u}; };
+
+  // A cutter warp that gives up still arrives once more on its group's stage: the
+  // X copy of the tile it did not cut may be in flight, and the copying thread's
+  // wait for it on the way out then ends with the copy
+  auto leave_stage = [&](int g) {
+    if (lane == 0) mbar_arrive(smem_u32(&st_full[g]));
   };
 
-  if (warp == W_TMA) {
-    // ---------------------------------------------------------- TMA of A
-    if (!GEN && lane == 0) {
-      int it = 0;
-      const uint64_t pol = l2_policy_evict_first();  // A is read once per call
-      for (int kt = next_active(0); kt < nkt; kt = next_active(kt + 1)) {
-        const int r = it % RSTAGES;
-        if (!mbar_wait(smem_u32(&raw_empty[r]), ((it / RSTAGES) & 1) ^ 1, &abort_flag,
-                       poll_limit))
-          break;
-        mbar_arrive_tx(smem_u32(&raw_full[r]), RAW_BYTES);
-        if (!TRANS)
-          tma_load_2d_hint(raw_addr + r * RAW_BYTES, &tmA, kt * TK, (int)m0,
-                           smem_u32(&raw_full[r]), pol);
-        else
-          tma_load_2d_hint(raw_addr + r * RAW_BYTES, &tmA, (int)m0, kt * TK,
-                           smem_u32(&raw_full[r]), pol);
-        ++it;
-      }
-      // the copies in flight land before the block's shared memory is given up
-      for (int j = (it > RSTAGES ? it - RSTAGES : 0); j < it; ++j)
-        mbar_wait_drain(smem_u32(&raw_full[j % RSTAGES]), (j / RSTAGES) & 1);
-    }
-  } else if (GEN && warp < 8) {
-    // ---------------------------------------------------------- generate A, cut, TMA of X
-    // A(i, j) = (S[|i - j|] + P[i + j]) in float pairs: fl((Sh + Ph) + (Sl + Pl)),
-    // 1 on the diagonal, 0 outside [0, n).  A tile's entries use TM + TK - 1
-    // values of each table, staged in the (unused) raw region: window entry e
-    // holds S[|d|] for i - j = d = m0 - k0 - (TK - 1) + e, and P[m0 + k0 + e].
-    int it = 0;
-    // Four shifted copies of each window (copy q holds window entry x + q at x),
-    // so that every thread reads its four consecutive entries of a table as one
-    // aligned float4: for row m the P entries start at m + 4 k4 and the S entries
-    // (descending) at m - 4 k4 + TK - 4, both congruent to m mod 4.
-    constexpr int WC = 164;  // floats per copy (16-byte multiple, covers index 161)
-    float* win = reinterpret_cast<float*>(sbase);  // [table (Sh, Sl, Ph, Pl)][q][WC]
-    // Thread e (< TM + TK - 1 <= NCONV) owns window entry e.  The next active
-    // tile's entry is loaded from the (L2-resident) tables one tile ahead, so the
-    // load latency hides behind the current tile's cut.
-    float pv[4] = {0.f, 0.f, 0.f, 0.f};
-    auto load_win = [&](int ktn) {
-      pv[0] = pv[1] = pv[2] = pv[3] = 0.f;
-      const int e = tid;
-      if (e < TM + TK - 1) {
-        const int64_t kn = (int64_t)ktn * TK;
-        const int64_t d = m0 - kn - (TK - 1) + e, ad = d < 0 ? -d : d, sidx = m0 + kn + e;
-        if (ad > 0 && ad < n) { pv[0] = tabS[ad]; pv[1] = tabS[n + ad]; }
-        if (sidx < 2 * n - 1) { pv[2] = tabP[sidx]; pv[3] = tabP[2 * n - 1 + sidx]; }
-      }
-    };
-    {
-      const int k1 = next_active(0);
-      if (k1 < nkt) load_win(k1);
-    }
-    constexpr int NP = TM * TK / 4 / NCONV;  // 4 passes: rows 32 p + tid / 8
-    float scs[NP];                           // this thread's row scales in window scw
-    int scw = -1;
-    for (int kt = next_active(0); kt < nkt; kt = next_active(kt + 1)) {
-      const int s = it % SSTAGES;
-      const bool ok = !abort_flag &&
-                      mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag,
-                                poll_limit);
-      // all cutters leave together (they share the table windows); the barrier
-      // also orders the previous tile's window reads before the new writes
-      if (!cutters_all(ok)) break;
-      const uint32_t st = stage_addr0 + (uint32_t)s * STAGE_BYTES;
-      const int64_t k0 = (int64_t)kt * TK;
-      {
-        const int e = tid;
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int x = e - q;
-          if (x >= 0 && x < WC)
-#pragma unroll
-            for (int a = 0; a < 4; ++a) win[(a * 4 + q) * WC + x] = pv[a];
+  if (warp < W_CUT0) {
+    if (warp == W_TMA) {
+      // -------------------------------------------------------- TMA of A
+      if (!GEN && lane == 0) {
+        int it = 0;
+        const uint64_t pol = l2_policy_evict_first();  // A is read once per call
+        TileIter ti = tiles();
+        for (int kt = ti.next(); kt < nkt; kt = ti.next()) {
+          const int r = it % RSTAGES;
+          if (!mbar_wait(smem_u32(&raw_empty[r]), ((it / RSTAGES) & 1) ^ 1, &abort_flag,
+                         poll_limit))
+            break;
+          mbar_arrive_tx(smem_u32(&raw_full[r]), RAW_BYTES);
+          if (!TRANS)
+            tma_load_2d_hint(raw_addr + r * RAW_BYTES, &tmA, kt * TK, (int)m0,
+                             smem_u32(&raw_full[r]), pol);
+          else
+            tma_load_2d_hint(raw_addr + r * RAW_BYTES, &tmA, (int)m0, kt * TK,
+                             smem_u32(&raw_full[r]), pol);
+          ++it;
         }
+        // the copies in flight land before the block's shared memory is given up
+        for (int j = (it > RSTAGES ? it - RSTAGES : 0); j < it; ++j)
+          mbar_wait_drain(smem_u32(&raw_full[j % RSTAGES]), (j / RSTAGES) & 1);
       }
-      {
-        const int k1 = next_active(kt + 1);
-        if (k1 < nkt) load_win(k1);
-      }
-      cutters_sync();
-      // tiles that hold a diagonal entry or reach past n take the per-entry fixes
-      const bool fix = (m0 + TM > n) || (k0 + TK > n) || (m0 < k0 + TK && k0 < m0 + TM);
-      const int dk = (int)(fix ? k0 - m0 : 0);  // i == j  <=>  m - (4 k4 + e) == dk
-      const int mrow = (int)(n - m0 < TM ? n - m0 : TM), kcol = (int)(n - k0 < TK ? n - k0 : TK);
-      unsigned char* sp = sbase + (st - base);
-      int bad = 0;
-      if (kt / WIN_TILES != scw) {
-        scw = kt / WIN_TILES;
-#pragma unroll
-        for (int p = 0; p < NP; ++p) scs[p] = row_scale((p * NCONV + tid) >> 3, scw);
-      }
-#pragma unroll
-      for (int p = 0; p < NP; ++p) {
-        const int f = p * NCONV + tid, m = f >> 3, k4 = f & 7;
-        const float sc = scs[p];
-        const int q = m & 3, ps = m + 4 * k4 - q, ds = m - 4 * k4 + (TK - 4) - q;
-        const float4 sh4 = *reinterpret_cast<const float4*>(win + (0 * 4 + q) * WC + ds);
-        const float4 sl4 = *reinterpret_cast<const float4*>(win + (1 * 4 + q) * WC + ds);
-        const float4 ph4 = *reinterpret_cast<const float4*>(win + (2 * 4 + q) * WC + ps);
-        const float4 pl4 = *reinterpret_cast<const float4*>(win + (3 * 4 + q) * WC + ps);
-        // entry e: S at window index m - 4 k4 + TK - 1 - e (component 3 - e of the
-        // S float4), P at m + 4 k4 + e (component e)
-        const float shv[4] = {sh4.w, sh4.z, sh4.y, sh4.x}, slv[4] = {sl4.w, sl4.z, sl4.y, sl4.x};
-        const float phv[4] = {ph4.x, ph4.y, ph4.z, ph4.w}, plv[4] = {pl4.x, pl4.y, pl4.z, pl4.w};
-        float a[4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          float v = (shv[e] + phv[e]) + (slv[e] + plv[e]);
-          if (fix) {
-            const int kk = 4 * k4 + e;
-            if (m - kk == dk) v = 1.f;
-            if (m >= mrow || kk >= kcol) v = 0.f;
+    } else if (warp == W_XTMA) {
+      // -------------------------------------------------------- bulk copies of the X slices
+      // the four pre-cut slices of a K tile are one contiguous 16 KB block of Xs,
+      // already in the stage's swizzled order
+      if (lane == 0) {
+        const int64_t nkt_pad = 2 * ((n + KPAD - 1) / KPAD);  // K tiles of the padded Xs
+        int it = 0;
+        const uint64_t pol = l2_policy_evict_last();  // every row block re-reads X
+        TileIter ti = tiles(), tp = tiles();
+        int kp = 0;  // the tile to prefetch, SSTAGES active ones ahead
+        for (int i = 0; i <= SSTAGES; ++i) kp = tp.next();
+        for (int kt = ti.next(); kt < nkt; kt = ti.next()) {
+          const int s = it % SSTAGES;
+          if (!mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag, poll_limit))
+            break;
+          const uint32_t st = stage_addr0 + (uint32_t)s * STAGE_BYTES;
+          mbar_arrive_tx(smem_u32(&st_full[s]), (uint32_t)(NSL * XB));
+          const int64_t tile = (int64_t)ct * nkt_pad + kt;
+          bulk_load_hint(st + NSL * A_SLICE + XZ * XB, Xs + tile * (NSL * TN * TK),
+                         (uint32_t)(NSL * XB), smem_u32(&st_full[s]), pol);
+          // the tile SSTAGES active tiles ahead, into L2 while this stage turns over
+          if (kp < nkt) {
+            bulk_prefetch_l2(Xs + ((int64_t)ct * nkt_pad + kp) * (NSL * TN * TK),
+                             (uint32_t)(NSL * XB));
+            kp = tp.next();
           }
-          a[e] = v * sc;
+          ++it;
         }
-        float sl[4][4];
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          bad |= !(fabsf(a[e]) < 128.f);
-          cut4(a[e], sl[0][e], sl[1][e], sl[2][e], sl[3][e]);
-        }
-        const uint32_t off = sw64_off(m, k4 >> 1) + (uint32_t)((k4 & 1) * 8);
-#pragma unroll
-        for (int t = 0; t < NSL; ++t)
-          *reinterpret_cast<uint2*>(sp + t * A_SLICE + off) =
-              make_uint2(pack_bf16(sl[t][0], sl[t][1]), pack_bf16(sl[t][2], sl[t][3]));
+        for (int j = (it > SSTAGES ? it - SSTAGES : 0); j < it; ++j)
+          mbar_wait_drain(smem_u32(&st_full[j % SSTAGES]), (j / SSTAGES) & 1);
       }
-      if (bad) abort_flag = 3;
-      fence_proxy_async();
-      mbar_arrive(smem_u32(&st_full[s]));
-      ++it;
+    } else if (warp == W_MMA) {
+      // -------------------------------------------------------- MMA issue
+      // The whole warp walks the tiles and one elected lane issues.  Loop control goes
+      // through votes, so that the stage, window and descriptor values are uniform
+      // over the warp and can live in uniform registers, which is what the MMA takes
+      // its operands from.
+      // The look at the next tile's barrier (~250 cycles) comes after the first eight
+      // of a tile's MMAs, so that it runs beside them.
+      constexpr uint32_t kAll = 0xffffffffu;
+      const bool leader = elect_one();
+      uint32_t s = 0, ph = 0, ab = 0, aph = 1;  // stage and phase; accumulator buffer and phase
+      uint32_t started = 0;
+      bool ready = false, fresh = true, ok = true;
+      const uint32_t id = idesc_bf16_f32_n(2 * TN);  // M = 128, N = 128
+      TileIter ti = tiles();
+      int kt = ti.next();
+      while (__any_sync(kAll, kt < nkt)) {
+        if (fresh) {
+          ok = __all_sync(kAll, mbar_wait(smem_u32(&acc_empty[ab]), aph, &abort_flag, poll_limit));
+          started = 0;
+        }
+        if (ok && !ready)
+          ok = __all_sync(kAll, mbar_wait(smem_u32(&st_full[s]), ph, &abort_flag, poll_limit));
+        if (!ok) break;
+        tc_fence_after();
+        const uint32_t dbase = tmem + ab * (4 * TN);
+        // descriptors of the stage's operands: the address field holds addr / 16
+        // (the stage lies below 256 KB, so offsets add without carry)
+        const uint64_t d0 = sw64_desc(stage_addr0 + s * STAGE_BYTES);
+        const uint32_t sn = s + 1 == SSTAGES ? 0 : s + 1, phn = s + 1 == SSTAGES ? ph ^ 1 : ph;
+        // the six products [A slice sl + 1] x [X blocks b, b + 1] of the tile: orders
+        // 2, 3 (accumulator half 0) take x1 x2 for slice 1 and 0 x1 for slice 2;
+        // orders 4, 5 (half 1) take x3 x4, x2 x3, x1 x2, 0 x1 for slices 1 to 4
+        auto product = [&](int sl, int half, int blk, uint32_t accum) {
+          const uint64_t ad = d0 + (uint64_t)((sl * A_SLICE) >> 4);
+          const uint64_t bd = d0 + (uint64_t)((NSL * A_SLICE + blk * XB) >> 4);
+          const uint32_t dt = dbase + (uint32_t)(half * 2 * TN);
+          mma_bf16(dt, ad, bd, id, accum);
+          mma_bf16(dt, ad + 2, bd + 2, id, 1);  // the second K step is 32 bytes on
+        };
+        if (leader) {
+          product(0, 0, 1, started);
+          product(0, 1, 3, started);
+          product(1, 0, 0, 1);
+          product(1, 1, 2, 1);
+        }
+        const int ktn = ti.next();
+        ready = __all_sync(kAll, ktn < nkt && mbar_test(smem_u32(&st_full[sn]), phn));
+        fresh = __any_sync(kAll, ktn >= nkt || ktn / WIN_TILES != kt / WIN_TILES);
+        if (leader) {
+          product(2, 1, 1, 1);
+          product(3, 1, 0, 1);
+          mma_commit(smem_u32(&st_empty[s]));
+          if (fresh) mma_commit(smem_u32(&acc_full[ab]));  // the window's last tile
+        }
+        started = 1;
+        if (fresh) {
+          ab ^= 1;
+          aph ^= ab ^ 1;  // the phase turns when buffer 0 comes round again
+        }
+        kt = ktn;
+        s = sn;
+        ph = phn;
+      }
+      // every MMA issued by this warp completes before TMEM is released: this wait
+      // ignores the other roles' abort and takes the full limit; only if even that
+      // runs out is TMEM left allocated (the error flag reports it)
+      if (leader) {
+        mma_commit(smem_u32(&bar_final));
+        if (!mbar_wait_drain(smem_u32(&bar_final), 0)) abort_flag = 2;
+      }
+      __syncwarp();
     }
-  } else if (warp < 8) {
-    // ---------------------------------------------------------- cut A, TMA of X
-    int it = 0;
-    constexpr int NP = TM * TK / 4 / NCONV;  // 4 passes: rows 32 p + tid / 8 (not TRANS)
-    float scs[NP];                           // this thread's row scales in window scw
-    int scw = -1;
-    for (int kt = next_active(0); kt < nkt && !abort_flag; kt = next_active(kt + 1)) {
-      const int s = it % SSTAGES, r = it % RSTAGES;
-      if (kt / WIN_TILES != scw) {  // (issued before the raw wait: the loads overlap it)
-        scw = kt / WIN_TILES;
-        if (!TRANS) {
+  } else if (warp < W_DRAIN0) {
+    if (GEN) {
+      // -------------------------------------------------------- generate A and cut
+      // A(i, j) = (S[|i - j|] + P[i + j]) in float pairs: fl((Sh + Ph) + (Sl + Pl)),
+      // 1 on the diagonal, 0 outside [0, n).  A tile's entries use TM + TK - 1
+      // values of each table, staged in the (unused) raw region: window entry e
+      // holds S[|d|] for i - j = d = m0 - k0 - (TK - 1) + e, and P[m0 + k0 + e].
+      const int g = (warp - W_CUT0) >> 2, t = threadIdx.x - W_CUT0 * 32 - g * GT;
+      // Four shifted copies of each window (copy q holds window entry x + q at x),
+      // so that every thread reads its four consecutive entries of a table as one
+      // aligned float4: for row m the P entries start at m + 4 k4 and the S entries
+      // (descending) at m - 4 k4 + TK - 4, both congruent to m mod 4.
+      constexpr int WC = 164;  // floats per copy (16-byte multiple, covers index 161)
+      static_assert(NG * 16 * WC * 4 <= RAW_REGION, "a group's windows in the raw region");
+      float* win = reinterpret_cast<float*>(sbase) + g * (16 * WC);  // [Sh, Sl, Ph, Pl][q][WC]
+      // Thread t owns window entries t and t + 128 (< TM + TK - 1).  The group's next
+      // tile's entries are loaded from the (L2-resident) tables one tile ahead, so
+      // the load latency hides behind the current tile's cut.
+      float pv[2][4];
+      auto load_win = [&](int ktn) {
 #pragma unroll
-          for (int p = 0; p < NP; ++p) scs[p] = row_scale((p * NCONV + tid) >> 3, scw);
-        } else {
-          scs[0] = row_scale(tid & (TM - 1), scw);
+        for (int i = 0; i < 2; ++i) {
+          pv[i][0] = pv[i][1] = pv[i][2] = pv[i][3] = 0.f;
+          const int e = t + i * GT;
+          if (e < TM + TK - 1) {
+            const int64_t kn = (int64_t)ktn * TK;
+            const int64_t d = m0 - kn - (TK - 1) + e, ad = d < 0 ? -d : d, sidx = m0 + kn + e;
+            if (ad > 0 && ad < n) { pv[i][0] = tabS[ad]; pv[i][1] = tabS[n + ad]; }
+            if (sidx < 2 * n - 1) { pv[i][2] = tabP[sidx]; pv[i][3] = tabP[2 * n - 1 + sidx]; }
+          }
         }
-      }
-      if (!mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag, poll_limit))
-        break;
-      const uint32_t st = stage_addr0 + (uint32_t)s * STAGE_BYTES;
-      if (!mbar_wait(smem_u32(&raw_full[r]), (it / RSTAGES) & 1, &abort_flag, poll_limit)) break;
-      const unsigned char* rw = sbase + r * RAW_BYTES;
-      unsigned char* sp = sbase + (st - base);
-      int bad = 0;
-      if (!TRANS) {
-        // raw [128 rows][32 k]; pass p: rows 32p .. 32p+31, 8 threads per row
-        float4 v[NP];
+      };
+      // the group's tiles: every NG-th active one, from the g-th
+      TileIter ti = tiles();
+      int kt = ti.next();
+      for (int i = 0; i < g; ++i) kt = ti.next();
+      if (kt < nkt) load_win(kt);
+      constexpr int NP = TM * TK / 4 / GT;  // 8 passes: rows 16 p + t / 8
+      float scs[NP];                        // this thread's row scales in window scw
+      int scw = -1;
+      uint32_t ph = 1;
+      while (kt < nkt) {
+        const bool ok = !abort_flag &&
+                        mbar_wait(smem_u32(&st_empty[g]), ph, &abort_flag, poll_limit);
+        ph ^= 1;
+        // the group leaves together (it shares the table windows); the barrier also
+        // orders the previous tile's window reads before the new writes
+        if (!group_all(g, ok)) { leave_stage(g); break; }
+        const int64_t k0 = (int64_t)kt * TK;
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int x = t + i * GT - q;
+            if (x >= 0 && x < WC)
+#pragma unroll
+              for (int a = 0; a < 4; ++a) win[(a * 4 + q) * WC + x] = pv[i][a];
+          }
+        int ktn = ti.next();
+#pragma unroll
+        for (int i = 1; i < NG; ++i) ktn = ti.next();
+        if (ktn < nkt) load_win(ktn);
+        group_sync(g);
+        // tiles that hold a diagonal entry or reach past n take the per-entry fixes
+        const bool fix = (m0 + TM > n) || (k0 + TK > n) || (m0 < k0 + TK && k0 < m0 + TM);
+        const int dk = (int)(fix ? k0 - m0 : 0);  // i == j  <=>  m - (4 k4 + e) == dk
+        const int mrow = (int)(n - m0 < TM ? n - m0 : TM), kcol = (int)(n - k0 < TK ? n - k0 : TK);
+        unsigned char* sp = sbase + RAW_REGION + g * STAGE_BYTES;
+        float mx = 0.f;
+        if (kt / WIN_TILES != scw) {
+          scw = kt / WIN_TILES;
+#pragma unroll
+          for (int p = 0; p < NP; ++p) scs[p] = row_scale((p * GT + t) >> 3, scw);
+        }
 #pragma unroll
         for (int p = 0; p < NP; ++p) {
-          const int f = p * NCONV + tid, m = f >> 3, k4 = f & 7;
-          v[p] = *reinterpret_cast<const float4*>(rw + m * (TK * 4) + k4 * 16);
+          const int f = p * GT + t, m = f >> 3, k4 = f & 7;
+          const float sc = scs[p];
+          const int q = m & 3, ps = m + 4 * k4 - q, ds = m - 4 * k4 + (TK - 4) - q;
+          const float4 sh4 = *reinterpret_cast<const float4*>(win + (0 * 4 + q) * WC + ds);
+          const float4 sl4 = *reinterpret_cast<const float4*>(win + (1 * 4 + q) * WC + ds);
+          const float4 ph4 = *reinterpret_cast<const float4*>(win + (2 * 4 + q) * WC + ps);
+          const float4 pl4 = *reinterpret_cast<const float4*>(win + (3 * 4 + q) * WC + ps);
+          // entry e: S at window index m - 4 k4 + TK - 1 - e (component 3 - e of the
+          // S float4), P at m + 4 k4 + e (component e)
+          const float shv[4] = {sh4.w, sh4.z, sh4.y, sh4.x}, slv[4] = {sl4.w, sl4.z, sl4.y, sl4.x};
+          const float phv[4] = {ph4.x, ph4.y, ph4.z, ph4.w}, plv[4] = {pl4.x, pl4.y, pl4.z, pl4.w};
+          float a[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            float v = (shv[e] + phv[e]) + (slv[e] + plv[e]);
+            if (fix) {
+              const int kk = 4 * k4 + e;
+              if (m - kk == dk) v = 1.f;
+              if (m >= mrow || kk >= kcol) v = 0.f;
+            }
+            a[e] = v * sc;
+          }
+          mx = max_abs(max_abs(mx, a[0], a[1]), a[2], a[3]);
+          f32x2 sl[4][2];
+#pragma unroll
+          for (int e = 0; e < 2; ++e)
+            cut4(pack2(a[2 * e], a[2 * e + 1]), sl[0][e], sl[1][e], sl[2][e], sl[3][e]);
+          const uint32_t off = sw64_off(m, k4 >> 1) + (uint32_t)((k4 & 1) * 8);
+#pragma unroll
+          for (int t4 = 0; t4 < NSL; ++t4)
+            *reinterpret_cast<uint2*>(sp + t4 * A_SLICE + off) =
+                make_uint2(pack_bf16(sl[t4][0]), pack_bf16(sl[t4][1]));
+        }
+        if (!(mx < 128.f)) abort_flag = 3;
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&st_full[g]));
+        kt = ktn;
+      }
+    } else {
+      // -------------------------------------------------------- cut A
+      const int g = (warp - W_CUT0) >> 2, t = threadIdx.x - W_CUT0 * 32 - g * GT;
+      constexpr int NP = TM * TK / 4 / GT;  // 8 passes: rows 16 p + t / 8 (not TRANS)
+      float scs[NP];                        // this thread's row scales in window scw
+      int scw = -1;
+      unsigned char* sp = sbase + RAW_REGION + g * STAGE_BYTES;
+      float v[TK];  // the thread's 32 entries of its tile
+      // the group's tiles: every NG-th active one, from the g-th
+      TileIter ti = tiles();
+      int kt = ti.next();
+      for (int i = 0; i < g; ++i) kt = ti.next();
+      uint32_t ph = 1;
+      while (kt < nkt) {
+        if (kt / WIN_TILES != scw) {  // (issued before the waits: the loads overlap them)
+          scw = kt / WIN_TILES;
+          if (!TRANS) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) scs[p] = row_scale((p * GT + t) >> 3, scw);
+          } else {
+            scs[0] = row_scale(t, scw);
+          }
+        }
+        // The warp's lanes leave together: one of them arrives for all.  The raw tile
+        // is waited for and read before the stage is free: safe because raw buffer g
+        // is this group's alone, so its phases cannot run ahead of the group (with
+        // buffers shared between groups, a group could meet the phase before the
+        // one it waits for, whose parity reads as complete).
+        if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&raw_full[g]), ph ^ 1, &abort_flag,
+                                               poll_limit))) {
+          leave_stage(g);
+          break;
+        }
+        // the raw tile into registers first (the wait for the stage follows), so that
+        // the raw buffer is free again early
+        const unsigned char* rw = sbase + g * RAW_BYTES;
+        if (!TRANS) {
+          // raw [128 rows][32 k]; pass p: rows 16 p .. 16 p + 15, 8 threads per row
+#pragma unroll
+          for (int p = 0; p < NP; ++p) {
+            const int f = p * GT + t, m = f >> 3, k4 = f & 7;
+            const float4 x = *reinterpret_cast<const float4*>(rw + m * (TK * 4) + k4 * 16);
+            v[4 * p] = x.x; v[4 * p + 1] = x.y; v[4 * p + 2] = x.z; v[4 * p + 3] = x.w;
+          }
+        } else {
+          // raw [32 k][128 m]; thread m = t takes all 32 k
+#pragma unroll
+          for (int i = 0; i < TK; ++i) v[i] = *reinterpret_cast<const float*>(rw + (i * TM + t) * 4);
         }
         // the next TMA write (async proxy) must follow these generic reads
         fence_proxy_async();
-        mbar_arrive(smem_u32(&raw_empty[r]));  // the raw stage is free for a later tile
-#pragma unroll
-        for (int p = 0; p < NP; ++p) {
-          const int f = p * NCONV + tid, m = f >> 3, k4 = f & 7;
-          const float sc = scs[p];
-          float a[4] = {v[p].x * sc, v[p].y * sc, v[p].z * sc, v[p].w * sc};
-          float sl[4][4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            bad |= !(fabsf(a[i]) < 128.f);
-            cut4(a[i], sl[0][i], sl[1][i], sl[2][i], sl[3][i]);
-          }
-          const uint32_t off = sw64_off(m, k4 >> 1) + (uint32_t)((k4 & 1) * 8);
-#pragma unroll
-          for (int t = 0; t < NSL; ++t)
-            *reinterpret_cast<uint2*>(sp + t * A_SLICE + off) =
-                make_uint2(pack_bf16(sl[t][0], sl[t][1]), pack_bf16(sl[t][2], sl[t][3]));
-        }
-      } else {
-        // raw [32 k][128 m]; thread (m, half) takes k = 16 half .. 16 half + 15
-        const int m = tid & (TM - 1), h = tid >> 7;
-        float v[16];
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-          v[i] = *reinterpret_cast<const float*>(rw + ((h * 16 + i) * TM + m) * 4);
-        fence_proxy_async();
-        mbar_arrive(smem_u32(&raw_empty[r]));
-        const float sc = scs[0];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {  // 16-byte chunk 2 h + q: k = 16 h + 8 q ..
-          float sl[4][8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const float a = v[q * 8 + i] * sc;
-            bad |= !(fabsf(a) < 128.f);
-            cut4(a, sl[0][i], sl[1][i], sl[2][i], sl[3][i]);
-          }
-          const uint32_t off = sw64_off(m, h * 2 + q);
-#pragma unroll
-          for (int t = 0; t < NSL; ++t)
-            *reinterpret_cast<uint4*>(sp + t * A_SLICE + off) =
-                make_uint4(pack_bf16(sl[t][0], sl[t][1]), pack_bf16(sl[t][2], sl[t][3]),
-                           pack_bf16(sl[t][4], sl[t][5]), pack_bf16(sl[t][6], sl[t][7]));
-        }
-      }
-      if (bad) abort_flag = 3;  // an entry outgrew its recorded row scale
-      fence_proxy_async();
-      mbar_arrive(smem_u32(&st_full[s]));
-      ++it;
-    }
-  } else if (warp == W_XTMA) {
-    // ---------------------------------------------------------- bulk copies of the X slices
-    // the four pre-cut slices of a K tile are one contiguous 16 KB block of Xs,
-    // already in the stage's swizzled order
-    if (lane == 0) {
-      const int64_t nkt_pad = 2 * ((n + KPAD - 1) / KPAD);  // K tiles of the padded Xs
-      int it = 0;
-      const uint64_t pol = l2_policy_evict_last();  // every row block re-reads X
-      for (int kt = next_active(0); kt < nkt; kt = next_active(kt + 1)) {
-        const int s = it % SSTAGES;
-        if (!mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag, poll_limit))
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&raw_empty[g]));
+        if (!__all_sync(0xffffffffu,
+                        mbar_wait(smem_u32(&st_empty[g]), ph, &abort_flag, poll_limit))) {
+          leave_stage(g);
           break;
-        const uint32_t st = stage_addr0 + (uint32_t)s * STAGE_BYTES;
-        mbar_arrive_tx(smem_u32(&x_full[s]), (uint32_t)(NSL * XB));
-        const int64_t tile = (int64_t)ct * nkt_pad + kt;
-        bulk_load_hint(st + NSL * A_SLICE + XZ * XB, Xs + tile * (NSL * TN * TK),
-                       (uint32_t)(NSL * XB), smem_u32(&x_full[s]), pol);
-        // the tile SSTAGES active tiles ahead, into L2 while this stage turns over
-        int kp = kt;
-        for (int i = 0; i < SSTAGES && kp < nkt; ++i) kp = next_active(kp + 1);
-        if (kp < nkt)
-          bulk_prefetch_l2(Xs + ((int64_t)ct * nkt_pad + kp) * (NSL * TN * TK),
-                           (uint32_t)(NSL * XB));
-        ++it;
-      }
-      for (int j = (it > SSTAGES ? it - SSTAGES : 0); j < it; ++j)
-        mbar_wait_drain(smem_u32(&x_full[j % SSTAGES]), (j / SSTAGES) & 1);
-    }
-  } else if (warp == W_MMA) {
-    // ---------------------------------------------------------- MMA issue
-    if (lane == 0) {
-      int it = 0, wc = 0, cur = -1;
-      uint32_t started = 0, dbase = 0;
-      bool ok = true;
-      const uint32_t id = idesc_bf16_f32_n(NSL * TN);  // M = 128, N = 256
-      for (int kt = next_active(0); kt < nkt && ok; kt = next_active(kt + 1)) {
-        const int w = kt / WIN_TILES;
-        if (w != cur) {
-          if (cur >= 0) {
-            mma_commit(smem_u32(&acc_full[wc & 1]));
-            ++wc;
-          }
-          cur = w;
-          ok = mbar_wait(smem_u32(&acc_empty[wc & 1]), ((wc >> 1) & 1) ^ 1, &abort_flag, poll_limit);
-          if (!ok) break;
-          dbase = tmem + (uint32_t)((wc & 1) * 4 * TN);
-          started = 0;
         }
-        const int s = it % SSTAGES;
-        ok = mbar_wait(smem_u32(&st_full[s]), (it / SSTAGES) & 1, &abort_flag, poll_limit) &&
-             mbar_wait(smem_u32(&x_full[s]), (it / SSTAGES) & 1, &abort_flag, poll_limit);
-        if (!ok) break;
-        tc_fence_after();
-        const uint32_t st = stage_addr0 + (uint32_t)s * STAGE_BYTES;
-        // descriptors of the stage's operands: the address field holds addr / 16
-        // (the stage lies below 256 KB, so offsets add without carry)
-        const uint64_t d0 = sw64_desc(st);
+        ph ^= 1;
+        float mx = 0.f;
+        if (!TRANS) {
 #pragma unroll
-        for (int sa = 0; sa < NSL; ++sa) {
-          // A slice sa + 1 times [0 .. x1 .. x(4 - sa)]: the 256 rows from block 3 - sa
-          const uint64_t ad = d0 + (uint64_t)((sa * A_SLICE) >> 4);
-          const uint64_t bd = d0 + (uint64_t)((NSL * A_SLICE + (XZ - sa) * XB) >> 4);
+          for (int p = 0; p < NP; ++p) {
+            const int f = p * GT + t, m = f >> 3, k4 = f & 7;
+            const float sc = scs[p];
+            f32x2 sl[4][2];
 #pragma unroll
-          for (int kk = 0; kk < TK / 16; ++kk) {  // K step kk is 32 bytes on
-            mma_bf16(dbase, ad + (uint64_t)(2 * kk), bd + (uint64_t)(2 * kk), id, started);
-            started = 1;
+            for (int i = 0; i < 2; ++i) {
+              const float a = v[4 * p + 2 * i] * sc, b = v[4 * p + 2 * i + 1] * sc;
+              mx = max_abs(mx, a, b);
+              cut4(pack2(a, b), sl[0][i], sl[1][i], sl[2][i], sl[3][i]);
+            }
+            const uint32_t off = sw64_off(m, k4 >> 1) + (uint32_t)((k4 & 1) * 8);
+#pragma unroll
+            for (int t4 = 0; t4 < NSL; ++t4)
+              *reinterpret_cast<uint2*>(sp + t4 * A_SLICE + off) =
+                  make_uint2(pack_bf16(sl[t4][0]), pack_bf16(sl[t4][1]));
+          }
+        } else {
+          const float sc = scs[0];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {  // 16-byte chunk q: k = 8 q ..
+            f32x2 sl[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float a = v[q * 8 + 2 * i] * sc, b = v[q * 8 + 2 * i + 1] * sc;
+              mx = max_abs(mx, a, b);
+              cut4(pack2(a, b), sl[0][i], sl[1][i], sl[2][i], sl[3][i]);
+            }
+            const uint32_t off = sw64_off(t, q);
+#pragma unroll
+            for (int t4 = 0; t4 < NSL; ++t4)
+              *reinterpret_cast<uint4*>(sp + t4 * A_SLICE + off) =
+                  make_uint4(pack_bf16(sl[t4][0]), pack_bf16(sl[t4][1]), pack_bf16(sl[t4][2]),
+                             pack_bf16(sl[t4][3]));
           }
         }
-        mma_commit(smem_u32(&st_empty[s]));
-        ++it;
+        if (!(mx < 128.f)) abort_flag = 3;  // an entry outgrew its recorded row scale
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(smem_u32(&st_full[g]));
+#pragma unroll
+        for (int i = 0; i < NG; ++i) kt = ti.next();
       }
-      if (ok && cur >= 0) mma_commit(smem_u32(&acc_full[wc & 1]));
-      // every MMA issued by this thread completes before TMEM is released: this
-      // wait ignores the other roles' abort and takes the full limit; only if
-      // even that runs out is TMEM left allocated (the error flag reports it)
-      mma_commit(smem_u32(&bar_final));
-      if (!mbar_wait_drain(smem_u32(&bar_final), 0)) abort_flag = 2;
     }
   } else {
     // ---------------------------------------------------------- drain / epilogue
-    const int dw = warp - W_DRAIN0;  // 0..7
+    const int dw = warp - W_DRAIN0;  // 0 .. 15
     const int q4 = warp & 3;         // TMEM lane quarter
-    const int half = dw >> 2;        // columns 32 half .. 32 half + 31
+    const int c0 = (dw >> 2) * DC;   // columns c0 .. c0 + 15 of the tile
     const int r = q4 * 32 + lane;
-    float hi[32], lo[32];
+    f32x2 hi[DC / 2], lo[DC / 2];  // columns 2 j, 2 j + 1 of them
 #pragma unroll
-    for (int j = 0; j < 32; ++j) { hi[j] = 0.f; lo[j] = 0.f; }
-    const int64_t colbase = (int64_t)ct * TN + half * 32;
+    for (int j = 0; j < DC / 2; ++j) { hi[j] = 0ull; lo[j] = 0ull; }
     int wc = 0;
     for (int w = 0; w < nwin; ++w) {
-      int any = 0;
-      for (int kt = w * WIN_TILES; kt < nkt && kt < (w + 1) * WIN_TILES; ++kt) any |= active(kt);
-      if (!any) continue;
+      // the window's eight K tiles are one byte of the activity mask
+      if (!((act_bits[w >> 2] >> ((w & 3) * 8)) & 0xffu)) continue;
       const int b = wc & 1;
-      const int exl = ex[((int64_t)w * nct + ct) * TN + half * 32 + lane];  // column lane
+      const int exl = ex[((int64_t)w * nct + ct) * TN + c0 + (lane & 15)];  // column lane
       const int ea = (m0 + r < n) ? e_rows[(m0 + r) * nwin + w] : 0;      // row, window
-      if (!mbar_wait(smem_u32(&acc_full[b]), (wc >> 1) & 1, &abort_flag, poll_limit)) break;
+      // every scale 2^(ea + exl - 14) of the warp in the normal range: its bits are a sum
+      const int emin = __reduce_min_sync(0xffffffffu, exl), emax = __reduce_max_sync(0xffffffffu, exl);
+      const bool normal = __all_sync(0xffffffffu, ea + emin - 14 >= -126 && ea + emax - 14 <= 127);
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), (wc >> 1) & 1, &abort_flag,
+                                             poll_limit)))
+        break;
       tc_fence_after();
-      const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 4 * TN + half * 32);
+      const uint32_t tl = tmem + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * 4 * TN + c0);
 #pragma unroll
-      for (int g = 0; g < 2; ++g) {
-        float sc[16], v[16];
+      for (int g = 0; g < DC / 8; ++g) {
+        float sc[8];
+        if (normal) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          const int e = ea + __shfl_sync(0xffffffffu, exl, g * 16 + j) - 14;
-          sc[j] = (e >= -126 && e <= 127) ? pow2f(e) : ldexpf(1.f, e);
+          for (int j = 0; j < 8; ++j)
+            sc[j] = __int_as_float(((ea + 113) << 23) + __shfl_sync(0xffffffffu, exl << 23, g * 8 + j));
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            sc[j] = ldexpf(1.f, ea + __shfl_sync(0xffffffffu, exl, g * 8 + j) - 14);
         }
-        // orders 2..5: exact integer sums times exact powers of two, each added
-        // into (hi, lo) through TwoSum, so that lo only gathers rounding residues
-        // (the lower orders are not small: their digits run up to 128 against a
-        // leading digit that may be much smaller)
+        // orders 2..5: exact sums (integers times 2^(-8 (d - 2))) times an exact power
+        // of two, each added into (hi, lo) through TwoSum, so that lo only gathers
+        // rounding residues (the lower orders are not small: their digits run up
+        // to 128 against a leading digit that may be much smaller)
 #pragma unroll
         for (int d = 0; d < 4; ++d) {
-          const float cd = d == 0 ? 1.f : (d == 1 ? 0.00390625f : (d == 2 ? 1.52587890625e-05f
-                                                                         : 5.9604644775390625e-08f));
-          tmem_ld16(tl + (uint32_t)(d * TN + g * 16), v);
+          float v[8];
+          tmem_ld8(tl + (uint32_t)(d * TN + g * 8), v);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int jj = g * 16 + j;
-            const float t = v[j] * (sc[j] * cd);
-            const float sum = hi[jj] + t;
-            const float bp = sum - hi[jj];
-            lo[jj] += (hi[jj] - (sum - bp)) + (t - bp);
+          for (int j = 0; j < 4; ++j) {
+            const int jj = g * 4 + j;
+            const f32x2 t = mul2(pack2(v[2 * j], v[2 * j + 1]), pack2(sc[2 * j], sc[2 * j + 1]));
+            const f32x2 sum = add2(hi[jj], t);
+            const f32x2 bp = sub2(sum, hi[jj]);
+            lo[jj] = add2(lo[jj], add2(sub2(hi[jj], sub2(sum, bp)), sub2(t, bp)));
             hi[jj] = sum;
           }
         }
       }
       tc_fence_before();
-      mbar_arrive(smem_u32(&acc_empty[b]));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
       ++wc;
     }
     const int64_t grow = m0 + r;
     const bool bad = abort_flag != 0;
     if (grow < n) {
 #pragma unroll
-      for (int j = 0; j < 32; ++j) {
-        const int64_t col = colbase + j;
+      for (int j = 0; j < DC; ++j) {
+        const int64_t col = (int64_t)ct * TN + c0 + j;
         if (col < ncols) {
+          float h[2], l[2];
+          unpack2(hi[j >> 1], h[0], h[1]);
+          unpack2(lo[j >> 1], l[0], l[1]);
           const double v = bad ? __longlong_as_double(0x7ff8000000000000ll)
-                               : (double)hi[j] + (double)lo[j];
+                               : (double)h[j & 1] + (double)l[j & 1];
           // split over K: Y was zeroed and every block adds its share
           if (gridDim.z > 1) atomicAdd(&Y[grow + col * ldy], v);
           else Y[grow + col * ldy] = v;
