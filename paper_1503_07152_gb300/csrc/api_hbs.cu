@@ -101,7 +101,8 @@ hm_status hbs_partial_apply(HbsState<T>& s, int m, const T* X, int64_t ldx, T* S
     T* qh = s.qhat;
     T* uh = s.uhat;
     launch_seg_tn<T>(pm.d_tn, pm.n_tn, pm.d_tn_begin, pm.nnodes, pm.node0, Vout, s.N, 0, 0, r,
-                     X + cb * ldx, ldx, 0, 0, w, s.partial, qh + pm.node0 * rw, st, s.df);
+                     X + cb * ldx, ldx, 0, 0, w, s.partial, qh + pm.node0 * rw, st, s.df,
+                     ncols == 2 * r && w == 2 * r ? r : 0);
     for (int lev = m - 1; lev >= 1; --lev) {
       for (int tau = 1 << lev; tau < (2 << lev); ++tau)
         it.add(Sout + (2 * tau) * rr, r, 1, qh + (2 * tau) * rw, r, 0, qh + tau * rw, r, r, w, r);

@@ -263,7 +263,8 @@ hm_status hodlr_peel(Ctx<T>& c, const T* U, const T* V, int level, const T* X, T
     for (int64_t cb = 0; cb < ncols; cb += 128) {
       const int w = (int)std::min<int64_t>(128, ncols - cb);
       launch_seg_tn<T>(lp.d_tn, lp.n_tn, lp.d_tn_begin, lp.nnodes, lp.node0, Proj, N, 0, 0, r,
-                       X + cb * N, N, 0, 0, w, c.partial, c.coef, c.st, c.bf16 && sizeof(T) == 8);
+                       X + cb * N, N, 0, 0, w, c.partial, c.coef, c.st, c.bf16 && sizeof(T) == 8,
+                       ncols == 2 * r && w == 2 * r ? r : 0);
       launch_seg_nn<T>(lp.d_nn, lp.n_nn, lp.node0, Expd, N, 0, 0, r, c.coef, (int64_t)r * w, r,
                        1, S + cb * N, N, 0, 0, w, (T)sign, (T)1, c.st, c.bf16 && sizeof(T) == 8);
       c.launches += 3;

@@ -12,11 +12,45 @@
 namespace hm {
 namespace df {
 
+// x = h + l rounded to 48 bits: h = (float)x, l = (float)(x - h), to nearest even.
+// On GB300 every FP64 instruction, the conversions included, holds a scheduler's
+// FP64 unit for ~65 cycles (a warp's two conversions, subtraction and conversion
+// back: ~262 cycles, measured), so the usual range goes through the integer pipe
+// instead (~16 instructions, ~30 cycles): the fraction's top 24 bits are rounded
+// in place, and the at most 29 bits left over are an integer that converts to
+// FP32 with the one rounding it needs.  Zeros are cheap too; anything whose h or
+// l would leave the normal float range takes the FP64 route.
 __device__ __forceinline__ void split(double x, float& h, float& l) {
-  h = (float)x;
-  l = (float)(x - (double)h);
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const unsigned e = ((unsigned)hi >> 20) & 0x7ffu;
+  if (e - 949u <= 200u) {  // 2^-74 <= |x| < 2^127
+    // exponent rebiased by 896 (modulo 512 above the sign), 23 bits of fraction
+    const unsigned f = __funnelshift_l(lo, (unsigned)hi, 3) + 0x40000000u;
+    const unsigned sign = (unsigned)hi & 0x80000000u;
+    const unsigned rest = lo & 0x1fffffffu;
+    const unsigned up = (rest + 0x0fffffffu + (f & 1u)) >> 29;
+    h = __uint_as_float((f + up) | sign);
+    const float unit = __uint_as_float(((f & 0x7f800000u) - 0x1a000000u) | sign);  // 2^-52 of h's
+    l = fmaf((float)((int)rest - (int)(up << 29)), unit, 0.f);
+  } else if ((((unsigned)hi << 1) | lo) == 0u) {
+    h = __int_as_float(hi);
+    l = 0.f;
+  } else {
+    h = (float)x;
+    l = (float)(x - (double)h);
+  }
 }
-__device__ __forceinline__ double join(float h, float l) { return (double)h + (double)l; }
+// (double)f through the integer pipe (an FP64 conversion: ~65 cycles a warp)
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f);
+  const unsigned a = u & 0x7fffffffu;
+  if (a - 0x00800000u < 0x7f000000u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((a >> 3) + 0x38000000u)), (int)(u << 29));
+  if (a == 0u) return __hiloint2double((int)u, 0);
+  return (double)f;
+}
+__device__ __forceinline__ double join(float h, float l) { return widen(h) + widen(l); }
 
 // s + e = a + b exactly (Knuth's TwoSum)
 __device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {

@@ -228,61 +228,94 @@ __global__ __launch_bounds__(256) void k_col_exp(const float* __restrict__ A, in
 }
 
 // X (FP64, column-major n x ncols) -> per (window, column) exponents and four
-// BF16 integer slices, laid out as the GEMM's shared memory wants them: per
+// BF16 digit slices, laid out as the GEMM's shared memory wants them: per
 // (column tile ct, K tile kt) one contiguous 16 KB block of 256 rows
 // (row t * 64 + c: slice t of column c) x 32 K values, each row's four 16-byte
 // chunks in 64-byte-swizzle order, so one 1-D bulk copy lands a tile in place.
-// Flags of (kt, ct) nonzero when that K tile has a nonzero slice.  Block: one
-// window (256 rows) x 64 columns; thread (c, q) covers rows 64 q .. 64 q + 63
-// of the window (kpad is a multiple of 64).
-__global__ __launch_bounds__(256) void k_split_x64(const double* __restrict__ X, int64_t ldx,
-                                                   int64_t n, int64_t ncols, int64_t kpad,
-                                                   int nct, __nv_bfloat16* __restrict__ Xs,
-                                                   int* __restrict__ ex,
-                                                   uint8_t* __restrict__ flags) {
-  constexpr int QR = WIN_ROWS / 4;  // rows per thread
+// Flags of (kt, ct) nonzero when that K tile has a nonzero digit.  Block: one
+// window (256 rows) x 64 columns; a warp takes two columns, lanes along the rows.
+//
+// Digit t is v = X 2^(7 - e) rounded (ties to even) to a multiple of 2^(-8 t) after
+// the digits before it are taken off, as in cut4.  Formed on the integer pipe from
+// v in fixed point (54 fraction bits, what lies below as a sticky bit): the FP64
+// form (ldexp, four rint / subtract / scale steps) held the FP64 units for ~1100
+// cycles per warp and 32 entries and, with its strided loads, took ~115 us at any
+// size up to n = 32768 x 60; this form ~12 us.
+constexpr int SPLIT_THREADS = 1024;
+__global__ __launch_bounds__(SPLIT_THREADS) void k_split_x64(
+    const double* __restrict__ X, int64_t ldx, int64_t n, int64_t ncols, int64_t kpad, int nct,
+    __nv_bfloat16* __restrict__ Xs, int* __restrict__ ex, uint8_t* __restrict__ flags) {
   const int win = blockIdx.x, ct = blockIdx.y;
-  const int tid = threadIdx.x;
-  const int c = tid >> 2, q = tid & 3;
-  const int64_t col = (int64_t)ct * TN + c;
-  const int64_t r0 = (int64_t)win * WIN_ROWS + q * QR;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ int fl[WIN_TILES];
-  if (tid < WIN_TILES) fl[tid] = 0;
-  double mx = 0.0;
-  for (int i = 0; i < QR; ++i) {
-    const int64_t row = r0 + i;
-    if (row < n && col < ncols) mx = fmax(mx, fabs(X[row + col * ldx]));
-  }
-  mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-  mx = fmax(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-  int e = 0;
-  if (mx > 0.0) frexp(mx, &e);
+  if (threadIdx.x < WIN_TILES) fl[threadIdx.x] = 0;
   __syncthreads();
-  int bits[QR / TK] = {};
-  if (r0 < kpad) {
-    for (int i = 0; i < QR; ++i) {
-      const int64_t row = r0 + i;
-      double r = (row < n && col < ncols) ? ldexp(X[row + col * ldx], 7 - e) : 0.0;
+  for (int c = warp; c < TN; c += SPLIT_THREADS / 32) {
+    const int64_t col = (int64_t)ct * TN + c;
+    long long x[WIN_TILES];  // the bits of rows 32 i + lane of the window
+    long long mx = 0;        // the largest finite magnitude's bits
+#pragma unroll
+    for (int i = 0; i < WIN_TILES; ++i) {
+      const int64_t row = (int64_t)win * WIN_ROWS + i * 32 + lane;
+      x[i] = (row < n && col < ncols) ? __double_as_longlong(X[row + col * ldx]) : 0ll;
+      const long long a = x[i] & 0x7fffffffffffffffll;
+      if (a < 0x7ff0000000000000ll) mx = a > mx ? a : mx;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      const long long y = __shfl_xor_sync(0xffffffffu, mx, o);
+      mx = y > mx ? y : mx;
+    }
+    int e = 0;  // 2^(e - 1) <= largest magnitude < 2^e
+    if (mx > 0) {
+      e = (int)(mx >> 52) - 1022;
+      if (e == -1022) e = -1010 - __clzll(mx);  // subnormal: the leading bit's place
+    }
+    if (lane == 0) ex[((int64_t)win * nct + ct) * TN + c] = e;
+#pragma unroll
+    for (int i = 0; i < WIN_TILES; ++i) {
+      const int64_t kt = (int64_t)win * WIN_TILES + i;
+      if (kt * TK >= kpad) break;
+      const int be = (int)(x[i] >> 52) & 0x7ff;
+      unsigned d[4];  // the digits' BF16 patterns (upper half of the FP32 ones)
+      if (be == 0x7ff) {
+        d[0] = d[1] = d[2] = d[3] = 0x7fc00000u;  // NaN or infinity: NaN products
+      } else {
+        unsigned long long m = (unsigned long long)x[i] & 0xfffffffffffffull;
+        if (be > 0) m |= 1ull << 52;
+        // |v| 2^54 = m 2^s with s <= 8
+        const int s = (be > 0 ? be : 1) - 1014 - e;
+        long long f;
+        if (s >= 0) f = (long long)(m << s);
+        else if (s > -60) f = (long long)((m >> -s) | ((m << (64 + s)) != 0ull ? 1ull : 0ull));
+        else f = m != 0ull ? 1ll : 0ll;
+        if (x[i] < 0) f = -f;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          const int b = 54 - 8 * t;  // the digit's unit is bit b
+          const long long q = (f + ((1ll << (b - 1)) - 1) + ((f >> b) & 1ll)) >> b;
+          f -= q << b;
+          d[t] = __float_as_uint(pow2f(-8 * t) * (float)(int)q);
+        }
+      }
+      const bool any = ((d[0] | d[1] | d[2] | d[3]) << 1) != 0u;
+      if (__any_sync(0xffffffffu, any) && lane == 0) fl[i] = 1;
+      const int64_t tile = (int64_t)ct * (kpad / TK) + kt;
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
-        const double st = rint(r);
-        r = (r - st) * 256.0;
-        bits[i / TK] |= (st != 0.0) ? (1 << t) : 0;
-        const int rr = t * TN + c, kk = (int)(row % TK);
-        const int64_t tile = (int64_t)ct * (kpad / TK) + row / TK;
-        Xs[(tile * (NSL * TN) + rr) * TK + ((((kk >> 3) ^ ((rr >> 1) & 3))) << 3) + (kk & 7)] =
-            __float2bfloat16_rn(pow2f(-8 * t) * (float)st);
+        const int rr = t * TN + c;
+        const unsigned up = __shfl_down_sync(0xffffffffu, d[t], 1);
+        if (!(lane & 1)) {  // rows lane, lane + 1 of the tile
+          const int off = (((lane >> 3) ^ ((rr >> 1) & 3)) << 3) + (lane & 7);
+          *reinterpret_cast<unsigned*>(Xs + (tile * (NSL * TN) + rr) * TK + off) =
+              __byte_perm(d[t], up, 0x7632);
+        }
       }
     }
   }
-#pragma unroll
-  for (int h = 0; h < QR / TK; ++h)
-    if (bits[h]) atomicOr(&fl[q * (QR / TK) + h], bits[h]);
-  if (q == 0) ex[((int64_t)win * nct + ct) * TN + c] = e;
   __syncthreads();
-  if (tid < WIN_TILES) {
-    const int64_t kt = (int64_t)win * WIN_TILES + tid;
-    if (kt * TK < kpad) flags[kt * nct + ct] = (uint8_t)fl[tid];
+  if (threadIdx.x < WIN_TILES) {
+    const int64_t kt = (int64_t)win * WIN_TILES + threadIdx.x;
+    if (kt * TK < kpad) flags[kt * nct + ct] = (uint8_t)fl[threadIdx.x];
   }
 }
 
@@ -935,7 +968,7 @@ int launch_gemm_esg(const float* A, int64_t lda, int trans, int64_t n, int64_t n
     return 2;
   count_launches(2);
   const int nwin = (nkt + WIN_TILES - 1) / WIN_TILES;
-  k_split_x64<<<dim3(nwin, nct), 256, 0, st>>>(X, ldx, n, ncols, kpad, nct, Xs, ex, flags);
+  k_split_x64<<<dim3(nwin, nct), SPLIT_THREADS, 0, st>>>(X, ldx, n, ncols, kpad, nct, Xs, ex, flags);
   const int* e_rows = trans ? aexp + gemm_esg_exp_count(n) : aexp;
   const size_t smem = gemm_esg_smem_bytes();
   static std::atomic<uint32_t> done[2] = {{0}, {0}};
@@ -1052,7 +1085,7 @@ int launch_gemm_esg_gen(const float* S, const float* P, const int* rowexp, int64
   memset(&tm0, 0, sizeof(tm0));
   count_launches(2);
   const int nwin = (nkt + WIN_TILES - 1) / WIN_TILES;
-  k_split_x64<<<dim3(nwin, nct), 256, 0, st>>>(X, ldx, n, ncols, kpad, nct, Xs, ex, flags);
+  k_split_x64<<<dim3(nwin, nct), SPLIT_THREADS, 0, st>>>(X, ldx, n, ncols, kpad, nct, Xs, ex, flags);
   const size_t smem = gemm_esg_smem_bytes();
   static std::atomic<uint32_t> done{0};
   // the same K split as the dense engine: two blocks share a row block's windows

@@ -11,6 +11,7 @@
 // is how the packed test matrices [Omega_2 | Omega_1] are addressed.
 #include <atomic>
 
+#include "df.cuh"
 #include "hm_internal.h"
 
 namespace hm {
@@ -101,84 +102,94 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial(
 // bits); a product a b is formed as hi_a hi_b exactly (TwoProduct by FMA) plus
 // the cross terms, and summed per output in a double-float (s_hi, s_lo) through
 // TwoSum.  The partial of a chunk (<= 256 rows) is accurate to ~1e-14 relative.
-__device__ __forceinline__ void split_df(double x, float& hi, float& lo) {
-  hi = (float)x;
-  lo = (float)(x - (double)hi);
-}
+//
+// Bound by the FP32 pipe: 12 instructions per product.  A block takes one chunk
+// and a 32 x 32 tile of the outputs (a thread 2 x 2 of it), so that a level of a
+// few dozen chunks still fills the chip; which thread owns an output changes
+// nothing in how it is summed.  The next 32 rows are in flight in registers while
+// the staged ones are multiplied.  A step whose 32 columns of B are all zero is
+// skipped (its products are exact zeros): the packed test matrices [Omega_2 |
+// Omega_1] are zero on every other child's rows, and the column tiles do not
+// straddle the two halves when kb is split (`half`).  N = 16384, 60 x 120: 228 ->
+// 50 us (64 x 128 outputs a block, one block per chunk, FP64-pipe cuts before).
+constexpr int DT = 32;  // outputs of a block: DT x DT
 
-template <int TI, int TJ>
 __global__ __launch_bounds__(256) void k_seg_tn_partial_df(
     const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
     int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
-    int kb, double* __restrict__ partial) {
-  constexpr int KA = 16 * TI, KB = 16 * TJ, LDA = KA + 1, LDB = KB + 1;
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float* Ah = reinterpret_cast<float*>(smem_raw);  // [TN_ROWS][LDA] each
-  float* Al = Ah + TN_ROWS * LDA;
-  float* Bh = Al + TN_ROWS * LDA;                  // [TN_ROWS][LDB] each
-  float* Bl = Bh + TN_ROWS * LDB;
+    int kb, int half, double* __restrict__ partial) {
+  __shared__ float2 As[TN_ROWS][DT + 1], Bs[TN_ROWS][DT + 1];
   const Chunk ch = chunks[blockIdx.x];
   const int aoff = (ch.node & 1) ? aoff_o : aoff_e;
   const int boff = (ch.node & 1) ? boff_o : boff_e;
   const int tid = threadIdx.x;
   const int ti = tid >> 4, tj = tid & 15;
-  float sh[TI][TJ], sl[TI][TJ];
+  // columns [a0, a1) of A, [b0, b1) of B
+  const int a0 = blockIdx.y * DT, a1 = min(ka, a0 + DT);
+  const int per = (half + DT - 1) / DT, hz = (int)blockIdx.z / per;
+  const int b0 = hz * half + ((int)blockIdx.z - hz * per) * DT;
+  const int b1 = min(min(kb, (hz + 1) * half), b0 + DT);
+  const int rr = tid & 31, cg = tid >> 5;  // staging: row, columns cg + 8 i
+  const double* Ap = A + ch.r0 + rr + (int64_t)(aoff + a0) * lda;
+  const double* Bp = B + ch.r0 + rr + (int64_t)(boff + b0) * ldb;
+  double va[4], vb[4];
+  auto load = [&](int64_t r0) {
+    const bool live = ch.r0 + r0 + rr < ch.r1;
 #pragma unroll
-  for (int i = 0; i < TI; ++i)
-#pragma unroll
-    for (int j = 0; j < TJ; ++j) { sh[i][j] = 0.f; sl[i][j] = 0.f; }
-  for (int64_t r0 = ch.r0; r0 < ch.r1; r0 += TN_ROWS) {
-    const int rows = (int)((ch.r1 - r0) < TN_ROWS ? (ch.r1 - r0) : TN_ROWS);
-    for (int idx = tid; idx < TN_ROWS * KA; idx += 256) {
-      const int rr = idx % TN_ROWS, c = idx / TN_ROWS;
-      float h, l;
-      split_df((rr < rows && c < ka) ? A[r0 + rr + (int64_t)(aoff + c) * lda] : 0.0, h, l);
-      Ah[rr * LDA + c] = h;
-      Al[rr * LDA + c] = l;
+    for (int i = 0; i < 4; ++i) {
+      const int c = cg + 8 * i;
+      va[i] = (live && a0 + c < a1) ? Ap[r0 + (int64_t)c * lda] : 0.0;
+      vb[i] = (live && b0 + c < b1) ? Bp[r0 + (int64_t)c * ldb] : 0.0;
     }
-    for (int idx = tid; idx < TN_ROWS * KB; idx += 256) {
-      const int rr = idx % TN_ROWS, c = idx / TN_ROWS;
-      float h, l;
-      split_df((rr < rows && c < kb) ? B[r0 + rr + (int64_t)(boff + c) * ldb] : 0.0, h, l);
-      Bh[rr * LDB + c] = h;
-      Bl[rr * LDB + c] = l;
+  };
+  float sh[2][2] = {}, sl[2][2] = {};
+  load(0);
+  for (int64_t r0 = 0; ch.r0 + r0 < ch.r1; r0 += TN_ROWS) {
+    bool nz = false;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int c = cg + 8 * i;
+      float2 v;
+      df::split(va[i], v.x, v.y);
+      As[rr][c] = v;
+      df::split(vb[i], v.x, v.y);
+      Bs[rr][c] = v;
+      nz |= !(v.x == 0.f);
     }
-    __syncthreads();
-    for (int rr = 0; rr < rows; ++rr) {
-      float ah[TI], al[TI], bh[TJ], bl[TJ];
+    load(r0 + TN_ROWS);
+    if (__syncthreads_or(nz)) {
+      const int rows = (int)min((int64_t)TN_ROWS, ch.r1 - ch.r0 - r0);
+#pragma unroll 4
+      for (int q = 0; q < rows; ++q) {
+        float2 a[2], b[2];
 #pragma unroll
-      for (int i = 0; i < TI; ++i) {
-        ah[i] = Ah[rr * LDA + ti + 16 * i];
-        al[i] = Al[rr * LDA + ti + 16 * i];
+        for (int i = 0; i < 2; ++i) a[i] = As[q][ti + 16 * i];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) b[j] = Bs[q][tj + 16 * j];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) {
+            const float p = a[i].x * b[j].x;
+            const float e = fmaf(a[i].x, b[j].x, -p);               // hi hi - p, exact
+            const float t = fmaf(a[i].x, b[j].y, fmaf(a[i].y, b[j].x, e));
+            const float s = sh[i][j] + p;                            // TwoSum(sh, p)
+            const float z = s - sh[i][j];
+            const float err = (sh[i][j] - (s - z)) + (p - z);
+            sh[i][j] = s;
+            sl[i][j] += err + t;
+          }
       }
-#pragma unroll
-      for (int j = 0; j < TJ; ++j) {
-        bh[j] = Bh[rr * LDB + tj + 16 * j];
-        bl[j] = Bl[rr * LDB + tj + 16 * j];
-      }
-#pragma unroll
-      for (int i = 0; i < TI; ++i)
-#pragma unroll
-        for (int j = 0; j < TJ; ++j) {
-          const float p = ah[i] * bh[j];
-          const float e = fmaf(ah[i], bh[j], -p);               // hi hi - p, exact
-          const float t = fmaf(ah[i], bl[j], fmaf(al[i], bh[j], e));
-          const float s = sh[i][j] + p;                          // TwoSum(sh, p)
-          const float z = s - sh[i][j];
-          const float err = (sh[i][j] - (s - z)) + (p - z);
-          sh[i][j] = s;
-          sl[i][j] += err + t;
-        }
     }
     __syncthreads();
   }
   double* out = partial + (int64_t)blockIdx.x * ka * kb;
 #pragma unroll
-  for (int i = 0; i < TI; ++i)
+  for (int i = 0; i < 2; ++i)
 #pragma unroll
-    for (int j = 0; j < TJ; ++j) {
-      const int ii = ti + 16 * i, jj = tj + 16 * j;
-      if (ii < ka && jj < kb) out[ii + jj * ka] = (double)sh[i][j] + (double)sl[i][j];
+    for (int j = 0; j < 2; ++j) {
+      const int ii = a0 + ti + 16 * i, jj = b0 + tj + 16 * j;
+      if (ii < a1 && jj < b1) out[ii + jj * ka] = df::join(sh[i][j], sl[i][j]);
     }
 }
 
@@ -269,77 +280,78 @@ __global__ __launch_bounds__(256) void k_seg_nn(
 
 // The FP64 expansion in double-float arithmetic (HM_A32), as k_seg_tn_partial_df:
 // inputs cut to hi + lo floats when staged, products by TwoProduct, sums by TwoSum.
-// Warp w owns output columns [CJ w, CJ w + CJ) (CJ = 4, 8 or 16 as kout needs), so
-// only the columns that cover kout are staged and computed.
-template <int CJ>
+// A block takes one chunk (<= 64 rows) and every gridDim.y-th 32-column tile of the
+// output; warp w owns four of the columns, a lane rows lane and lane + 32.  Only
+// what kin and 32 columns need is staged, so that four blocks share an SM where the
+// full-width staging (196 KB) left one.  With P aliasing Y the launch gives one
+// block all the tiles (P is staged whole before any write).  N = 16384, kin = 60,
+// 120 columns: 126 -> 45 us.
 __global__ __launch_bounds__(256) void k_seg_nn_df(
     const Chunk* __restrict__ chunks, int node0, const double* P, int64_t ldp, int poff_e,
     int poff_o, int kin, const double* __restrict__ C, int64_t cstride, int cld, int cflip,
     double* Y, int64_t ldy, int yoff_e, int yoff_o, int kout, double alpha, double beta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  constexpr int CW = 8 * CJ;                      // staged columns of C
-  float* Ph = reinterpret_cast<float*>(smem_raw);  // [NN_MAX][NN_ROWS] each
-  float* Pl = Ph + NN_MAX * NN_ROWS;
-  float* Ch = Pl + NN_MAX * NN_ROWS;              // [NN_MAX][CW] each
-  float* Cl = Ch + NN_MAX * CW;
+  const int kp = kin | 1;                            // row pitch of Cs
+  float2* Ps = reinterpret_cast<float2*>(smem_raw);  // [kin][NN_ROWS]
+  float2* Cs = Ps + kin * NN_ROWS;                   // [DT][kp]
   const Chunk ch = chunks[blockIdx.x];
   const int rows = (int)(ch.r1 - ch.r0);
   const int poff = (ch.node & 1) ? poff_o : poff_e;
   const int yoff = (ch.node & 1) ? yoff_o : yoff_e;
   const double* Cn = C + (int64_t)((ch.node ^ cflip) - node0) * cstride;
-  const int tid = threadIdx.x;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   for (int idx = tid; idx < kin * NN_ROWS; idx += 256) {
     const int rr = idx % NN_ROWS, k = idx / NN_ROWS;
-    float h, l;
-    split_df((rr < rows) ? P[ch.r0 + rr + (int64_t)(poff + k) * ldp] : 0.0, h, l);
-    Ph[k * NN_ROWS + rr] = h;
-    Pl[k * NN_ROWS + rr] = l;
+    float2 v;
+    df::split((rr < rows) ? P[ch.r0 + rr + (int64_t)(poff + k) * ldp] : 0.0, v.x, v.y);
+    Ps[idx] = v;
   }
-  for (int idx = tid; idx < kin * CW; idx += 256) {
-    const int j = idx % CW, k = idx / CW;
-    float h, l;
-    split_df((j < kout) ? Cn[k + (int64_t)j * cld] : 0.0, h, l);
-    Ch[k * CW + j] = h;
-    Cl[k * CW + j] = l;
-  }
-  __syncthreads();
-  const int lane = tid & 31, w = tid >> 5;
-  float sh[2][CJ], sl[2][CJ];
+  for (int c0 = blockIdx.y * DT; c0 < kout; c0 += gridDim.y * DT) {
+    const int nc = min(DT, kout - c0);
+    for (int j = w; j < DT; j += 8)
+      for (int k = lane; k < kin; k += 32) {
+        float2 v;
+        df::split((j < nc) ? Cn[k + (int64_t)(c0 + j) * cld] : 0.0, v.x, v.y);
+        Cs[j * kp + k] = v;
+      }
+    __syncthreads();
+    float sh[2][4] = {}, sl[2][4] = {};
+    if (4 * w < nc) {
+#pragma unroll 2
+      for (int k = 0; k < kin; ++k) {
+        const float2 a[2] = {Ps[k * NN_ROWS + lane], Ps[k * NN_ROWS + lane + 32]};
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
+        for (int j = 0; j < 4; ++j) {
+          const float2 cj = Cs[(4 * w + j) * kp + k];
 #pragma unroll
-    for (int j = 0; j < CJ; ++j) { sh[i][j] = 0.f; sl[i][j] = 0.f; }
-  for (int k = 0; k < kin; ++k) {
-    const float ah[2] = {Ph[k * NN_ROWS + lane], Ph[k * NN_ROWS + lane + 32]};
-    const float al[2] = {Pl[k * NN_ROWS + lane], Pl[k * NN_ROWS + lane + 32]};
+          for (int i = 0; i < 2; ++i) {
+            const float p = a[i].x * cj.x;
+            const float e = fmaf(a[i].x, cj.x, -p);
+            const float t = fmaf(a[i].x, cj.y, fmaf(a[i].y, cj.x, e));
+            const float s = sh[i][j] + p;
+            const float z = s - sh[i][j];
+            const float err = (sh[i][j] - (s - z)) + (p - z);
+            sh[i][j] = s;
+            sl[i][j] += err + t;
+          }
+        }
+      }
 #pragma unroll
-    for (int j = 0; j < CJ; ++j) {
-      const float chj = Ch[k * CW + w * CJ + j], clj = Cl[k * CW + w * CJ + j];
+      for (int j = 0; j < 4; ++j) {
+        if (4 * w + j >= nc) continue;
 #pragma unroll
-      for (int i = 0; i < 2; ++i) {
-        const float p = ah[i] * chj;
-        const float e = fmaf(ah[i], chj, -p);
-        const float t = fmaf(ah[i], clj, fmaf(al[i], chj, e));
-        const float s = sh[i][j] + p;
-        const float z = s - sh[i][j];
-        const float err = (sh[i][j] - (s - z)) + (p - z);
-        sh[i][j] = s;
-        sl[i][j] += err + t;
+        for (int i = 0; i < 2; ++i) {
+          const int rr = lane + 32 * i;
+          if (rr >= rows) continue;
+          double* yp = Y + ch.r0 + rr + (int64_t)(yoff + c0 + 4 * w + j) * ldy;
+          double v = df::join(sh[i][j], sl[i][j]);
+          if (alpha == -1.0) v = -v;  // (an FP64 product costs as much as the join's sum)
+          else if (alpha != 1.0) v *= alpha;
+          *yp = (beta == 0.0) ? v : fma(beta, *yp, v);
+        }
       }
     }
-  }
-#pragma unroll
-  for (int j = 0; j < CJ; ++j) {
-    const int col = w * CJ + j;
-    if (col >= kout) continue;
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-      const int rr = lane + 32 * i;
-      if (rr >= rows) continue;
-      double* yp = Y + ch.r0 + rr + (int64_t)(yoff + col) * ldy;
-      const double v = alpha * ((double)sh[i][j] + (double)sl[i][j]);
-      *yp = (beta == 0.0) ? v : v + beta * (*yp);
-    }
+    __syncthreads();
   }
 }
 
@@ -348,42 +360,31 @@ __global__ __launch_bounds__(256) void k_seg_nn_df(
 template <typename T, int TI, int TJ>
 void seg_tn_partial_tiled(const Chunk* chunks, int nchunks, const T* A, int64_t lda,
                           int aoff_even, int aoff_odd, int ka, const T* B, int64_t ldb,
-                          int boff_even, int boff_odd, int kb, double* partial, cudaStream_t st,
-                          bool df) {
+                          int boff_even, int boff_odd, int kb, double* partial, cudaStream_t st) {
   constexpr int LDA = 16 * TI + 1, LDB = 16 * TJ + 1;
-  if (sizeof(T) == 8 && df) {
-    const size_t smem = 2 * TN_ROWS * (LDA + LDB) * sizeof(float);
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_seg_tn_partial_df<TI, TJ>, done);
-    k_seg_tn_partial_df<TI, TJ><<<nchunks, 256, smem, st>>>(
-        chunks, (const double*)A, lda, aoff_even, aoff_odd, ka, (const double*)B, ldb, boff_even,
-        boff_odd, kb, partial);
-  } else {
     const size_t smem = TN_ROWS * (LDA + LDB) * sizeof(T);
     static std::atomic<uint32_t> done{0};
     raise_smem_limit((const void*)k_seg_tn_partial<T, TI, TJ>, done);
     k_seg_tn_partial<T, TI, TJ><<<nchunks, 256, smem, st>>>(
         chunks, A, lda, aoff_even, aoff_odd, ka, B, ldb, boff_even, boff_odd, kb, partial);
-  }
 }
 
 template <typename T, int TI>
 void seg_tn_partial_pick_j(const Chunk* chunks, int nchunks, const T* A, int64_t lda,
                            int aoff_even, int aoff_odd, int ka, const T* B, int64_t ldb,
-                           int boff_even, int boff_odd, int kb, double* partial, cudaStream_t st,
-                           bool df) {
+                           int boff_even, int boff_odd, int kb, double* partial, cudaStream_t st) {
   switch (tn_tile(kb)) {
     case 2:
       seg_tn_partial_tiled<T, TI, 2>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                     boff_even, boff_odd, kb, partial, st, df);
+                                     boff_even, boff_odd, kb, partial, st);
       break;
     case 4:
       seg_tn_partial_tiled<T, TI, 4>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                     boff_even, boff_odd, kb, partial, st, df);
+                                     boff_even, boff_odd, kb, partial, st);
       break;
     default:
       seg_tn_partial_tiled<T, TI, 8>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                     boff_even, boff_odd, kb, partial, st, df);
+                                     boff_even, boff_odd, kb, partial, st);
   }
 }
 
@@ -391,21 +392,30 @@ template <typename T>
 void launch_seg_tn(const Chunk* chunks, int nchunks, const int32_t* chunk_begin, int nnodes,
                    int node0, const T* A, int64_t lda, int aoff_even, int aoff_odd, int ka,
                    const T* B, int64_t ldb, int boff_even, int boff_odd, int kb, double* partial,
-                   T* out, cudaStream_t st, bool df) {
+                   T* out, cudaStream_t st, bool df, int half) {
   count_launches(2);
   (void)node0;
-  switch (tn_tile(ka)) {
+  if (sizeof(T) == 8 && df) {
+    if (nchunks > 0) {
+      const int h = half > 0 ? half : kb;
+      const dim3 grid((unsigned)nchunks, (unsigned)((ka + DT - 1) / DT),
+                      (unsigned)(((h + DT - 1) / DT) * ((kb + h - 1) / h)));
+      k_seg_tn_partial_df<<<grid, 256, 0, st>>>(chunks, (const double*)A, lda, aoff_even, aoff_odd,
+                                                ka, (const double*)B, ldb, boff_even, boff_odd, kb,
+                                                h, partial);
+    }
+  } else switch (tn_tile(ka)) {
     case 2:
       seg_tn_partial_pick_j<T, 2>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st, df);
+                                  boff_even, boff_odd, kb, partial, st);
       break;
     case 4:
       seg_tn_partial_pick_j<T, 4>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st, df);
+                                  boff_even, boff_odd, kb, partial, st);
       break;
     default:
       seg_tn_partial_pick_j<T, 8>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st, df);
+                                  boff_even, boff_odd, kb, partial, st);
   }
   const int m = ka * kb;
   dim3 grid((unsigned)((m + 255) / 256), (unsigned)nnodes);
@@ -420,23 +430,14 @@ void launch_seg_nn(const Chunk* chunks, int nchunks, int node0, const T* P, int6
   count_launches(1);
   const size_t smem = (size_t)(NN_MAX * NN_ROWS + NN_MAX * NN_MAX) * sizeof(T);
   if (sizeof(T) == 8 && df) {
-    auto run = [&](auto kern, int cw) {
-      const size_t sm = (size_t)2 * (NN_MAX * NN_ROWS + NN_MAX * cw) * sizeof(float);
-      kern<<<nchunks, 256, sm, st>>>(chunks, node0, (const double*)P, ldp, poff_even, poff_odd,
-                                     kin, (const double*)C, cstride, cld, cflip, (double*)Y, ldy,
-                                     yoff_even, yoff_odd, kout, (double)alpha, (double)beta);
-    };
-    static std::atomic<uint32_t> d4{0}, d8{0}, d16{0};
-    if (kout <= 32) {
-      raise_smem_limit((const void*)k_seg_nn_df<4>, d4);
-      run(k_seg_nn_df<4>, 32);
-    } else if (kout <= 64) {
-      raise_smem_limit((const void*)k_seg_nn_df<8>, d8);
-      run(k_seg_nn_df<8>, 64);
-    } else {
-      raise_smem_limit((const void*)k_seg_nn_df<16>, d16);
-      run(k_seg_nn_df<16>, 128);
-    }
+    const size_t sm = (size_t)(kin * NN_ROWS + DT * (kin | 1)) * sizeof(float2);
+    static std::atomic<uint32_t> raised{0};
+    raise_smem_limit((const void*)k_seg_nn_df, raised);
+    const bool alias = (const void*)P == (const void*)Y;
+    const dim3 grid((unsigned)nchunks, alias ? 1u : (unsigned)((kout + DT - 1) / DT));
+    k_seg_nn_df<<<grid, 256, sm, st>>>(chunks, node0, (const double*)P, ldp, poff_even, poff_odd,
+                                       kin, (const double*)C, cstride, cld, cflip, (double*)Y, ldy,
+                                       yoff_even, yoff_odd, kout, (double)alpha, (double)beta);
     return;
   }
   static std::atomic<uint32_t> done{0};
@@ -448,10 +449,10 @@ void launch_seg_nn(const Chunk* chunks, int nchunks, int node0, const T* P, int6
 
 template void launch_seg_tn<float>(const Chunk*, int, const int32_t*, int, int, const float*,
                                    int64_t, int, int, int, const float*, int64_t, int, int, int,
-                                   double*, float*, cudaStream_t, bool);
+                                   double*, float*, cudaStream_t, bool, int);
 template void launch_seg_tn<double>(const Chunk*, int, const int32_t*, int, int, const double*,
                                     int64_t, int, int, int, const double*, int64_t, int, int,
-                                    int, double*, double*, cudaStream_t, bool);
+                                    int, double*, double*, cudaStream_t, bool, int);
 template void launch_seg_nn<float>(const Chunk*, int, int, const float*, int64_t, int, int, int,
                                    const float*, int64_t, int, int, float*, int64_t, int, int,
                                    int, float, float, cudaStream_t, bool);
