@@ -7,9 +7,14 @@
 // (K-tile, column-tile) blocks of X and the GEMM skips them: the work and the
 // A bytes read follow the nonzero structure of X.
 //
-// This is the CUDA-core form: 128 x 64 output tile per block of 256 threads,
-// 8 x 4 register tile per thread.  In FP32 every K-tile is accumulated in a
-// fresh register tile and added to the running sum with Kahan compensation.
+// These are the CUDA-core forms: FP32 (128 x 64 output tile per block of 256
+// threads, 8 x 4 register tile per thread; every K-tile is accumulated in a fresh
+// register tile and added to the running sum with Kahan compensation) and FP64
+// sums over an FP64 or an FP32 operator (k_dense_gemm64).
+#include <algorithm>
+#include <cooperative_groups.h>
+
+#include "df.cuh"
 #include "hm_internal.h"
 
 namespace hm {
@@ -18,19 +23,17 @@ namespace {
 constexpr int BM = 128;
 constexpr int BN = 64;
 
-template <typename T> struct KTile { static constexpr int BK = 32; };
-template <> struct KTile<double> { static constexpr int BK = 16; };
+constexpr int BK = 32;
 
-// flags[kt * nct + ct] = 1 iff X(kt*BK .. , ct*BN ..) has a nonzero entry.
-template <typename T>
+// flags[kt * nct + ct] = 1 iff X(kt*BK .. , ct*CN ..) has a nonzero entry.
+template <typename T, int CN>
 __global__ void k_tile_flags(const T* __restrict__ X, int64_t ldx, int64_t n, int64_t ncols,
                              uint8_t* __restrict__ flags, int nct) {
-  constexpr int BK = KTile<T>::BK;
   const int kt = blockIdx.x, ct = blockIdx.y;
   bool nz = false;
-  for (int idx = threadIdx.x; idx < BK * BN; idx += blockDim.x) {
+  for (int idx = threadIdx.x; idx < BK * CN; idx += blockDim.x) {
     const int k = idx % BK, c = idx / BK;
-    const int64_t row = (int64_t)kt * BK + k, col = (int64_t)ct * BN + c;
+    const int64_t row = (int64_t)kt * BK + k, col = (int64_t)ct * CN + c;
     if (row < n && col < ncols) nz |= (X[row + col * ldx] != (T)0);
   }
   nz = __syncthreads_or(nz);
@@ -43,7 +46,6 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
                                                     const T* __restrict__ X, int64_t ldx,
                                                     T* __restrict__ Y, int64_t ldy,
                                                     const uint8_t* __restrict__ flags, int nct) {
-  constexpr int BK = KTile<T>::BK;
   __shared__ __align__(16) T As[BK][BM + 4];
   __shared__ __align__(16) T Xs[BK][BN + 4];
   const int64_t m0 = (int64_t)blockIdx.x * BM;
@@ -101,19 +103,15 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
 #pragma unroll
         for (int j = 0; j < 4; ++j) tmp[i][j] = fma(a[i], x[j], tmp[i][j]);
     }
-    // running sum: compensated in FP32, plain in FP64
+    // compensated running sum
 #pragma unroll
     for (int i = 0; i < 8; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        if (sizeof(T) == 4) {
-          const T y = tmp[i][j] - cmp[i][j];
-          const T t = acc[i][j] + y;
-          cmp[i][j] = (t - acc[i][j]) - y;
-          acc[i][j] = t;
-        } else {
-          acc[i][j] += tmp[i][j];
-        }
+        const T y = tmp[i][j] - cmp[i][j];
+        const T t = acc[i][j] + y;
+        cmp[i][j] = (t - acc[i][j]) - y;
+        acc[i][j] = t;
       }
     __syncthreads();
   }
@@ -129,119 +127,141 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
   }
 }
 
-// FP32 operator, FP64 samples: every product a * x is formed and summed in FP64
-// (an FP32 value converts to FP64 exactly).
-template <int TRANS>
-__global__ __launch_bounds__(256) void k_dense_gemm_a32(const float* __restrict__ A, int64_t lda,
-                                                        int64_t n, int64_t ncols,
-                                                        const double* __restrict__ X, int64_t ldx,
-                                                        double* __restrict__ Y, int64_t ldy,
-                                                        const uint8_t* __restrict__ flags,
-                                                        int nct) {
-  constexpr int BK = 16;
-  __shared__ __align__(16) double As[BK][BM + 2];
-  __shared__ __align__(16) double Xs[BK][BN + 2];
-  const int64_t m0 = (int64_t)blockIdx.x * BM;
-  const int ct = blockIdx.y;
-  const int64_t c0 = (int64_t)ct * BN;
-  const int tid = threadIdx.x;
-  const int rg = tid >> 4, cg = tid & 15;
-  double acc[8][4];
-#pragma unroll
-  for (int i = 0; i < 8; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+// FP64 samples with an FP64 operator, or an FP32 one (an FP32 value is an FP64 value;
+// widened on the integer pipe): every product formed and summed in FP64.
+//
+// Bound by the FP64 pipe (64 cycles per warp FMA and scheduler), so the aim is FMAs
+// on every scheduler and none for padding: a block of four warps takes 32 rows
+// (lanes) x 32 columns (warp w: columns w, w + 4, ..), only columns that exist are
+// multiplied, and where the row blocks alone would not fill the chip a cluster of S
+// blocks shares a tile's active K tiles (dealt out in turn) and sums its shares over
+// distributed shared memory in rank order (deterministic, no workspace).  N = 1024,
+// 20 columns, half of K active: 1200 us as 8 blocks of 128 x 64 outputs, 24 us so.
+template <typename TA, int TRANS>
+__global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, int64_t lda,
+                                                      int64_t n, int64_t ncols,
+                                                      const double* __restrict__ X, int64_t ldx,
+                                                      double* __restrict__ Y, int64_t ldy,
+                                                      const uint8_t* __restrict__ flags,
+                                                      int nct, int S) {
+  __shared__ double As[32][33];  // [k][row] (TRANS) or [row][k]
+  __shared__ double Xs[32][33];  // [column][k], later the sums [column][row]
+  const int64_t m0 = (int64_t)blockIdx.x * 32;
+  const int part = blockIdx.y, ct = blockIdx.z;
+  const int64_t c0 = (int64_t)ct * 32;
+  const int nc = (int)min((int64_t)32, ncols - c0);
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int nq = w < nc ? (nc - w + 3) / 4 : 0;  // this warp's columns
+  double acc[8] = {};
   const int nkt = (int)((n + BK - 1) / BK);
+  int turn = 0;
   for (int kt = 0; kt < nkt; ++kt) {
-    if (flags && !flags[(int64_t)kt * nct + ct]) continue;
+    if (flags && !flags[(int64_t)kt * nct + ct]) continue;  // uniform over the cluster
+    const bool mine = turn == part;
+    turn = turn + 1 == S ? 0 : turn + 1;
+    if (!mine) continue;
     const int64_t k0 = (int64_t)kt * BK;
-    if (!TRANS) {
-      for (int idx = tid; idx < BM * BK; idx += 256) {
-        const int k = idx % BK, m = idx / BK;
-        const int64_t row = m0 + m, col = k0 + k;
-        As[k][m] = (row < n && col < n) ? (double)A[row * lda + col] : 0.0;
-      }
-    } else {
-      for (int idx = tid; idx < BM * BK; idx += 256) {
-        const int m = idx % BM, k = idx / BM;
-        const int64_t row = k0 + k, col = m0 + m;
-        As[k][m] = (row < n && col < n) ? (double)A[row * lda + col] : 0.0;
-      }
-    }
-    for (int idx = tid; idx < BK * BN; idx += 256) {
-      const int k = idx % BK, c = idx / BK;
-      const int64_t row = k0 + k, col = c0 + c;
-      Xs[k][c] = (row < n && col < ncols) ? X[row + col * ldx] : 0.0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      // lanes along the contiguous index of A: k, or the row of op(A)
+      const int r = w + 4 * i;
+      const int64_t row = TRANS ? k0 + r : m0 + r, col = (TRANS ? m0 : k0) + lane;
+      const TA a = (row < n && col < n) ? A[row * lda + col] : (TA)0;
+      if constexpr (sizeof(TA) == 8) As[r][lane] = a;
+      else As[r][lane] = df::widen(a);
+      if (r < nc) Xs[r][lane] = (k0 + lane < n) ? X[k0 + lane + (c0 + r) * ldx] : 0.0;
     }
     __syncthreads();
 #pragma unroll 4
-    for (int kk = 0; kk < BK; ++kk) {
-      double a[8], x[4];
+    for (int k = 0; k < BK; ++k) {
+      const double a = TRANS ? As[k][lane] : As[lane][k];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = As[kk][rg * 8 + i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) x[j] = Xs[kk][cg * 4 + j];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], x[j], acc[i][j]);
+      for (int q = 0; q < 8; ++q)
+        if (q < nq) acc[q] = fma(a, Xs[w + 4 * q][k], acc[q]);
     }
     __syncthreads();
   }
-#pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int64_t col = c0 + cg * 4 + j;
-    if (col >= ncols) continue;
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int64_t row = m0 + rg * 8 + i;
-      if (row < n) Y[row + col * ldy] = acc[i][j];
-    }
+  if (S == 1) {
+    if (m0 + lane < n)
+      for (int q = 0; q < 8; ++q)
+        if (q < nq) Y[m0 + lane + (c0 + w + 4 * q) * ldy] = acc[q];
+    return;
   }
+#pragma unroll
+  for (int q = 0; q < 8; ++q)
+    if (q < nq) Xs[w + 4 * q][lane] = acc[q];
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.sync();
+  for (int c = part + S * w; c < nc; c += 4 * S) {
+    double s = 0.0;
+    for (int p = 0; p < S; ++p) s += cl.map_shared_rank(&Xs[c][lane], p)[0];
+    if (m0 + lane < n) Y[m0 + lane + (c0 + c) * ldy] = s;
+  }
+  cl.sync();  // no block leaves while another may still read its sums
 }
 
 }  // namespace
 
+// The FP64 GEMM with its cluster size: doubled while the blocks are fewer than three
+// per SM (152 SMs) and there is a K tile for each (N = 1024 x 20: 8 blocks a tile;
+// from N ~ 15000 on: 1).
+template <typename TA>
+static void dense_gemm64(const TA* A, int64_t lda, int trans, int64_t n, int64_t ncols,
+                         const double* X, int64_t ldx, double* Y, int64_t ldy, uint8_t* flags,
+                         cudaStream_t st) {
+  count_launches(flags ? 2 : 1);
+  const int nct = (int)((ncols + 31) / 32), nkt = (int)((n + BK - 1) / BK);
+  if (flags) k_tile_flags<double, 32><<<dim3(nkt, nct), 256, 0, st>>>(X, ldx, n, ncols, flags, nct);
+  const int64_t rows = (n + 31) / 32;
+  int S = 1;
+  while (S < 8 && rows * nct * S < 456 && 2 * S <= nkt) S *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)rows, (unsigned)S, (unsigned)nct);
+  cfg.blockDim = dim3(128);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 1;
+  at[0].val.clusterDim.y = (unsigned)S;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const uint8_t* fl = flags;
+  if (trans)
+    cudaLaunchKernelEx(&cfg, k_dense_gemm64<TA, 1>, A, lda, n, ncols, X, ldx, Y, ldy, fl, nct, S);
+  else
+    cudaLaunchKernelEx(&cfg, k_dense_gemm64<TA, 0>, A, lda, n, ncols, X, ldx, Y, ldy, fl, nct, S);
+}
+
 void launch_dense_gemm_a32(const float* A, int64_t lda, int trans, int64_t n, int64_t ncols,
                            const double* X, int64_t ldx, double* Y, int64_t ldy, uint8_t* flags,
                            cudaStream_t st) {
-  count_launches(flags ? 2 : 1);
-  constexpr int BK = 16;
-  const int nct = (int)((ncols + BN - 1) / BN);
-  const int nkt = (int)((n + BK - 1) / BK);
-  if (flags) {
-    dim3 gf(nkt, nct);
-    k_tile_flags<double><<<gf, 256, 0, st>>>(X, ldx, n, ncols, flags, nct);
-  }
-  dim3 grid((unsigned)((n + BM - 1) / BM), (unsigned)nct);
-  if (trans)
-    k_dense_gemm_a32<1><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
-  else
-    k_dense_gemm_a32<0><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
+  dense_gemm64<float>(A, lda, trans, n, ncols, X, ldx, Y, ldy, flags, st);
 }
 
 template <typename T>
 void launch_dense_gemm(const T* A, int64_t lda, int trans, int64_t n, int64_t ncols, const T* X,
                        int64_t ldx, T* Y, int64_t ldy, uint8_t* flags, cudaStream_t st) {
-  count_launches(flags ? 2 : 1);
-  constexpr int BK = KTile<T>::BK;
-  const int nct = (int)((ncols + BN - 1) / BN);
-  const int nkt = (int)((n + BK - 1) / BK);
-  if (flags) {
-    dim3 gf(nkt, nct);
-    k_tile_flags<T><<<gf, 256, 0, st>>>(X, ldx, n, ncols, flags, nct);
+  if constexpr (sizeof(T) == 8) {
+    dense_gemm64<double>(A, lda, trans, n, ncols, X, ldx, Y, ldy, flags, st);
+  } else {
+    count_launches(flags ? 2 : 1);
+    const int nct = (int)((ncols + BN - 1) / BN);
+    const int nkt = (int)((n + BK - 1) / BK);
+    if (flags)
+      k_tile_flags<T, BN><<<dim3(nkt, nct), 256, 0, st>>>(X, ldx, n, ncols, flags, nct);
+    dim3 grid((unsigned)((n + BM - 1) / BM), (unsigned)nct);
+    if (trans)
+      k_dense_gemm<T, 1><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
+    else
+      k_dense_gemm<T, 0><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
   }
-  dim3 grid((unsigned)((n + BM - 1) / BM), (unsigned)nct);
-  if (trans)
-    k_dense_gemm<T, 1><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
-  else
-    k_dense_gemm<T, 0><<<grid, 256, 0, st>>>(A, lda, n, ncols, X, ldx, Y, ldy, flags, nct);
 }
 
 int64_t dense_flags_bytes(int64_t n, int64_t ncols, int is_double) {
   (void)is_double;
-  const int BK = 16;  // the smallest K tile of any variant
-  return ((n + BK - 1) / BK) * ((ncols + BN - 1) / BN);
+  // the smallest K tile and column tile of any variant
+  return ((n + 15) / 16) * ((ncols + 31) / 32);
 }
 
 template void launch_dense_gemm<float>(const float*, int64_t, int, int64_t, int64_t,

@@ -9,6 +9,7 @@
 // A node's rows are split into chunks; uneven node sizes go into one launch.
 // Column offsets can depend on the node's parity (left child / right child), which
 // is how the packed test matrices [Omega_2 | Omega_1] are addressed.
+#include <algorithm>
 #include <atomic>
 
 #include "df.cuh"
@@ -27,7 +28,7 @@ constexpr int TN_MAX = 128;   // max ka, kb
 // Which thread owns an output changes nothing in how it is summed.
 constexpr int tn_tile(int k) { return k <= 32 ? 2 : (k <= 64 ? 4 : 8); }
 
-// Partial products of one chunk (<= 256 rows).
+// FP32 partial products of one chunk (<= 256 rows).
 template <typename T, int TI, int TJ>
 __global__ __launch_bounds__(256) void k_seg_tn_partial(
     const Chunk* __restrict__ chunks, const T* __restrict__ A, int64_t lda, int aoff_e,
@@ -94,6 +95,60 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial(
       const int ii = ti + 16 * i, jj = tj + 16 * j;
       if (ii < ka && jj < kb) out[ii + jj * ka] = acc[i][j];
     }
+}
+
+// FP64 partial products of one chunk.  Bound by the FP64 pipe (a warp's FMA holds a
+// scheduler's FP64 unit for 64 cycles on GB300), so what counts is that every
+// scheduler has FMAs to issue and that none is issued for padding: the ka x kb
+// outputs of a chunk are dealt out flat, M to a thread and 128 M to a block (a
+// grid of output tiles would idle lanes at every edge, and one block per chunk
+// left most of the chip idle: 128 chunks x 60 x 37 at N = 16384 took 278 us, this
+// 92; 16 chunks x 20 x 40 at N = 1024 141 us, this 9).
+template <int M>
+__global__ __launch_bounds__(128) void k_seg_tn_partial64(
+    const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
+    int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
+    int kb, double* __restrict__ partial) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const Chunk ch = chunks[blockIdx.x];
+  const int aoff = (ch.node & 1) ? aoff_o : aoff_e;
+  const int boff = (ch.node & 1) ? boff_o : boff_e;
+  const int tid = threadIdx.x, mtot = ka * kb, e0 = blockIdx.y * 128 * M;
+  // the columns of B that outputs e0 .. need
+  const int jlo = e0 / ka, nb = (min(e0 + 128 * M, mtot) - 1) / ka - jlo + 1;
+  const int pa = ka | 1, pb = nb | 1;
+  double* As = reinterpret_cast<double*>(smem_raw);  // [TN_ROWS][pa]
+  double* Bs = As + TN_ROWS * pa;                    // [TN_ROWS][pb]
+  int ia[M], jb[M];
+  double acc[M];
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int e = e0 + tid + 128 * m;
+    ia[m] = e < mtot ? e % ka : 0;
+    jb[m] = e < mtot ? e / ka - jlo : 0;
+    acc[m] = 0.0;
+  }
+  const int rr = tid & 31, cg = tid >> 5;
+  for (int64_t r0 = ch.r0; r0 < ch.r1; r0 += TN_ROWS) {
+    const int rows = (int)min((int64_t)TN_ROWS, ch.r1 - r0);
+    if (rr < rows) {
+      for (int c = cg; c < ka; c += 4) As[rr * pa + c] = A[r0 + rr + (int64_t)(aoff + c) * lda];
+      for (int c = cg; c < nb; c += 4)
+        Bs[rr * pb + c] = B[r0 + rr + (int64_t)(boff + jlo + c) * ldb];
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int q = 0; q < rows; ++q)
+#pragma unroll
+      for (int m = 0; m < M; ++m) acc[m] = fma(As[q * pa + ia[m]], Bs[q * pb + jb[m]], acc[m]);
+    __syncthreads();
+  }
+  double* out = partial + (int64_t)blockIdx.x * mtot;  // output (i, j) at i + j ka
+#pragma unroll
+  for (int m = 0; m < M; ++m) {
+    const int e = e0 + tid + 128 * m;
+    if (e < mtot) out[e] = acc[m];
+  }
 }
 
 // The FP64 form of the partial products in double-float arithmetic on the FP32
@@ -242,7 +297,7 @@ __global__ __launch_bounds__(256) void k_seg_nn(
   for (int i = 0; i < 2; ++i)
 #pragma unroll
     for (int j = 0; j < 16; ++j) acc[i][j] = 0.0;
-  for (int k0 = 0; k0 < kin; k0 += 16) {
+  for (int k0 = 0; k0 < kin && w * 16 < kout; k0 += 16) {
     const int k1 = (k0 + 16 < kin) ? k0 + 16 : kin;
     T tmp[2][16];
 #pragma unroll
@@ -275,6 +330,62 @@ __global__ __launch_bounds__(256) void k_seg_nn(
       const double v = (double)alpha * acc[i][j];
       *yp = (beta == (T)0) ? (T)v : (T)(v + (double)beta * (double)(*yp));
     }
+  }
+}
+
+// The FP64 expansion.  Bound by the FP64 pipe, as k_seg_tn_partial64: a block takes
+// one chunk (<= 64 rows) and every gridDim.y-th tile of CT columns, its four warps
+// the (row half, column group) pairs that exist, so that no FMA is issued for a
+// column past kout or a row half past the chunk (the form with 16 columns a warp
+// issued 128 columns whatever kout: 308 us for N = 16384, 60 x 37, this 93).  CT = 4
+// where CT = 8 would leave schedulers without a block.  P aliasing Y: one block has
+// all the tiles (P is staged whole before any write).
+template <int CT>
+__global__ __launch_bounds__(128) void k_seg_nn64(
+    const Chunk* __restrict__ chunks, int node0, const double* P, int64_t ldp, int poff_e,
+    int poff_o, int kin, const double* __restrict__ C, int64_t cstride, int cld, int cflip,
+    double* Y, int64_t ldy, int yoff_e, int yoff_o, int kout, double alpha, double beta) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  double* Ps = reinterpret_cast<double*>(smem_raw);  // [kin][NN_ROWS]
+  double* Cs = Ps + kin * NN_ROWS;                   // [CT][kin]
+  const Chunk ch = chunks[blockIdx.x];
+  const int rows = (int)(ch.r1 - ch.r0);
+  const int poff = (ch.node & 1) ? poff_o : poff_e;
+  const int yoff = (ch.node & 1) ? yoff_o : yoff_e;
+  const double* Cn = C + (int64_t)((ch.node ^ cflip) - node0) * cstride;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  for (int idx = tid; idx < kin * NN_ROWS; idx += 128) {
+    const int rr = idx % NN_ROWS, k = idx / NN_ROWS;
+    Ps[idx] = (rr < rows) ? P[ch.r0 + rr + (int64_t)(poff + k) * ldp] : 0.0;
+  }
+  const int nh = rows > 32 ? 2 : 1, ng = 4 / nh;  // row halves, column groups
+  const int rr = (nh == 2 ? (w & 1) * 32 : 0) + lane, g = w / nh;
+  for (int c0 = blockIdx.y * CT; c0 < kout; c0 += gridDim.y * CT) {
+    const int nc = min(CT, kout - c0);
+    for (int idx = tid; idx < nc * kin; idx += 128) {
+      const int k = idx % kin, j = idx / kin;
+      Cs[idx] = Cn[k + (int64_t)(c0 + j) * cld];
+    }
+    __syncthreads();
+    // this warp's columns g, g + ng, .. of the tile (at most CT / 2)
+    const int nj = g < nc ? (nc - g + ng - 1) / ng : 0;
+    double acc[CT / 2] = {};
+    for (int k = 0; k < kin; ++k) {
+      const double a = Ps[k * NN_ROWS + rr];
+#pragma unroll
+      for (int j = 0; j < CT / 2; ++j)
+        if (j < nj) acc[j] = fma(a, Cs[(g + ng * j) * kin + k], acc[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < CT / 2; ++j) {
+      if (j >= nj || rr >= rows) continue;
+      double* yp = Y + ch.r0 + rr + (int64_t)(yoff + c0 + g + ng * j) * ldy;
+      double v = acc[j];
+      if (alpha == -1.0) v = -v;
+      else if (alpha != 1.0) v *= alpha;
+      *yp = (beta == 0.0) ? v : fma(beta, *yp, v);
+    }
+    __syncthreads();
   }
 }
 
@@ -388,6 +499,32 @@ void seg_tn_partial_pick_j(const Chunk* chunks, int nchunks, const T* A, int64_t
   }
 }
 
+// FP64 TN: outputs per thread (4, 2 or 1) so that the blocks of 4 warps cover the
+// schedulers several times over (a block's time is set by its FMAs, 64 cycles each)
+static void seg_tn64(const Chunk* chunks, int nchunks, const double* A, int64_t lda, int aoff_even,
+                     int aoff_odd, int ka, const double* B, int64_t ldb, int boff_even,
+                     int boff_odd, int kb, double* partial, cudaStream_t st) {
+  auto run = [&](auto kern, int m) {
+    const int nb = std::min(kb, (128 * m - 1) / ka + 2);
+    const size_t smem = (size_t)TN_ROWS * ((ka | 1) + (nb | 1)) * sizeof(double);
+    const dim3 grid((unsigned)nchunks, (unsigned)((ka * kb + 128 * m - 1) / (128 * m)));
+    kern<<<grid, 128, smem, st>>>(chunks, A, lda, aoff_even, aoff_odd, ka, B, ldb, boff_even,
+                                  boff_odd, kb, partial);
+  };
+  static std::atomic<uint32_t> d1{0}, d2{0}, d4{0};
+  const int64_t warps = (int64_t)nchunks * ((ka * kb + 31) / 32);  // one output a lane
+  if (warps >= 16 * 608) {
+    raise_smem_limit((const void*)k_seg_tn_partial64<4>, d4);
+    run(k_seg_tn_partial64<4>, 4);
+  } else if (warps >= 8 * 608) {
+    raise_smem_limit((const void*)k_seg_tn_partial64<2>, d2);
+    run(k_seg_tn_partial64<2>, 2);
+  } else {
+    raise_smem_limit((const void*)k_seg_tn_partial64<1>, d1);
+    run(k_seg_tn_partial64<1>, 1);
+  }
+}
+
 template <typename T>
 void launch_seg_tn(const Chunk* chunks, int nchunks, const int32_t* chunk_begin, int nnodes,
                    int node0, const T* A, int64_t lda, int aoff_even, int aoff_odd, int ka,
@@ -395,27 +532,31 @@ void launch_seg_tn(const Chunk* chunks, int nchunks, const int32_t* chunk_begin,
                    T* out, cudaStream_t st, bool df, int half) {
   count_launches(2);
   (void)node0;
-  if (sizeof(T) == 8 && df) {
-    if (nchunks > 0) {
+  if constexpr (sizeof(T) == 8) {
+    if (df) {
       const int h = half > 0 ? half : kb;
       const dim3 grid((unsigned)nchunks, (unsigned)((ka + DT - 1) / DT),
                       (unsigned)(((h + DT - 1) / DT) * ((kb + h - 1) / h)));
-      k_seg_tn_partial_df<<<grid, 256, 0, st>>>(chunks, (const double*)A, lda, aoff_even, aoff_odd,
-                                                ka, (const double*)B, ldb, boff_even, boff_odd, kb,
-                                                h, partial);
+      k_seg_tn_partial_df<<<grid, 256, 0, st>>>(chunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
+                                                boff_even, boff_odd, kb, h, partial);
+    } else {
+      seg_tn64(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb, boff_even, boff_odd, kb,
+               partial, st);
     }
-  } else switch (tn_tile(ka)) {
-    case 2:
-      seg_tn_partial_pick_j<T, 2>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st);
-      break;
-    case 4:
-      seg_tn_partial_pick_j<T, 4>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st);
-      break;
-    default:
-      seg_tn_partial_pick_j<T, 8>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
-                                  boff_even, boff_odd, kb, partial, st);
+  } else {
+    switch (tn_tile(ka)) {
+      case 2:
+        seg_tn_partial_pick_j<T, 2>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
+                                    boff_even, boff_odd, kb, partial, st);
+        break;
+      case 4:
+        seg_tn_partial_pick_j<T, 4>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
+                                    boff_even, boff_odd, kb, partial, st);
+        break;
+      default:
+        seg_tn_partial_pick_j<T, 8>(chunks, nchunks, A, lda, aoff_even, aoff_odd, ka, B, ldb,
+                                    boff_even, boff_odd, kb, partial, st);
+    }
   }
   const int m = ka * kb;
   dim3 grid((unsigned)((m + 255) / 256), (unsigned)nnodes);
@@ -428,23 +569,32 @@ void launch_seg_nn(const Chunk* chunks, int nchunks, int node0, const T* P, int6
                    int cflip, T* Y, int64_t ldy, int yoff_even, int yoff_odd, int kout, T alpha,
                    T beta, cudaStream_t st, bool df) {
   count_launches(1);
-  const size_t smem = (size_t)(NN_MAX * NN_ROWS + NN_MAX * NN_MAX) * sizeof(T);
-  if (sizeof(T) == 8 && df) {
-    const size_t sm = (size_t)(kin * NN_ROWS + DT * (kin | 1)) * sizeof(float2);
-    static std::atomic<uint32_t> raised{0};
-    raise_smem_limit((const void*)k_seg_nn_df, raised);
+  if constexpr (sizeof(T) == 8) {
     const bool alias = (const void*)P == (const void*)Y;
-    const dim3 grid((unsigned)nchunks, alias ? 1u : (unsigned)((kout + DT - 1) / DT));
-    k_seg_nn_df<<<grid, 256, sm, st>>>(chunks, node0, (const double*)P, ldp, poff_even, poff_odd,
-                                       kin, (const double*)C, cstride, cld, cflip, (double*)Y, ldy,
-                                       yoff_even, yoff_odd, kout, (double)alpha, (double)beta);
-    return;
+    auto run = [&](auto kern, int threads, int ct, size_t smem) {
+      const dim3 grid((unsigned)nchunks, alias ? 1u : (unsigned)((kout + ct - 1) / ct));
+      kern<<<grid, threads, smem, st>>>(chunks, node0, P, ldp, poff_even, poff_odd, kin, C, cstride,
+                                        cld, cflip, Y, ldy, yoff_even, yoff_odd, kout, alpha, beta);
+    };
+    static std::atomic<uint32_t> ddf{0}, d4{0}, d8{0};
+    if (df) {
+      raise_smem_limit((const void*)k_seg_nn_df, ddf);
+      run(k_seg_nn_df, 256, DT, (size_t)(kin * NN_ROWS + DT * (kin | 1)) * sizeof(float2));
+    } else if (alias || (int64_t)nchunks * ((kout + 7) / 8) >= 304) {  // two blocks per SM
+      raise_smem_limit((const void*)k_seg_nn64<8>, d8);
+      run(k_seg_nn64<8>, 128, 8, (size_t)kin * (NN_ROWS + 8) * sizeof(double));
+    } else {
+      raise_smem_limit((const void*)k_seg_nn64<4>, d4);
+      run(k_seg_nn64<4>, 128, 4, (size_t)kin * (NN_ROWS + 4) * sizeof(double));
+    }
+  } else {
+    const size_t smem = (size_t)(NN_MAX * NN_ROWS + NN_MAX * NN_MAX) * sizeof(T);
+    static std::atomic<uint32_t> done{0};
+    raise_smem_limit((const void*)k_seg_nn<T>, done);
+    k_seg_nn<T><<<nchunks, 256, smem, st>>>(chunks, node0, P, ldp, poff_even, poff_odd, kin, C,
+                                            cstride, cld, cflip, Y, ldy, yoff_even, yoff_odd, kout,
+                                            alpha, beta);
   }
-  static std::atomic<uint32_t> done{0};
-  raise_smem_limit((const void*)k_seg_nn<T>, done);
-  k_seg_nn<T><<<nchunks, 256, smem, st>>>(chunks, node0, P, ldp, poff_even, poff_odd, kin, C,
-                                          cstride, cld, cflip, Y, ldy, yoff_even, yoff_odd, kout,
-                                          alpha, beta);
 }
 
 template void launch_seg_tn<float>(const Chunk*, int, const int32_t*, int, int, const float*,
