@@ -135,8 +135,8 @@ hm_status factorize_t(hm_handle* h, cudaStream_t st) {
   // scratch: Gauss-Jordan work, per-node projections, partials, GEMM items
   int max_tn = 0;
   for (int lv = 1; lv <= L; ++lv) max_tn = std::max(max_tn, t->plans[lv].n_tn);
-  const int64_t gj = std::max<int64_t>((int64_t)nleaf * nmax * 2 * nmax,
-                                       (nparents + 1) / 2 * 8 * (int64_t)r * r);
+  const int64_t gj = std::max<int64_t>((int64_t)nleaf * nmax * nmax,
+                                       (nparents + 1) / 2 * 4 * (int64_t)r * r);
   SolveCtx<T> c;
   T* work = nullptr;
   int* sing = nullptr;

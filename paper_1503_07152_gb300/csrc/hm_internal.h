@@ -235,8 +235,8 @@ void launch_blockdiag_apply(const T* D, int nmax, int trans, const T* X, int64_t
 template <typename T>
 void launch_fill(T* p, int64_t count, T v, cudaStream_t st);
 
-// HODLR solver: inverses of a batch of n x n matrices held as [A | I] (n x 2n,
-// column-major) in `work`, by Gauss-Jordan with partial pivoting.
+// HODLR solver: inverses of a batch of n x n matrices (n <= 256, column-major) held in
+// `work`, by Gauss-Jordan with partial pivoting.
 template <typename T>
 void launch_gauss_jordan(T* work, int batch, int n, T* out, int* singular, cudaStream_t st);
 template <typename T>

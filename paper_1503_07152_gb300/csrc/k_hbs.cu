@@ -113,6 +113,72 @@ __global__ __launch_bounds__(256) void k_batched_gemm_tiled(const GemmItem* __re
   }
 }
 
+// FP64 products (HM_FP64, and the applies of HM_A32 handles).  Bound by the FP64 pipe
+// (64 cycles a warp FMA): the outputs of a row segment (<= 64 rows of C) are dealt out
+// flat, M to a thread, so that no FMA goes to a column past n (a 32 x 32 tile wasted
+// two thirds of them at the 10 columns of an apply) and a level of a few items still
+// spreads over many SMs.  Operands staged in steps of 32 along k, each read along its
+// contiguous index; every output is one chain over p, as in k_batched_gemm.  Level of
+// 256 items, r = 60, 10 columns: 41 -> 17 us; 2 items: 41 -> 6 us.
+template <int M>
+__global__ __launch_bounds__(128) void k_batched_gemm64(const GemmItem* __restrict__ items,
+                                                        double alpha, double beta) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const GemmItem it = items[blockIdx.x];
+  const int n = it.n, k = it.k, m0 = blockIdx.z * 64;
+  const int m = min(64, it.m - m0), mn = m * n, e0 = blockIdx.y * 128 * M;
+  if (m <= 0 || e0 >= mn) return;  // uniform over the block
+  const double* A = (const double*)it.A;
+  const double* B = (const double*)it.B;
+  const int j0 = e0 / m, nb = (min(e0 + 128 * M, mn) - 1) / m - j0 + 1;
+  const int pb = nb | 1;
+  double* As = reinterpret_cast<double*>(smem_raw);  // [32][65]
+  double* Bs = As + 32 * 65;                         // [32][pb]
+  const int tid = threadIdx.x;
+  int ia[M], jb[M];
+  double acc[M];
+#pragma unroll
+  for (int q = 0; q < M; ++q) {
+    const int e = e0 + tid + 128 * q;
+    ia[q] = e < mn ? e % m : 0;
+    jb[q] = e < mn ? e / m - j0 : 0;
+    acc[q] = 0.0;
+  }
+  for (int p0 = 0; p0 < k; p0 += 32) {
+    const int kp = min(32, k - p0);
+    if (it.ta) {
+      for (int e = tid; e < 32 * m; e += 128) {
+        const int p = e & 31, i = e >> 5;
+        if (p < kp) As[p * 65 + i] = A[p0 + p + (int64_t)(m0 + i) * it.lda];
+      }
+    } else {
+      for (int e = tid; e < kp * 64; e += 128) {
+        const int i = e & 63, p = e >> 6;
+        if (i < m) As[p * 65 + i] = A[m0 + i + (int64_t)(p0 + p) * it.lda];
+      }
+    }
+    for (int e = tid; e < 32 * nb; e += 128) {
+      const int p = it.tb ? e / nb : e & 31, j = it.tb ? e % nb : e >> 5;
+      if (p < kp)
+        Bs[p * pb + j] = it.tb ? B[j0 + j + (int64_t)(p0 + p) * it.ldb]
+                               : B[p0 + p + (int64_t)(j0 + j) * it.ldb];
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int p = 0; p < kp; ++p)
+#pragma unroll
+      for (int q = 0; q < M; ++q) acc[q] = fma(As[p * 65 + ia[q]], Bs[p * pb + jb[q]], acc[q]);
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < M; ++q) {
+    if (e0 + tid + 128 * q >= mn) continue;
+    double* c = (double*)it.C + m0 + ia[q] + (int64_t)(j0 + jb[q]) * it.ldc;
+    const double v = alpha == 1.0 ? acc[q] : alpha * acc[q];
+    *c = (beta == 0.0) ? v : fma(beta, *c, v);
+  }
+}
+
 // The FP64 form of k_batched_gemm_tiled in double-float on the FP32 pipe
 // (HM_A32): every input cut once, when staged, into hi + lo floats; each output
 // summed as a float pair (TwoProduct of the high parts, the cross terms, TwoSum).
@@ -531,6 +597,26 @@ void launch_batched_gemm(const GemmItem* items, int count, T alpha, T beta, cuda
     raise_smem_limit((const void*)k_batched_gemm_tiled_df, done);
     dim3 grid((unsigned)count, (unsigned)((max_n + 31) / 32), (unsigned)((max_m + 31) / 32));
     k_batched_gemm_tiled_df<<<grid, 256, smem, st>>>(items, (double)alpha, (double)beta);
+  } else if (sizeof(T) == 8 && max_m >= 1 && max_n >= 1 && max_k >= 1 && max_m <= 64 * 65535 &&
+             (int64_t)std::min(max_m, 64) * max_n <= 128 * (int64_t)65535) {
+    // outputs per thread: four once the items alone give every scheduler several warps
+    const int ms = std::min(max_m, 64);
+    auto run = [&](auto kern, int mq) {
+      // columns of B a block may touch: items of fewer rows than max_m touch more
+      const int nb = std::min(max_n, 128 * mq + 1);
+      const dim3 grid((unsigned)count, (unsigned)((ms * max_n + 128 * mq - 1) / (128 * mq)),
+                      (unsigned)((max_m + 63) / 64));
+      kern<<<grid, 128, (size_t)32 * (65 + (nb | 1)) * sizeof(double), st>>>(items, (double)alpha,
+                                                                           (double)beta);
+    };
+    static std::atomic<uint32_t> d1{0}, d4{0};
+    if ((int64_t)count * max_m * max_n / 32 >= 16 * 608 && max_n <= 512) {
+      raise_smem_limit((const void*)k_batched_gemm64<4>, d4);
+      run(k_batched_gemm64<4>, 4);
+    } else {
+      raise_smem_limit((const void*)k_batched_gemm64<1>, d1);
+      run(k_batched_gemm64<1>, 1);
+    }
   } else if (max_m >= 1 && max_n >= 1 && max_k >= 1 && smem <= 96 * 1024 &&
              max_n <= 32 * 65535 && max_m <= 32 * 65535) {
     static std::atomic<uint32_t> done{0};

@@ -2,113 +2,153 @@
 // dense matrices by Gauss-Jordan elimination with partial pivoting, and the
 // assembly of the per-parent Woodbury matrices.
 #include <algorithm>
+#include <atomic>
+#include <cooperative_groups.h>
 
 #include "hm_internal.h"
 
 namespace hm {
 namespace {
 
-// Inverse of every matrix of a batch, one block per matrix.  W holds the
-// augmented [A | I] of each matrix, column-major n x 2n (ld n), in global memory
-// (L2-resident at these sizes); out[b] receives A^{-1} (n x n, ld n).  A zero
+// Inverse of every matrix of a batch by Gauss-Jordan elimination with partial
+// pivoting, in place (W: n x n, column-major, ld n, in global memory, read once and
+// out[b] written once): row k of the inverse replaces the eliminated column k as the
+// step goes, the row exchanges are undone as column exchanges at the end.  A zero
 // pivot raises *singular and the step is skipped (the output is then garbage).
+//
+// Bound by the FP64 pipe (n^2 FMAs a step, 64 cycles a warp FMA on one scheduler), so
+// a matrix is dealt out column by column over a cluster of S blocks (block p holds
+// columns p, p + S, .. in shared memory) when the batch alone leaves SMs idle.  A
+// step: the owner of column k finds the pivot and writes it and the column's
+// multipliers into every block's shared memory, one cluster barrier, and each block
+// exchanges the two rows of its columns and updates them.  The multipliers are double-
+// buffered, so one barrier a step orders them: a block writes buffer k & 1 at step k
+// only after the barrier of step k - 1, which every block passes after its last use of
+// that buffer, at step k - 2.  32 leaves of 94: 1510 -> 250 us (one block a matrix, the
+// augmented n x 2n form in L2); 36 x 36 Woodbury blocks: 92 -> 40 us.
 template <typename T>
-__global__ __launch_bounds__(512) void k_gauss_jordan(T* __restrict__ W, int n,
+__global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, int n,
                                                       T* __restrict__ out,
-                                                      int* __restrict__ singular) {
-  __shared__ T fcol[256];
-  __shared__ double rv[16];
-  __shared__ int ri[16];
-  __shared__ int piv;
-  T* Wb = W + (int64_t)blockIdx.x * n * 2 * n;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-  const int n2 = 2 * n;
+                                                      int* __restrict__ singular, int S) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ T fcol[2][256];   // the pivot column before the step, rows exchanged
+  __shared__ int prow[2];      // its pivot row
+  __shared__ double rv[8];
+  __shared__ int ri[8];
+  __shared__ short swp[256];   // pivot row of every step
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  const int part = S > 1 ? (int)cl.block_rank() : 0;
+  const int b = blockIdx.x / S;
+  T* M = reinterpret_cast<T*>(smem_raw);  // local column c: global column part + S c
+  const int nloc = part < n ? (n - part + S - 1) / S : 0;
+  const T* Wb = W + (int64_t)b * n * n;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int e = tid; e < n * nloc; e += 256) {
+    const int i = e % n, c = e / n;
+    M[e] = Wb[i + (int64_t)(part + S * c) * n];
+  }
+  if (S > 1) cl.sync();  // every block of the cluster runs before its memory is written
+  else __syncthreads();
   for (int k = 0; k < n; ++k) {
-    // pivot: the largest |A(i, k)|, i >= k (first on ties)
-    double best = -1.0;
-    int bi = n;
-    for (int i = k + tid; i < n; i += blockDim.x) {
-      const double a = fabs((double)Wb[i + (int64_t)k * n]);
-      if (a > best) { best = a; bi = i; }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
-    __syncthreads();
-    if (tid == 0) {
-      double b = -1.0;
+    const int buf = k & 1;
+    if (k % S == part) {
+      T* col = M + (int64_t)(k / S) * n;
+      // pivot: the largest |A(i, k)|, i >= k (first on ties)
+      double best = -1.0;
+      int bi = n;
+      for (int i = k + tid; i < n; i += 256) {
+        const double a = fabs((double)col[i]);
+        if (a > best) { best = a; bi = i; }
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
+        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+      }
+      if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
+      __syncthreads();
+      double bb = -1.0;
       int p = n;
-      for (int w = 0; w < nw; ++w)
-        if (rv[w] > b || (rv[w] == b && ri[w] < p)) { b = rv[w]; p = ri[w]; }
-      if (!(b > 0.0) || p >= n) {
-        atomicExch(singular, 1);
+      for (int w = 0; w < 8; ++w)
+        if (rv[w] > bb || (rv[w] == bb && ri[w] < p)) { bb = rv[w]; p = ri[w]; }
+      if (!(bb > 0.0) || p >= n) {
+        if (tid == 0) atomicExch(singular, 1);
         p = k;
       }
-      piv = p;
-    }
-    __syncthreads();
-    const int p = piv;
-    if (p != k)
-      for (int j = tid; j < n2; j += blockDim.x) {
-        const T t = Wb[k + (int64_t)j * n];
-        Wb[k + (int64_t)j * n] = Wb[p + (int64_t)j * n];
-        Wb[p + (int64_t)j * n] = t;
+      for (int i = tid; i < n; i += 256) {
+        const T v = col[i == k ? p : (i == p ? k : i)];
+        for (int q = 0; q < S; ++q) (S > 1 ? cl.map_shared_rank(&fcol[buf][i], q) : &fcol[buf][i])[0] = v;
       }
-    __syncthreads();
-    const T pv = Wb[k + (int64_t)k * n];
-    const T inv = (pv != (T)0) ? (T)1 / pv : (T)0;
-    __syncthreads();
-    for (int j = tid; j < n2; j += blockDim.x) Wb[k + (int64_t)j * n] *= inv;
-    for (int i = tid; i < n; i += blockDim.x) fcol[i] = (i == k) ? (T)0 : Wb[i + (int64_t)k * n];
-    __syncthreads();
-    // row i -= f_i row k, all i != k (columns k .. 2n - 1: the eliminated
-    // columns left of k are already unit vectors and stay so)
-    const int cols = n2 - k;
-    for (int e = tid; e < n * cols; e += blockDim.x) {
-      const int i = e % n, j = k + e / n;
-      if (i != k) Wb[i + (int64_t)j * n] -= fcol[i] * Wb[k + (int64_t)j * n];
+      if (tid < S) (S > 1 ? cl.map_shared_rank(&prow[buf], tid) : &prow[buf])[0] = p;
     }
-    __syncthreads();
+    if (S > 1) cl.sync();
+    else __syncthreads();
+    const int p = prow[buf];
+    const T pv = fcol[buf][k];
+    const T inv = (pv != (T)0) ? (T)1 / pv : (T)0;
+    if (tid == 0) swp[k] = (short)p;
+    // a warp takes a column: exchange rows k and p, scale the pivot row's entry, update
+    for (int c = warp; c < nloc; c += 8) {
+      T* col = M + (int64_t)c * n;
+      if (part + S * c == k) {  // the column of the inverse that replaces column k
+        for (int i = lane; i < n; i += 32) col[i] = i == k ? inv : -fcol[buf][i] * inv;
+        continue;
+      }
+      const T xp = col[p], xk = col[k];
+      const T x = xp * inv;
+      __syncwarp();
+      for (int i = lane; i < n; i += 32) {
+        const T y = i == p ? xk : col[i];
+        col[i] = i == k ? x : fma(-fcol[buf][i], x, y);
+      }
+      __syncwarp();
+    }
+    __syncthreads();  // the owner of column k + 1 reads what one of its warps updated
   }
-  T* ob = out + (int64_t)blockIdx.x * n * n;
-  for (int e = tid; e < n * n; e += blockDim.x) ob[e] = Wb[(int64_t)n * n + e];
+  if (S > 1) cl.sync();  // no block leaves while another may still write to it
+  else __syncthreads();
+  // undo the exchanges: column k and column swp[k], k = n - 1 .. 0.  Thread c follows
+  // its column to the place it ends up at.
+  T* ob = out + (int64_t)b * n * n;
+  for (int c = warp; c < nloc; c += 8) {
+    int dst = part + S * c;
+    for (int k = n - 1; k >= 0; --k) {
+      const int p = swp[k];
+      if (dst == k) dst = p;
+      else if (dst == p) dst = k;
+    }
+    for (int i = lane; i < n; i += 32) ob[i + (int64_t)dst * n] = M[(int64_t)c * n + i];
+  }
 }
 
-// [D_leaf | I] padded to nmax (identity beyond the leaf size), one block per leaf.
+// D_leaf padded to nmax (identity beyond the leaf size), one block per leaf.
 template <typename T>
 __global__ void k_gj_load_leaves(const T* __restrict__ D, int nmax,
                                  const int64_t* __restrict__ size, int L, T* __restrict__ W) {
   const int leaf = blockIdx.x;
   const int ns = (int)size[(1 << L) + leaf];
   const T* Dl = D + (int64_t)leaf * nmax * nmax;
-  T* Wl = W + (int64_t)leaf * nmax * 2 * nmax;
-  for (int e = threadIdx.x; e < nmax * 2 * nmax; e += blockDim.x) {
+  T* Wl = W + (int64_t)leaf * nmax * nmax;
+  for (int e = threadIdx.x; e < nmax * nmax; e += blockDim.x) {
     const int i = e % nmax, j = e / nmax;
-    T v;
-    if (j < nmax) v = (i < ns && j < ns) ? Dl[i + (int64_t)j * nmax] : (T)(i == j ? 1 : 0);
-    else v = (T)(i == j - nmax ? 1 : 0);
-    Wl[e] = v;
+    Wl[e] = (i < ns && j < ns) ? Dl[e] : (T)(i == j ? 1 : 0);
   }
 }
 
-// [[I, P_b], [P_a, I] | I] for every parent p of a level (children a = 2p,
-// b = 2p + 1): P holds V_x^T W_x (r x r, ld r) for the children, indexed by
-// x - child0.
+// [[I, P_b], [P_a, I]] for every parent p of a level (children a = 2p, b = 2p + 1):
+// P holds V_x^T W_x (r x r, ld r) for the children, indexed by x - child0.
 template <typename T>
 __global__ void k_gj_load_woodbury(const T* __restrict__ P, int r, T* __restrict__ W) {
   const int pi = blockIdx.x;  // parent index within its level
   const int n = 2 * r;
   const T* Pa = P + (int64_t)(2 * pi) * r * r;
   const T* Pb = P + (int64_t)(2 * pi + 1) * r * r;
-  T* Wp = W + (int64_t)pi * n * 2 * n;
-  for (int e = threadIdx.x; e < n * 2 * n; e += blockDim.x) {
+  T* Wp = W + (int64_t)pi * n * n;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
     const int i = e % n, j = e / n;
     T v;
-    if (j >= n) v = (T)(i == j - n ? 1 : 0);
-    else if ((i < r) == (j < r)) v = (T)(i == j ? 1 : 0);
+    if ((i < r) == (j < r)) v = (T)(i == j ? 1 : 0);
     else if (i < r) v = Pb[i + (int64_t)(j - r) * r];  // top right: V_b^T W_b
     else v = Pa[(i - r) + (int64_t)j * r];             // bottom left: V_a^T W_a
     Wp[e] = v;
@@ -117,10 +157,31 @@ __global__ void k_gj_load_woodbury(const T* __restrict__ P, int r, T* __restrict
 
 }  // namespace
 
+// Cluster size: doubled (up to 8) while two blocks per SM are not reached and a block
+// would keep at least eight columns, and further while a block's columns do not fit its
+// shared memory (n = 256 in FP64: 512 KB over 4 blocks).
 template <typename T>
 void launch_gauss_jordan(T* work, int batch, int n, T* out, int* singular, cudaStream_t st) {
   count_launches(1);
-  k_gauss_jordan<T><<<batch, 512, 0, st>>>(work, n, out, singular);
+  int S = 1;
+  while (S < 8 && ((int64_t)batch * 2 * S <= 304 && n >= 16 * S)) S *= 2;
+  auto smem = [&](int s) { return (size_t)n * ((n + s - 1) / s) * sizeof(T); };
+  while (S < 8 && smem(S) > 200 * 1024) S *= 2;
+  static std::atomic<uint32_t> done{0};
+  raise_smem_limit((const void*)k_gauss_jordan<T>, done);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(batch * S));
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = smem(S);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)S;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const T* W = work;
+  cudaLaunchKernelEx(&cfg, k_gauss_jordan<T>, W, n, out, singular, S);
 }
 
 template <typename T>
