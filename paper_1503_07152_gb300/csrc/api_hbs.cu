@@ -103,6 +103,32 @@ hm_status hbs_partial_apply(HbsState<T>& s, int m, const T* X, int64_t ldx, T* S
     launch_seg_tn<T>(pm.d_tn, pm.n_tn, pm.d_tn_begin, pm.nnodes, pm.node0, Vout, s.N, 0, 0, r,
                      X + cb * ldx, ldx, 0, 0, w, s.partial, qh + pm.node0 * rw, st, s.df,
                      ncols == 2 * r && w == 2 * r ? r : 0);
+    if constexpr (sizeof(T) == 8) {
+      NodeGemm g{};
+      g.r = r;
+      g.w = w;
+      g.q = qh;
+      g.u = uh;
+      g.mode = NodeGemm::kUp;
+      g.A0 = Sout;
+      g.ta0 = 1;
+      for (int lev = m - 1; lev >= 1; --lev) {
+        g.node0 = 1 << lev;
+        launch_node_gemm(g, 1 << lev, st, s.df);
+      }
+      g.mode = NodeGemm::kDown;
+      g.A0 = s.Bm;
+      g.ta0 = trans;
+      g.ta1 = 0;
+      for (int lev = 1; lev <= m; ++lev) {
+        g.node0 = 1 << lev;
+        g.A1 = lev >= 2 ? Sin : nullptr;
+        launch_node_gemm(g, 1 << lev, st, s.df);
+      }
+      launch_seg_nn<T>(pm.d_nn, pm.n_nn, pm.node0, Uin, s.N, 0, 0, r, uh + pm.node0 * rw, rw, r, 0,
+                       S + cb * lds, lds, 0, 0, w, sign, (T)1, st, s.df);
+      continue;
+    }
     for (int lev = m - 1; lev >= 1; --lev) {
       for (int tau = 1 << lev; tau < (2 << lev); ++tau)
         it.add(Sout + (2 * tau) * rr, r, 1, qh + (2 * tau) * rw, r, 0, qh + tau * rw, r, r, w, r);
@@ -337,13 +363,13 @@ hm_status hbsid_sweep(Ctx<T>& c, HbsState<T>& s, const T* D, hm_handle* h) {
 
 // ------------------------------------------------------------ applies ------
 template <typename T>
-hm_status hbsid_apply_block(const hm_handle* h, int trans, int w, const T* X, T* Y, T* qh, T* uh,
-                            GemmItem* items, size_t cap, cudaStream_t st) {
+hm_status hbsid_apply_block(const hm_handle* h, int trans, int w, const T* X, int64_t ldx, T* Y,
+                            int64_t ldy, T* qh, T* uh, GemmItem* items, size_t cap,
+                            cudaStream_t st) {
   const hm_tree* t = &h->tree;
   const int r = h->r;
   const int L = t->L;
   const int nmax = (int)t->nmax;
-  const int64_t N = h->n;
   const int64_t rr = (int64_t)r * r, rw = (int64_t)r * w;
   const int64_t total = h->tin_off[4];
   const T* sin = (const T*)h->hbs_store;
@@ -356,10 +382,51 @@ hm_status hbsid_apply_block(const hm_handle* h, int trans, int w, const T* X, T*
     if (node >= (1 << L)) return base + (int64_t)(node - (1 << L)) * r * nmax;
     return base + h->tin_off[1] + (int64_t)(node - 1) * 2 * rr;
   };
+  if constexpr (sizeof(T) == 8) {
+    NodeGemm g{};
+    g.r = r;
+    g.w = w;
+    g.nmax = nmax;
+    g.q = qh;
+    g.u = uh;
+    g.X = X;
+    g.Y = Y;
+    g.ldx = ldx;
+    g.ldy = ldy;
+    g.start = t->d_start;
+    g.size = t->d_size;
+    g.node0 = 1 << L;
+    g.mode = NodeGemm::kLeafUp;
+    g.A0 = Tout;
+    launch_node_gemm(g, 1 << L, st, false);
+    // a parent's interpolation matrix is r x 2r: its halves are where child 2 x + h of
+    // node x would be in a heap of r x r blocks starting two blocks earlier
+    g.mode = NodeGemm::kUp;
+    g.A0 = Tout + h->tin_off[1] - 2 * rr;
+    for (int lev = L - 1; lev >= 1; --lev) {
+      g.node0 = 1 << lev;
+      launch_node_gemm(g, 1 << lev, st, false);
+    }
+    g.mode = NodeGemm::kDown;
+    g.A0 = Bsk;
+    g.ta0 = trans;
+    g.ta1 = 1;
+    for (int lev = 1; lev <= L; ++lev) {
+      g.node0 = 1 << lev;
+      g.A1 = lev >= 2 ? Tin + h->tin_off[1] - 2 * rr : nullptr;
+      launch_node_gemm(g, 1 << lev, st, false);
+    }
+    g.mode = NodeGemm::kLeafDown;
+    g.A0 = Tin;
+    g.node0 = 1 << L;
+    launch_node_gemm(g, 1 << L, st, false);
+    launch_blockdiag_apply<T>(D, nmax, trans, X, ldx, Y, ldy, w, 1, t->d_start, t->d_size, L, st);
+    return check_launch("hbs-id apply");
+  }
   Items<T> it;
   // upward: leaves then parents
   for (int leaf = 1 << L; leaf < (2 << L); ++leaf)
-    it.add(tcol(Tout, leaf), r, 0, X + t->start[leaf], N, 0, qh + leaf * rw, r, r, w,
+    it.add(tcol(Tout, leaf), r, 0, X + t->start[leaf], (int)ldx, 0, qh + leaf * rw, r, r, w,
            (int)t->size[leaf]);
   HM_TRY(it.run(items, cap, (T)1, (T)0, st));
   for (int lev = L - 1; lev >= 1; --lev) {
@@ -386,10 +453,10 @@ hm_status hbsid_apply_block(const hm_handle* h, int trans, int w, const T* X, T*
     }
   }
   for (int leaf = 1 << L; leaf < (2 << L); ++leaf)
-    it.add(tcol(Tin, leaf), r, 1, uh + leaf * rw, r, 0, Y + t->start[leaf], N, (int)t->size[leaf],
+    it.add(tcol(Tin, leaf), r, 1, uh + leaf * rw, r, 0, Y + t->start[leaf], (int)ldy, (int)t->size[leaf],
            w, r);
   HM_TRY(it.run(items, cap, (T)1, (T)0, st));
-  launch_blockdiag_apply<T>(D, nmax, trans, X, N, Y, N, w, t->d_start, t->d_size, L, st);
+  launch_blockdiag_apply<T>(D, nmax, trans, X, ldx, Y, ldy, w, 1, t->d_start, t->d_size, L, st);
   return check_launch("hbs-id apply");
 }
 
@@ -401,13 +468,18 @@ hm_status hbs_apply_t(const hm_handle* h, int trans, int64_t ncols, const T* X, 
   const int nheap = 1 << (h->L + 1);
   const int64_t cbw = 128;
   const size_t cap = 4 * (size_t)nheap + 16;
-  T *qh, *uh, *Xc, *Yc;
+  T *qh, *uh, *Xc = nullptr, *Yc = nullptr;
   GemmItem* items;
+  // FP32 handles go through item lists whose leading dimensions are 32-bit: their blocks
+  // are copied to ld = N when the caller's are longer
+  const bool copy = sizeof(T) == 4 && (ldx > INT32_MAX || ldy > INT32_MAX);
   auto layout = [&](Arena& a) {
     qh = a.take<T>((size_t)nheap * r * cbw);
     uh = a.take<T>((size_t)nheap * r * cbw);
-    Xc = a.take<T>(N * cbw);
-    Yc = a.take<T>(N * cbw);
+    if (copy) {
+      Xc = a.take<T>(N * cbw);
+      Yc = a.take<T>(N * cbw);
+    }
     items = a.take<GemmItem>(cap);
   };
   Arena m;
@@ -421,14 +493,21 @@ hm_status hbs_apply_t(const hm_handle* h, int trans, int64_t ncols, const T* X, 
   hm_status s = HM_OK;
   for (int64_t cb = 0; cb < ncols && s == HM_OK; cb += cbw) {
     const int w = (int)std::min<int64_t>(cbw, ncols - cb);
-    launch_copy_cols<T>(X + cb * ldx, ldx, Xc, N, N, w, st);
+    const T* Xb = X + cb * ldx;
+    T* Yb = Y + cb * ldy;
+    if (copy) {
+      launch_copy_cols<T>(Xb, ldx, Xc, N, N, w, st);
+      Xb = Xc;
+      Yb = Yc;
+    }
     if (h->format == HM_FORMAT_HBSID) {
-      s = hbsid_apply_block<T>(h, trans, w, Xc, Yc, qh, uh, items, cap, st);
+      s = hbsid_apply_block<T>(h, trans, w, Xb, copy ? N : ldx, Yb, copy ? N : ldy, qh, uh, items,
+                               cap, st);
     } else {
       s = HM_EUNSUPPORTED;
       set_error("apply of the plain HBS format is served through HBS-ID handles");
     }
-    if (s == HM_OK) launch_copy_cols<T>(Yc, N, Y + cb * ldy, ldy, N, w, st);
+    if (s == HM_OK && copy) launch_copy_cols<T>(Yc, N, Y + cb * ldy, ldy, N, w, st);
   }
   cudaFreeAsync(blk, st);
   if (s != HM_OK) return s;

@@ -522,15 +522,12 @@ hm_status hodlr_apply_t(const hm_handle* h, int trans, int64_t ncols, const T* X
   int max_tn = 0;
   for (int lv = 1; lv <= t->L; ++lv) max_tn = std::max(max_tn, t->plans[lv].n_tn);
   const int64_t nn = (int64_t)1 << t->L;
-  // contiguous copies of X / Y blocks so that the kernels see ld = N
   const int64_t cbw = 128;
   double* partial = nullptr;
-  T *coef = nullptr, *Xc = nullptr, *Yc = nullptr;
+  T* coef = nullptr;
   auto layout = [&](Arena& a) {
     partial = a.take<double>((size_t)max_tn * r * cbw);
     coef = a.take<T>(nn * r * cbw);
-    Xc = a.take<T>(N * cbw);
-    Yc = a.take<T>(N * cbw);
   };
   Arena m;
   layout(m);
@@ -544,10 +541,10 @@ hm_status hodlr_apply_t(const hm_handle* h, int trans, int64_t ncols, const T* X
   const T* V = (const T*)h->V;
   for (int64_t cb = 0; cb < ncols; cb += cbw) {
     const int w = (int)std::min<int64_t>(cbw, ncols - cb);
-    launch_copy_cols<T>(X + cb * ldx, ldx, Xc, N, N, w, st);
-    launch_fill<T>(Yc, N * w, (T)0, st);
-    launch_blockdiag_apply<T>((const T*)h->D, (int)t->nmax, trans, Xc, N, Yc, N, w, t->d_start,
-                              t->d_size, t->L, st);
+    const T* Xc = X + cb * ldx;
+    T* Yc = Y + cb * ldy;
+    launch_blockdiag_apply<T>((const T*)h->D, (int)t->nmax, trans, Xc, ldx, Yc, ldy, w, 0,
+                              t->d_start, t->d_size, t->L, st);
     for (int j = 1; j <= t->L; ++j) {
       const LevelPlan& lp = t->plans[j];
       const T* Uj = U + (int64_t)(j - 1) * N * r;
@@ -555,11 +552,10 @@ hm_status hodlr_apply_t(const hm_handle* h, int trans, int64_t ncols, const T* X
       const T* Proj = trans ? Uj : Vj;
       const T* Expd = trans ? Vj : Uj;
       launch_seg_tn<T>(lp.d_tn, lp.n_tn, lp.d_tn_begin, lp.nnodes, lp.node0, Proj, N, 0, 0, r, Xc,
-                       N, 0, 0, w, partial, coef, st);
+                       ldx, 0, 0, w, partial, coef, st);
       launch_seg_nn<T>(lp.d_nn, lp.n_nn, lp.node0, Expd, N, 0, 0, r, coef, (int64_t)r * w, r, 1,
-                       Yc, N, 0, 0, w, (T)1, (T)1, st);
+                       Yc, ldy, 0, 0, w, (T)1, (T)1, st);
     }
-    launch_copy_cols<T>(Yc, N, Y + cb * ldy, ldy, N, w, st);
   }
   HM_CUDA_TRY(cudaFreeAsync(blk, st));
   return check_launch("hodlr apply");

@@ -82,7 +82,18 @@ struct SolveCtx {
     // then y_a -= W_a s_a, y_b -= W_b s_b (forward) or y_a -= V_a s_a, y_b -= V_b s_b
     // with s_a = (M^T [q_a; q_b])[r:2r], s_b = (...)[0:r] (transposed)
     const int np = lp.nnodes / 2;
-    for (int pass = 0; pass < 2; ++pass) {
+    if constexpr (sizeof(T) == 8) {
+      NodeGemm g{};
+      g.mode = NodeGemm::kSolve;
+      g.node0 = lp.node0;
+      g.r = r;
+      g.w = w;
+      g.ta0 = trans;
+      g.A0 = M + (int64_t)((1 << (j - 1)) - 1) * rr2;  // parents of levels < j first
+      g.q = q;
+      g.u = s;
+      launch_node_gemm(g, lp.nnodes, st, false);
+    } else for (int pass = 0; pass < 2; ++pass) {
       for (int pi = 0; pi < np; ++pi) {
         const T* Mp = M + (int64_t)((1 << (j - 1)) - 1 + pi) * rr2;  // parents of levels < j first
         const T* qa = q + (int64_t)(2 * pi) * rw;
@@ -165,8 +176,7 @@ hm_status factorize_t(hm_handle* h, cudaStream_t st) {
     T* Wj = Wall + (int64_t)(j - 1) * N * r;
     const T* Uj = (const T*)h->U + (int64_t)(j - 1) * N * r;
     // W_j = D^{-1} U_j, then through the factors of the finer levels
-    launch_fill<T>(Wj, N * r, (T)0, st);
-    launch_blockdiag_apply<T>(Dinv, nmax, 0, Uj, N, Wj, N, r, t->d_start, t->d_size, L, st);
+    launch_blockdiag_apply<T>(Dinv, nmax, 0, Uj, N, Wj, N, r, 0, t->d_start, t->d_size, L, st);
     for (int i = L; i > j && s == HM_OK; --i) s = c.level_inverse(i, Wj, r, 0);
     if (s != HM_OK) break;
     // M for the parents of level j: P_x = V_x^T W_x per child x on level j
@@ -244,13 +254,11 @@ hm_status solve_t(const hm_handle* h, int trans, int64_t ncols, const T* B, int6
     const int w = (int)std::min<int64_t>(cbw, ncols - cb);
     launch_copy_cols<T>(B + cb * ldb, ldb, Bc, N, N, w, st);
     if (!trans) {
-      launch_fill<T>(Yc, N * w, (T)0, st);
-      launch_blockdiag_apply<T>(c.Dinv, nmax, 0, Bc, N, Yc, N, w, t->d_start, t->d_size, L, st);
+      launch_blockdiag_apply<T>(c.Dinv, nmax, 0, Bc, N, Yc, N, w, 0, t->d_start, t->d_size, L, st);
       for (int j = L; j >= 1 && s == HM_OK; --j) s = c.level_inverse(j, Yc, w, 0);
     } else {
       for (int j = 1; j <= L && s == HM_OK; ++j) s = c.level_inverse(j, Bc, w, 1);
-      launch_fill<T>(Yc, N * w, (T)0, st);
-      launch_blockdiag_apply<T>(c.Dinv, nmax, 1, Bc, N, Yc, N, w, t->d_start, t->d_size, L, st);
+      launch_blockdiag_apply<T>(c.Dinv, nmax, 1, Bc, N, Yc, N, w, 0, t->d_start, t->d_size, L, st);
     }
     if (s == HM_OK) launch_copy_cols<T>(Yc, N, X + cb * ldx, ldx, N, w, st);
   }

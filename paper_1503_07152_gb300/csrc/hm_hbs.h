@@ -15,6 +15,32 @@ struct GemmItem {
   int32_t ta, tb;
 };
 
+// One level's small FP64 products in one launch, the operands of every node found from
+// its index on the device (no item list to build and copy): node x gets
+//   C = op(A_0) B_0 [+ op(A_1) B_1],
+// each product summed on its own and the two added last.  q, u hold one r x w block
+// per heap node (the solver: per node of the level, x - node0).
+struct NodeGemm {
+  enum Mode {
+    kUp,        // q[x] = op(A_0) q[2x] + op(A_1) q[2x + 1], A_h = A0 + (2x + h) r^2
+    kDown,      // u[x] = B_x q[x ^ 1] + op(A) u[x / 2]: B_x = A0 + x r^2 (ta0: the sibling's,
+                //   transposed), A = A1 + x r^2 (ta1); no second term when A1 is null
+    kLeafUp,    // q[x] = A X(I_x), A = A0 + leaf r nmax (r x n_x)
+    kLeafDown,  // Y(I_x) = A^T u[x], A as above
+    kSolve      // u[x] = the rows of M [q_b; q_a] (ta0: of M^T [q_a; q_b]) that child x of
+                //   its parent takes, M = A0 + parent (2r)^2, parents of level node0 / 2
+  };
+  int32_t mode;
+  int32_t node0, r, w, nmax, ta0, ta1;
+  const double *A0, *A1;
+  double *q, *u;
+  const double* X;
+  double* Y;
+  int64_t ldx, ldy;
+  const int64_t *start, *size;
+};
+void launch_node_gemm(const NodeGemm& a, int nodes, cudaStream_t st, bool df);
+
 template <typename T>
 void launch_gather_parent_scaled(const T* U, int64_t ldu, T* P, int64_t ldp, int64_t n, int r,
                                  int lv, const int64_t* d_start, const T* y, int col0,

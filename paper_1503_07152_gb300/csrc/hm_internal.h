@@ -226,14 +226,11 @@ template <typename T>
 void launch_extract_diag(const T* Y, int64_t ldy, T* D, int nmax, const int64_t* d_start,
                          const int64_t* d_size, int L, cudaStream_t st);
 
-// Y(I_t, :) += op(D_t) X(I_t, :) for every leaf.
+// Y(I_t, :) = [Y(I_t, :) +] op(D_t) X(I_t, :) for every leaf (added to Y when `add`).
 template <typename T>
 void launch_blockdiag_apply(const T* D, int nmax, int trans, const T* X, int64_t ldx, T* Y,
-                            int64_t ldy, int64_t ncols, const int64_t* d_start,
+                            int64_t ldy, int64_t ncols, int add, const int64_t* d_start,
                             const int64_t* d_size, int L, cudaStream_t st);
-
-template <typename T>
-void launch_fill(T* p, int64_t count, T v, cudaStream_t st);
 
 // HODLR solver: inverses of a batch of n x n matrices (n <= 256, column-major) held in
 // `work`, by Gauss-Jordan with partial pivoting.

@@ -141,7 +141,7 @@ __global__ void k_extract_diag(const T* __restrict__ Y, int64_t ldy, T* __restri
   }
 }
 
-// Y(I_t, c) += sum_j op(D_t)(i, j) X(I_t(j), c) for every leaf t.  Block: 64 rows of a
+// Y(I_t, c) = [Y +] sum_j op(D_t)(i, j) X(I_t(j), c) for every leaf t.  Block: 64 rows of a
 // leaf x 16 columns, K in steps of 32 staged in shared memory (both orders of D read
 // along its contiguous index); warp w owns row half w & 1 and columns w / 2, w / 2 +
 // 2, .. of the tile.  In FP64 it is bound by the FP64 pipe (64 cycles a warp FMA), so
@@ -152,7 +152,7 @@ constexpr int BD_COLS = 16;
 template <typename T>
 __global__ __launch_bounds__(128) void k_blockdiag_apply(
     const T* __restrict__ D, int nmax, int trans, const T* __restrict__ X, int64_t ldx,
-    T* __restrict__ Y, int64_t ldy, int64_t ncols, const int64_t* __restrict__ start,
+    T* __restrict__ Y, int64_t ldy, int64_t ncols, int add, const int64_t* __restrict__ start,
     const int64_t* __restrict__ size, int L) {
   __shared__ T Ds[32][65];  // [k][row]
   __shared__ T Xs[BD_COLS][33];
@@ -195,14 +195,10 @@ __global__ __launch_bounds__(128) void k_blockdiag_apply(
   if (i0 + rr < ns)
 #pragma unroll
     for (int j = 0; j < BD_COLS / 2; ++j)
-      if (j < nj) Y[s + i0 + rr + (c0 + g + 2 * j) * ldy] += acc[j];
-}
-
-template <typename T>
-__global__ void k_fill(T* p, int64_t count, T v) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count;
-       i += (int64_t)gridDim.x * blockDim.x)
-    p[i] = v;
+      if (j < nj) {
+        T* y = Y + s + i0 + rr + (c0 + g + 2 * j) * ldy;
+        *y = add ? *y + acc[j] : acc[j];
+      }
 }
 
 template <typename T>
@@ -330,20 +326,12 @@ void launch_extract_diag(const T* Y, int64_t ldy, T* D, int nmax, const int64_t*
 
 template <typename T>
 void launch_blockdiag_apply(const T* D, int nmax, int trans, const T* X, int64_t ldx, T* Y,
-                            int64_t ldy, int64_t ncols, const int64_t* d_start,
+                            int64_t ldy, int64_t ncols, int add, const int64_t* d_start,
                             const int64_t* d_size, int L, cudaStream_t st) {
   count_launches(1);
   dim3 grid(1u << L, (unsigned)((nmax + 63) / 64), (unsigned)((ncols + BD_COLS - 1) / BD_COLS));
-  k_blockdiag_apply<T><<<grid, 128, 0, st>>>(D, nmax, trans, X, ldx, Y, ldy, ncols, d_start,
-                                             d_size, L);
-}
-
-template <typename T>
-void launch_fill(T* p, int64_t count, T v, cudaStream_t st) {
-  if (count <= 0) return;
-  count_launches(1);
-  unsigned g = blocks_for(count, 256);
-  k_fill<T><<<g > 4096 ? 4096 : g, 256, 0, st>>>(p, count, v);
+  k_blockdiag_apply<T><<<grid, 128, 0, st>>>(D, nmax, trans, X, ldx, Y, ldy, ncols, add,
+                                             d_start, d_size, L);
 }
 
 template <typename T>
@@ -408,9 +396,8 @@ void launch_gen_log_kernel(float* A, int64_t n, int64_t lda, cudaStream_t st) {
   template void launch_extract_diag<T>(const T*, int64_t, T*, int, const int64_t*,          \
                                        const int64_t*, int, cudaStream_t);                  \
   template void launch_blockdiag_apply<T>(const T*, int, int, const T*, int64_t, T*,        \
-                                          int64_t, int64_t, const int64_t*, const int64_t*, \
+                                          int64_t, int64_t, int, const int64_t*, const int64_t*, \
                                           int, cudaStream_t);                               \
-  template void launch_fill<T>(T*, int64_t, T, cudaStream_t);                               \
   template void launch_copy_cols<T>(const T*, int64_t, T*, int64_t, int64_t, int64_t,       \
                                     cudaStream_t);                                          \
   template void launch_identity_cols<T>(T*, int64_t, int64_t, int64_t, int64_t,            \

@@ -8,6 +8,7 @@
 //    for computing the HBS-ID representation"): column-pivoted Householder QR
 //    (Businger-Golub, largest remaining column norm, lowest index on ties) and
 //    T = R11^{-1} [R11 R12] in FP64, one block per node.
+#include <algorithm>
 #include <atomic>
 
 #include "df.cuh"
@@ -113,122 +114,244 @@ __global__ __launch_bounds__(256) void k_batched_gemm_tiled(const GemmItem* __re
   }
 }
 
-// FP64 products (HM_FP64, and the applies of HM_A32 handles).  Bound by the FP64 pipe
-// (64 cycles a warp FMA): the outputs of a row segment (<= 64 rows of C) are dealt out
-// flat, M to a thread, so that no FMA goes to a column past n (a 32 x 32 tile wasted
-// two thirds of them at the 10 columns of an apply) and a level of a few items still
-// spreads over many SMs.  Operands staged in steps of 32 along k, each read along its
-// contiguous index; every output is one chain over p, as in k_batched_gemm.  Level of
-// 256 items, r = 60, 10 columns: 41 -> 17 us; 2 items: 41 -> 6 us.
+// One product op(A) B of a small-GEMM block: A (lda) m x k or its transpose, B (ldb)
+// k x n or its transpose.
+struct GemmSeg {
+  const double *A, *B;
+  int64_t lda, ldb;
+  int k, ta, tb;
+};
+
+// FP64 products (HM_FP64, and the applies of HM_A32 handles): C = sum over the segments
+// (1 or 2), times alpha, plus beta C.  Bound by the FP64 pipe (64 cycles a warp FMA):
+// the outputs of a row segment (<= 64 rows of C) are dealt out flat, M to a thread, so
+// that no FMA goes to a column past n (a 32 x 32 tile wasted two thirds of them at the
+// 10 columns of an apply) and a level of a few items still spreads over many SMs.
+// Operands staged in steps of 32 along k, each read along its contiguous index; every
+// product is one chain over p, as in k_batched_gemm.
 template <int M>
-__global__ __launch_bounds__(128) void k_batched_gemm64(const GemmItem* __restrict__ items,
-                                                        double alpha, double beta) {
+__device__ __forceinline__ void gemm64_block(const GemmSeg* seg, int nseg, int mtot, int n,
+                                             double* C, int64_t ldc, double alpha, double beta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const GemmItem it = items[blockIdx.x];
-  const int n = it.n, k = it.k, m0 = blockIdx.z * 64;
-  const int m = min(64, it.m - m0), mn = m * n, e0 = blockIdx.y * 128 * M;
+  const int m0 = blockIdx.z * 64;
+  const int m = min(64, mtot - m0), mn = m * n, e0 = blockIdx.y * 128 * M;
   if (m <= 0 || e0 >= mn) return;  // uniform over the block
-  const double* A = (const double*)it.A;
-  const double* B = (const double*)it.B;
   const int j0 = e0 / m, nb = (min(e0 + 128 * M, mn) - 1) / m - j0 + 1;
   const int pb = nb | 1;
   double* As = reinterpret_cast<double*>(smem_raw);  // [32][65]
   double* Bs = As + 32 * 65;                         // [32][pb]
   const int tid = threadIdx.x;
   int ia[M], jb[M];
-  double acc[M];
+  double tot[M];
 #pragma unroll
   for (int q = 0; q < M; ++q) {
     const int e = e0 + tid + 128 * q;
     ia[q] = e < mn ? e % m : 0;
     jb[q] = e < mn ? e / m - j0 : 0;
-    acc[q] = 0.0;
+    tot[q] = 0.0;
   }
-  for (int p0 = 0; p0 < k; p0 += 32) {
-    const int kp = min(32, k - p0);
-    if (it.ta) {
-      for (int e = tid; e < 32 * m; e += 128) {
-        const int p = e & 31, i = e >> 5;
-        if (p < kp) As[p * 65 + i] = A[p0 + p + (int64_t)(m0 + i) * it.lda];
+  for (int s = 0; s < nseg; ++s) {
+    const GemmSeg g = seg[s];
+    double acc[M] = {};
+    for (int p0 = 0; p0 < g.k; p0 += 32) {
+      const int kp = min(32, g.k - p0);
+      if (g.ta) {
+        for (int e = tid; e < 32 * m; e += 128) {
+          const int p = e & 31, i = e >> 5;
+          if (p < kp) As[p * 65 + i] = g.A[p0 + p + (int64_t)(m0 + i) * g.lda];
+        }
+      } else {
+        for (int e = tid; e < kp * 64; e += 128) {
+          const int i = e & 63, p = e >> 6;
+          if (i < m) As[p * 65 + i] = g.A[m0 + i + (int64_t)(p0 + p) * g.lda];
+        }
       }
-    } else {
-      for (int e = tid; e < kp * 64; e += 128) {
-        const int i = e & 63, p = e >> 6;
-        if (i < m) As[p * 65 + i] = A[m0 + i + (int64_t)(p0 + p) * it.lda];
+      for (int e = tid; e < 32 * nb; e += 128) {
+        const int p = g.tb ? e / nb : e & 31, j = g.tb ? e % nb : e >> 5;
+        if (p < kp)
+          Bs[p * pb + j] = g.tb ? g.B[j0 + j + (int64_t)(p0 + p) * g.ldb]
+                                : g.B[p0 + p + (int64_t)(j0 + j) * g.ldb];
       }
-    }
-    for (int e = tid; e < 32 * nb; e += 128) {
-      const int p = it.tb ? e / nb : e & 31, j = it.tb ? e % nb : e >> 5;
-      if (p < kp)
-        Bs[p * pb + j] = it.tb ? B[j0 + j + (int64_t)(p0 + p) * it.ldb]
-                               : B[p0 + p + (int64_t)(j0 + j) * it.ldb];
-    }
-    __syncthreads();
+      __syncthreads();
 #pragma unroll 4
-    for (int p = 0; p < kp; ++p)
+      for (int p = 0; p < kp; ++p)
 #pragma unroll
-      for (int q = 0; q < M; ++q) acc[q] = fma(As[p * 65 + ia[q]], Bs[p * pb + jb[q]], acc[q]);
-    __syncthreads();
+        for (int q = 0; q < M; ++q) acc[q] = fma(As[p * 65 + ia[q]], Bs[p * pb + jb[q]], acc[q]);
+      __syncthreads();
+    }
+#pragma unroll
+    for (int q = 0; q < M; ++q) tot[q] = s == 0 ? acc[q] : acc[q] + tot[q];
   }
 #pragma unroll
   for (int q = 0; q < M; ++q) {
     if (e0 + tid + 128 * q >= mn) continue;
-    double* c = (double*)it.C + m0 + ia[q] + (int64_t)(j0 + jb[q]) * it.ldc;
-    const double v = alpha == 1.0 ? acc[q] : alpha * acc[q];
+    double* c = C + m0 + ia[q] + (int64_t)(j0 + jb[q]) * ldc;
+    const double v = alpha == 1.0 ? tot[q] : alpha * tot[q];
     *c = (beta == 0.0) ? v : fma(beta, *c, v);
   }
 }
 
-// The FP64 form of k_batched_gemm_tiled in double-float on the FP32 pipe
-// (HM_A32): every input cut once, when staged, into hi + lo floats; each output
-// summed as a float pair (TwoProduct of the high parts, the cross terms, TwoSum).
-__global__ __launch_bounds__(256) void k_batched_gemm_tiled_df(const GemmItem* __restrict__ items,
-                                                               double alpha, double beta) {
+// The same in double-float on the FP32 pipe (HM_A32): a 32 x 32 tile of C per block,
+// every input cut once, when staged, into hi + lo floats; each output summed as a float
+// pair (TwoProduct of the high parts, the cross terms, TwoSum), the segments' sums added
+// in FP64.  (pitch kp odd: the staging writes along k fall on different banks.)
+__device__ __forceinline__ void gemm_df_block(const GemmSeg* seg, int nseg, int m, int n,
+                                              double* C, int64_t ldc, double alpha, double beta) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const GemmItem it = items[blockIdx.x];
-  const int m = it.m, n = it.n, k = it.k;
   const int j0 = blockIdx.y * 32, m0 = blockIdx.z * 32;
   if (j0 >= n || m0 >= m) return;  // uniform over the block
-  const double* A = (const double*)it.A;
-  const double* B = (const double*)it.B;
-  double* Cm = (double*)it.C;
-  float* Ah = reinterpret_cast<float*>(smem_raw);  // [32][k]: rows m0 .. m0 + 31 of op(A)
-  float* Al = Ah + 32 * k;
-  float* Bh = Al + 32 * k;                         // [k][32]: columns j0 .. j0 + 31 of op(B)
-  float* Bl = Bh + 32 * k;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < 32 * k; e += 256) {
-    const int ii = e / k, p = e % k, i = m0 + ii;
-    const double v = (i < m) ? (it.ta ? A[p + (int64_t)i * it.lda] : A[i + (int64_t)p * it.lda]) : 0.0;
-    df::split(v, Ah[e], Al[e]);
-  }
-  for (int e = tid; e < k * 32; e += 256) {
-    const int p = e >> 5, col = j0 + (e & 31);
-    const double v = (col < n) ? (it.tb ? B[col + (int64_t)p * it.ldb] : B[p + (int64_t)col * it.ldb])
-                               : 0.0;
-    df::split(v, Bh[e], Bl[e]);
-  }
-  __syncthreads();
-  const int j = tid & 31, i0 = tid >> 5;
-  float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-  for (int p = 0; p < k; ++p) {
-    const float bh = Bh[p * 32 + j], bl = Bl[p * 32 + j];
+  const int tid = threadIdx.x, j = tid & 31, i0 = tid >> 5;
+  double tot[4];
+  for (int s = 0; s < nseg; ++s) {
+    const GemmSeg g = seg[s];
+    const int k = g.k, kp = k | 1;
+    float2* As = reinterpret_cast<float2*>(smem_raw);  // [32][kp]: rows m0 .. of op(A)
+    float2* Bs = As + 32 * kp;                          // [32][kp]: columns j0 .. of op(B)
+    for (int e = tid; e < 32 * k; e += 256) {
+      // along the contiguous index of the operand
+      const int ia = g.ta ? e / k : e & 31, pa = g.ta ? e % k : e >> 5;
+      float2 v;
+      df::split(m0 + ia < m ? (g.ta ? g.A[pa + (int64_t)(m0 + ia) * g.lda]
+                                    : g.A[m0 + ia + (int64_t)pa * g.lda])
+                            : 0.0,
+                v.x, v.y);
+      As[ia * kp + pa] = v;
+      const int jb = g.tb ? e & 31 : e / k, pb = g.tb ? e >> 5 : e % k;
+      df::split(j0 + jb < n ? (g.tb ? g.B[j0 + jb + (int64_t)pb * g.ldb]
+                                    : g.B[pb + (int64_t)(j0 + jb) * g.ldb])
+                            : 0.0,
+                v.x, v.y);
+      Bs[jb * kp + pb] = v;
+    }
+    __syncthreads();
+    float sh[4] = {}, sl[4] = {};
+#pragma unroll 2
+    for (int p = 0; p < k; ++p) {
+      const float2 b = Bs[j * kp + p];
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
-      df::dot_acc(Ah[(i0 + 8 * q) * k + p], Al[(i0 + 8 * q) * k + p], bh, bl, sh[q], sl[q]);
+      for (int q = 0; q < 4; ++q) {
+        const float2 a = As[(i0 + 8 * q) * kp + p];
+        df::dot_acc(a.x, a.y, b.x, b.y, sh[q], sl[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const double v = df::join(sh[q], sl[q]);
+      tot[q] = s == 0 ? v : v + tot[q];
+    }
+    __syncthreads();
   }
-  const int col = j0 + j;
-  if (col < n) {
+  if (j0 + j < n) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int i = m0 + i0 + 8 * q;
-      if (i < m) {
-        double* c = Cm + i + (int64_t)col * it.ldc;
-        const double a = df::join(sh[q], sl[q]);
-        *c = (beta == 0.0) ? alpha * a : alpha * a + beta * (*c);
-      }
+      if (i >= m) continue;
+      double* c = C + i + (int64_t)(j0 + j) * ldc;
+      const double v = alpha == 1.0 ? tot[q] : alpha * tot[q];
+      *c = (beta == 0.0) ? v : fma(beta, *c, v);
     }
   }
+}
+
+template <int M>
+__global__ __launch_bounds__(128) void k_batched_gemm64(const GemmItem* __restrict__ items,
+                                                        double alpha, double beta) {
+  const GemmItem it = items[blockIdx.x];
+  const GemmSeg g{(const double*)it.A, (const double*)it.B, it.lda, it.ldb, it.k, it.ta, it.tb};
+  gemm64_block<M>(&g, 1, it.m, it.n, (double*)it.C, it.ldc, alpha, beta);
+}
+__global__ __launch_bounds__(256) void k_batched_gemm_tiled_df(const GemmItem* __restrict__ items,
+                                                               double alpha, double beta) {
+  const GemmItem it = items[blockIdx.x];
+  const GemmSeg g{(const double*)it.A, (const double*)it.B, it.lda, it.ldb, it.k, it.ta, it.tb};
+  gemm_df_block(&g, 1, it.m, it.n, (double*)it.C, it.ldc, alpha, beta);
+}
+
+// A level's products with the operands of node x found here (see NodeGemm).  One launch
+// a level and direction: as item lists built on the host and copied over, a level took
+// two launches and two copies, and the levels' products waited for the host (HBS-ID
+// apply, N = 65536, 10 columns, both directions: 2.57 -> 1.07 ms).
+__device__ __forceinline__ int node_segs(const NodeGemm& a, GemmSeg* g, int& m, double*& C,
+                                         int64_t& ldc) {
+  const int x = a.node0 + blockIdx.x, r = a.r;
+  const int64_t rr = (int64_t)r * r, rw = (int64_t)r * a.w;
+  m = r;
+  ldc = r;
+  g[0].lda = g[1].lda = r;
+  g[0].ldb = g[1].ldb = r;
+  g[0].k = g[1].k = r;
+  g[0].ta = g[1].ta = a.ta0;
+  g[0].tb = g[1].tb = 0;
+  switch (a.mode) {
+    case NodeGemm::kUp:
+      for (int h = 0; h < 2; ++h) {
+        g[h].A = a.A0 + (2 * x + h) * rr;
+        g[h].B = a.q + (2 * x + h) * rw;
+      }
+      C = a.q + x * rw;
+      return 2;
+    case NodeGemm::kDown:
+      g[0].A = a.A0 + (a.ta0 ? x ^ 1 : x) * rr;
+      g[0].B = a.q + (x ^ 1) * rw;
+      C = a.u + x * rw;
+      if (!a.A1) return 1;
+      g[1].A = a.A1 + x * rr;
+      g[1].ta = a.ta1;
+      g[1].B = a.u + (x >> 1) * rw;
+      return 2;
+    case NodeGemm::kLeafUp:
+      g[0].A = a.A0 + (int64_t)blockIdx.x * r * a.nmax;
+      g[0].B = a.X + a.start[x];
+      g[0].ldb = a.ldx;
+      g[0].k = (int)a.size[x];
+      C = a.q + x * rw;
+      return 1;
+    case NodeGemm::kLeafDown:
+      g[0].A = a.A0 + (int64_t)blockIdx.x * r * a.nmax;
+      g[0].ta = 1;
+      g[0].B = a.u + x * rw;
+      m = (int)a.size[x];
+      C = a.Y + a.start[x];
+      ldc = a.ldy;
+      return 1;
+    default: {  // kSolve
+      const int c = blockIdx.x & 1;
+      const double* Mp = a.A0 + (int64_t)(blockIdx.x >> 1) * 4 * rr;
+      const double *qa = a.q + (int64_t)(blockIdx.x - c) * rw, *qb = qa + rw;
+      g[0].lda = g[1].lda = 2 * r;
+      if (!a.ta0) {  // child c: M(c r .., 0 .. r) q_b + M(c r .., r .. 2r) q_a
+        g[0].A = Mp + c * r;
+        g[0].B = qb;
+        g[1].A = Mp + c * r + 2 * rr;
+        g[1].B = qa;
+      } else {  // child a: columns r .. 2r of M, child b: columns 0 .. r, transposed
+        const double* Mc = Mp + (c ? 0 : 2 * rr);
+        g[0].A = Mc;
+        g[0].B = qa;
+        g[1].A = Mc + r;
+        g[1].B = qb;
+      }
+      C = a.u + (int64_t)blockIdx.x * rw;
+      return 2;
+    }
+  }
+}
+template <int M>
+__global__ __launch_bounds__(128) void k_node_gemm64(const __grid_constant__ NodeGemm a) {
+  GemmSeg g[2];
+  int m;
+  double* C;
+  int64_t ldc;
+  const int ns = node_segs(a, g, m, C, ldc);
+  gemm64_block<M>(g, ns, m, a.w, C, ldc, 1.0, 0.0);
+}
+__global__ __launch_bounds__(256) void k_node_gemm_df(const __grid_constant__ NodeGemm a) {
+  GemmSeg g[2];
+  int m;
+  double* C;
+  int64_t ldc;
+  const int ns = node_segs(a, g, m, C, ldc);
+  gemm_df_block(g, ns, m, a.w, C, ldc, 1.0, 0.0);
 }
 
 // dst[(node0 + i) ^ flip] (rows x cols, ld dld) = src[i] (ld sld); heap-indexed dst.
@@ -585,47 +708,88 @@ void launch_gather_parent_scaled(const T* U, int64_t ldu, T* P, int64_t ldp, int
   k_gather_parent_scaled<T><<<grid, 256, 0, st>>>(U, ldu, P, ldp, n, r, lv, d_start, y, col0);
 }
 
+// Launch shape of the FP64 form: outputs per thread four once the items alone give
+// every scheduler several warps.  A block may touch as many columns of B as it has
+// outputs (items of a single row).
+template <typename F1, typename F4>
+static void gemm64_shape(int count, int max_m, int max_n, F1 run1, F4 run4) {
+  const int ms = std::min(max_m, 64);
+  const int mq = ((int64_t)count * max_m * max_n / 32 >= 16 * 608 && max_n <= 512) ? 4 : 1;
+  const int nb = std::min(max_n, 128 * mq + 1);
+  const dim3 grid((unsigned)count, (unsigned)((ms * max_n + 128 * mq - 1) / (128 * mq)),
+                  (unsigned)((max_m + 63) / 64));
+  const size_t smem = (size_t)32 * (65 + (nb | 1)) * sizeof(double);
+  if (mq == 4) run4(grid, smem);
+  else run1(grid, smem);
+}
+
 template <typename T>
 void launch_batched_gemm(const GemmItem* items, int count, T alpha, T beta, cudaStream_t st,
                          int max_m, int max_n, int max_k, bool df) {
   if (count <= 0) return;
   count_launches(1);
-  const size_t smem = (size_t)64 * max_k * sizeof(T);
-  if (max_m >= 1 && max_n >= 1 && max_k >= 1 && smem <= 96 * 1024 && max_n <= 32 * 65535 &&
-      max_m <= 32 * 65535 && sizeof(T) == 8 && df) {
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_batched_gemm_tiled_df, done);
-    dim3 grid((unsigned)count, (unsigned)((max_n + 31) / 32), (unsigned)((max_m + 31) / 32));
-    k_batched_gemm_tiled_df<<<grid, 256, smem, st>>>(items, (double)alpha, (double)beta);
-  } else if (sizeof(T) == 8 && max_m >= 1 && max_n >= 1 && max_k >= 1 && max_m <= 64 * 65535 &&
-             (int64_t)std::min(max_m, 64) * max_n <= 128 * (int64_t)65535) {
-    // outputs per thread: four once the items alone give every scheduler several warps
-    const int ms = std::min(max_m, 64);
-    auto run = [&](auto kern, int mq) {
-      // columns of B a block may touch: items of fewer rows than max_m touch more
-      const int nb = std::min(max_n, 128 * mq + 1);
-      const dim3 grid((unsigned)count, (unsigned)((ms * max_n + 128 * mq - 1) / (128 * mq)),
-                      (unsigned)((max_m + 63) / 64));
-      kern<<<grid, 128, (size_t)32 * (65 + (nb | 1)) * sizeof(double), st>>>(items, (double)alpha,
-                                                                           (double)beta);
-    };
-    static std::atomic<uint32_t> d1{0}, d4{0};
-    if ((int64_t)count * max_m * max_n / 32 >= 16 * 608 && max_n <= 512) {
-      raise_smem_limit((const void*)k_batched_gemm64<4>, d4);
-      run(k_batched_gemm64<4>, 4);
-    } else {
-      raise_smem_limit((const void*)k_batched_gemm64<1>, d1);
-      run(k_batched_gemm64<1>, 1);
+  const size_t smem = (size_t)64 * (max_k | 1) * sizeof(T);
+  const bool any = max_m >= 1 && max_n >= 1 && max_k >= 1;
+  const bool tiles = any && smem <= 96 * 1024 && max_n <= 32 * 65535 && max_m <= 32 * 65535;
+  if constexpr (sizeof(T) == 8) {
+    if (df && tiles) {
+      static std::atomic<uint32_t> done{0};
+      raise_smem_limit((const void*)k_batched_gemm_tiled_df, done);
+      dim3 grid((unsigned)count, (unsigned)((max_n + 31) / 32), (unsigned)((max_m + 31) / 32));
+      k_batched_gemm_tiled_df<<<grid, 256, smem, st>>>(items, alpha, beta);
+      return;
     }
-  } else if (max_m >= 1 && max_n >= 1 && max_k >= 1 && smem <= 96 * 1024 &&
-             max_n <= 32 * 65535 && max_m <= 32 * 65535) {
+    if (any && max_m <= 64 * 65535 &&
+        (int64_t)std::min(max_m, 64) * max_n <= 128 * (int64_t)65535) {
+      gemm64_shape(
+          count, max_m, max_n,
+          [&](dim3 grid, size_t sm) {
+            static std::atomic<uint32_t> done{0};
+            raise_smem_limit((const void*)k_batched_gemm64<1>, done);
+            k_batched_gemm64<1><<<grid, 128, sm, st>>>(items, alpha, beta);
+          },
+          [&](dim3 grid, size_t sm) {
+            static std::atomic<uint32_t> done{0};
+            raise_smem_limit((const void*)k_batched_gemm64<4>, done);
+            k_batched_gemm64<4><<<grid, 128, sm, st>>>(items, alpha, beta);
+          });
+      return;
+    }
+  } else if (tiles) {
     static std::atomic<uint32_t> done{0};
     raise_smem_limit((const void*)k_batched_gemm_tiled<T>, done);
     dim3 grid((unsigned)count, (unsigned)((max_n + 31) / 32), (unsigned)((max_m + 31) / 32));
     k_batched_gemm_tiled<T><<<grid, 256, smem, st>>>(items, alpha, beta);
-  } else {
-    k_batched_gemm<T><<<count, 256, 0, st>>>(items, alpha, beta);
+    return;
   }
+  k_batched_gemm<T><<<count, 256, 0, st>>>(items, alpha, beta);
+}
+
+// r <= 128 and w <= 128 here (panel widths and column blocks); leaf rows are segmented.
+void launch_node_gemm(const NodeGemm& a, int nodes, cudaStream_t st, bool df) {
+  if (nodes <= 0) return;
+  count_launches(1);
+  const int max_m = a.mode == NodeGemm::kLeafDown ? a.nmax : a.r;
+  if (df) {
+    static std::atomic<uint32_t> done{0};
+    raise_smem_limit((const void*)k_node_gemm_df, done);
+    const int k = a.mode == NodeGemm::kLeafUp ? a.nmax : a.r;
+    const dim3 grid((unsigned)nodes, (unsigned)((a.w + 31) / 32), (unsigned)((max_m + 31) / 32));
+    k_node_gemm_df<<<grid, 256, (size_t)64 * (k | 1) * sizeof(float2), st>>>(a);
+    return;
+  }
+  gemm64_shape(
+      nodes, max_m, a.w,
+      [&](dim3 grid, size_t sm) {
+        static std::atomic<uint32_t> done{0};
+        raise_smem_limit((const void*)k_node_gemm64<1>, done);
+        k_node_gemm64<1><<<grid, 128, sm, st>>>(a);
+      },
+      [&](dim3 grid, size_t sm) {
+        static std::atomic<uint32_t> done{0};
+        raise_smem_limit((const void*)k_node_gemm64<4>, done);
+        k_node_gemm64<4><<<grid, 128, sm, st>>>(a);
+      });
 }
 
 template <typename TS, typename TD>
