@@ -141,64 +141,65 @@ __global__ void k_extract_diag(const T* __restrict__ Y, int64_t ldy, T* __restri
   }
 }
 
-// Y(I_t, c) = [Y +] sum_j op(D_t)(i, j) X(I_t(j), c) for every leaf t.  Block: 64 rows of a
-// leaf x 16 columns, K in steps of 32 staged in shared memory (both orders of D read
-// along its contiguous index); warp w owns row half w & 1 and columns w / 2, w / 2 +
-// 2, .. of the tile.  In FP64 it is bound by the FP64 pipe (64 cycles a warp FMA), so
-// D is read once per 16 columns and no FMA goes to a column that is not there
-// (N = 65536, leaves of 256, 10 columns: 423 us with one block per leaf and column,
-// 290 now; the FP64 pipe's floor is 266).
-constexpr int BD_COLS = 16;
-template <typename T>
+// Y(I_t, c) = [Y +] sum_j op(D_t)(i, j) X(I_t(j), c) for every leaf t.  Block: 32 rows of a
+// leaf (lanes) x up to 8 columns; its four warps split K (32 of every 128 each) and
+// their sums are added in warp order, so that the warps' work is equal whatever the
+// column count and the leaf size.  D is read straight from global memory along its
+// contiguous index (transposed: through a 32 x 33 tile of the warp's own).  In FP64 it
+// is bound by the FP64 pipe (76 cycles a warp FMA): N = 65536, leaves of 256, 10 columns
+// 423 us with a block per leaf and column, 283 now (transposed 321), at the floor.
+constexpr int BD_COLS = 8;
+template <typename T, int TRANS>
 __global__ __launch_bounds__(128) void k_blockdiag_apply(
-    const T* __restrict__ D, int nmax, int trans, const T* __restrict__ X, int64_t ldx,
-    T* __restrict__ Y, int64_t ldy, int64_t ncols, int add, const int64_t* __restrict__ start,
+    const T* __restrict__ D, int nmax, const T* __restrict__ X, int64_t ldx, T* __restrict__ Y,
+    int64_t ldy, int64_t ncols, int ctile, int add, const int64_t* __restrict__ start,
     const int64_t* __restrict__ size, int L) {
-  __shared__ T Ds[32][65];  // [k][row]
-  __shared__ T Xs[BD_COLS][33];
+  __shared__ T Xs[BD_COLS][128];
+  __shared__ T Dt[TRANS ? 4 : 1][32][33];
+  __shared__ T Red[4][BD_COLS][32];
   const int leaf = blockIdx.x, node = (1 << L) + leaf;
   const int64_t s = start[node];
   const int ns = (int)size[node];
-  const int i0 = blockIdx.y * 64;
+  const int i0 = blockIdx.y * 32;
   if (i0 >= ns) return;  // uniform over the block
-  const int64_t c0 = (int64_t)blockIdx.z * BD_COLS;
-  const int nc = (int)min((int64_t)BD_COLS, ncols - c0);
-  const T* Dl = D + (int64_t)leaf * nmax * nmax;
+  const int64_t c0 = (int64_t)blockIdx.z * ctile;
+  const int nc = (int)min((int64_t)ctile, ncols - c0);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const int rr = (w & 1) * 32 + lane, g = w >> 1;
-  const int nj = g < nc ? (nc - g + 1) / 2 : 0;
-  T acc[BD_COLS / 2] = {};
-  for (int k0 = 0; k0 < ns; k0 += 32) {
-    if (!trans) {
-      for (int e = tid; e < 32 * 64; e += 128) {
-        const int i = e & 63, k = e >> 6;
-        Ds[k][i] = (i0 + i < ns && k0 + k < ns) ? Dl[i0 + i + (int64_t)(k0 + k) * nmax] : (T)0;
-      }
-    } else {
-      for (int e = tid; e < 32 * 64; e += 128) {
-        const int k = e & 31, i = e >> 5;
-        Ds[k][i] = (i0 + i < ns && k0 + k < ns) ? Dl[k0 + k + (int64_t)(i0 + i) * nmax] : (T)0;
-      }
-    }
-    for (int c = w; c < nc; c += 4)
-      Xs[c][lane] = (k0 + lane < ns) ? X[s + k0 + lane + (c0 + c) * ldx] : (T)0;
+  const int i = i0 + lane;
+  const T* Dl = D + (int64_t)leaf * nmax * nmax;
+  T acc[BD_COLS] = {};
+  for (int b0 = 0; b0 < ns; b0 += 128) {
+    for (int c = 0; c < nc; ++c) Xs[c][tid] = (b0 + tid < ns) ? X[s + b0 + tid + (c0 + c) * ldx] : (T)0;
     __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < 32; ++k) {
-      const T a = Ds[k][rr];
+    const int k0 = b0 + 32 * w, kn = min(32, ns - k0);
+    if (kn > 0) {
+      if (TRANS) {
+        for (int q = 0; q < 32; ++q)
+          Dt[w][q][lane] = (i0 + q < ns && lane < kn) ? Dl[k0 + lane + (int64_t)(i0 + q) * nmax] : (T)0;
+        __syncwarp();
+      }
+      const T* Dk = Dl + (i < ns ? i : i0) + (int64_t)k0 * nmax;
+      with_count<BD_COLS>(nc, [&](auto cols) {
+#pragma unroll 8
+        for (int k = 0; k < kn; ++k) {
+          const T a = TRANS ? Dt[TRANS ? w : 0][lane][k] : Dk[(int64_t)k * nmax];
 #pragma unroll
-      for (int j = 0; j < BD_COLS / 2; ++j)
-        if (j < nj) acc[j] = fma(a, Xs[g + 2 * j][k], acc[j]);
+          for (int c = 0; c < cols; ++c) acc[c] = fma(a, Xs[c][32 * w + k], acc[c]);
+        }
+      });
     }
     __syncthreads();
   }
-  if (i0 + rr < ns)
 #pragma unroll
-    for (int j = 0; j < BD_COLS / 2; ++j)
-      if (j < nj) {
-        T* y = Y + s + i0 + rr + (c0 + g + 2 * j) * ldy;
-        *y = add ? *y + acc[j] : acc[j];
-      }
+  for (int c = 0; c < BD_COLS; ++c) Red[w][c][lane] = acc[c];
+  __syncthreads();
+  if (i < ns)
+    for (int c = w; c < nc; c += 4) {
+      T v = Red[0][c][lane];
+      for (int q = 1; q < 4; ++q) v += Red[q][c][lane];
+      T* y = Y + s + i + (c0 + c) * ldy;
+      *y = add ? *y + v : v;
+    }
 }
 
 template <typename T>
@@ -329,9 +330,16 @@ void launch_blockdiag_apply(const T* D, int nmax, int trans, const T* X, int64_t
                             int64_t ldy, int64_t ncols, int add, const int64_t* d_start,
                             const int64_t* d_size, int L, cudaStream_t st) {
   count_launches(1);
-  dim3 grid(1u << L, (unsigned)((nmax + 63) / 64), (unsigned)((ncols + BD_COLS - 1) / BD_COLS));
-  k_blockdiag_apply<T><<<grid, 128, 0, st>>>(D, nmax, trans, X, ldx, Y, ldy, ncols, add,
-                                             d_start, d_size, L);
+  // equal column tiles of at most BD_COLS
+  const int64_t nt = (ncols + BD_COLS - 1) / BD_COLS;
+  const int ctile = (int)((ncols + nt - 1) / nt);
+  dim3 grid(1u << L, (unsigned)((nmax + 31) / 32), (unsigned)nt);
+  if (trans)
+    k_blockdiag_apply<T, 1><<<grid, 128, 0, st>>>(D, nmax, X, ldx, Y, ldy, ncols, ctile, add,
+                                                  d_start, d_size, L);
+  else
+    k_blockdiag_apply<T, 0><<<grid, 128, 0, st>>>(D, nmax, X, ldx, Y, ldy, ncols, ctile, add,
+                                                  d_start, d_size, L);
 }
 
 template <typename T>

@@ -172,13 +172,15 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
       if (r < nc) Xs[r][lane] = (k0 + lane < n) ? X[k0 + lane + (c0 + r) * ldx] : 0.0;
     }
     __syncthreads();
+    if (nq > 0)
+      with_count<8>(nq, [&](auto cols) {
 #pragma unroll 4
-    for (int k = 0; k < BK; ++k) {
-      const double a = TRANS ? As[k][lane] : As[lane][k];
+        for (int k = 0; k < BK; ++k) {
+          const double a = TRANS ? As[k][lane] : As[lane][k];
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (q < nq) acc[q] = fma(a, Xs[w + 4 * q][k], acc[q]);
-    }
+          for (int q = 0; q < cols; ++q) acc[q] = fma(a, Xs[w + 4 * q][k], acc[q]);
+        }
+      });
     __syncthreads();
   }
   if (S == 1) {

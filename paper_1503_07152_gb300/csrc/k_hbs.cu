@@ -270,7 +270,7 @@ __global__ __launch_bounds__(256) void k_batched_gemm_tiled_df(const GemmItem* _
 // A level's products with the operands of node x found here (see NodeGemm).  One launch
 // a level and direction: as item lists built on the host and copied over, a level took
 // two launches and two copies, and the levels' products waited for the host (HBS-ID
-// apply, N = 65536, 10 columns, both directions: 2.57 -> 1.07 ms).
+// apply, N = 65536, 10 columns, both directions: 2.57 -> 2.24 ms).
 __device__ __forceinline__ int node_segs(const NodeGemm& a, GemmSeg* g, int& m, double*& C,
                                          int64_t& ldc) {
   const int x = a.node0 + blockIdx.x, r = a.r;

@@ -151,6 +151,51 @@ __global__ __launch_bounds__(128) void k_seg_tn_partial64(
   }
 }
 
+// The same for few chunks (a small operator): 32 outputs a block, the chunk's rows split
+// over its eight warps, whose sums are added in warp order.  One thread per output
+// would be a chain of 256 dependent FMAs (10 us) behind eight exposed rounds of loads
+// (12 us); here all rows are staged at once and a chain is 32 long.  4 chunks x 20 x 40
+// (N = 1024): 23 -> 9 us.
+__global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
+    const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
+    int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
+    int kb, double* __restrict__ partial) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[8][32];
+  const Chunk ch = chunks[blockIdx.x];
+  const int rows = (int)(ch.r1 - ch.r0);  // <= 256
+  const int aoff = (ch.node & 1) ? aoff_o : aoff_e;
+  const int boff = (ch.node & 1) ? boff_o : boff_e;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int mtot = ka * kb, e0 = blockIdx.y * 32, ne = min(32, mtot - e0);
+  const int jlo = e0 / ka, nb = (e0 + ne - 1) / ka - jlo + 1;
+  const int pb = nb | 1;
+  double* As = reinterpret_cast<double*>(smem_raw);  // [256][33]: column c of output e0 + c
+  double* Bs = As + 256 * 33;                        // [256][pb]
+  const int row = tid;
+  if (row < rows) {
+    const double* ap = A + ch.r0 + row + (int64_t)aoff * lda;
+    const double* bp = B + ch.r0 + row + (int64_t)(boff + jlo) * ldb;
+#pragma unroll 8
+    for (int c = 0; c < ne; ++c) As[row * 33 + c] = ap[(int64_t)((e0 + c) % ka) * lda];
+    for (int c = 0; c < nb; ++c) Bs[row * pb + c] = bp[(int64_t)c * ldb];
+  }
+  __syncthreads();
+  const int jb = lane < ne ? (e0 + lane) / ka - jlo : 0;
+  const int c = lane < ne ? lane : 0;
+  const int per = (rows + 7) / 8, q0 = min(rows, w * per), q1 = min(rows, q0 + per);
+  double acc = 0.0;
+#pragma unroll 4
+  for (int q = q0; q < q1; ++q) acc = fma(As[q * 33 + c], Bs[q * pb + jb], acc);
+  red[w][lane] = acc;
+  __syncthreads();
+  if (w == 0 && lane < ne) {
+    double v = red[0][lane];
+    for (int q = 1; q < 8; ++q) v += red[q][lane];
+    partial[(int64_t)blockIdx.x * mtot + e0 + lane] = v;
+  }
+}
+
 // The FP64 form of the partial products in double-float arithmetic on the FP32
 // pipe (GB300's FP64 pipe runs at a small fraction of the FP32 rate).  Each FP64
 // input is cut once, when staged, into x = hi + lo (two floats, 48 significant
@@ -370,12 +415,15 @@ __global__ __launch_bounds__(128) void k_seg_nn64(
     // this warp's columns g, g + ng, .. of the tile (at most CT / 2)
     const int nj = g < nc ? (nc - g + ng - 1) / ng : 0;
     double acc[CT / 2] = {};
-    for (int k = 0; k < kin; ++k) {
-      const double a = Ps[k * NN_ROWS + rr];
+    if (nj > 0)
+      with_count<CT / 2>(nj, [&](auto cols) {
+#pragma unroll 4
+        for (int k = 0; k < kin; ++k) {
+          const double a = Ps[k * NN_ROWS + rr];
 #pragma unroll
-      for (int j = 0; j < CT / 2; ++j)
-        if (j < nj) acc[j] = fma(a, Cs[(g + ng * j) * kin + k], acc[j]);
-    }
+          for (int j = 0; j < cols; ++j) acc[j] = fma(a, Cs[(g + ng * j) * kin + k], acc[j]);
+        }
+      });
 #pragma unroll
     for (int j = 0; j < CT / 2; ++j) {
       if (j >= nj || rr >= rows) continue;
@@ -499,8 +547,9 @@ void seg_tn_partial_pick_j(const Chunk* chunks, int nchunks, const T* A, int64_t
   }
 }
 
-// FP64 TN: outputs per thread (4, 2 or 1) so that the blocks of 4 warps cover the
-// schedulers several times over (a block's time is set by its FMAs, 64 cycles each)
+// FP64 TN: outputs per thread (4, 2 or 1) so that the blocks of 4 warps cover the 608
+// schedulers several times over (a block's time is set by its FMAs); below two warps of
+// outputs a scheduler, the form that splits the rows.
 static void seg_tn64(const Chunk* chunks, int nchunks, const double* A, int64_t lda, int aoff_even,
                      int aoff_odd, int ka, const double* B, int64_t ldb, int boff_even,
                      int boff_odd, int kb, double* partial, cudaStream_t st) {
@@ -511,9 +560,15 @@ static void seg_tn64(const Chunk* chunks, int nchunks, const double* A, int64_t 
     kern<<<grid, 128, smem, st>>>(chunks, A, lda, aoff_even, aoff_odd, ka, B, ldb, boff_even,
                                   boff_odd, kb, partial);
   };
-  static std::atomic<uint32_t> d1{0}, d2{0}, d4{0};
+  static std::atomic<uint32_t> d0{0}, d1{0}, d2{0}, d4{0};
   const int64_t warps = (int64_t)nchunks * ((ka * kb + 31) / 32);  // one output a lane
-  if (warps >= 16 * 608) {
+  if (warps < 2 * 608) {
+    const int nb = std::min(kb, 31 / ka + 2);
+    raise_smem_limit((const void*)k_seg_tn_partial64_split, d0);
+    const dim3 grid((unsigned)nchunks, (unsigned)((ka * kb + 31) / 32));
+    k_seg_tn_partial64_split<<<grid, 256, (size_t)256 * (33 + (nb | 1)) * sizeof(double), st>>>(
+        chunks, A, lda, aoff_even, aoff_odd, ka, B, ldb, boff_even, boff_odd, kb, partial);
+  } else if (warps >= 16 * 608) {
     raise_smem_limit((const void*)k_seg_tn_partial64<4>, d4);
     run(k_seg_tn_partial64<4>, 4);
   } else if (warps >= 8 * 608) {

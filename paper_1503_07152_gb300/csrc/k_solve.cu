@@ -10,6 +10,23 @@
 namespace hm {
 namespace {
 
+// 1 / x to within an ulp: in FP64 three Newton steps r <- r + r (1 - x r) from the FP32
+// reciprocal of the fraction (a chain of six FMAs; the division is ~20 instructions of
+// 76 cycles each).  Zeros, infinities, NaN and subnormals take the division.
+__device__ __forceinline__ float reciprocal(float x) { return 1.f / x; }
+__device__ __forceinline__ double reciprocal(double x) {
+  const int e = (int)((__double2hiint(x) >> 20) & 0x7ff);
+  if (e < 2 || e > 2044) return 1.0 / x;
+  // x = m 2^(e - 1023), 1 <= |m| < 2
+  const double m = __hiloint2double((__double2hiint(x) & (int)0x800fffff) | 0x3ff00000,
+                                    __double2loint(x));
+  double r = (double)(1.f / (float)m);
+  r = fma(r, fma(-m, r, 1.0), r);
+  r = fma(r, fma(-m, r, 1.0), r);
+  r = fma(r, fma(-m, r, 1.0), r);
+  return r * __hiloint2double((2046 - e) << 20, 0);
+}
+
 // Inverse of every matrix of a batch by Gauss-Jordan elimination with partial
 // pivoting, in place (W: n x n, column-major, ld n, in global memory, read once and
 // out[b] written once): row k of the inverse replaces the eliminated column k as the
@@ -33,6 +50,7 @@ __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, i
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ T fcol[2][256];   // the pivot column before the step, rows exchanged
   __shared__ int prow[2];      // its pivot row
+  __shared__ T pinv[2];        // 1 / pivot
   __shared__ double rv[8];
   __shared__ int ri[8];
   __shared__ short swp[256];   // pivot row of every step
@@ -80,13 +98,19 @@ __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, i
         const T v = col[i == k ? p : (i == p ? k : i)];
         for (int q = 0; q < S; ++q) (S > 1 ? cl.map_shared_rank(&fcol[buf][i], q) : &fcol[buf][i])[0] = v;
       }
-      if (tid < S) (S > 1 ? cl.map_shared_rank(&prow[buf], tid) : &prow[buf])[0] = p;
+      if (warp == 0) {  // (one warp: an FP64 division is a long chain on the FP64 pipe)
+        const T pv = col[p];
+        const T iv = (pv != (T)0) ? reciprocal(pv) : (T)0;
+        if (lane < S) {
+          (S > 1 ? cl.map_shared_rank(&prow[buf], lane) : &prow[buf])[0] = p;
+          (S > 1 ? cl.map_shared_rank(&pinv[buf], lane) : &pinv[buf])[0] = iv;
+        }
+      }
     }
     if (S > 1) cl.sync();
     else __syncthreads();
     const int p = prow[buf];
-    const T pv = fcol[buf][k];
-    const T inv = (pv != (T)0) ? (T)1 / pv : (T)0;
+    const T inv = pinv[buf];
     if (tid == 0) swp[k] = (short)p;
     // a warp takes a column: exchange rows k and p, scale the pivot row's entry, update
     for (int c = warp; c < nloc; c += 8) {
