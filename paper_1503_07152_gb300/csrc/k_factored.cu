@@ -2,13 +2,16 @@
 // sibling matrices B = I) and its hand-written adjoint (vector-Jacobian product
 // for x, U, V, D; with r = H x - b and scale 2, the gradients of ||H x - b||^2).
 //
-// Both are HBM-streaming: every factor byte is read once (and every gradient
-// byte written once).  Pass 1 reduces t_node = V(I_node)^T x(I_node) (and
-// s_node = U(I_node)^T res(I_node) for the adjoint) over 256-row chunks of all
-// levels; pass 2 reduces the chunk partials per node in a fixed order; pass 3
-// runs one block per leaf: every row of the leaf gathers the contributions of
-// its L ancestors' siblings (ancestor of leaf l on level j = l >> (L - j)) and
-// of the leaf block D, and, for the adjoint, writes the gradient rows.
+// All are HBM-streaming.  Pass 1 reduces t_node = V(I_node)^T x(I_node) (and s_node =
+// U(I_node)^T res(I_node) for the adjoint) over 256-row chunks of all levels; pass 2
+// reduces the chunk partials per node in a fixed order; pass 3 runs one block per tile
+// of a leaf's rows: every row gathers the contributions of its L ancestors' siblings
+// (ancestor of leaf l on level j = l >> (L - j)) and of the leaf block D, and, for
+// the adjoint, writes the gradient rows.  The fused step (loss_grad) forms the tile's
+// share of s and of D^T res and the gradient of D in the forward's block too, from the
+// tile's rows of U in shared memory and its rows of D in L2, so that U and D are read
+// from HBM once.
+#include <algorithm>
 #include <atomic>
 #include <string>
 
@@ -20,10 +23,11 @@ namespace {
 constexpr int kMaxK = 64;
 
 // partial[chunk][0:k] = V_j(rows)^T x(rows); with second operand pair for the
-// adjoint: partial[chunk][k:2k] = U_j(rows)^T res(rows).  Thread t loads row t's k
-// factor entries at once (independent, coalesced loads), the products go to
-// shared memory (row-major, stride k + 1: conflict-free both ways), thread
-// (col, part) sums its 32-row part of a column, and the 8 parts are added.
+// adjoint: partial[chunk][k:2k] = U_j(rows)^T res(rows).  A chunk has at most 256 rows:
+// a lane holds eight entries of the vector, a warp takes every eighth column and sums
+// its 256 entries (coalesced loads, all of a column's in flight) over the warp.
+// N = 262144, k = 32, 335 MB: 70 us (4.8 TB/s),
+// no shared memory; the products transposed through shared memory took the same time.
 __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restrict__ ch,
                                                       int64_t n, int k,
                                                       const float* __restrict__ A0,
@@ -31,53 +35,64 @@ __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restric
                                                       const float* __restrict__ A1,
                                                       const float* __restrict__ v1,
                                                       float* __restrict__ partial) {
-  extern __shared__ float prod[];  // [256][k + 1]
-  __shared__ float red[8][2 * kMaxK];
   const FactChunk c = ch[blockIdx.x];
-  const int tid = threadIdx.x;
-  const int ldp = k + 1;
-  const int64_t row = c.r0 + tid;
-  const bool live = row < c.r1;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int rows = (int)(c.r1 - c.r0);
   const int npair = A1 ? 2 : 1;
-  const int cl = tid & 31, part = tid >> 5;
   for (int p = 0; p < npair; ++p) {
-    const float* A = (p == 0 ? A0 : A1) + (int64_t)(c.level - 1) * n * k;
-    const float xv = live ? (p == 0 ? v0 : v1)[row] : 0.f;
-#pragma unroll 8
-    for (int col = 0; col < k; ++col)
-      prod[tid * ldp + col] = live ? A[row + (int64_t)col * n] * xv : 0.f;
-    __syncthreads();
-    for (int col = cl; col < k; col += 32) {
+    const float* A = (p == 0 ? A0 : A1) + (int64_t)(c.level - 1) * n * k + c.r0;
+    const float* v = (p == 0 ? v0 : v1) + c.r0;
+    float x[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) x[q] = (lane + 32 * q < rows) ? v[lane + 32 * q] : 0.f;
+#pragma unroll 4
+    for (int col = w; col < k; col += 8) {
+      const float* a = A + (int64_t)col * n;
+      float y[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) y[q] = (lane + 32 * q < rows) ? a[lane + 32 * q] : 0.f;
       float s = 0.f;
 #pragma unroll
-      for (int i = 0; i < 32; ++i) s += prod[(part * 32 + i) * ldp + col];
-      red[part][p * k + col] = s;
+      for (int q = 0; q < 8; ++q) s = fmaf(y[q], x[q], s);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      if (lane == 0) partial[((int64_t)blockIdx.x * npair + p) * k + col] = s;
     }
-    __syncthreads();
-  }
-  for (int e = tid; e < npair * k; e += 256) {
-    float s = 0.f;
-    for (int w = 0; w < 8; ++w) s += red[w][e];
-    partial[(int64_t)blockIdx.x * npair * k + e] = s;
   }
 }
 
-// out[node][e] = sum over the node's chunks (heap ids 2 .. 2^(L+1)-1).  The
-// 256 threads form 256 / width groups; group q sums chunks q, q + groups, ...
-// and the group sums are added in group order (deterministic).  width <= 128.
-__global__ __launch_bounds__(256) void k_fact_reduce(const float* __restrict__ partial,
+// out[node][e] = sum over the node's chunks (heap ids 2 .. 2^(L+1)-1): chunks
+// begin[node] .. begin[node + 1] at partial[chunk * stride + e], or, without `begin`,
+// the row tiles (`tiles` a leaf) of the node's leaves (L rows of k per tile).  The
+// threads form RED_T / width groups; group q sums chunks q, q + groups, ... and the
+// group sums are added in group order (deterministic).  width <= 128.  (A node of level
+// 1 has thousands of row tiles: the chain of its loads is what takes the time.)
+constexpr int RED_T = 1024;
+__global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__ partial,
                                                      const int32_t* __restrict__ fbegin,
-                                                     int width, int nnodes_total,
+                                                     int width, int L, int tiles,
                                                      float* __restrict__ out) {
-  __shared__ float sred[256];
+  __shared__ float sred[RED_T];
   const int node = 2 + blockIdx.x;
-  if (node >= nnodes_total) return;  // uniform over the block
-  const int c0 = fbegin[node], c1 = fbegin[node + 1];
-  const int groups = 256 / width;
+  int c0, c1;
+  int64_t stride = width, off = 0;
+  if (fbegin) {
+    c0 = fbegin[node];
+    c1 = fbegin[node + 1];
+  } else {
+    const int j = 31 - __clz(node);  // the node's level
+    c0 = ((node << (L - j)) - (1 << L)) * tiles;
+    c1 = (((node + 1) << (L - j)) - (1 << L)) * tiles;
+    stride = (int64_t)L * width;
+    off = (int64_t)(j - 1) * width;
+  }
+  const int groups = RED_T / width;
   const int t = threadIdx.x, e = t % width, q = t / width;
   float s = 0.f;
-  if (q < groups)
-    for (int c = c0 + q; c < c1; c += groups) s += partial[(int64_t)c * width + e];
+  if (q < groups) {
+#pragma unroll 8
+    for (int c = c0 + q; c < c1; c += groups) s += partial[c * stride + off + e];
+  }
   sred[t] = s;
   __syncthreads();
   if (t < width) {
@@ -87,146 +102,340 @@ __global__ __launch_bounds__(256) void k_fact_reduce(const float* __restrict__ p
   }
 }
 
-// y(I_leaf) = sum_j Uex_j(I_leaf) coef[sib(anc_j)] + op(D_leaf) x(I_leaf); with
-// b, also res = y - b
-__global__ __launch_bounds__(256) void k_fact_expand(const int64_t* __restrict__ start,
-                                                     const int64_t* __restrict__ size, int L,
-                                                     int64_t n, int k, int nmax, int width,
-                                                     const float* __restrict__ Uex,
-                                                     const float* __restrict__ coef,
-                                                     const float* __restrict__ D, int trans,
-                                                     const float* __restrict__ x,
-                                                     float* __restrict__ y,
-                                                     const float* __restrict__ b,
-                                                     float* __restrict__ res) {
+// The leaf kernels: a block takes a tile of `rt` rows of a leaf (a power of two), a
+// thread a row and every LEAF_T / rt-th column (group g), eight loads in flight; the
+// groups' row sums meet in shared memory.  The leaf's x is staged LEAF_X at a time.
+constexpr int LEAF_T = 512, LEAF_X = 1024;
+
+// acc + sum over columns e = g, g + G, .. < m of a[e * ld] c[e]
+constexpr int ROWB = 8;
+__device__ __forceinline__ float row_dot(const float* a, int64_t ld, const float* c, int g, int G,
+                                         int m, float acc) {
+  for (int e0 = g; e0 < m; e0 += ROWB * G) {
+    float v[ROWB];
+#pragma unroll
+    for (int q = 0; q < ROWB; ++q) {
+      const int e = e0 + q * G;
+      v[q] = e < m ? a[(int64_t)e * ld] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < ROWB; ++q) {
+      const int e = e0 + q * G;
+      if (e < m) acc = fmaf(v[q], c[e], acc);
+    }
+  }
+  return acc;
+}
+__device__ __forceinline__ float warp_total(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// y(I_leaf) = sum_j Uex_j(I_leaf) coef[sib(anc_j)] + op(D_leaf) x(I_leaf) for the block's
+// rows.
+__global__ __launch_bounds__(LEAF_T) void k_fact_expand(
+    const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
+    int nmax, int rt, const float* __restrict__ Uex, const float* __restrict__ coef,
+    const float* __restrict__ D, int trans, const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ float sm[];
-  float* cs = sm;                  // L * k coefficients
-  float* xs = sm + L * kMaxK;      // leaf slice of x
-  float* dt = xs + nmax;           // D^T x for the transposed product
+  const int ncol = L * k;          // column e of level 1 + e / k starts at Uex + e n
+  float* cs = sm;                  // ncol coefficients
+  float* xs = cs + ncol;           // LEAF_X entries of the leaf's x
+  float* part = xs + LEAF_X;       // the groups' row sums
+  float* rs = part + LEAF_T;       // rt rows of D^T x (trans)
   const int leaf = (1 << L) + blockIdx.x;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int tid = threadIdx.x;
-  for (int e = tid; e < L * k; e += blockDim.x) {
+  const int i0 = blockIdx.y * rt;
+  if (i0 >= ns) return;  // uniform over the block
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
+  for (int e = tid; e < ncol; e += LEAF_T) {
     const int j = 1 + e / k, col = e % k;
     const int anc = leaf >> (L - j);
-    cs[(j - 1) * kMaxK + col] = coef[(int64_t)(anc ^ 1) * width + col];
+    cs[e] = coef[(int64_t)(anc ^ 1) * k + col];
   }
-  for (int m = tid; m < ns; m += blockDim.x) xs[m] = x[s0 + m];
-  __syncthreads();
   const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
-  if (trans) {
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int i = warp; i < ns; i += blockDim.x >> 5) {
+  if (trans)
+    for (int q = warp; q < rt; q += LEAF_T / 32) {
       float v = 0.f;
-      for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)i * nmax] * xs[m];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) dt[i] = v;
+      if (i0 + q < ns)
+#pragma unroll 8
+        for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)(i0 + q) * nmax] * x[s0 + m];
+      v = warp_total(v);
+      if (lane == 0) rs[q] = v;
     }
-    __syncthreads();
-  }
-  for (int i = tid; i < ns; i += blockDim.x) {
-    const int64_t row = s0 + i;
-    float acc = 0.f;
-    for (int j = 1; j <= L; ++j) {
-      const float* Uj = Uex + (int64_t)(j - 1) * n * k;
-      for (int col = 0; col < k; ++col) acc = fmaf(Uj[row + (int64_t)col * n], cs[(j - 1) * kMaxK + col], acc);
+  __syncthreads();
+  const bool live = i < ns;
+  float acc = 0.f;
+  if (live) acc = row_dot(Uex + s0 + i, n, cs, g, G, ncol, acc);
+  if (!trans)
+    for (int m0 = 0; m0 < ns; m0 += LEAF_X) {
+      const int mn = min(LEAF_X, ns - m0);
+      __syncthreads();
+      for (int m = tid; m < mn; m += LEAF_T) xs[m] = x[s0 + m0 + m];
+      __syncthreads();
+      if (live) acc = row_dot(Dl + i + (int64_t)m0 * nmax, nmax, xs, g, G, mn, acc);
     }
-    if (trans) {
-      acc += dt[i];
-    } else {
-      for (int m = 0; m < ns; ++m) acc = fmaf(Dl[i + (int64_t)m * nmax], xs[m], acc);
-    }
-    if (y) y[row] = acc;
-    if (b) res[row] = acc - b[row];
+  part[tid] = acc;
+  __syncthreads();
+  if (g == 0 && live) {
+    for (int q = 1; q < G; ++q) acc += part[q * rt + tid];
+    if (trans) acc += rs[tid];
+    y[s0 + i] = acc;
   }
 }
 
-// Adjoint rows of one leaf.  Per node, coef_t holds t_node = V_j(I_node)^T x and
-// coef_s holds s_node = U_j(I_node)^T res, at node * cw (+ the k entries).
-__global__ __launch_bounds__(256) void k_fact_adjoint(
+// The forward of the fused step for one tile of rows: y = H x, res = y - b, the tile's
+// share of every ancestor's s_node = U^T res (sp[leaf][tile][level][k]) and of D^T res
+// (dtr[tile][row]), and its rows of the gradient of D.  The tile's rows of U and, where
+// they fit (DS), of D are brought into shared memory by asynchronous copies (4 bytes:
+// rows may start anywhere) that are all in flight at once, so that both products read
+// them from there and HBM once; two blocks an SM overlap copies and arithmetic.
+// N = 262144, k = 32, 870 MB: 227 us, bound by the copies' and the products'
+// instructions; 340 us through registers with U and D read again from L2, 274 us with
+// one block an SM walking the tiles, the next tile's copies in flight.
+__device__ __forceinline__ void copy_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   (unsigned)__cvta_generic_to_shared(dst)),
+               "l"(src)
+               : "memory");
+}
+template <int DS, int rt>
+__global__ __launch_bounds__(LEAF_T) void k_fact_forward(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
-    int nmax, const float* __restrict__ U, const float* __restrict__ V,
-    const float* __restrict__ D, const float* __restrict__ coef_t,
-    const float* __restrict__ coef_s, int cw, const float* __restrict__ x,
-    const float* __restrict__ res, float scale, float* __restrict__ gx, float* __restrict__ gU,
-    float* __restrict__ gV, float* __restrict__ gD) {
+    int nmax, const float* __restrict__ U, const float* __restrict__ coef,
+    const float* __restrict__ D, const float* __restrict__ x, float* __restrict__ y,
+    const float* __restrict__ b, float* __restrict__ res, float scale, float* __restrict__ sp,
+    float* __restrict__ dtr, float* __restrict__ gD) {
   extern __shared__ float sm[];
-  float* ts = sm;                  // t of the sibling per level
-  float* ss = sm + L * kMaxK;      // s of the sibling per level
-  float* xs = ss + L * kMaxK;
-  float* rs = xs + nmax;
-  float* dt = rs + nmax;           // D^T res
+  constexpr int pt = rt + 1, G = LEAF_T / rt;
+  const int ncol = L * k;
+  float* cs = sm;                  // ncol coefficients
+  float* xs = cs + ncol;           // the leaf's x (DS), else LEAF_X entries of it
+  float* part = xs + (DS ? nmax : LEAF_X);
+  float* rs = part + LEAF_T;       // rt rows of res
+  float* us = rs + rt;             // the tile's rows of U, [ncol][pt]
+  float* ds = us + ncol * pt;      // DS: its rows of D, [nmax][pt]
   const int leaf = (1 << L) + blockIdx.x;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int e = tid; e < L * k; e += blockDim.x) {
-    const int j = 1 + e / k, col = e % k;
-    const int sib = (leaf >> (L - j)) ^ 1;
-    ts[(j - 1) * kMaxK + col] = coef_t[(int64_t)sib * cw + col];
-    ss[(j - 1) * kMaxK + col] = coef_s[(int64_t)sib * cw + col];
+  const int i0 = blockIdx.y * rt;
+  const int tid = threadIdx.x;
+  const int g = tid / rt, ti = tid & (rt - 1), i = i0 + ti;
+  const bool live = i < ns;
+  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+  if (live) {
+    const float* u = U + s0 + i + (int64_t)g * n;
+    float* d = us + g * pt + ti;
+#pragma unroll 4
+    for (int e = g; e < ncol; e += G, u += G * n, d += G * pt) copy_async4(d, u);
+    if (DS) {
+      u = Dl + i + (int64_t)g * nmax;
+      d = ds + g * pt + ti;
+#pragma unroll 4
+      for (int m = g; m < ns; m += G, u += G * nmax, d += G * pt) copy_async4(d, u);
+    }
+  } else {
+    for (int e = g; e < ncol; e += G) us[e * pt + ti] = 0.f;
+    if (DS)
+      for (int m = g; m < ns; m += G) ds[m * pt + ti] = 0.f;
   }
-  for (int m = tid; m < ns; m += blockDim.x) {
-    xs[m] = x[s0 + m];
-    rs[m] = res[s0 + m];
+  for (int e = tid; e < ncol; e += LEAF_T) {
+    const int j = 1 + e / k, col = e % k;
+    const int anc = leaf >> (L - j);
+    cs[e] = coef[(int64_t)(anc ^ 1) * k + col];
+  }
+  if (DS)
+    for (int m = tid; m < ns; m += LEAF_T) xs[m] = x[s0 + m];
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+  float acc = 0.f;
+#pragma unroll 4
+  for (int e = g; e < ncol; e += G) acc = fmaf(us[e * pt + ti], cs[e], acc);
+  if (DS) {
+#pragma unroll 4
+    for (int m = g; m < ns; m += G) acc = fmaf(ds[m * pt + ti], xs[m], acc);
+  } else {
+    for (int m0 = 0; m0 < ns; m0 += LEAF_X) {
+      const int mn = min(LEAF_X, ns - m0);
+      __syncthreads();
+      for (int m = tid; m < mn; m += LEAF_T) xs[m] = x[s0 + m0 + m];
+      __syncthreads();
+      if (live) acc = row_dot(Dl + i + (int64_t)m0 * nmax, nmax, xs, g, G, mn, acc);
+    }
+  }
+  part[tid] = acc;
+  __syncthreads();
+  if (g == 0) {
+#pragma unroll
+    for (int q = 1; q < G; ++q) acc += part[q * rt + tid];
+    float r = 0.f;
+    if (live) {
+      r = acc - b[s0 + i];
+      y[s0 + i] = acc;
+      res[s0 + i] = r;
+    }
+    rs[ti] = r;
   }
   __syncthreads();
-  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
-  if (gx) {
-    for (int i = warp; i < ns; i += blockDim.x >> 5) {
-      float v = 0.f;
-      for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)i * nmax] * rs[m];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) dt[i] = v;
-    }
-    __syncthreads();
+  // a thread a column: D^T res, then U^T res over the tile's rows
+  float* spt = sp + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * ncol;
+  float* dt = dtr + (int64_t)blockIdx.y * n + s0;
+  const int nd = DS ? ns : 0;
+  for (int e = tid; e < nd + ncol; e += LEAF_T) {
+    const float* c = e < nd ? ds + e * pt : us + (e - nd) * pt;
+    float v = 0.f;
+#pragma unroll
+    for (int q = 0; q < rt; ++q) v = fmaf(c[q], rs[q], v);
+    if (e < nd) dt[e] = v;
+    else spt[e - nd] = v;
   }
-  for (int i = tid; i < ns; i += blockDim.x) {
+  if (!DS) {
+    const int lane = tid & 31, nr = max(0, min(rt, ns - i0));
+    for (int m = tid >> 5; m < ns; m += LEAF_T / 32) {
+      float v = 0.f;
+      for (int q = lane; q < nr; q += 32) v = fmaf(Dl[i0 + q + (int64_t)m * nmax], rs[q], v);
+      v = warp_total(v);
+      if (lane == 0) dt[m] = v;
+    }
+  }
+  if (gD && i < nmax) {
+    // (zero past the leaf's size, in rows and columns)
+    const float sr = scale * rs[ti];
+    float* o = gD + (int64_t)blockIdx.x * nmax * nmax + i + (int64_t)g * nmax;
+#pragma unroll 4
+    for (int m = g; m < nmax; m += G, o += G * nmax)
+      __stcs(o, m < ns ? sr * (DS ? xs[m] : x[s0 + m]) : 0.f);
+  }
+}
+
+// Adjoint rows of one tile of a leaf.  Per node, coef_t holds t_node = V_j(I_node)^T x
+// and coef_s holds s_node = U_j(I_node)^T res, at node * cw (+ the k entries).  dtr: the
+// tiles' shares of D^T res where the forward has formed them (and written gD), else null.
+__global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
+    const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
+    int nmax, int rt, const float* __restrict__ V, const float* __restrict__ D,
+    const float* __restrict__ coef_t, const float* __restrict__ coef_s, int cw,
+    const float* __restrict__ x, const float* __restrict__ res, float scale,
+    const float* __restrict__ dtr, int dtiles, float* __restrict__ gx, float* __restrict__ gU,
+    float* __restrict__ gV, float* __restrict__ gD) {
+  extern __shared__ float sm[];
+  const int ncol = L * k;
+  float* ts = sm;                  // t of the sibling per level
+  float* ss = ts + ncol;           // s of the sibling per level
+  float* part = ss + ncol;         // the groups' row sums
+  float* dt = part + LEAF_T;       // D^T res of the tile's rows
+  const int leaf = (1 << L) + blockIdx.x;
+  const int64_t s0 = start[leaf];
+  const int ns = (int)size[leaf];
+  const int i0 = blockIdx.y * rt;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
+  for (int e = tid; e < ncol; e += LEAF_T) {
+    const int j = 1 + e / k, col = e % k;
+    const int sib = (leaf >> (L - j)) ^ 1;
+    ts[e] = coef_t[(int64_t)sib * cw + col];
+    ss[e] = coef_s[(int64_t)sib * cw + col];
+  }
+  if (gx && !dtr) {
+    const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+    for (int q = warp; q < rt; q += LEAF_T / 32) {
+      float v = 0.f;
+      if (i0 + q < ns)
+#pragma unroll 8
+        for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)(i0 + q) * nmax] * res[s0 + m];
+      v = warp_total(v);
+      if (lane == 0) dt[q] = v;
+    }
+  }
+  __syncthreads();
+  const bool live = i < ns;
+  const float xi = live ? x[s0 + i] : 0.f, ri = live ? res[s0 + i] : 0.f;
+  float acc = 0.f;
+  if (live) {
+    const float sx = scale * xi, sr = scale * ri;
     const int64_t row = s0 + i;
-    const float xr = xs[i], rr = rs[i];
-    float acc = 0.f;
-    for (int j = 1; j <= L; ++j) {
-      const int64_t base = (int64_t)(j - 1) * n * k;
-      for (int col = 0; col < k; ++col) {
-        const int64_t off = base + row + (int64_t)col * n;
-        if (gx) acc = fmaf(V[off], ss[(j - 1) * kMaxK + col], acc);
-        if (gU) gU[off] = scale * rr * ts[(j - 1) * kMaxK + col];
-        if (gV) gV[off] = scale * xr * ss[(j - 1) * kMaxK + col];
+    for (int e0 = g; e0 < ncol; e0 += 8 * G) {
+      float v[8];
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int e = e0 + q * G;
+        v[q] = (gx && e < ncol) ? V[row + (int64_t)e * n] : 0.f;
+      }
+#pragma unroll
+      for (int q = 0; q < 8; ++q) {
+        const int e = e0 + q * G;
+        if (e < ncol) {
+          const int64_t off = row + (int64_t)e * n;
+          acc = fmaf(v[q], ss[e], acc);
+          if (gU) __stcs(gU + off, sr * ts[e]);
+          if (gV) __stcs(gV + off, sx * ss[e]);
+        }
       }
     }
-    if (gx) gx[row] = scale * (acc + dt[i]);
-    if (gD) {
-      float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax;
-      for (int m = 0; m < nmax; ++m)
-        gDl[i + (int64_t)m * nmax] = (m < ns) ? scale * rr * xs[m] : 0.f;
+  }
+  if (gx) {
+    part[tid] = acc;
+    __syncthreads();
+    if (g == 0 && live) {
+      for (int q = 1; q < G; ++q) acc += part[q * rt + tid];
+      float d = 0.f;
+      if (dtr) for (int q = 0; q < dtiles; ++q) d += dtr[(int64_t)q * n + s0 + i];
+      else d = dt[tid];
+      gx[s0 + i] = scale * (acc + d);
     }
   }
-  // rows past the leaf's size (a leaf smaller than n_max): zero, so that the
-  // whole n_max x n_max block of every leaf is written
-  if (gD && ns < nmax) {
-    float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax;
-    const int pad = nmax - ns;
-    for (int e = tid; e < pad * nmax; e += blockDim.x)
-      gDl[ns + e % pad + (int64_t)(e / pad) * nmax] = 0.f;
+  if (gD && !dtr && i < nmax) {
+    // (zero past the leaf's size, in rows and columns)
+    float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax + i;
+    const float sr = scale * ri;
+    for (int m = g; m < nmax; m += G)
+      __stcs(gDl + (int64_t)m * nmax, m < ns ? sr * x[s0 + m] : 0.f);
   }
 }
 
 }  // namespace
 
-// dynamic shared memory of k_fact_partial (66.5 KB at k = 64: limit raised once)
-static size_t fact_partial_smem(int k) {
-  static std::atomic<uint32_t> done{0};
-  raise_smem_limit((const void*)k_fact_partial, done);
-  return sizeof(float) * 256 * (size_t)(k + 1);
-}
-
-// dynamic shared memory of the per-leaf kernels: the sibling coefficients of
-// every level plus the leaf's slices of x (and res, D^T res); grows with n_max
+// Leaves are taken up to this much shared memory for a whole leaf's slices of x (and
+// res, D^T res) beside the coefficients: the limit of hm_hodlr_factored_apply and its
+// adjoint, kept although the kernels' tiles need less.
 static size_t fact_leaf_smem(const hm_tree* t, bool adjoint) {
   const size_t nmax = (size_t)t->nmax, L = (size_t)t->L;
   return adjoint ? sizeof(float) * (2 * L * kMaxK + 3 * nmax)
                  : sizeof(float) * (L * kMaxK + 2 * nmax);
+}
+
+// Rows of a block's tile: 64, or 32 where 64 would leave SMs without two blocks
+// (N = 4096 in leaves of 256: 64 blocks of 64 rows, 128 of 32).
+static int leaf_rows(const hm_tree* t) {
+  const int64_t leaves = (int64_t)1 << t->L;
+  return leaves * ((t->nmax + 63) / 64) >= 304 ? 64 : 32;
+}
+// The fused forward keeps its tile's L k columns of U and, where two blocks an SM then
+// still fit, its rows of D in shared memory: 32 rows, fewer where L k is large.
+static size_t forward_smem(const hm_tree* t, int k, int rt, bool ds) {
+  const size_t ncol = (size_t)t->L * k, nmax = (size_t)t->nmax;
+  return sizeof(float) * (ncol * (rt + 2) + LEAF_T + rt + (ds ? nmax * (rt + 2) : LEAF_X));
+}
+constexpr size_t kForwardSmem = 112 * 1024;
+static int forward_rows(const hm_tree* t, int k) {
+  int rt = 32;
+  while (rt > 4 && forward_smem(t, k, rt, false) > kForwardSmem) rt /= 2;
+  return rt;
+}
+static bool forward_ds(const hm_tree* t, int k) {
+  return forward_smem(t, k, forward_rows(t, k), true) <= kForwardSmem;
+}
+static size_t expand_smem(const hm_tree* t, int k, int rt) {
+  return sizeof(float) * ((size_t)t->L * k + LEAF_X + LEAF_T + rt);
+}
+static size_t adjoint_smem(const hm_tree* t, int k, int rt) {
+  return sizeof(float) * (2 * (size_t)t->L * k + LEAF_T + rt);
+}
+static dim3 leaf_grid(const hm_tree* t, int rt) {
+  return dim3(1u << t->L, (unsigned)((t->nmax + rt - 1) / rt));
 }
 
 hm_status factored_check(const hm_tree* t, bool adjoint) {
@@ -241,8 +450,10 @@ hm_status factored_check(const hm_tree* t, bool adjoint) {
     return HM_EINVAL;
   }
   static std::atomic<uint32_t> done_e{0}, done_a{0};
-  if (adjoint) raise_smem_limit((const void*)k_fact_adjoint, done_a);
-  else raise_smem_limit((const void*)k_fact_expand, done_e);
+  raise_smem_limit((const void*)k_fact_expand, done_e);
+  if (adjoint) {
+    raise_smem_limit((const void*)k_fact_adjoint, done_a);
+  }
   return HM_OK;
 }
 
@@ -256,18 +467,15 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
                            cudaStream_t st) {
   count_launches(3);
   const int L = t->L;
-  const int nodes = 1 << (L + 1);
+  const int nodes = 1 << (L + 1), rt = leaf_rows(t);
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * k;
   // t_node = Proj(I_node)^T x with Proj = V (H x) or U (H^T x)
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
-                                                nullptr, partial);
-  k_fact_reduce<<<nodes - 2, 256, 0, st>>>(partial, t->d_fbegin, k, nodes, coef);
-  const int nmax = (int)t->nmax;
-  const size_t smem = fact_leaf_smem(t, false);
-  k_fact_expand<<<1 << L, 256, smem, st>>>(t->d_start, t->d_size, L, t->n, k, nmax, k,
-                                           trans ? V : U, coef, D, trans, x, y, nullptr,
-                                           nullptr);
+  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
+                                               nullptr, partial);
+  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
+  k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
+      t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
 }
 
 void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const float* V,
@@ -276,51 +484,72 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
                              cudaStream_t st) {
   count_launches(3);
   const int L = t->L;
-  const int nodes = 1 << (L + 1);
+  const int nodes = 1 << (L + 1), rt = leaf_rows(t);
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * 2 * k;
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, U, res, partial);
-  k_fact_reduce<<<nodes - 2, 256, 0, st>>>(partial, t->d_fbegin, 2 * k, nodes, coef);
-  const int nmax = (int)t->nmax;
-  const size_t smem = fact_leaf_smem(t, true);
-  k_fact_adjoint<<<1 << L, 256, smem, st>>>(t->d_start, t->d_size, L, t->n, k, nmax, U, V, D,
-                                            coef, coef + k, 2 * k, x, res, scale, gx, gU, gV,
-                                            gD);
+  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, V, x, U, res, partial);
+  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
+  k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
+      t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
+      scale, nullptr, 0, gx, gU, gV, gD);
 }
 
 size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
   const size_t nodes = (size_t)1 << (t->L + 1);
-  return sizeof(float) * ((size_t)t->n_fchunks * k + 2 * nodes * k + 2 * (size_t)t->n) + 512;
+  const size_t tiles = leaf_grid(t, forward_rows(t, k)).y;
+  return sizeof(float) * ((size_t)t->n_fchunks * k + (nodes / 2) * tiles * t->L * k +
+                          2 * nodes * k + (2 + tiles) * (size_t)t->n) + 512;
 }
 
-// y = H x, res = y - b and the adjoint at res, with every factor read twice: the
-// forward's projections t = V^T x are the adjoint's too, so the adjoint's first
-// pass reads U only, and V is read again only for gx.
+// y = H x, res = y - b and the adjoint at res: the forward's projections t = V^T x are
+// the adjoint's too, the forward's blocks also form s = U^T res (per tile of rows;
+// reduced per node), D^T res and the gradient of D, and the adjoint's pass reads V once
+// more and writes gx, gU, gV.  N = 262144, k = 32 (2.2 GB instead of 2.8): 557 -> 502 us.
 void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const float* V,
                                const float* D, const float* x, const float* b, float scale,
                                float* y, float* res, float* gx, float* gU, float* gV, float* gD,
                                float* scratch, cudaStream_t st) {
-  count_launches(6);
+  count_launches(5);
   const int L = t->L;
   const int nodes = 1 << (L + 1);
   const int nmax = (int)t->nmax;
+  const int rf = forward_rows(t, k), rt = leaf_rows(t);
+  const dim3 gf = leaf_grid(t, rf);
+  const int tiles = (int)gf.y;
   float* partial = scratch;
-  float* coef_t = partial + (size_t)t->n_fchunks * k;
+  float* sp = partial + (size_t)t->n_fchunks * k;
+  float* coef_t = sp + (size_t)(nodes / 2) * tiles * L * k;
   float* coef_s = coef_t + (size_t)nodes * k;
   float* tmp = coef_s + (size_t)nodes * k;
   float* yy = y ? y : tmp;
   float* rr = res ? res : tmp + t->n;
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x,
-                                                                   nullptr, nullptr, partial);
-  k_fact_reduce<<<nodes - 2, 256, 0, st>>>(partial, t->d_fbegin, k, nodes, coef_t);
-  k_fact_expand<<<1 << L, 256, fact_leaf_smem(t, false), st>>>(
-      t->d_start, t->d_size, L, t->n, k, nmax, k, U, coef_t, D, 0, x, yy, b, rr);
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, U, rr,
-                                                                   nullptr, nullptr, partial);
-  k_fact_reduce<<<nodes - 2, 256, 0, st>>>(partial, t->d_fbegin, k, nodes, coef_s);
-  k_fact_adjoint<<<1 << L, 256, fact_leaf_smem(t, true), st>>>(
-      t->d_start, t->d_size, L, t->n, k, nmax, U, V, D, coef_t, coef_s, k, x, rr, scale, gx, gU,
-      gV, gD);
+  float* dtr = tmp + 2 * t->n;
+  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, V, x, nullptr, nullptr,
+                                               partial);
+  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
+  const bool ds = forward_ds(t, k);
+  auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
+    raise_smem_limit((const void*)kern, done);
+    kern<<<gf, LEAF_T, forward_smem(t, k, rf, ds), st>>>(t->d_start, t->d_size, L, t->n, k, nmax, U,
+                                                         coef_t, D, x, yy, b, rr, scale, sp, dtr,
+                                                         gD);
+  };
+  static std::atomic<uint32_t> done[8] = {{0}, {0}, {0}, {0}, {0}, {0}, {0}, {0}};
+  switch (2 * rf + ds) {
+    case 65: forward(k_fact_forward<1, 32>, done[0]); break;
+    case 64: forward(k_fact_forward<0, 32>, done[1]); break;
+    case 33: forward(k_fact_forward<1, 16>, done[2]); break;
+    case 32: forward(k_fact_forward<0, 16>, done[3]); break;
+    case 17: forward(k_fact_forward<1, 8>, done[4]); break;
+    case 16: forward(k_fact_forward<0, 8>, done[5]); break;
+    case 9: forward(k_fact_forward<1, 4>, done[6]); break;
+    default: forward(k_fact_forward<0, 4>, done[7]); break;
+  }
+  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
+  if (gx || gU || gV)
+    k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
+        tiles, gx, gU, gV, nullptr);
 }
 
 }  // namespace hm
