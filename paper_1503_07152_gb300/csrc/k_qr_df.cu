@@ -658,6 +658,100 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
 
 
 constexpr int TQ_THREADS = 512;  // threads of the double-float TSQR kernels
+constexpr int TQ_G = TQ_THREADS / 8;  // 8-lane groups: group p holds columns p, p + TQ_G
+constexpr int TQ_Q = kTsqrRows / 8;   // a lane's rows of a column: 8 q + lane
+
+// The trailing columns' update of step j of a double-float Householder QR held in
+// registers: column k = grp + TQ_G s of the block has row 8 q + gl in (mh, ml)[s][q] of
+// lane gl of group grp.  v (smem): the reflector, zero outside its rows, which lie in
+// the eight-row slices qa .. qb (taken four slices at a time: a branch per slice kept the
+// loads from overlapping).  d[s] = v^T column s over the group, in two chains (even and
+// odd slices) for latency.
+//
+// The lane of a row is fixed (row mod 8) where the shared-memory form gave it to
+// lane (row - j) mod 8: lanes are only rotated by j, which neither the lanes' sums (a
+// lane's rows are the same set in the same order; the two chains trade places) nor the
+// group sum (xor 4, 2, 1 pairs classes mod 8, 4, 2) sees, so the results are the same
+// bit for bit.
+template <int NC>
+__device__ __forceinline__ void hh_dots(const float2* v, int qa, int qb, int gl,
+                                        const float (&mh)[NC][TQ_Q], const float (&ml)[NC][TQ_Q],
+                                        float (&dh)[NC], float (&dl)[NC]) {
+  float eh[NC], el[NC];
+#pragma unroll
+  for (int s = 0; s < NC; ++s) dh[s] = dl[s] = eh[s] = el[s] = 0.f;
+#pragma unroll
+  for (int q0 = 0; q0 < TQ_Q; q0 += 4) {
+    if (q0 + 3 < qa || q0 > qb) continue;  // uniform over the block
+    float2 x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = v[8 * (q0 + q) + gl];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+#pragma unroll
+      for (int s = 0; s < NC; ++s) {
+        if (q & 1) df::dot_acc(x[q].x, x[q].y, mh[s][q0 + q], ml[s][q0 + q], eh[s], el[s]);
+        else df::dot_acc(x[q].x, x[q].y, mh[s][q0 + q], ml[s][q0 + q], dh[s], dl[s]);
+      }
+  }
+#pragma unroll
+  for (int s = 0; s < NC; ++s) {
+    df::add_to(dh[s], dl[s], eh[s], el[s]);
+    df::group8_sum(dh[s], dl[s]);
+  }
+}
+template <int NC>
+__device__ __forceinline__ void hh_axpy(const float2* v, int qa, int qb, int gl,
+                                        float (&mh)[NC][TQ_Q], float (&ml)[NC][TQ_Q],
+                                        const bool (&on)[NC], const float (&fh)[NC],
+                                        const float (&fl)[NC]) {
+#pragma unroll
+  for (int q0 = 0; q0 < TQ_Q; q0 += 4) {
+    if (q0 + 3 < qa || q0 > qb) continue;
+    float2 x[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) x[q] = v[8 * (q0 + q) + gl];
+#pragma unroll
+    for (int s = 0; s < NC; ++s)
+      if (on[s])
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          df::axpy_neg(fh[s], fl[s], x[q].x, x[q].y, mh[s][q0 + q], ml[s][q0 + q]);
+  }
+}
+
+// |x|^2 of v[first .. last] (at most 160 entries), one warp: each lane's entries of
+// every 32-row piece summed over the warp, the pieces in order
+__device__ __forceinline__ void hh_norm2(const float2* v, int first, int last, int lane, float& th,
+                                         float& tl) {
+  float sh[TQ_Q / 4], sl[TQ_Q / 4];
+#pragma unroll
+  for (int w = 0; w < TQ_Q / 4; ++w) {
+    sh[w] = sl[w] = 0.f;
+    const int i = first + 32 * w + lane;
+    if (i <= last) df::dot_acc(v[i].x, v[i].y, v[i].x, v[i].y, sh[w], sl[w]);
+  }
+  // (an empty piece's sum is zero, and adding zero renormalizes th, tl once: below)
+  if (last - first < 32) {
+    df::warp_sum(sh[0], sl[0]);
+    th = sh[0];
+    tl = sl[0];
+  } else if (last - first < 64) {
+#pragma unroll
+    for (int w = 0; w < 2; ++w) df::warp_sum(sh[w], sl[w]);
+    th = sh[0];
+    tl = sl[0];
+    df::add_to(th, tl, sh[1], sl[1]);
+  } else {
+#pragma unroll
+    for (int w = 0; w < TQ_Q / 4; ++w) df::warp_sum(sh[w], sl[w]);
+    th = sh[0];
+    tl = sl[0];
+#pragma unroll
+    for (int w = 1; w < TQ_Q / 4; ++w) df::add_to(th, tl, sh[w], sl[w]);
+  }
+  df::add_to(th, tl, 0.f, 0.f);
+}
 
 // Householder QR of one row block of a panel (the first TSQR round, <= 128 rows,
 // FP64 data) in double-float: the steps of k_tsqr with every operation (the
@@ -665,11 +759,19 @@ constexpr int TQ_THREADS = 512;  // threads of the double-float TSQR kernels
 // columns) carried by float pairs on the FP32 pipe.  v^T v is formed as
 // 2 nrm (nrm + |x0|), the cancellation-free form of |x|^2 - x0^2 + v0^2.
 // Writes the c x c R (row-major, upper triangle) in FP64.
+//
+// The block is held in registers (an 8-lane group per column, NC columns a group); only
+// the reflector passes through shared memory, written with its norm and scalars by the
+// warp that owns the column, so a step has one barrier (the reflector is double-
+// buffered) and its updates no shared-memory stores.  Bound by the step's chain (norm,
+// square root, division: ~1300 cycles) and by the updates' FP32 instructions.  N = 16384,
+// 60 columns: 181 -> 139 us; N = 20001, 120 columns: 672 -> 567 us (before: six barriers a
+// step and the block in shared memory).
+template <int NC>
 __global__ __launch_bounds__(TQ_THREADS) void k_tsqr_df(const TsqrTask* __restrict__ tasks,
                                                  const double* __restrict__ P, int64_t ldp,
-                                                 int c, double* __restrict__ R, int ldm,
+                                                 int c, double* __restrict__ R,
                                                  const NodeJob* __restrict__ jobs) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
   const TsqrTask* tkp = tasks + blockIdx.x;
   if (jobs) {  // a level-wide launch over several operators' nodes
     const NodeJob& jb = jobs[blockIdx.x];
@@ -679,111 +781,102 @@ __global__ __launch_bounds__(TQ_THREADS) void k_tsqr_df(const TsqrTask* __restri
     c = jb.c;
     R = jb.R;
   }
-  const TsqrTask tk = *tkp;
-  float* Mh = reinterpret_cast<float*>(smem_raw);  // column-major, ld = ldm, high parts
-  float* Ml = Mh + (size_t)ldm * c;                 // low parts
-  __shared__ float red_h[TQ_THREADS / 32], red_l[TQ_THREADS / 32];
-  __shared__ float sh_ah, sh_al, sh_bh, sh_bl;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int m = 0;
-  for (int s = 0; s < tk.nsrc; ++s) {
-    if (tk.kind[s] == 0) {
-      const int rows = (int)(tk.r1[s] - tk.r0[s]);
-      for (int idx = tid; idx < rows * c; idx += TQ_THREADS) {
-        const int rr = idx % rows, col = idx / rows;
-        df::split(P[tk.r0[s] + rr + (int64_t)col * ldp], Mh[col * ldm + m + rr],
-                  Ml[col * ldm + m + rr]);
-      }
-      m += rows;
-    } else {
-      const double* Rs = R + (int64_t)tk.slot[s] * c * c;
-      for (int idx = tid; idx < c * c; idx += TQ_THREADS) {
-        const int rr = idx / c, col = idx % c;
-        df::split(Rs[rr * c + col], Mh[col * ldm + m + rr], Ml[col * ldm + m + rr]);
-      }
-      m += c;
+  __shared__ float2 vbuf[2][kTsqrRows];
+  __shared__ float4 scal[2];  // beta, alpha
+  const int64_t r0 = tkp->r0[0];
+  const int m = (int)(tkp->r1[0] - r0);
+  const int tid = threadIdx.x, lane = tid & 31, gl = tid & 7, grp = tid >> 3;
+  float mh[NC][TQ_Q], ml[NC][TQ_Q];
+#pragma unroll
+  for (int s = 0; s < NC; ++s) {
+    const int k = grp + TQ_G * s;
+#pragma unroll
+    for (int q = 0; q < TQ_Q; ++q) {
+      const int i = 8 * q + gl;
+      df::split((k < c && i < m) ? P[r0 + i + (int64_t)k * ldp] : 0.0, mh[s][q], ml[s][q]);
     }
   }
-  __syncthreads();
   const int steps = m < c ? m : c;
+  const int qb = (m - 1) >> 3;
   for (int j = 0; j < steps; ++j) {
-    float* mjh = Mh + j * ldm;
-    float* mjl = Ml + j * ldm;
-    float sh = 0.f, sl = 0.f;
-    for (int i = j + tid; i < m; i += TQ_THREADS) df::dot_acc(mjh[i], mjl[i], mjh[i], mjl[i], sh, sl);
-    df::warp_sum(sh, sl);
-    if (lane == 0) { red_h[warp] = sh; red_l[warp] = sl; }
-    __syncthreads();
-    if (tid == 0) {
-      // the reflector's scalars in double-float too (an FP64 square root or
-      // division is a long dependent chain on the FP64 pipe)
-      float th = red_h[0], tl = red_l[0];
-      for (int w = 1; w < TQ_THREADS / 32; ++w) df::add_to(th, tl, red_h[w], red_l[w]);
-      const float xh = mjh[j], xl = mjl[j];
+    float2* v = vbuf[j & 1];
+    const int og = j % TQ_G, os = j / TQ_G;
+    if ((tid >> 5) == (og >> 2)) {  // the warp that holds column j
+      if (grp == og) {
+#pragma unroll
+        for (int s = 0; s < NC; ++s)
+          if (s == os)
+#pragma unroll
+            for (int q = 0; q < TQ_Q; ++q) {
+              const bool in = 8 * q + gl >= j;
+              v[8 * q + gl] = make_float2(in ? mh[s][q] : 0.f, in ? ml[s][q] : 0.f);
+            }
+      }
+      __syncwarp();
+      float th, tl;
+      hh_norm2(v, j, m - 1, lane, th, tl);
+      const float xh = v[j].x, xl = v[j].y;
       float nh, nl;
       df::sqrt_df(th, tl, nh, nl);
       const float ah = (xh > 0.f) ? -nh : nh, al = (xh > 0.f) ? -nl : nl;
-      float vh, vl, wh = nh, wl = nl, qh, ql;
+      float vh, vl, wh = nh, wl = nl, qh, ql, bh = 0.f, bl = 0.f;
       df::sub(xh, xl, ah, al, vh, vl);                                 // v0 = x0 - alpha
       df::add_to(wh, wl, fabsf(xh), xh < 0.f ? -xl : xl);               // nrm + |x0|
       df::mul(nh, nl, wh, wl, qh, ql);                                  // v^T v / 2
-      sh_ah = ah;
-      sh_al = al;
-      if (qh > 0.f) {
-        df::div_df(1.f, 0.f, qh, ql, sh_bh, sh_bl);                     // beta = 2 / v^T v
-      } else {
-        sh_bh = 0.f;
-        sh_bl = 0.f;
-      }
-      mjh[j] = vh;
-      mjl[j] = vl;
-    }
-    __syncthreads();
-    const float bh = sh_bh, bl = sh_bl;
-    if (bh != 0.f) {
-      // one aligned 8-lane group per trailing column, TQ_THREADS / 8 columns per round
-      for (int k0 = j + 1; k0 < c; k0 += TQ_THREADS / 8) {
-        const int k = k0 + (tid >> 3), gl = tid & 7;
-        const bool on = k < c;
-        float* mkh = Mh + (on ? k : j) * ldm;
-        float* mkl = Ml + (on ? k : j) * ldm;
-        float dh = 0.f, dl = 0.f, eh = 0.f, el = 0.f;  // two chains for latency
-        if (on) {
-#pragma unroll
-          for (int ii = 0; ii < 17; ii += 2) {  // rows j .. m - 1, m <= 136
-            const int i = j + gl + 8 * ii, i2 = i + 8;
-            if (i < m) df::dot_acc(mjh[i], mjl[i], mkh[i], mkl[i], dh, dl);
-            if (ii + 1 < 17 && i2 < m) df::dot_acc(mjh[i2], mjl[i2], mkh[i2], mkl[i2], eh, el);
-          }
-          df::add_to(dh, dl, eh, el);
-        }
-        df::group8_sum(dh, dl);
-        if (on) {
-          float fh, fl;
-          df::fast_two_sum(dh, dl, dh, dl);
-          df::mul(bh, bl, dh, dl, fh, fl);
-#pragma unroll
-          for (int ii = 0; ii < 17; ++ii) {
-            const int i = j + gl + 8 * ii;
-            if (i < m) df::axpy_neg(fh, fl, mjh[i], mjl[i], mkh[i], mkl[i]);
-          }
-        }
+      if (qh > 0.f) df::div_df(1.f, 0.f, qh, ql, bh, bl);               // beta = 2 / v^T v
+      __syncwarp();
+      if (lane == 0) {
+        v[j] = make_float2(vh, vl);
+        scal[j & 1] = make_float4(bh, bl, ah, al);
       }
     }
     __syncthreads();
-    if (tid == 0) { mjh[j] = sh_ah; mjl[j] = sh_al; }
-    __syncthreads();
+    const float4 sc = scal[j & 1];
+    bool on[NC], any = false;
+#pragma unroll
+    for (int s = 0; s < NC; ++s) {
+      const int k = grp + TQ_G * s;
+      on[s] = k > j && k < c;
+      any |= on[s];
+    }
+    if (sc.x != 0.f && __any_sync(0xffffffffu, any)) {
+      float dh[NC], dl[NC], fh[NC], fl[NC];
+      hh_dots<NC>(v, j >> 3, qb, gl, mh, ml, dh, dl);
+#pragma unroll
+      for (int s = 0; s < NC; ++s) {
+        df::fast_two_sum(dh[s], dl[s], dh[s], dl[s]);
+        df::mul(sc.x, sc.y, dh[s], dl[s], fh[s], fl[s]);
+      }
+      hh_axpy<NC>(v, j >> 3, qb, gl, mh, ml, on, fh, fl);
+    }
+    if (grp == og) {  // R(j, j) = alpha
+#pragma unroll
+      for (int s = 0; s < NC; ++s)
+        if (s == os)
+#pragma unroll
+          for (int q = 0; q < TQ_Q; ++q)
+            if (8 * q + gl == j) { mh[s][q] = sc.z; ml[s][q] = sc.w; }
+    }
   }
-  double* Ro = R + (int64_t)tk.out_slot * c * c;
-  for (int idx = tid; idx < c * c; idx += TQ_THREADS) {
-    const int rr = idx / c, col = idx % c;
-    Ro[idx] = (rr <= col && rr < steps) ? df::join(Mh[col * ldm + rr], Ml[col * ldm + rr]) : 0.0;
+  double* Ro = R + (int64_t)tkp->out_slot * c * c;
+#pragma unroll
+  for (int s = 0; s < NC; ++s) {
+    const int k = grp + TQ_G * s;
+#pragma unroll
+    for (int q = 0; q < TQ_Q; ++q) {
+      const int i = 8 * q + gl;
+      if (k < c && i < c)
+        Ro[i * c + k] = (i <= k && i < steps) ? df::join(mh[s][q], ml[s][q]) : 0.0;
+    }
   }
 }
 
 // The merge of two c x c triangles R = qr([R1; R2]) of k_tsqr_merge (packed
 // triangles, the j-th reflector touching row j of R1 and rows 0..j of R2) in
-// double-float; FP64 in and out.
+// double-float; FP64 in and out.  R2 is held in registers as in k_tsqr_df, R1 (one row
+// a step) in shared memory, packed.  120 columns: 433 -> 293 us a round; 60 columns: 148
+// -> 100.
+template <int NC>
 __global__ __launch_bounds__(TQ_THREADS) void k_tsqr_merge_df(const TsqrTask* __restrict__ tasks,
                                                               int c, double* __restrict__ R,
                                                               const NodeJob* __restrict__ jobs) {
@@ -795,102 +888,104 @@ __global__ __launch_bounds__(TQ_THREADS) void k_tsqr_merge_df(const TsqrTask* __
     c = jb.c;
     R = jb.R;
   }
-  const TsqrTask tk = *tkp;
-  const int pk = c * (c + 1) / 2;
-  float* Ah = reinterpret_cast<float*>(smem_raw);  // R1, packed upper
-  float* Al = Ah + pk;
-  float* Bh = Al + pk;                              // R2, packed upper
-  float* Bl = Bh + pk;
-  __shared__ float red_h[TQ_THREADS / 32], red_l[TQ_THREADS / 32];
-  __shared__ float sh_ah, sh_al, sh_bh, sh_bl, sh_vh, sh_vl;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const double* R1 = R + (int64_t)tk.slot[0] * c * c;
-  const double* R2 = R + (int64_t)tk.slot[1] * c * c;
+  float2* A = reinterpret_cast<float2*>(smem_raw);  // R1, packed upper: column k at k(k+1)/2
+  __shared__ float2 vbuf[2][kTsqrRows];
+  __shared__ float4 scal[2], vtop[2];  // beta, alpha; v0 (the reflector's entry in R1)
+  const int tid = threadIdx.x, lane = tid & 31, gl = tid & 7, grp = tid >> 3;
+  const double* R1 = R + (int64_t)tkp->slot[0] * c * c;
+  const double* R2 = R + (int64_t)tkp->slot[1] * c * c;
   for (int idx = tid; idx < c * c; idx += TQ_THREADS) {
     const int rr = idx / c, col = idx % c;
     if (rr <= col) {
-      const int o = col * (col + 1) / 2 + rr;
-      df::split(R1[idx], Ah[o], Al[o]);
-      df::split(R2[idx], Bh[o], Bl[o]);
+      float2 x;
+      df::split(R1[idx], x.x, x.y);
+      A[col * (col + 1) / 2 + rr] = x;
+    }
+  }
+  float mh[NC][TQ_Q], ml[NC][TQ_Q];
+#pragma unroll
+  for (int s = 0; s < NC; ++s) {
+    const int k = grp + TQ_G * s;
+#pragma unroll
+    for (int q = 0; q < TQ_Q; ++q) {
+      const int i = 8 * q + gl;
+      df::split((k < c && i <= k) ? R2[i * c + k] : 0.0, mh[s][q], ml[s][q]);
     }
   }
   __syncthreads();
   for (int j = 0; j < c; ++j) {
-    const int oj = j * (j + 1) / 2;  // rows 0..j of column j of R2
-    float sh = 0.f, sl = 0.f;
-    for (int i = tid; i <= j; i += TQ_THREADS) df::dot_acc(Bh[oj + i], Bl[oj + i], Bh[oj + i], Bl[oj + i], sh, sl);
-    df::warp_sum(sh, sl);
-    if (lane == 0) { red_h[warp] = sh; red_l[warp] = sl; }
-    __syncthreads();
-    if (tid == 0) {
-      // the reflector's scalars in double-float (see k_tsqr_df)
-      float th = red_h[0], tl = red_l[0];
-      for (int w = 1; w < TQ_THREADS / 32; ++w) df::add_to(th, tl, red_h[w], red_l[w]);
-      const float xh = Ah[oj + j], xl = Al[oj + j];
+    float2* v = vbuf[j & 1];
+    const int og = j % TQ_G, os = j / TQ_G;
+    if ((tid >> 5) == (og >> 2)) {  // the warp that holds column j of R2
+      if (grp == og) {
+#pragma unroll
+        for (int s = 0; s < NC; ++s)
+          if (s == os)
+#pragma unroll
+            for (int q = 0; q < TQ_Q; ++q) {
+              const bool in = 8 * q + gl <= j;
+              v[8 * q + gl] = make_float2(in ? mh[s][q] : 0.f, in ? ml[s][q] : 0.f);
+            }
+      }
+      __syncwarp();
+      float th, tl;
+      hh_norm2(v, 0, j, lane, th, tl);
+      const float2 x0 = A[j * (j + 1) / 2 + j];
+      const float xh = x0.x, xl = x0.y;
       float sh2, sl2, nh, nl;
       df::mul(xh, xl, xh, xl, sh2, sl2);
       df::add_to(sh2, sl2, th, tl);                                     // x0^2 + tail
       df::sqrt_df(sh2, sl2, nh, nl);
       const float ah = (xh > 0.f) ? -nh : nh, al = (xh > 0.f) ? -nl : nl;
-      float vh, vl, wh = nh, wl = nl, qh, ql;
+      float vh, vl, wh = nh, wl = nl, qh, ql, bh = 0.f, bl = 0.f;
       df::sub(xh, xl, ah, al, vh, vl);                                 // v0 = x0 - alpha
       df::add_to(wh, wl, fabsf(xh), xh < 0.f ? -xl : xl);               // nrm + |x0|
       df::mul(nh, nl, wh, wl, qh, ql);                                  // v^T v / 2
-      sh_ah = ah;
-      sh_al = al;
-      sh_vh = vh;
-      sh_vl = vl;
-      if (qh > 0.f) {
-        df::div_df(1.f, 0.f, qh, ql, sh_bh, sh_bl);                     // beta = 2 / v^T v
-      } else {
-        sh_bh = 0.f;
-        sh_bl = 0.f;
+      if (qh > 0.f) df::div_df(1.f, 0.f, qh, ql, bh, bl);               // beta = 2 / v^T v
+      __syncwarp();
+      if (lane == 0) {
+        scal[j & 1] = make_float4(bh, bl, ah, al);
+        vtop[j & 1] = make_float4(vh, vl, 0.f, 0.f);
+        if (bh != 0.f) A[j * (j + 1) / 2 + j] = make_float2(ah, al);
       }
     }
     __syncthreads();
-    const float bh = sh_bh, bl = sh_bl, vh = sh_vh, vl = sh_vl;
-    if (bh != 0.f) {
-      // one aligned 8-lane group per trailing column, TQ_THREADS / 8 columns per round
-      for (int k0 = j + 1; k0 < c; k0 += TQ_THREADS / 8) {
-        const int k = k0 + (tid >> 3), gl = tid & 7;
-        const bool on = k < c;
-        const int kk = on ? k : j;
-        const int ok = kk * (kk + 1) / 2;
-        float dh = 0.f, dl = 0.f, eh = 0.f, el = 0.f;  // two chains for latency
-        if (on) {
+    const float4 sc = scal[j & 1], v0 = vtop[j & 1];
+    bool on[NC], any = false;
 #pragma unroll
-          for (int ii = 0; ii < 16; ii += 2) {  // rows 0 .. j, j < c <= 128
-            const int i = gl + 8 * ii, i2 = i + 8;
-            if (i <= j) df::dot_acc(Bh[oj + i], Bl[oj + i], Bh[ok + i], Bl[ok + i], dh, dl);
-            if (i2 <= j) df::dot_acc(Bh[oj + i2], Bl[oj + i2], Bh[ok + i2], Bl[ok + i2], eh, el);
-          }
-          df::add_to(dh, dl, eh, el);
-        }
-        df::group8_sum(dh, dl);
-        if (on) {
-          // f = beta (dot + v0 A(j, k))
-          df::dot_acc(vh, vl, Ah[ok + j], Al[ok + j], dh, dl);
-          float fh, fl;
-          df::fast_two_sum(dh, dl, dh, dl);
-          df::mul(bh, bl, dh, dl, fh, fl);
+    for (int s = 0; s < NC; ++s) {
+      const int k = grp + TQ_G * s;
+      on[s] = k > j && k < c;
+      any |= on[s];
+    }
+    if (sc.x != 0.f && __any_sync(0xffffffffu, any)) {
+      float dh[NC], dl[NC], fh[NC], fl[NC];
+      hh_dots<NC>(v, 0, j >> 3, gl, mh, ml, dh, dl);
 #pragma unroll
-          for (int ii = 0; ii < 16; ++ii) {
-            const int i = gl + 8 * ii;
-            if (i <= j) df::axpy_neg(fh, fl, Bh[oj + i], Bl[oj + i], Bh[ok + i], Bl[ok + i]);
-          }
-          if (gl == 0) df::axpy_neg(fh, fl, vh, vl, Ah[ok + j], Al[ok + j]);
+      for (int s = 0; s < NC; ++s) {
+        const int k = grp + TQ_G * s;
+        float2* a = A + k * (k + 1) / 2 + j;
+        const float2 x = on[s] ? *a : make_float2(0.f, 0.f);
+        // f = beta (dot + v0 A(j, k))
+        df::dot_acc(v0.x, v0.y, x.x, x.y, dh[s], dl[s]);
+        df::fast_two_sum(dh[s], dl[s], dh[s], dl[s]);
+        df::mul(sc.x, sc.y, dh[s], dl[s], fh[s], fl[s]);
+        __syncwarp();
+        if (on[s] && gl == 0) {
+          float2 y = x;
+          df::axpy_neg(fh[s], fl[s], v0.x, v0.y, y.x, y.y);
+          *a = y;
         }
       }
+      hh_axpy<NC>(v, 0, j >> 3, gl, mh, ml, on, fh, fl);
     }
-    __syncthreads();
-    if (tid == 0 && bh != 0.f) { Ah[oj + j] = sh_ah; Al[oj + j] = sh_al; }
-    __syncthreads();
   }
-  double* Ro = R + (int64_t)tk.out_slot * c * c;
+  __syncthreads();
+  double* Ro = R + (int64_t)tkp->out_slot * c * c;
   for (int idx = tid; idx < c * c; idx += TQ_THREADS) {
     const int rr = idx / c, col = idx % c;
-    const int o = col * (col + 1) / 2 + rr;
-    Ro[idx] = (rr <= col) ? df::join(Ah[o], Al[o]) : 0.0;
+    const float2 x = (rr <= col) ? A[col * (col + 1) / 2 + rr] : make_float2(0.f, 0.f);
+    Ro[idx] = (rr <= col) ? df::join(x.x, x.y) : 0.0;
   }
 }
 }  // namespace
@@ -913,38 +1008,35 @@ void launch_jacobi_df_jobs(const NodeJob* jobs, int njobs, int cmax, cudaStream_
   k_jacobi_df<<<njobs, 512, smem, st>>>(nullptr, nullptr, cmax, nullptr, nullptr, jobs);
 }
 
-void launch_tsqr_df(const TsqrTask* tasks, int ntasks, int merge, const double* P, int64_t ldp,
-                    int c, double* R, cudaStream_t st) {
+// One column a group up to 64 columns (two blocks an SM), two above.
+static void tsqr_df_launch(const TsqrTask* tasks, int ntasks, int merge, const double* P,
+                           int64_t ldp, int c, int cmax, double* R, const NodeJob* jobs,
+                           cudaStream_t st) {
   count_launches(1);
   if (!merge) {
-    const int ldm = kTsqrRows + 8;
-    const size_t smem = (size_t)2 * ldm * c * sizeof(float);
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_tsqr_df, done);
-    k_tsqr_df<<<ntasks, TQ_THREADS, smem, st>>>(tasks, P, ldp, c, R, ldm, nullptr);
-  } else {
-    const size_t smem = (size_t)2 * c * (c + 1) * sizeof(float);
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_tsqr_merge_df, done);
-    k_tsqr_merge_df<<<ntasks, TQ_THREADS, smem, st>>>(tasks, c, R, nullptr);
+    if (cmax <= TQ_G) k_tsqr_df<1><<<ntasks, TQ_THREADS, 0, st>>>(tasks, P, ldp, c, R, jobs);
+    else k_tsqr_df<2><<<ntasks, TQ_THREADS, 0, st>>>(tasks, P, ldp, c, R, jobs);
+    return;
   }
+  const size_t smem = (size_t)cmax * (cmax + 1) / 2 * sizeof(float2);
+  static std::atomic<uint32_t> d1{0}, d2{0};
+  if (cmax <= TQ_G) {
+    raise_smem_limit((const void*)k_tsqr_merge_df<1>, d1);
+    k_tsqr_merge_df<1><<<ntasks, TQ_THREADS, smem, st>>>(tasks, c, R, jobs);
+  } else {
+    raise_smem_limit((const void*)k_tsqr_merge_df<2>, d2);
+    k_tsqr_merge_df<2><<<ntasks, TQ_THREADS, smem, st>>>(tasks, c, R, jobs);
+  }
+}
+
+void launch_tsqr_df(const TsqrTask* tasks, int ntasks, int merge, const double* P, int64_t ldp,
+                    int c, double* R, cudaStream_t st) {
+  tsqr_df_launch(tasks, ntasks, merge, P, ldp, c, c, R, nullptr, st);
 }
 
 void launch_tsqr_df_jobs(const NodeJob* jobs, int njobs, int merge, int cmax, cudaStream_t st) {
   if (njobs <= 0) return;
-  count_launches(1);
-  if (!merge) {
-    const int ldm = kTsqrRows + 8;
-    const size_t smem = (size_t)2 * ldm * cmax * sizeof(float);
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_tsqr_df, done);
-    k_tsqr_df<<<njobs, TQ_THREADS, smem, st>>>(nullptr, nullptr, 0, cmax, nullptr, ldm, jobs);
-  } else {
-    const size_t smem = (size_t)2 * cmax * (cmax + 1) * sizeof(float);
-    static std::atomic<uint32_t> done{0};
-    raise_smem_limit((const void*)k_tsqr_merge_df, done);
-    k_tsqr_merge_df<<<njobs, TQ_THREADS, smem, st>>>(nullptr, cmax, nullptr, jobs);
-  }
+  tsqr_df_launch(nullptr, njobs, merge, nullptr, 0, cmax, cmax, nullptr, jobs, st);
 }
 
 }  // namespace hm
