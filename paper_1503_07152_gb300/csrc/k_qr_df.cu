@@ -54,6 +54,15 @@ __device__ __forceinline__ bool jacobi_angle32(float ga, float al, float be, flo
   ts = tc * t;
   return true;
 }
+// The rotation of an FP32 pair with its roundings spelled out: left to the compiler, the
+// contraction of the two products can differ between instantiations of the kernel, and
+// a node's result must not depend on the widths it shares a launch with.
+__device__ __forceinline__ float rot_c(float tc, float ts, float x, float y) {
+  return fmaf(tc, x, -__fmul_rn(ts, y));
+}
+__device__ __forceinline__ float rot_s(float tc, float ts, float x, float y) {
+  return fmaf(ts, x, __fmul_rn(tc, y));
+}
 // the pair's squared norms after the rotation (c^2 al - 2cs ga + s^2 be and
 // s^2 al + 2cs ga + c^2 be, clamped at 0)
 __device__ __forceinline__ void jacobi_norms32(float tc, float ts, float ga, float& np,
@@ -81,6 +90,7 @@ __device__ __forceinline__ void jacobi_norms32(float tc, float ts, float ga, flo
 //      descending, the sign convention of k_jacobi_mp.
 // R is scaled by a power of two (exact) so that its largest entry lies in
 // [1, 2): squared column norms then stay inside the float range.
+template <int NB>
 __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict__ node_slot,
                                                       const double* __restrict__ R, int c,
                                                       double* __restrict__ W,
@@ -100,10 +110,15 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
     Wn = W + (int64_t)blockIdx.x * c * c;
     sig = sigma + (int64_t)blockIdx.x * c;
   }
+  // Columns are LD apart and their rows padded with zeros to 32 NB >= c, so that every
+  // element loop has a fixed count and no condition (a condition per element kept the
+  // loads of a loop from overlapping); LD = 8 mod 32 puts the columns that the four
+  // groups of a warp work on in different banks.
+  constexpr int LD = 32 * NB + 8, NE = 4 * NB;  // NE: an 8-lane group's elements per lane
   const int cc = c * c;
   float* reg0 = reinterpret_cast<float*>(smem_raw);
-  float* reg1 = reg0 + cc;
-  float* reg2 = reg1 + cc;
+  float* reg1 = reg0 + c * LD;
+  float* reg2 = reg1 + c * LD;
   float* Mh = reg0;   // A: R, then R2 (column-major)
   float* Ml = reg1;
   float* V32 = reg0;  // B, C
@@ -119,8 +134,9 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   __shared__ double red_v[16];
   __shared__ int red_i[16];
   __shared__ float pnh[128], pnl[128], ph0[128];  // A: pivoting norms
-  __shared__ float sh_ah, sh_al, sh_sh, sh_sl;
+  __shared__ float sh_ah, sh_al, sh_sh, sh_sl, sh_vh, sh_vl;
   __shared__ int sh_exp;
+  __shared__ float2 vb[32 * NB];  // A: the reflector, zero outside its rows
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   const int nthr = blockDim.x;
   const int pg = tid >> 3, gl = tid & 7;
@@ -144,7 +160,12 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   // ---------------------------------------------------------------- A
   for (int idx = tid; idx < cc; idx += nthr) {
     const int rr = idx / c, col = idx % c;
-    df::split(ldexp(Rs[idx], -ex), Mh[col * c + rr], Ml[col * c + rr]);
+    df::split(ldexp(Rs[idx], -ex), Mh[col * LD + rr], Ml[col * LD + rr]);
+  }
+  for (int idx = tid; idx < c * (LD - c); idx += nthr) {
+    const int o = idx / (LD - c) * LD + c + idx % (LD - c);
+    Mh[o] = 0.f;
+    Ml[o] = 0.f;
   }
   for (int j = tid; j < c; j += nthr) perm[j] = j;
   __syncthreads();
@@ -154,7 +175,7 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   // instructions (a square root, a division) is very long on GB300's FP64 pipe.
   for (int k = warp; k < c; k += nwarps) {
     float sh = 0.f, sl = 0.f;
-    for (int i = lane; i < c; i += 32) df::dot_acc(Mh[k * c + i], Ml[k * c + i], Mh[k * c + i], Ml[k * c + i], sh, sl);
+    for (int i = lane; i < c; i += 32) df::dot_acc(Mh[k * LD + i], Ml[k * LD + i], Mh[k * LD + i], Ml[k * LD + i], sh, sl);
     df::warp_sum(sh, sl);
     if (lane == 0) { df::fast_two_sum(sh, sl, pnh[k], pnl[k]); ph0[k] = pnh[k]; }
   }
@@ -165,7 +186,7 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
       if (!(pnh[k] > 5.9604644775390625e-08f * ph0[k])) {
         float sh = 0.f, sl = 0.f;
         for (int i = j + lane; i < c; i += 32)
-          df::dot_acc(Mh[k * c + i], Ml[k * c + i], Mh[k * c + i], Ml[k * c + i], sh, sl);
+          df::dot_acc(Mh[k * LD + i], Ml[k * LD + i], Mh[k * LD + i], Ml[k * LD + i], sh, sl);
         df::warp_sum(sh, sl);
         if (lane == 0) { df::fast_two_sum(sh, sl, pnh[k], pnl[k]); ph0[k] = pnh[k]; }
       }
@@ -188,8 +209,8 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
     const int p = red_i[0];
     if (p != j && p < c) {
       for (int i = tid; i < c; i += nthr) {
-        float t = Mh[j * c + i]; Mh[j * c + i] = Mh[p * c + i]; Mh[p * c + i] = t;
-        t = Ml[j * c + i]; Ml[j * c + i] = Ml[p * c + i]; Ml[p * c + i] = t;
+        float t = Mh[j * LD + i]; Mh[j * LD + i] = Mh[p * LD + i]; Mh[p * LD + i] = t;
+        t = Ml[j * LD + i]; Ml[j * LD + i] = Ml[p * LD + i]; Ml[p * LD + i] = t;
       }
       if (tid == 0) {
         const int t = perm[j]; perm[j] = perm[p]; perm[p] = t;
@@ -199,8 +220,8 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
       }
     }
     __syncthreads();
-    float* mjh = Mh + j * c;
-    float* mjl = Ml + j * c;
+    float* mjh = Mh + j * LD;
+    float* mjl = Ml + j * LD;
     if (warp == 0) {  // the reflector needs the pivot column's exact norm
       float sh = 0.f, sl = 0.f;
       for (int i = j + lane; i < c; i += 32) df::dot_acc(mjh[i], mjl[i], mjh[i], mjl[i], sh, sl);
@@ -224,25 +245,40 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
         sh_al = al;
         sh_sh = sch;
         sh_sl = scl;
-        df::mul(vh, vl, sch, scl, mjh[j], mjl[j]);
+        df::mul(vh, vl, sch, scl, sh_vh, sh_vl);
       }
     }
     __syncthreads();
     const float sch = sh_sh, scl = sh_sl;
-    for (int i = j + 1 + tid; i < c; i += nthr) df::mul(sch, scl, mjh[i], mjl[i], mjh[i], mjl[i]);
+    if (tid < 32 * NB) {
+      float2 v = make_float2(0.f, 0.f);
+      if (tid == j) v = make_float2(sh_vh, sh_vl);
+      else if (tid > j) df::mul(sch, scl, mjh[tid], mjl[tid], v.x, v.y);
+      vb[tid] = v;
+    }
     __syncthreads();
     if (sch != 0.f) {
-      for (int k0 = j + 1; k0 < c; k0 += 64) {  // one 8-lane group per trailing column
+      // One 8-lane group per trailing column; lane gl holds rows 8 q + gl (the group sum
+      // does not see by how many lanes the rows are rotated: k_tsqr_df), four slices of
+      // rows at a time
+      for (int k0 = j + 1; k0 < c; k0 += 64) {
         const int k = k0 + pg;
         const bool on = k < c;
-        float* mkh = Mh + (on ? k : j) * c;
-        float* mkl = Ml + (on ? k : j) * c;
+        float* mkh = Mh + (on ? k : j) * LD + gl;
+        float* mkl = Ml + (on ? k : j) * LD + gl;
         float dh = 0.f, dl = 0.f;
         if (on) {
 #pragma unroll
-          for (int ii = 0; ii < 16; ++ii) {
-            const int i = j + gl + 8 * ii;
-            if (i < c) df::dot_acc(mjh[i], mjl[i], mkh[i], mkl[i], dh, dl);
+          for (int q0 = 0; q0 < NE; q0 += 4) {
+            if (8 * q0 + 31 < j) continue;
+            float2 v[4], m[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              v[q] = vb[8 * (q0 + q) + gl];
+              m[q] = make_float2(mkh[8 * (q0 + q)], mkl[8 * (q0 + q)]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) df::dot_acc(v[q].x, v[q].y, m[q].x, m[q].y, dh, dl);
           }
         }
         df::group8_sum(dh, dl);
@@ -250,18 +286,32 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
           float fh, fl;
           df::fast_two_sum(dh, dl, fh, fl);
 #pragma unroll
-          for (int ii = 0; ii < 16; ++ii) {
-            const int i = j + gl + 8 * ii;
-            if (i < c) df::axpy_neg(fh, fl, mjh[i], mjl[i], mkh[i], mkl[i]);
+          for (int q0 = 0; q0 < NE; q0 += 4) {
+            if (8 * q0 + 31 < j) continue;
+            float2 v[4], m[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              v[q] = vb[8 * (q0 + q) + gl];
+              m[q] = make_float2(mkh[8 * (q0 + q)], mkl[8 * (q0 + q)]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              df::axpy_neg(fh, fl, v[q].x, v[q].y, m[q].x, m[q].y);
+              mkh[8 * (q0 + q)] = m[q].x;
+              mkl[8 * (q0 + q)] = m[q].y;
+            }
           }
         }
       }
     }
     __syncthreads();
-    if (tid == 0 && sch != 0.f) { mjh[j] = sh_ah; mjl[j] = sh_al; }
+    if (tid == 0) {  // R2(j, j)
+      mjh[j] = sch != 0.f ? sh_ah : 0.f;
+      mjl[j] = sch != 0.f ? sh_al : 0.f;
+    }
     for (int k = j + 1 + tid; k < c; k += nthr) {  // downdate: |col k|^2 -= R(j, k)^2
       float rh, rl;
-      df::mul(Mh[k * c + j], Ml[k * c + j], Mh[k * c + j], Ml[k * c + j], rh, rl);
+      df::mul(Mh[k * LD + j], Ml[k * LD + j], Mh[k * LD + j], Ml[k * LD + j], rh, rl);
       df::sub(pnh[k], pnl[k], rh, rl, pnh[k], pnl[k]);
     }
     __syncthreads();
@@ -274,28 +324,27 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   for (int idx = tid; idx < cc; idx += nthr) {
     const int col = idx / c, row = idx % c;  // X(row, col) = R2(col, row), zero above
     const bool low = row >= col;
-    Xph[idx] = low ? Mh[row * c + col] : 0.f;
-    Xpl[idx] = low ? Ml[row * c + col] : 0.f;
+    Xph[idx] = low ? Mh[row * LD + col] : 0.f;
+    Xpl[idx] = low ? Ml[row * LD + col] : 0.f;
   }
   __syncthreads();
   // ---------------------------------------------------------------- B
-  for (int idx = tid; idx < cc; idx += nthr) {
-    X32[idx] = Xph[idx];
-    V32[idx] = (idx / c == idx % c) ? 1.f : 0.f;
+  for (int idx = tid; idx < c * LD; idx += nthr) {
+    const int col = idx / LD, row = idx - col * LD;
+    X32[idx] = row < c ? Xph[col * c + row] : 0.f;
+    V32[idx] = col == row ? 1.f : 0.f;
   }
   __syncthreads();
   const int cp = (c + 1) & ~1;
   float* cn32 = cnh;  // FP32 squared column norms of X32 (cnh is free until E)
   for (int j = warp; j < c; j += nwarps) {
     float s2 = 0.f;
-    for (int i = lane; i < c; i += 32) s2 = fmaf(X32[j * c + i], X32[j * c + i], s2);
+    for (int i = lane; i < c; i += 32) s2 = fmaf(X32[j * LD + i], X32[j * LD + i], s2);
     for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
     if (lane == 0) cn32[j] = s2;
   }
   __syncthreads();
   {
-    // (element loops over a fixed 16 strided elements per lane, c <= 128, so
-    // that they unroll; the arithmetic and its order are those of the plain loops)
     const float tol = (float)(5.960464477539063e-08 * sqrt((double)c));
     const float big2 = tol;
     const bool vec = (c & 3) == 0;
@@ -314,54 +363,54 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
           q = vb + 1;
         }
         const bool valid = p < c && q < c;
-        float* ap = X32 + (valid ? p : 0) * c;
-        float* aq = X32 + (valid ? q : 0) * c;
+        float* ap = X32 + (valid ? p : 0) * LD;
+        float* aq = X32 + (valid ? q : 0) * LD;
         if (vec) {
           // c a multiple of 4: lane gl holds the 16-byte chunks gl, gl + 8, ..
           // of both columns in registers (one 128-byte row of shared memory per
           // group and load: no bank conflicts) for the dot product and the
           // rotation
-          const int c4 = c >> 2;
-          float4 xa[4], xb[4];
+          float4 xa[NB], xb[NB];
           float ga = 0.f;
-          if (valid) {
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-              const int ch = gl + 8 * k;
-              if (ch < c4) {
-                xa[k] = reinterpret_cast<const float4*>(ap)[ch];
-                xb[k] = reinterpret_cast<const float4*>(aq)[ch];
-                ga = fmaf(xa[k].x, xb[k].x, ga);
-                ga = fmaf(xa[k].y, xb[k].y, ga);
-                ga = fmaf(xa[k].z, xb[k].z, ga);
-                ga = fmaf(xa[k].w, xb[k].w, ga);
-              }
-            }
+          for (int k = 0; k < NB; ++k) {
+            xa[k] = reinterpret_cast<const float4*>(ap)[gl + 8 * k];
+            xb[k] = reinterpret_cast<const float4*>(aq)[gl + 8 * k];
+          }
+#pragma unroll
+          for (int k = 0; k < NB; ++k) {
+            ga = fmaf(xa[k].x, xb[k].x, ga);
+            ga = fmaf(xa[k].y, xb[k].y, ga);
+            ga = fmaf(xa[k].z, xb[k].z, ga);
+            ga = fmaf(xa[k].w, xb[k].w, ga);
           }
           ga += __shfl_xor_sync(0xffffffffu, ga, 4);
           ga += __shfl_xor_sync(0xffffffffu, ga, 2);
           ga += __shfl_xor_sync(0xffffffffu, ga, 1);
           float tc, ts;
           if (valid && jacobi_angle32(ga, cn32[p], cn32[q], tol, big2, gl, large, tc, ts)) {
-            float4* vp = reinterpret_cast<float4*>(V32 + p * c);
-            float4* vq = reinterpret_cast<float4*>(V32 + q * c);
+            float4* vp = reinterpret_cast<float4*>(V32 + p * LD);
+            float4* vq = reinterpret_cast<float4*>(V32 + q * LD);
+            float4 u[NB], w[NB];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
+            for (int k = 0; k < NB; ++k) {
+              u[k] = vp[gl + 8 * k];
+              w[k] = vq[gl + 8 * k];
+            }
+#pragma unroll
+            for (int k = 0; k < NB; ++k) {
               const int ch = gl + 8 * k;
-              if (ch < c4) {
-                const float4 x = xa[k], y = xb[k];
-                reinterpret_cast<float4*>(ap)[ch] =
-                    make_float4(tc * x.x - ts * y.x, tc * x.y - ts * y.y, tc * x.z - ts * y.z,
-                                tc * x.w - ts * y.w);
-                reinterpret_cast<float4*>(aq)[ch] =
-                    make_float4(ts * x.x + tc * y.x, ts * x.y + tc * y.y, ts * x.z + tc * y.z,
-                                ts * x.w + tc * y.w);
-                const float4 u = vp[ch], w = vq[ch];
-                vp[ch] = make_float4(tc * u.x - ts * w.x, tc * u.y - ts * w.y,
-                                     tc * u.z - ts * w.z, tc * u.w - ts * w.w);
-                vq[ch] = make_float4(ts * u.x + tc * w.x, ts * u.y + tc * w.y,
-                                     ts * u.z + tc * w.z, ts * u.w + tc * w.w);
-              }
+              const float4 x = xa[k], y = xb[k];
+              reinterpret_cast<float4*>(ap)[ch] =
+                  make_float4(rot_c(tc, ts, x.x, y.x), rot_c(tc, ts, x.y, y.y), rot_c(tc, ts, x.z, y.z),
+                              rot_c(tc, ts, x.w, y.w));
+              reinterpret_cast<float4*>(aq)[ch] =
+                  make_float4(rot_s(tc, ts, x.x, y.x), rot_s(tc, ts, x.y, y.y), rot_s(tc, ts, x.z, y.z),
+                              rot_s(tc, ts, x.w, y.w));
+              vp[ch] = make_float4(rot_c(tc, ts, u[k].x, w[k].x), rot_c(tc, ts, u[k].y, w[k].y),
+                                   rot_c(tc, ts, u[k].z, w[k].z), rot_c(tc, ts, u[k].w, w[k].w));
+              vq[ch] = make_float4(rot_s(tc, ts, u[k].x, w[k].x), rot_s(tc, ts, u[k].y, w[k].y),
+                                   rot_s(tc, ts, u[k].z, w[k].z), rot_s(tc, ts, u[k].w, w[k].w));
             }
             __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of the norms first
             if (gl == 0) {
@@ -371,37 +420,28 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
           }
         } else {
           float ga = 0;
-          if (valid) {
 #pragma unroll
-            for (int ii = 0; ii < 16; ++ii) {
-              const int i = gl + 8 * ii;
-              if (i < c) ga = fmaf(ap[i], aq[i], ga);
-            }
-          }
+          for (int ii = 0; ii < NE; ++ii) ga = fmaf(ap[gl + 8 * ii], aq[gl + 8 * ii], ga);
           ga += __shfl_xor_sync(0xffffffffu, ga, 4);
           ga += __shfl_xor_sync(0xffffffffu, ga, 2);
           ga += __shfl_xor_sync(0xffffffffu, ga, 1);
           float tc, ts;
           if (valid && jacobi_angle32(ga, cn32[p], cn32[q], tol, big2, gl, large, tc, ts)) {
-            float* vp = V32 + p * c;
-            float* vq = V32 + q * c;
+            float* vp = V32 + p * LD;
+            float* vq = V32 + q * LD;
 #pragma unroll
-            for (int ii = 0; ii < 16; ++ii) {
+            for (int ii = 0; ii < NE; ++ii) {
               const int i = gl + 8 * ii;
-              if (i < c) {
-                const float x = ap[i], y = aq[i];
-                ap[i] = tc * x - ts * y;
-                aq[i] = ts * x + tc * y;
-              }
+              const float x = ap[i], y = aq[i];
+              ap[i] = rot_c(tc, ts, x, y);
+              aq[i] = rot_s(tc, ts, x, y);
             }
 #pragma unroll
-            for (int ii = 0; ii < 16; ++ii) {
+            for (int ii = 0; ii < NE; ++ii) {
               const int i = gl + 8 * ii;
-              if (i < c) {
-                const float x = vp[i], y = vq[i];
-                vp[i] = tc * x - ts * y;
-                vq[i] = ts * x + tc * y;
-              }
+              const float x = vp[i], y = vq[i];
+              vp[i] = rot_c(tc, ts, x, y);
+              vq[i] = rot_s(tc, ts, x, y);
             }
             __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of the norms first
             if (gl == 0) {
@@ -420,21 +460,27 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   // ---------------------------------------------------------------- C
   // (X32 is dead; Q overlays it and the third region)
   for (int j = 0; j < c; ++j) {
-    float* qjh = Qh + j * c;
-    float* qjl = Ql + j * c;
-    for (int i = tid; i < c; i += nthr) { qjh[i] = V32[j * c + i]; qjl[i] = 0.f; }
+    float* qjh = Qh + j * LD;
+    float* qjl = Ql + j * LD;
+    for (int i = tid; i < LD; i += nthr) { qjh[i] = V32[j * LD + i]; qjl[i] = 0.f; }
     __syncthreads();
     for (int i0 = 0; i0 < j; i0 += 64) {  // one 8-lane group per earlier column
       const int i = i0 + pg;
       const bool on = i < j;
-      const float* qih = Qh + (on ? i : 0) * c;
-      const float* qil = Ql + (on ? i : 0) * c;
+      const float* qih = Qh + (on ? i : 0) * LD + gl;
+      const float* qil = Ql + (on ? i : 0) * LD + gl;
       float sh = 0.f, sl = 0.f;
       if (on) {
 #pragma unroll
-        for (int ee = 0; ee < 16; ++ee) {
-          const int e = gl + 8 * ee;
-          if (e < c) df::dot_acc(qih[e], qil[e], qjh[e], qjl[e], sh, sl);
+        for (int e0 = 0; e0 < NE; e0 += 4) {
+          float xh[4], xl[4], yh[4], yl[4];
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int o = 8 * (e0 + e);
+            xh[e] = qih[o]; xl[e] = qil[o]; yh[e] = qjh[gl + o]; yl[e] = qjl[gl + o];
+          }
+#pragma unroll
+          for (int e = 0; e < 4; ++e) df::dot_acc(xh[e], xl[e], yh[e], yl[e], sh, sl);
         }
       }
       df::group8_sum(sh, sl);
@@ -445,8 +491,10 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
       const int e = tid & 127, part = tid >> 7;
       const int i0 = (j * part) >> 2, i1 = (j * (part + 1)) >> 2;
       float sh = 0.f, sl = 0.f;
-      if (e < c)
-        for (int i = i0; i < i1; ++i) df::dot_acc(hbh[i], hbl[i], Qh[i * c + e], Ql[i * c + e], sh, sl);
+      if (e < c) {
+#pragma unroll 4
+        for (int i = i0; i < i1; ++i) df::dot_acc(hbh[i], hbl[i], Qh[i * LD + e], Ql[i * LD + e], sh, sl);
+      }
       df::add_to(sh, sl, 0.f, 0.f);
       psh[part][e] = sh;
       psl[part][e] = sl;
@@ -476,29 +524,31 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   }
   // ---------------------------------------------------------------- D
   for (int j = warp; j < c; j += nwarps) {
-    float ah[4] = {0.f, 0.f, 0.f, 0.f}, alo[4] = {0.f, 0.f, 0.f, 0.f};
+    float ah[NB] = {}, alo[NB] = {};
+#pragma unroll 4
     for (int k = 0; k < c; ++k) {
-      const float qh = Qh[j * c + k], ql = Ql[j * c + k];
+      const float qh = Qh[j * LD + k], ql = Ql[j * LD + k];
       const float* xkh = Xph + k * c;
       const float* xkl = Xpl + k * c;
 #pragma unroll
-      for (int rr = 0; rr < 4; ++rr) {
+      for (int rr = 0; rr < NB; ++rr) {
         const int row = lane + 32 * rr;
-        if (row < c) df::dot_acc(xkh[row], xkl[row], qh, ql, ah[rr], alo[rr]);
+        const float xh = row < c ? xkh[row] : 0.f, xl = row < c ? xkl[row] : 0.f;
+        df::dot_acc(xh, xl, qh, ql, ah[rr], alo[rr]);
       }
     }
     __syncwarp();
 #pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
+    for (int rr = 0; rr < NB; ++rr) {  // (zero in the padding)
       const int row = lane + 32 * rr;
-      if (row < c) df::fast_two_sum(ah[rr], alo[rr], Qh[j * c + row], Ql[j * c + row]);
+      df::fast_two_sum(ah[rr], alo[rr], Qh[j * LD + row], Ql[j * LD + row]);
     }
   }
   __syncthreads();
   // ---------------------------------------------------------------- E
   for (int j = warp; j < c; j += nwarps) {
     float sh = 0.f, sl = 0.f;
-    for (int i = lane; i < c; i += 32) df::dot_acc(Qh[j * c + i], Ql[j * c + i], Qh[j * c + i], Ql[j * c + i], sh, sl);
+    for (int i = lane; i < c; i += 32) df::dot_acc(Qh[j * LD + i], Ql[j * LD + i], Qh[j * LD + i], Ql[j * LD + i], sh, sl);
     df::warp_sum(sh, sl);
     if (lane == 0) df::fast_two_sum(sh, sl, cnh[j], cnl[j]);
   }
@@ -522,16 +572,22 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
           q = vb + 1;
         }
         const bool valid = p < c && q < c;
-        float* aph = Qh + (valid ? p : 0) * c;
-        float* apl = Ql + (valid ? p : 0) * c;
-        float* aqh = Qh + (valid ? q : 0) * c;
-        float* aql = Ql + (valid ? q : 0) * c;
+        float* aph = Qh + (valid ? p : 0) * LD + gl;
+        float* apl = Ql + (valid ? p : 0) * LD + gl;
+        float* aqh = Qh + (valid ? q : 0) * LD + gl;
+        float* aql = Ql + (valid ? q : 0) * LD + gl;
         float gh = 0.f, glo = 0.f;
         if (valid) {
 #pragma unroll
-          for (int ii = 0; ii < 16; ++ii) {
-            const int i = gl + 8 * ii;
-            if (i < c) df::dot_acc(aph[i], apl[i], aqh[i], aql[i], gh, glo);
+          for (int e0 = 0; e0 < NE; e0 += 4) {
+            float xh[4], xl[4], yh[4], yl[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+              const int o = 8 * (e0 + e);
+              xh[e] = aph[o]; xl[e] = apl[o]; yh[e] = aqh[o]; yl[e] = aql[o];
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) df::dot_acc(xh[e], xl[e], yh[e], yl[e], gh, glo);
           }
         }
         df::group8_sum(gh, glo);
@@ -569,9 +625,19 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
               df::mul(ch, cl, th, tl, sh, sl);                     // sin = t cos
             }
 #pragma unroll
-            for (int ii = 0; ii < 16; ++ii) {
-              const int i = gl + 8 * ii;
-              if (i < c) rot_df(ch, cl, sh, sl, aph[i], apl[i], aqh[i], aql[i]);
+            for (int e0 = 0; e0 < NE; e0 += 4) {
+              float xh[4], xl[4], yh[4], yl[4];
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const int o = 8 * (e0 + e);
+                xh[e] = aph[o]; xl[e] = apl[o]; yh[e] = aqh[o]; yl[e] = aql[o];
+              }
+#pragma unroll
+              for (int e = 0; e < 4; ++e) {
+                const int o = 8 * (e0 + e);
+                rot_df(ch, cl, sh, sl, xh[e], xl[e], yh[e], yl[e]);
+                aph[o] = xh[e]; apl[o] = xl[e]; aqh[o] = yh[e]; aql[o] = yl[e];
+              }
             }
             if (gl == 0) {
               // norms after the rotation: c^2 al - 2cs ga + s^2 be, s^2 al + 2cs ga + c^2 be
@@ -609,7 +675,7 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   // ---------------------------------------------------------------- F
   for (int j = warp; j < c; j += nwarps) {
     float sh = 0.f, sl = 0.f;
-    for (int i = lane; i < c; i += 32) df::dot_acc(Qh[j * c + i], Ql[j * c + i], Qh[j * c + i], Ql[j * c + i], sh, sl);
+    for (int i = lane; i < c; i += 32) df::dot_acc(Qh[j * LD + i], Ql[j * LD + i], Qh[j * LD + i], Ql[j * LD + i], sh, sl);
     df::warp_sum(sh, sl);
     if (lane == 0) {
       const double s = df::join(sh, sl);
@@ -624,8 +690,8 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   }
   __syncthreads();
   for (int j = warp; j < c; j += nwarps) {
-    const float* xh = Qh + order[j] * c;
-    const float* xl = Ql + order[j] * c;
+    const float* xh = Qh + order[j] * LD;
+    const float* xl = Ql + order[j] * LD;
     double best = -1.0, bv = 0.0;
     int bi = c;
     for (int i = lane; i < c; i += 32) {
@@ -649,7 +715,7 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
   for (int idx = tid; idx < cc; idx += nthr) {
     const int i = idx % c, col = idx / c;
     const int j = order[col];
-    const double u = df::join(Qh[j * c + i], Ql[j * c + i]) * hb[col];
+    const double u = df::join(Qh[j * LD + i], Ql[j * LD + i]) * hb[col];
     Wn[perm[i] + col * c] = sgn[col] < 0 ? -u : u;
   }
   for (int j = tid; j < c; j += nthr)
@@ -990,22 +1056,32 @@ __global__ __launch_bounds__(TQ_THREADS) void k_tsqr_merge_df(const TsqrTask* __
 }
 }  // namespace
 
+template <int NB>
+static void jacobi_df_run(const int32_t* node_slot, int nblocks, const double* R, int c, double* W,
+                          double* sigma, const NodeJob* jobs, cudaStream_t st) {
+  const size_t smem = (size_t)3 * c * (32 * NB + 8) * sizeof(float);
+  static std::atomic<uint32_t> done{0};
+  raise_smem_limit((const void*)k_jacobi_df<NB>, done);
+  k_jacobi_df<NB><<<nblocks, 512, smem, st>>>(node_slot, R, c, W, sigma, jobs);
+}
+// rows padded to the next multiple of 32
+static void jacobi_df_launch(const int32_t* node_slot, int nblocks, const double* R, int c,
+                             double* W, double* sigma, const NodeJob* jobs, cudaStream_t st) {
+  count_launches(1);
+  if (c <= 32) jacobi_df_run<1>(node_slot, nblocks, R, c, W, sigma, jobs, st);
+  else if (c <= 64) jacobi_df_run<2>(node_slot, nblocks, R, c, W, sigma, jobs, st);
+  else if (c <= 96) jacobi_df_run<3>(node_slot, nblocks, R, c, W, sigma, jobs, st);
+  else jacobi_df_run<4>(node_slot, nblocks, R, c, W, sigma, jobs, st);
+}
+
 void launch_jacobi_df(const int32_t* node_slot, int nnodes, const double* R, int c, double* W,
                       double* sigma, cudaStream_t st) {
-  count_launches(1);
-  const size_t smem = (size_t)3 * c * c * sizeof(float);
-  static std::atomic<uint32_t> done{0};
-  raise_smem_limit((const void*)k_jacobi_df, done);
-  k_jacobi_df<<<nnodes, 512, smem, st>>>(node_slot, R, c, W, sigma, nullptr);
+  jacobi_df_launch(node_slot, nnodes, R, c, W, sigma, nullptr, st);
 }
 
 void launch_jacobi_df_jobs(const NodeJob* jobs, int njobs, int cmax, cudaStream_t st) {
   if (njobs <= 0) return;
-  count_launches(1);
-  const size_t smem = (size_t)3 * cmax * cmax * sizeof(float);
-  static std::atomic<uint32_t> done{0};
-  raise_smem_limit((const void*)k_jacobi_df, done);
-  k_jacobi_df<<<njobs, 512, smem, st>>>(nullptr, nullptr, cmax, nullptr, nullptr, jobs);
+  jacobi_df_launch(nullptr, njobs, nullptr, cmax, nullptr, nullptr, jobs, st);
 }
 
 // One column a group up to 64 columns (two blocks an SM), two above.
