@@ -22,8 +22,25 @@ void hbs_free(hm_handle* h);
 template <typename T>
 static hm_status apply_any(const hm_handle* h, int trans, int64_t ncols, const T* X, int64_t ldx,
                            T* Y, int64_t ldy, cudaStream_t st) {
-  if (h->format == HM_FORMAT_HODLR) return hodlr_apply_t<T>(h, trans, ncols, X, ldx, Y, ldy, st);
-  return hbs_apply_t<T>(h, trans, ncols, X, ldx, Y, ldy, st);
+  auto run = [&](int64_t w, const T* Xb, int64_t ld, T* Yb) {
+    if (h->format == HM_FORMAT_HODLR) return hodlr_apply_t<T>(h, trans, w, Xb, ld, Yb, ldy, st);
+    return hbs_apply_t<T>(h, trans, w, Xb, ld, Yb, ldy, st);
+  };
+  // the products read X while they write Y: where the two share memory (one buffer, or
+  // alternating columns of one), from a copy of X, 128 columns at a time
+  if (X + (ncols - 1) * ldx + h->n <= Y || Y + (ncols - 1) * ldy + h->n <= X)
+    return run(ncols, X, ldx, Y);
+  const int64_t cbw = 128, N = h->n;
+  T* Xc = nullptr;
+  HM_CUDA_TRY(cudaMallocAsync((void**)&Xc, sizeof(T) * N * std::min(cbw, ncols), st));
+  hm_status s = HM_OK;
+  for (int64_t cb = 0; cb < ncols && s == HM_OK; cb += cbw) {
+    const int64_t w = std::min(cbw, ncols - cb);
+    launch_copy_cols<T>(X + cb * ldx, ldx, Xc, N, N, w, st);
+    s = run(w, Xc, N, Y + cb * ldy);
+  }
+  cudaFreeAsync(Xc, st);
+  return s;
 }
 
 static size_t elem(const hm_handle* h) { return h->prec == HM_MIXED ? 4 : 8; }
@@ -270,9 +287,18 @@ hm_status hm_hodlr_factored_adjoint(const hm_tree* tree, int32_t k, const float*
   cudaStream_t st = (cudaStream_t)stream;
   HM_TRY(factored_check(tree, true));
   HM_TRY(tree_device(const_cast<hm_tree*>(tree), st));
+  const int64_t n = tree->n;
+  const bool in_place = gx && (factored_overlap(gx, n, x, n) || factored_overlap(gx, n, res, n));
   float* scratch = nullptr;
   const size_t sbytes = factored_scratch_bytes(tree, k);
-  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes, st));
+  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes + (in_place ? 2 * n * sizeof(float) : 0), st));
+  if (in_place) {
+    float* own = (float*)((char*)scratch + sbytes);
+    launch_copy_cols<float>(x, n, own, n, n, 1, st);
+    launch_copy_cols<float>(res, n, own + n, n, n, 1, st);
+    x = own;
+    res = own + n;
+  }
   launch_factored_adjoint(tree, k, U, V, D, x, res, scale, gx, gU, gV, gD, scratch, st);
   cudaFreeAsync(scratch, st);
   return check_launch("hm_hodlr_factored_adjoint");
@@ -291,9 +317,17 @@ hm_status hm_hodlr_factored_loss_grad(const hm_tree* tree, int32_t k, const floa
   HM_TRY(factored_check(tree, false));
   HM_TRY(factored_check(tree, true));
   HM_TRY(tree_device(const_cast<hm_tree*>(tree), st));
+  const int64_t n = tree->n;
+  const bool in_place =
+      (y && factored_overlap(y, n, x, n)) || (res && factored_overlap(res, n, x, n));
   float* scratch = nullptr;
   const size_t sbytes = factored_loss_grad_scratch_bytes(tree, k);
-  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes, st));
+  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes + (in_place ? n * sizeof(float) : 0), st));
+  if (in_place) {
+    float* own = (float*)((char*)scratch + sbytes);
+    launch_copy_cols<float>(x, n, own, n, n, 1, st);
+    x = own;
+  }
   launch_factored_loss_grad(tree, k, U, V, D, x, b, scale, y, res, gx, gU, gV, gD, scratch, st);
   cudaFreeAsync(scratch, st);
   return check_launch("hm_hodlr_factored_loss_grad");

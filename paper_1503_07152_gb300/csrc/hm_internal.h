@@ -298,6 +298,7 @@ namespace hm {
 size_t factored_scratch_bytes(const hm_tree* t, int k);
 // Checks that the per-leaf kernels' shared memory fits the device (HM_EINVAL
 // naming the sizes otherwise) and raises their limit once per device.
+bool factored_overlap(const float* a, size_t na, const float* b, size_t nb);
 hm_status factored_check(const hm_tree* t, bool adjoint);
 void launch_factored_apply(const hm_tree* t, int k, const float* U, const float* V,
                            const float* D, int trans, const float* x, float* y, float* scratch,

@@ -187,6 +187,31 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
   }
 }
 
+// The same with y in x's place: a block takes the whole leaf and holds its x before it
+// writes.  (The tiles above read x over the whole leaf while other tiles write.)
+__global__ __launch_bounds__(256) void k_fact_expand_inplace(
+    const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
+    int nmax, const float* __restrict__ Uex, const float* __restrict__ coef,
+    const float* __restrict__ D, int trans, const float* x, float* y) {
+  extern __shared__ float sm[];
+  const int ncol = L * k;
+  float* cs = sm;          // ncol coefficients
+  float* xs = cs + ncol;   // the leaf's x
+  const int leaf = (1 << L) + blockIdx.x;
+  const int64_t s0 = start[leaf];
+  const int ns = (int)size[leaf];
+  for (int e = threadIdx.x; e < ncol; e += blockDim.x)
+    cs[e] = coef[(int64_t)((leaf >> (L - 1 - e / k)) ^ 1) * k + e % k];
+  for (int m = threadIdx.x; m < ns; m += blockDim.x) xs[m] = x[s0 + m];
+  __syncthreads();
+  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+  for (int i = threadIdx.x; i < ns; i += blockDim.x) {
+    const float acc = row_dot(Uex + s0 + i, n, cs, 0, 1, ncol, 0.f);
+    y[s0 + i] = trans ? row_dot(Dl + (int64_t)i * nmax, 1, xs, 0, 1, ns, acc)
+                      : row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
+  }
+}
+
 // The forward of the fused step for one tile of rows: y = H x, res = y - b, the tile's
 // share of every ancestor's s_node = U^T res (sp[leaf][tile][level][k]) and of D^T res
 // (dtr[tile][row]), and its rows of the gradient of D.  The tile's rows of U and, where
@@ -434,6 +459,14 @@ static size_t expand_smem(const hm_tree* t, int k, int rt) {
 static size_t adjoint_smem(const hm_tree* t, int k, int rt) {
   return sizeof(float) * (2 * (size_t)t->L * k + LEAF_T + rt);
 }
+static size_t dsize(const hm_tree* t) { return ((size_t)1 << t->L) * t->nmax * t->nmax; }
+
+// An output in an input's place: the tiles of a leaf read its whole slices of x, res and
+// D while others write, so such calls take a copy or a form of their own.
+bool factored_overlap(const float* a, size_t na, const float* b, size_t nb) {
+  return a < b + nb && b < a + na;
+}
+
 static dim3 leaf_grid(const hm_tree* t, int rt) {
   return dim3(1u << t->L, (unsigned)((t->nmax + rt - 1) / rt));
 }
@@ -449,8 +482,9 @@ hm_status factored_check(const hm_tree* t, bool adjoint) {
               " bytes of shared memory per block; the device allows " + std::to_string(optin));
     return HM_EINVAL;
   }
-  static std::atomic<uint32_t> done_e{0}, done_a{0};
+  static std::atomic<uint32_t> done_e{0}, done_i{0}, done_a{0};
   raise_smem_limit((const void*)k_fact_expand, done_e);
+  raise_smem_limit((const void*)k_fact_expand_inplace, done_i);
   if (adjoint) {
     raise_smem_limit((const void*)k_fact_adjoint, done_a);
   }
@@ -474,8 +508,12 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
   k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
                                                nullptr, partial);
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
-  k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
-      t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
+  if (factored_overlap(x, t->n, y, t->n))
+    k_fact_expand_inplace<<<1u << L, 256, sizeof(float) * ((size_t)L * k + t->nmax), st>>>(
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, x, y);
+  else
+    k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
 }
 
 void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const float* V,
@@ -489,9 +527,14 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
   float* coef = scratch + (size_t)t->n_fchunks * 2 * k;
   k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, V, x, U, res, partial);
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
+  const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
       t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
-      scale, nullptr, 0, gx, gU, gV, gD);
+      scale, nullptr, 0, gx, gU, gV, d_in_place ? nullptr : gD);
+  if (d_in_place)  // once every tile has read D
+    k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
+        scale, nullptr, 0, nullptr, nullptr, nullptr, gD);
 }
 
 size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
@@ -528,11 +571,12 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
                                                partial);
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
   const bool ds = forward_ds(t, k);
+  const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
     raise_smem_limit((const void*)kern, done);
     kern<<<gf, LEAF_T, forward_smem(t, k, rf, ds), st>>>(t->d_start, t->d_size, L, t->n, k, nmax, U,
                                                          coef_t, D, x, yy, b, rr, scale, sp, dtr,
-                                                         gD);
+                                                         d_in_place ? nullptr : gD);
   };
   static std::atomic<uint32_t> done[8] = {{0}, {0}, {0}, {0}, {0}, {0}, {0}, {0}};
   switch (2 * rf + ds) {
@@ -546,6 +590,10 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
     default: forward(k_fact_forward<0, 4>, done[7]); break;
   }
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
+  if (d_in_place)  // once every tile has read D
+    k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, nullptr,
+        0, nullptr, nullptr, nullptr, gD);
   if (gx || gU || gV)
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
         t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
