@@ -9,15 +9,16 @@
 // values (the Gaussian test matrices of the sweeps) its m and l slices are zero
 // and only the three products with x_h are issued.
 //
-// Block: 128 rows of op(A) x 64 columns of X, ten warps in four roles.
-//   warp 9 (one lane): TMA loads of the FP32 tile of A (128 x 64 for Y = A X,
+// Block: 128 rows of op(A) x 64 columns of X, nineteen warps in five roles.
+//   warp 17 (one lane): TMA loads of the FP32 tile of A (128 x 64 for Y = A X,
 //     64 x 128 for Y = A^T X) into a ring of raw stages;
-//   warps 0-3: split each raw tile into three BF16 slices stored as K-major
-//     tiles with the 128-byte swizzle (the transpose of A^T is taken here), and
-//     one lane loads the matching pre-split X slices by TMA (128-byte swizzle);
-//   warp 4: allocates TMEM; one lane issues the MMAs;
-//   warps 5-8: drain the accumulators into compensated FP32 sums in registers
-//     and write Y.
+//   warp 18 (one lane): TMA loads of the matching pre-split X slices (128-byte
+//     swizzle) into the operand stages;
+//   warps 0-7: split each raw tile into three BF16 slices stored as K-major
+//     tiles with the 128-byte swizzle (the transpose of A^T is taken here);
+//   warp 8: allocates TMEM; one lane issues the MMAs;
+//   warps 9-16: drain the accumulators into compensated FP32 sums in registers
+//     (two warps per TMEM lane quarter, 32 columns each) and write Y.
 // The tensor cores round (toward zero) whenever they add into an FP32
 // accumulator, so the accumulators are kept short: every 64-wide K tile gets a
 // fresh pair of accumulators, one for the leading product h*h and one for the
@@ -27,6 +28,13 @@
 // the nonzero structure of X.  When no tile of the block's columns of X needs
 // the m and l slices, the X stage area shrinks to one slice and a third raw
 // stage of A is kept in flight.
+//
+// What bounds it: the cycle of an operand stage (split, fence, 24 MMAs of N = 64,
+// release, refill of X; two stages fit beside the raw ring), not HBM, the tensor
+// pipe or the split's instructions.  Eight split warps instead of four, eight drain
+// warps of 32 columns instead of four of 64, one arrival a warp instead of one a
+// thread and a warp of its own for the X loads: N = 10000, 130 columns, FP32 X:
+// 639 -> 554 us.
 //
 // Every wait on an mbarrier is bounded; on timeout the block raises an error
 // flag, writes NaN to its outputs, waits (bounded) for its own TMA copies still
@@ -51,7 +59,10 @@ constexpr int MAX_RAW = 3;              // raw stages with one X slice; two with
 // both layouts need the same room: 3 raw + 2 x (3 A + 1 X) = 2 raw + 2 x (3 A + 3 X)
 constexpr int LAYOUT_BYTES = 3 * RAW_BYTES + SSTAGES * (3 * A_SLICE + B_SLICE);
 static_assert(LAYOUT_BYTES == 2 * RAW_BYTES + SSTAGES * (3 * A_SLICE + 3 * B_SLICE), "layout");
-constexpr int NCONV = 128, NTHREADS = 320;
+constexpr int NCONV = 256, NDRAIN = 256, NTHREADS = NCONV + NDRAIN + 96;
+constexpr int W_MMA = NCONV / 32, W_DRAIN0 = W_MMA + 1, W_TMA = W_DRAIN0 + NDRAIN / 32,
+              W_XTMA = W_TMA + 1;
+constexpr int DC = TN * TM / NDRAIN;  // columns of a drain thread: 32
 constexpr uint32_t TMEM_COLS = 4 * TN;  // two (leading, correction) pairs
 
 // Three-way BF16 split of an FP32 value.
@@ -132,21 +143,21 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
     abort_flag = 0;
     for (int i = 0; i < MAX_RAW; ++i) {
       mbar_init(smem_u32(&raw_full[i]), 1);
-      mbar_init(smem_u32(&raw_empty[i]), NCONV);
+      mbar_init(smem_u32(&raw_empty[i]), NCONV / 32);
     }
     for (int i = 0; i < SSTAGES; ++i) {
-      mbar_init(smem_u32(&st_full[i]), NCONV);
+      mbar_init(smem_u32(&st_full[i]), NCONV / 32);
       mbar_init(smem_u32(&x_full[i]), 1);
       mbar_init(smem_u32(&st_empty[i]), 1);
     }
     for (int b = 0; b < 2; ++b) {
       mbar_init(smem_u32(&acc_full[b]), 1);
-      mbar_init(smem_u32(&acc_empty[b]), 128);
+      mbar_init(smem_u32(&acc_empty[b]), NDRAIN / 32);
     }
     mbar_init(smem_u32(&bar_final), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 4) {
+  if (warp == W_MMA) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                      smem_u32(&tmem_base_slot)),
                  "r"(TMEM_COLS)
@@ -166,7 +177,7 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
   const uint32_t stage_bytes = 3 * A_SLICE + (need_ml ? 3 : 1) * B_SLICE;
   const uint32_t raw_addr0 = base, stage_addr0 = base + (uint32_t)nraw * RAW_BYTES;
 
-  if (warp == 9) {
+  if (warp == W_TMA) {
     // ---------------------------------------------------------- TMA of A
     if (lane == 0) {
       int it = 0;
@@ -186,31 +197,48 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
       for (int j = (it > nraw ? it - nraw : 0); j < it; ++j)
         mbar_wait_drain(smem_u32(&raw_full[j % nraw]), (j / nraw) & 1);
     }
-  } else if (warp < 4) {
-    // ---------------------------------------------------------- split A, TMA of X
-    int it = 0, xissued = 0;
-    for (int kt = 0; kt < nkt && !abort_flag; ++kt) {
+  } else if (warp == W_XTMA) {
+    // ---------------------------------------------------------- TMA of X
+    if (lane == 0) {
+      int it = 0;
+      for (int kt = 0; kt < nkt; ++kt) {
+        const int fl = active(kt);
+        if (!fl) continue;
+        const int s = it % SSTAGES;
+        if (!mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag, poll_limit)) break;
+        const uint32_t xs = stage_addr0 + (uint32_t)s * stage_bytes + 3 * A_SLICE;
+        const uint32_t bar = smem_u32(&x_full[s]);
+        const int y = ct * 3 * TN;
+        mbar_arrive_tx(bar, (uint32_t)__popc(fl & 7) * B_SLICE);
+        if (fl & 1) tma_load_2d(xs, &tmX, kt * TK, y, bar);
+        if (fl & 2) tma_load_2d(xs + B_SLICE, &tmX, kt * TK, y + TN, bar);
+        if (fl & 4) tma_load_2d(xs + 2 * B_SLICE, &tmX, kt * TK, y + 2 * TN, bar);
+        ++it;
+      }
+      for (int j = (it > SSTAGES ? it - SSTAGES : 0); j < it; ++j)
+        mbar_wait_drain(smem_u32(&x_full[j % SSTAGES]), (j / SSTAGES) & 1);
+    }
+  } else if (warp < W_MMA) {
+    // ---------------------------------------------------------- split A
+    // (a warp's lanes leave together: one of them arrives for all)
+    int it = 0;
+    for (int kt = 0; kt < nkt; ++kt) {
       const int fl = active(kt);
       if (!fl) continue;
       const int rs = it % nraw, s = it % SSTAGES;
-      if (!mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1, &abort_flag, poll_limit)) break;
+      const bool free_ = !abort_flag && mbar_wait(smem_u32(&st_empty[s]), ((it / SSTAGES) & 1) ^ 1,
+                                                  &abort_flag, poll_limit);
+      if (!__all_sync(0xffffffffu, free_)) break;
       const uint32_t st = stage_addr0 + (uint32_t)s * stage_bytes;
-      if (tid == 0) {
-        const uint32_t nsl = (uint32_t)__popc(fl & 7);
-        mbar_arrive_tx(smem_u32(&x_full[s]), nsl * B_SLICE);
-        for (int sl = 0; sl < 3; ++sl)
-          if (fl & (1 << sl))
-            tma_load_2d(st + 3 * A_SLICE + sl * B_SLICE, &tmX, kt * TK, (ct * 3 + sl) * TN,
-                        smem_u32(&x_full[s]));
-        xissued = it + 1;
-      }
-      if (!mbar_wait(smem_u32(&raw_full[rs]), (it / nraw) & 1, &abort_flag, poll_limit)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&raw_full[rs]), (it / nraw) & 1, &abort_flag,
+                                             poll_limit)))
+        break;
       const unsigned char* rw = sbase + (size_t)(raw_addr0 - base) + (size_t)rs * RAW_BYTES;
       unsigned char* sp = sbase + (st - base);
       if (!TRANS) {
-        // raw: [128 rows][64 k] FP32; a pass covers 8 rows, 16 float4 per row
+        // raw: [128 rows][64 k] FP32; a pass covers 16 rows, 16 float4 per row
 #pragma unroll 4
-        for (int p = 0; p < 16; ++p) {
+        for (int p = 0; p < TM * TK / 4 / NCONV; ++p) {
           const int f = p * NCONV + tid, m = f >> 4, k4 = f & 15;
           const float4 v = *reinterpret_cast<const float4*>(rw + m * 256 + k4 * 16);
           uint32_t h0, m0_, l0, h1, m1_, l1;
@@ -222,10 +250,10 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
           *reinterpret_cast<uint2*>(sp + 2 * A_SLICE + off) = make_uint2(l0, l1);
         }
       } else {
-        // raw: [64 k][128 m] FP32; thread m gathers its column, 8 k at a time
-        const int m = tid;
+        // raw: [64 k][128 m] FP32; two threads a column m gather it, 8 k at a time
+        const int m = tid & (TM - 1), q0 = tid / TM;
 #pragma unroll 2
-        for (int q = 0; q < 8; ++q) {
+        for (int q = q0; q < 8; q += NCONV / TM) {
           float v[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e)
@@ -240,14 +268,14 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
         }
       }
       fence_proxy_async();
-      mbar_arrive(smem_u32(&raw_empty[rs]));
-      mbar_arrive(smem_u32(&st_full[s]));
+      __syncwarp();
+      if (lane == 0) {
+        mbar_arrive(smem_u32(&raw_empty[rs]));
+        mbar_arrive(smem_u32(&st_full[s]));
+      }
       ++it;
     }
-    if (tid == 0)
-      for (int j = (xissued > SSTAGES ? xissued - SSTAGES : 0); j < xissued; ++j)
-        mbar_wait_drain(smem_u32(&x_full[j % SSTAGES]), (j / SSTAGES) & 1);
-  } else if (warp == 4) {
+  } else if (warp == W_MMA) {
     // ---------------------------------------------------------- MMA issue
     if (lane == 0) {
       const uint32_t idesc = idesc_bf16_f32();
@@ -299,10 +327,10 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
   } else {
     // ---------------------------------------------------------- drain / epilogue
     const int q4 = warp & 3;  // TMEM lane quarter of this warp
-    const int r = q4 * 32 + lane;
-    float acc[TN], cmp[TN];
+    const int r = q4 * 32 + lane, c0 = ((warp - W_DRAIN0) >> 2) * DC;
+    float acc[DC], cmp[DC];
 #pragma unroll
-    for (int j = 0; j < TN; ++j) { acc[j] = 0.f; cmp[j] = 0.f; }
+    for (int j = 0; j < DC; ++j) { acc[j] = 0.f; cmp[j] = 0.f; }
     // per active K tile: acc += lead + corr, compensated; the correction term is
     // folded into the compensation (it is far below the leading term)
     int it = 0;
@@ -310,26 +338,28 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
       const int fl = active(kt);
       if (!fl) continue;
       const int b = it & 1;
-      if (!mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1, &abort_flag, poll_limit)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1, &abort_flag,
+                                             poll_limit)))
+        break;
       tc_fence_after();
       const uint32_t t_lane = (uint32_t)(q4 * 32) << 16;
-      const uint32_t t_lead = tmem + t_lane + (uint32_t)(b * 2 * TN), t_corr = t_lead + TN;
+      const uint32_t t_lead = tmem + t_lane + (uint32_t)(b * 2 * TN + c0), t_corr = t_lead + TN;
       // the leading accumulator is written only when the h slice of X is present
       const bool has_lead = (fl & 1) != 0;
 #pragma unroll
-      for (int g = 0; g < TN / 16; ++g) {
-        float d0[16], d1[16];
-        tmem_ld16(t_corr + (uint32_t)(g * 16), d1);
+      for (int g = 0; g < DC / 8; ++g) {
+        float d0[8], d1[8];
+        tmem_ld8(t_corr + (uint32_t)(g * 8), d1);
         if (has_lead) {
-          tmem_ld16(t_lead + (uint32_t)(g * 16), d0);
+          tmem_ld8(t_lead + (uint32_t)(g * 8), d0);
         } else {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) d0[j] = 0.f;
+          for (int j = 0; j < 8; ++j) d0[j] = 0.f;
         }
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          float& a = acc[g * 16 + j];
-          float& c = cmp[g * 16 + j];
+        for (int j = 0; j < 8; ++j) {
+          float& a = acc[g * 8 + j];
+          float& c = cmp[g * 8 + j];
           const float y = d0[j] - c;
           const float t = a + y;
           c = ((t - a) - y) - d1[j];
@@ -337,15 +367,16 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
         }
       }
       tc_fence_before();
-      mbar_arrive(smem_u32(&acc_empty[b]));
+      __syncwarp();
+      if (lane == 0) mbar_arrive(smem_u32(&acc_empty[b]));
       ++it;
     }
     const int64_t grow = m0 + r;
     const bool bad = abort_flag != 0;
     if (grow < n) {
 #pragma unroll
-      for (int j = 0; j < TN; ++j) {
-        const int64_t col = (int64_t)ct * TN + j;
+      for (int j = 0; j < DC; ++j) {
+        const int64_t col = (int64_t)ct * TN + c0 + j;
         if (col < ncols)
           Y[grow + col * ldy] = bad ? __int_as_float(0x7fc00000)
                                     : (float)((double)acc[j] - (double)cmp[j]);
@@ -355,7 +386,7 @@ __global__ __launch_bounds__(NTHREADS, 1) void k_gemm_tc(
   tc_fence_before();
   __syncthreads();
   if (abort_flag && tid == 0) atomicExch(err, 1);
-  if (warp == 4 && abort_flag != 2) {
+  if (warp == W_MMA && abort_flag != 2) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem),
                  "r"(TMEM_COLS)
