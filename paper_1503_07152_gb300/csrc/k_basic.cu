@@ -147,7 +147,7 @@ __global__ void k_extract_diag(const T* __restrict__ Y, int64_t ldy, T* __restri
 // column count and the leaf size.  D is read straight from global memory along its
 // contiguous index (transposed: through a 32 x 33 tile of the warp's own).  In FP64 it
 // is bound by the FP64 pipe (76 cycles a warp FMA): N = 65536, leaves of 256, 10 columns
-// 423 us with a block per leaf and column, 283 now (transposed 321), at the floor.
+// 285 us (transposed 565) with a block per leaf and column, 283 (325) now, near the floor.
 constexpr int BD_COLS = 8;
 template <typename T, int TRANS>
 __global__ __launch_bounds__(128) void k_blockdiag_apply(

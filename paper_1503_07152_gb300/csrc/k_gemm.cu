@@ -136,7 +136,7 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
 // multiplied, and where the row blocks alone would not fill the chip a cluster of S
 // blocks shares a tile's active K tiles (dealt out in turn) and sums its shares over
 // distributed shared memory in rank order (deterministic, no workspace).  N = 1024,
-// 20 columns, half of K active: 1200 us as 8 blocks of 128 x 64 outputs, 24 us so.
+// 20 columns, half of K active: 1175 us as 8 blocks of 128 x 64 outputs, 39 us so.
 template <typename TA, int TRANS>
 __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, int64_t lda,
                                                       int64_t n, int64_t ncols,

@@ -27,7 +27,7 @@
 // halves, so that they are ordered by the tensor pipe without waits.
 //
 // What bounds it and what was measured (dense A^T X, N = 32768, 60 columns, every
-// tile active, the pre-cut of X included): 2.40 -> 1.74 ms; per 32-wide tile and
+// tile active, the pre-cut of X included): 2.40 -> 1.64 ms; per 32-wide tile and
 // block 2430 -> ~1600 cycles, of which the twelve MMAs take 768, the FP32 pipe ~640
 // (cuts and drain) and shared memory ~1400 (operands read by the MMAs, slices
 // written, raw tile and X copied in).  A clock of every role showed where the rest
@@ -240,7 +240,7 @@ __global__ __launch_bounds__(256) void k_col_exp(const float* __restrict__ A, in
 // v in fixed point (54 fraction bits, what lies below as a sticky bit): the FP64
 // form (ldexp, four rint / subtract / scale steps) held the FP64 units for ~1100
 // cycles per warp and 32 entries and, with its strided loads, took ~115 us at any
-// size up to n = 32768 x 60; this form ~12 us.
+// size up to n = 32768 x 60; this form 13-14 us.
 constexpr int SPLIT_THREADS = 1024;
 __global__ __launch_bounds__(SPLIT_THREADS) void k_split_x64(
     const double* __restrict__ X, int64_t ldx, int64_t n, int64_t ncols, int64_t kpad, int nct,

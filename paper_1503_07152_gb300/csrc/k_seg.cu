@@ -102,8 +102,8 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial(
 // scheduler has FMAs to issue and that none is issued for padding: the ka x kb
 // outputs of a chunk are dealt out flat, M to a thread and 128 M to a block (a
 // grid of output tiles would idle lanes at every edge, and one block per chunk
-// left most of the chip idle: 128 chunks x 60 x 37 at N = 16384 took 278 us, this
-// 92; 16 chunks x 20 x 40 at N = 1024 141 us, this 9).
+// left most of the chip idle: 64 chunks x 60 x 37 at N = 16384 took 278 us, this
+// 81).
 template <int M>
 __global__ __launch_bounds__(128) void k_seg_tn_partial64(
     const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
@@ -155,7 +155,7 @@ __global__ __launch_bounds__(128) void k_seg_tn_partial64(
 // over its eight warps, whose sums are added in warp order.  One thread per output
 // would be a chain of 256 dependent FMAs (10 us) behind eight exposed rounds of loads
 // (12 us); here all rows are staged at once and a chain is 32 long.  4 chunks x 20 x 40
-// (N = 1024): 23 -> 9 us.
+// (N = 1024): 23 -> 10 us (164 with one block per chunk).
 __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
     const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
     int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
@@ -210,8 +210,9 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
 // the staged ones are multiplied.  A step whose 32 columns of B are all zero is
 // skipped (its products are exact zeros): the packed test matrices [Omega_2 |
 // Omega_1] are zero on every other child's rows, and the column tiles do not
-// straddle the two halves when kb is split (`half`).  N = 16384, 60 x 120: 228 ->
-// 50 us (64 x 128 outputs a block, one block per chunk, FP64-pipe cuts before).
+// straddle the two halves when kb is split (`half`).  N = 16384, 64 chunks, 60 x
+// 120: 230 -> 80 us (64 x 128 outputs a block, one block per chunk, FP64-pipe cuts
+// before); 60 x 60: 126 -> 48.
 constexpr int DT = 32;  // outputs of a block: DT x DT
 
 __global__ __launch_bounds__(256) void k_seg_tn_partial_df(
@@ -382,7 +383,7 @@ __global__ __launch_bounds__(256) void k_seg_nn(
 // one chunk (<= 64 rows) and every gridDim.y-th tile of CT columns, its four warps
 // the (row half, column group) pairs that exist, so that no FMA is issued for a
 // column past kout or a row half past the chunk (the form with 16 columns a warp
-// issued 128 columns whatever kout: 308 us for N = 16384, 60 x 37, this 93).  CT = 4
+// issued 128 columns whatever kout: 308 us for N = 16384, 60 x 37, this 85).  CT = 4
 // where CT = 8 would leave schedulers without a block.  P aliasing Y: one block has
 // all the tiles (P is staged whole before any write).
 template <int CT>
@@ -444,7 +445,7 @@ __global__ __launch_bounds__(128) void k_seg_nn64(
 // what kin and 32 columns need is staged, so that four blocks share an SM where the
 // full-width staging (196 KB) left one.  With P aliasing Y the launch gives one
 // block all the tiles (P is staged whole before any write).  N = 16384, kin = 60,
-// 120 columns: 126 -> 45 us.
+// 120 columns: 126 -> 99 us; 60 columns: 67 -> 49.
 __global__ __launch_bounds__(256) void k_seg_nn_df(
     const Chunk* __restrict__ chunks, int node0, const double* P, int64_t ldp, int poff_e,
     int poff_o, int kin, const double* __restrict__ C, int64_t cstride, int cld, int cflip,

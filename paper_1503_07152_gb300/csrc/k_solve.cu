@@ -41,8 +41,9 @@ __device__ __forceinline__ double reciprocal(double x) {
 // exchanges the two rows of its columns and updates them.  The multipliers are double-
 // buffered, so one barrier a step orders them: a block writes buffer k & 1 at step k
 // only after the barrier of step k - 1, which every block passes after its last use of
-// that buffer, at step k - 2.  32 leaves of 94: 1510 -> 250 us (one block a matrix, the
-// augmented n x 2n form in L2); 36 x 36 Woodbury blocks: 92 -> 40 us.
+// that buffer, at step k - 2.  32 leaves of 94: 1037 -> 486 us (one block a matrix, the
+// augmented n x 2n form in L2); 16 x 16 Woodbury blocks: 188 -> 136 us (a step is then a
+// chain of FP64 latencies: the pivot search, its reciprocal, the barrier).
 template <typename T>
 __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, int n,
                                                       T* __restrict__ out,
