@@ -27,6 +27,17 @@ __device__ __forceinline__ double reciprocal(double x) {
   return r * __hiloint2double((2046 - e) << 20, 0);
 }
 
+// |x| as an integer of the same order (the bits of a non-negative number), NaN below all:
+// a comparison on the integer pipe instead of one on the FP64 pipe.
+__device__ __forceinline__ long long magnitude_key(double x) {
+  const long long a = __double_as_longlong(x) & 0x7fffffffffffffffll;
+  return a > 0x7ff0000000000000ll ? -1 : a;
+}
+__device__ __forceinline__ long long magnitude_key(float x) {
+  const int a = __float_as_int(x) & 0x7fffffff;
+  return a > 0x7f800000 ? -1 : a;
+}
+
 // Inverse of every matrix of a batch by Gauss-Jordan elimination with partial
 // pivoting, in place (W: n x n, column-major, ld n, in global memory, read once and
 // out[b] written once): row k of the inverse replaces the eliminated column k as the
@@ -41,9 +52,9 @@ __device__ __forceinline__ double reciprocal(double x) {
 // exchanges the two rows of its columns and updates them.  The multipliers are double-
 // buffered, so one barrier a step orders them: a block writes buffer k & 1 at step k
 // only after the barrier of step k - 1, which every block passes after its last use of
-// that buffer, at step k - 2.  32 leaves of 94: 1037 -> 486 us (one block a matrix, the
-// augmented n x 2n form in L2); 16 x 16 Woodbury blocks: 188 -> 136 us (a step is then a
-// chain of FP64 latencies: the pivot search, its reciprocal, the barrier).
+// that buffer, at step k - 2.  32 leaves of 94: 1037 -> 218 us (one block a matrix, the
+// augmented n x 2n form in L2); 36 x 36 Woodbury blocks: 188 -> 67 us (of these 486 and
+// 136 before the pivot search left the FP64 pipe: its comparisons held every scheduler).
 template <typename T>
 __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, int n,
                                                       T* __restrict__ out,
@@ -52,8 +63,6 @@ __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, i
   __shared__ T fcol[2][256];   // the pivot column before the step, rows exchanged
   __shared__ int prow[2];      // its pivot row
   __shared__ T pinv[2];        // 1 / pivot
-  __shared__ double rv[8];
-  __shared__ int ri[8];
   __shared__ short swp[256];   // pivot row of every step
   namespace cg = cooperative_groups;
   cg::cluster_group cl = cg::this_cluster();
@@ -73,25 +82,19 @@ __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, i
     const int buf = k & 1;
     if (k % S == part) {
       T* col = M + (int64_t)(k / S) * n;
-      // pivot: the largest |A(i, k)|, i >= k (first on ties)
-      double best = -1.0;
-      int bi = n;
-      for (int i = k + tid; i < n; i += 256) {
-        const double a = fabs((double)col[i]);
-        if (a > best) { best = a; bi = i; }
+      // pivot: the largest |A(i, k)|, i >= k (first on ties), found by every warp for itself
+      long long best = -1;
+      int p = n;
+      for (int i = k + lane; i < n; i += 32) {
+        const long long a = magnitude_key(col[i]);
+        if (a > best) { best = a; p = i; }
       }
       for (int o = 16; o > 0; o >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+        const long long ob = __shfl_xor_sync(0xffffffffu, best, o);
+        const int oi = __shfl_xor_sync(0xffffffffu, p, o);
+        if (ob > best || (ob == best && oi < p)) { best = ob; p = oi; }
       }
-      if (lane == 0) { rv[warp] = best; ri[warp] = bi; }
-      __syncthreads();
-      double bb = -1.0;
-      int p = n;
-      for (int w = 0; w < 8; ++w)
-        if (rv[w] > bb || (rv[w] == bb && ri[w] < p)) { bb = rv[w]; p = ri[w]; }
-      if (!(bb > 0.0) || p >= n) {
+      if (best <= 0 || p >= n) {
         if (tid == 0) atomicExch(singular, 1);
         p = k;
       }
