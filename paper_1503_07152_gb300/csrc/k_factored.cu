@@ -23,11 +23,13 @@ namespace {
 constexpr int kMaxK = 64;
 
 // partial[chunk][0:k] = V_j(rows)^T x(rows); with second operand pair for the
-// adjoint: partial[chunk][k:2k] = U_j(rows)^T res(rows).  A chunk has at most 256 rows:
-// a lane holds eight entries of the vector, a warp takes every eighth column and sums
-// its 256 entries (coalesced loads, all of a column's in flight) over the warp.
-// N = 262144, k = 32, 335 MB: 70 us (4.8 TB/s),
-// no shared memory; the products transposed through shared memory took the same time.
+// adjoint: partial[chunk][k:2k] = U_j(rows)^T res(rows).  Thread t loads row t's k
+// factor entries at once (independent, coalesced loads), the products go to
+// shared memory (row-major, stride k + 1: conflict-free both ways), thread
+// (col, part) sums its 32-row part of a column, and the 8 parts are added.
+// N = 262144, k = 32: 70 us for one operand (335 MB, 4.8 TB/s), 126 for two.  A form with
+// a warp a column and no shared memory measured 67 for one operand but 241 for two (177
+// with the operands in separate blocks, which cost 93 for one).
 __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restrict__ ch,
                                                       int64_t n, int k,
                                                       const float* __restrict__ A0,
@@ -35,39 +37,44 @@ __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restric
                                                       const float* __restrict__ A1,
                                                       const float* __restrict__ v1,
                                                       float* __restrict__ partial) {
+  extern __shared__ float prod[];  // [256][k + 1]
+  __shared__ float red[8][2 * kMaxK];
   const FactChunk c = ch[blockIdx.x];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int rows = (int)(c.r1 - c.r0);
+  const int tid = threadIdx.x;
+  const int ldp = k + 1;
+  const int64_t row = c.r0 + tid;
+  const bool live = row < c.r1;
   const int npair = A1 ? 2 : 1;
+  const int cl = tid & 31, part = tid >> 5;
   for (int p = 0; p < npair; ++p) {
-    const float* A = (p == 0 ? A0 : A1) + (int64_t)(c.level - 1) * n * k + c.r0;
-    const float* v = (p == 0 ? v0 : v1) + c.r0;
-    float x[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) x[q] = (lane + 32 * q < rows) ? v[lane + 32 * q] : 0.f;
-#pragma unroll 4
-    for (int col = w; col < k; col += 8) {
-      const float* a = A + (int64_t)col * n;
-      float y[8];
-#pragma unroll
-      for (int q = 0; q < 8; ++q) y[q] = (lane + 32 * q < rows) ? a[lane + 32 * q] : 0.f;
+    const float* A = (p == 0 ? A0 : A1) + (int64_t)(c.level - 1) * n * k;
+    const float xv = live ? (p == 0 ? v0 : v1)[row] : 0.f;
+#pragma unroll 8
+    for (int col = 0; col < k; ++col)
+      prod[tid * ldp + col] = live ? A[row + (int64_t)col * n] * xv : 0.f;
+    __syncthreads();
+    for (int col = cl; col < k; col += 32) {
       float s = 0.f;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) s = fmaf(y[q], x[q], s);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-      if (lane == 0) partial[((int64_t)blockIdx.x * npair + p) * k + col] = s;
+      for (int i = 0; i < 32; ++i) s += prod[(part * 32 + i) * ldp + col];
+      red[part][p * k + col] = s;
     }
+    __syncthreads();
+  }
+  for (int e = tid; e < npair * k; e += 256) {
+    float s = 0.f;
+    for (int w = 0; w < 8; ++w) s += red[w][e];
+    partial[(int64_t)blockIdx.x * npair * k + e] = s;
   }
 }
 
 // out[node][e] = sum over the node's chunks (heap ids 2 .. 2^(L+1)-1): chunks
 // begin[node] .. begin[node + 1] at partial[chunk * stride + e], or, without `begin`,
 // the row tiles (`tiles` a leaf) of the node's leaves (L rows of k per tile).  The
-// threads form RED_T / width groups; group q sums chunks q, q + groups, ... and the
+// threads (RED_T over row tiles, RED_C over chunks) form blockDim / width groups; group q sums chunks q, q + groups, ... and the
 // group sums are added in group order (deterministic).  width <= 128.  (A node of level
 // 1 has thousands of row tiles: the chain of its loads is what takes the time.)
-constexpr int RED_T = 1024;
+constexpr int RED_T = 1024, RED_C = 256;
 __global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__ partial,
                                                      const int32_t* __restrict__ fbegin,
                                                      int width, int L, int tiles,
@@ -86,7 +93,7 @@ __global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__
     stride = (int64_t)L * width;
     off = (int64_t)(j - 1) * width;
   }
-  const int groups = RED_T / width;
+  const int groups = blockDim.x / width;
   const int t = threadIdx.x, e = t % width, q = t / width;
   float s = 0.f;
   if (q < groups) {
@@ -187,9 +194,13 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
   }
 }
 
-// The same with y in x's place: a block takes the whole leaf and holds its x before it
-// writes.  (The tiles above read x over the whole leaf while other tiles write.)
-__global__ __launch_bounds__(256) void k_fact_expand_inplace(
+// The same by whole leaves: a block of 256 threads holds the leaf's x (and D^T x) in shared
+// memory, a thread takes a row.  For y in x's place (the tiles above read x over the whole
+// leaf while other tiles write), and where the leaves alone fill the chip and the factors
+// come from HBM (leaf_form): N = 262144, k = 32, 604 MB: 100 us, the tiles 113-128 (shorter
+// runs of each column); N = 65536, k = 16, leaves of 128 (71 MB, in L2): 36 us, the tiles
+// 24-32.
+__global__ __launch_bounds__(256) void k_fact_expand_leaf(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
     int nmax, const float* __restrict__ Uex, const float* __restrict__ coef,
     const float* __restrict__ D, int trans, const float* x, float* y) {
@@ -197,18 +208,36 @@ __global__ __launch_bounds__(256) void k_fact_expand_inplace(
   const int ncol = L * k;
   float* cs = sm;          // ncol coefficients
   float* xs = cs + ncol;   // the leaf's x
+  float* dt = xs + nmax;   // D^T x (trans)
   const int leaf = (1 << L) + blockIdx.x;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  for (int e = threadIdx.x; e < ncol; e += blockDim.x)
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int e = tid; e < ncol; e += 256)
     cs[e] = coef[(int64_t)((leaf >> (L - 1 - e / k)) ^ 1) * k + e % k];
-  for (int m = threadIdx.x; m < ns; m += blockDim.x) xs[m] = x[s0 + m];
+  for (int m = tid; m < ns; m += 256) xs[m] = x[s0 + m];
   __syncthreads();
   const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
-  for (int i = threadIdx.x; i < ns; i += blockDim.x) {
-    const float acc = row_dot(Uex + s0 + i, n, cs, 0, 1, ncol, 0.f);
-    y[s0 + i] = trans ? row_dot(Dl + (int64_t)i * nmax, 1, xs, 0, 1, ns, acc)
-                      : row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
+  if (trans) {
+    for (int i = warp; i < ns; i += 8) {
+      float v = 0.f;
+      for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)i * nmax] * xs[m];
+      v = warp_total(v);
+      if (lane == 0) dt[i] = v;
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < ns; i += 256) {
+    const float* u = Uex + s0 + i;
+    float acc = 0.f;
+    if (trans) {  // (plain loops and batches of loads: each measured the faster one here)
+      for (int e = 0; e < ncol; ++e) acc = fmaf(u[(int64_t)e * n], cs[e], acc);
+      acc += dt[i];
+    } else {
+      acc = row_dot(u, n, cs, 0, 1, ncol, 0.f);
+      acc = row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
+    }
+    y[s0 + i] = acc;
   }
 }
 
@@ -332,7 +361,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
     float* o = gD + (int64_t)blockIdx.x * nmax * nmax + i + (int64_t)g * nmax;
 #pragma unroll 4
     for (int m = g; m < nmax; m += G, o += G * nmax)
-      __stcs(o, m < ns ? sr * (DS ? xs[m] : x[s0 + m]) : 0.f);
+      __stcs(o, live && m < ns ? sr * (DS ? xs[m] : x[s0 + m]) : 0.f);
   }
 }
 
@@ -416,8 +445,71 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
     // (zero past the leaf's size, in rows and columns)
     float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax + i;
     const float sr = scale * ri;
+#pragma unroll 4
     for (int m = g; m < nmax; m += G)
-      __stcs(gDl + (int64_t)m * nmax, m < ns ? sr * x[s0 + m] : 0.f);
+      __stcs(gDl + (int64_t)m * nmax, live && m < ns ? sr * x[s0 + m] : 0.f);
+  }
+}
+
+// The same by whole leaves (leaf_form), coefficients of t and s in one array: a thread a
+// row of the leaf, x, res and D^T res in shared memory.  N = 262144, leaves of 256: 276 us
+// at k = 32 (the tiles 301); the whole adjoint at k = 8 208 us (231).
+__global__ __launch_bounds__(256) void k_fact_adjoint_leaf(
+    const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
+    int nmax, const float* __restrict__ V, const float* __restrict__ D,
+    const float* __restrict__ coef, const float* __restrict__ x, const float* __restrict__ res,
+    float scale, float* __restrict__ gx, float* __restrict__ gU, float* __restrict__ gV,
+    float* __restrict__ gD) {
+  extern __shared__ float sm[];
+  const int ncol = L * k;
+  float* ts = sm;           // t of the sibling per level
+  float* ss = ts + ncol;    // s of the sibling per level
+  float* xs = ss + ncol;
+  float* rs = xs + nmax;
+  float* dt = rs + nmax;    // D^T res
+  const int leaf = (1 << L) + blockIdx.x;
+  const int64_t s0 = start[leaf];
+  const int ns = (int)size[leaf];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  for (int e = tid; e < ncol; e += 256) {
+    const float* c = coef + (int64_t)((leaf >> (L - 1 - e / k)) ^ 1) * 2 * k + e % k;
+    ts[e] = c[0];
+    ss[e] = c[k];
+  }
+  for (int m = tid; m < ns; m += 256) {
+    xs[m] = x[s0 + m];
+    rs[m] = res[s0 + m];
+  }
+  __syncthreads();
+  if (gx) {
+    const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+    for (int i = warp; i < ns; i += 8) {
+      float v = 0.f;
+      for (int m = lane; m < ns; m += 32) v += Dl[m + (int64_t)i * nmax] * rs[m];
+      v = warp_total(v);
+      if (lane == 0) dt[i] = v;
+    }
+    __syncthreads();
+  }
+  float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax;
+  for (int i = tid; i < ns; i += 256) {
+    const int64_t row = s0 + i;
+    const float xr = xs[i], rr = rs[i];
+    float acc = 0.f;
+    for (int e = 0; e < ncol; ++e) {
+      const int64_t off = row + (int64_t)e * n;
+      if (gx) acc = fmaf(V[off], ss[e], acc);
+      if (gU) gU[off] = scale * rr * ts[e];
+      if (gV) gV[off] = scale * xr * ss[e];
+    }
+    if (gx) gx[row] = scale * (acc + dt[i]);
+    if (gD)
+      for (int m = 0; m < nmax; ++m) gDl[i + (int64_t)m * nmax] = m < ns ? scale * rr * xs[m] : 0.f;
+  }
+  if (gD && ns < nmax) {  // rows past the leaf's size
+    const int pad = nmax - ns;
+    for (int e = tid; e < pad * nmax; e += 256)
+      gDl[ns + e % pad + (int64_t)(e / pad) * nmax] = 0.f;
   }
 }
 
@@ -432,6 +524,22 @@ static size_t fact_leaf_smem(const hm_tree* t, bool adjoint) {
                  : sizeof(float) * (L * kMaxK + 2 * nmax);
 }
 
+// dynamic shared memory of k_fact_partial (66.5 KB at k = 64: limit raised once)
+static size_t fact_partial_smem(int k) {
+  static std::atomic<uint32_t> done{0};
+  raise_smem_limit((const void*)k_fact_partial, done);
+  return sizeof(float) * 256 * (size_t)(k + 1);
+}
+
+// Whole leaves where they fill the chip (four blocks an SM) and the factors exceed L2
+// twice over (once for the transposed product): then long runs of each column count, not
+// the number of blocks.  N = 131072, k = 32, leaves of 128 (235 MB), the apply's three
+// kernels: 115 us by leaves and 109 by tiles, transposed 119 and 124.
+static bool leaf_form(const hm_tree* t, int k, int mib = 256) {
+  const size_t leaves = (size_t)1 << t->L;
+  return leaves >= 608 &&
+         sizeof(float) * (size_t)t->n * ((size_t)t->L * k + t->nmax) >= (size_t)mib << 20;
+}
 // Rows of a block's tile: 64, or 32 where 64 would leave SMs without two blocks
 // (N = 4096 in leaves of 256: 64 blocks of 64 rows, 128 of 32).
 static int leaf_rows(const hm_tree* t) {
@@ -482,11 +590,12 @@ hm_status factored_check(const hm_tree* t, bool adjoint) {
               " bytes of shared memory per block; the device allows " + std::to_string(optin));
     return HM_EINVAL;
   }
-  static std::atomic<uint32_t> done_e{0}, done_i{0}, done_a{0};
+  static std::atomic<uint32_t> done_e{0}, done_i{0}, done_a{0}, done_l{0};
   raise_smem_limit((const void*)k_fact_expand, done_e);
-  raise_smem_limit((const void*)k_fact_expand_inplace, done_i);
+  raise_smem_limit((const void*)k_fact_expand_leaf, done_i);
   if (adjoint) {
     raise_smem_limit((const void*)k_fact_adjoint, done_a);
+    raise_smem_limit((const void*)k_fact_adjoint_leaf, done_l);
   }
   return HM_OK;
 }
@@ -505,11 +614,11 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * k;
   // t_node = Proj(I_node)^T x with Proj = V (H x) or U (H^T x)
-  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
                                                nullptr, partial);
-  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
-  if (factored_overlap(x, t->n, y, t->n))
-    k_fact_expand_inplace<<<1u << L, 256, sizeof(float) * ((size_t)L * k + t->nmax), st>>>(
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
+  if (leaf_form(t, k, trans ? 128 : 256) || factored_overlap(x, t->n, y, t->n))
+    k_fact_expand_leaf<<<1u << L, 256, sizeof(float) * ((size_t)L * k + 2 * t->nmax), st>>>(
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, x, y);
   else
     k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
@@ -525,16 +634,22 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
   const int nodes = 1 << (L + 1), rt = leaf_rows(t);
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * 2 * k;
-  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, V, x, U, res, partial);
-  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, U, res,
+                                                        partial);
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
-  k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-      t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
-      scale, nullptr, 0, gx, gU, gV, d_in_place ? nullptr : gD);
-  if (d_in_place)  // once every tile has read D
-    k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
-        scale, nullptr, 0, nullptr, nullptr, nullptr, gD);
+  auto run = [&](float* ox, float* oU, float* oV, float* oD) {
+    if (leaf_form(t, k))
+      k_fact_adjoint_leaf<<<1u << L, 256, sizeof(float) * (2 * (size_t)L * k + 3 * t->nmax), st>>>(
+          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, V, D, coef, x, res, scale, ox, oU, oV,
+          oD);
+    else
+      k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
+          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
+          scale, nullptr, 0, ox, oU, oV, oD);
+  };
+  run(gx, gU, gV, d_in_place ? nullptr : gD);
+  if (d_in_place) run(nullptr, nullptr, nullptr, gD);  // once every tile has read D
 }
 
 size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
@@ -567,9 +682,9 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   float* yy = y ? y : tmp;
   float* rr = res ? res : tmp + t->n;
   float* dtr = tmp + 2 * t->n;
-  k_fact_partial<<<t->n_fchunks, 256, 0, st>>>(t->d_fchunks, t->n, k, V, x, nullptr, nullptr,
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, nullptr, nullptr,
                                                partial);
-  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
   const bool ds = forward_ds(t, k);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
