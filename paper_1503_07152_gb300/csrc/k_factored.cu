@@ -230,13 +230,9 @@ __global__ __launch_bounds__(256) void k_fact_expand_leaf(
   for (int i = tid; i < ns; i += 256) {
     const float* u = Uex + s0 + i;
     float acc = 0.f;
-    if (trans) {  // (plain loops and batches of loads: each measured the faster one here)
-      for (int e = 0; e < ncol; ++e) acc = fmaf(u[(int64_t)e * n], cs[e], acc);
-      acc += dt[i];
-    } else {
-      acc = row_dot(u, n, cs, 0, 1, ncol, 0.f);
-      acc = row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
-    }
+    for (int e = 0; e < ncol; ++e) acc = fmaf(u[(int64_t)e * n], cs[e], acc);
+    if (trans) acc += dt[i];
+    else acc = row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
     y[s0 + i] = acc;
   }
 }
