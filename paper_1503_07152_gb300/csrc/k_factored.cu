@@ -200,10 +200,14 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
 // come from HBM (leaf_form): N = 262144, k = 32, 604 MB: 100 us, the tiles 113-128 (shorter
 // runs of each column); N = 65536, k = 16, leaves of 128 (71 MB, in L2): 36 us, the tiles
 // 24-32.
+// x and y may be one buffer: a block reads its leaf of x before its first barrier, writes
+// its leaf of y after, and touches no other.  Plain loops over qualified pointers: the
+// whole apply 181 us at k = 32; 189 with batches of eight conditional loads, 235 with the
+// same loops unqualified.
 __global__ __launch_bounds__(256) void k_fact_expand_leaf(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
     int nmax, const float* __restrict__ Uex, const float* __restrict__ coef,
-    const float* __restrict__ D, int trans, const float* x, float* y) {
+    const float* __restrict__ D, int trans, const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ float sm[];
   const int ncol = L * k;
   float* cs = sm;          // ncol coefficients
@@ -230,9 +234,13 @@ __global__ __launch_bounds__(256) void k_fact_expand_leaf(
   for (int i = tid; i < ns; i += 256) {
     const float* u = Uex + s0 + i;
     float acc = 0.f;
-    for (int e = 0; e < ncol; ++e) acc = fmaf(u[(int64_t)e * n], cs[e], acc);
-    if (trans) acc += dt[i];
-    else acc = row_dot(Dl + i, nmax, xs, 0, 1, ns, acc);
+    for (int j = 0; j < L; ++j)
+      for (int c = 0; c < k; ++c) acc = fmaf(u[(int64_t)(j * k + c) * n], cs[j * k + c], acc);
+    if (trans) {
+      acc += dt[i];
+    } else {
+      for (int m = 0; m < ns; ++m) acc = fmaf(Dl[i + (int64_t)m * nmax], xs[m], acc);
+    }
     y[s0 + i] = acc;
   }
 }
