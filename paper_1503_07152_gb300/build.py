@@ -32,7 +32,8 @@ def nvcc() -> str:
 
 
 def _headers_mtime() -> float:
-    hs = glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
+    pats = (os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"), os.path.join(ROOT, "include", "*.h"))
+    hs = [h for pat in pats for h in glob.glob(pat)]
     return max((os.path.getmtime(h) for h in hs), default=0.0)
 
 
