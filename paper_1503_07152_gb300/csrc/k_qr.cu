@@ -186,6 +186,7 @@ __global__ __launch_bounds__(256) void k_tsqr_merge(const TsqrTask* __restrict__
         if (on) {
           const T f = beta * (dot + v0 * ak[j]);
           for (int i = gl; i <= j; i += 8) bk[i] = fma(-f, bj[i], bk[i]);
+          __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of A(j, k) first
           if (gl == 0) ak[j] = fma(-f, v0, ak[j]);
         }
       }
@@ -519,6 +520,7 @@ __global__ __launch_bounds__(512) void k_jacobi_mp(const int32_t* __restrict__ n
               vp[i] = tc * x - ts * y;
               vq[i] = ts * x + tc * y;
             }
+            __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of the norms first
             if (gl == 0) {
               const float cs2 = 2.f * tc * ts, c2 = tc * tc, s2 = ts * ts;
               cn32[p] = fmaxf(fmaf(c2, al, fmaf(-cs2, ga, s2 * be)), 0.f);
@@ -667,6 +669,7 @@ __global__ __launch_bounds__(512) void k_jacobi_mp(const int32_t* __restrict__ n
               ap[i] = tc * x - ts * y;
               aq[i] = ts * x + tc * y;
             }
+            __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of the norms first
             if (gl == 0) {
               // norms after the rotation (whatever the angle's accuracy)
               const double cs2 = 2.0 * tc * ts, c2 = tc * tc, s2 = ts * ts;

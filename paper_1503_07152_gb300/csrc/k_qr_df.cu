@@ -639,6 +639,7 @@ __global__ __launch_bounds__(512, 1) void k_jacobi_df(const int32_t* __restrict_
                 aph[o] = xh[e]; apl[o] = xl[e]; aqh[o] = yh[e]; aql[o] = yl[e];
               }
             }
+            __syncwarp(0xffu << (8 * (lane >> 3)));  // the group's reads of the norms first
             if (gl == 0) {
               // norms after the rotation: c^2 al - 2cs ga + s^2 be, s^2 al + 2cs ga + c^2 be
               float c2h, c2l, s2h, s2l, csh, csl, th, tl;
