@@ -479,7 +479,9 @@ void hm_destroy(hm_handle* h);
  *        at offset (j - 1) * N * k.
  *  D:    device float, one n_max x n_max column-major block per leaf
  *        (ld n_max, entries beyond the leaf size are ignored).
- *  x, y: device float vectors of length N (y is overwritten).
+ *  x, y: device float vectors of length N (y is overwritten).  y may be x, or
+ *        share part of x's memory (then x is copied first); it must not share
+ *        memory with U, V or D.
  * trans = 1 applies H^T.  1 <= k <= 64.  Stream-ordered scratch as for the
  * adjoint below.  The per-leaf kernel keeps the leaf's slice of x in shared
  * memory: leaves too large for the device's per-block shared memory (about
@@ -501,8 +503,9 @@ hm_status hm_hodlr_factored_apply(const hm_tree* tree, int32_t k, const float* U
  *  - Scratch: a fixed 8 MiB buffer compiled into the library (reserved on every
  *    device where the library's device code is loaded).  A call needs
  *    4 * k * (c + 2^(L+1)) bytes, c = the number of 256-row chunks over all
- *    nodes of levels 1..L (about L * N / 256); larger requests return
- *    HM_EINVAL naming the size, before anything is launched.
+ *    nodes of levels 1..L (about L * N / 256), and 4 * N more where y shares part
+ *    of x's memory (none for y = x); larger requests return HM_EINVAL naming the
+ *    size, before anything is launched.
  *  - Nothing in the scratch needs to start at zero: every element a call reads
  *    is written earlier in the same call.
  *  - All calls on one device share the one buffer: two calls whose work may
@@ -531,6 +534,9 @@ hm_status hm_hodlr_factored_apply_noalloc(const hm_tree* tree, int32_t k, const 
  * (same layouts as x, U, V, D; outputs are overwritten; any output may be NULL
  * to skip it; gD entries beyond a leaf's size are written as zero).  With
  * r = H x - b and scale = 2 these are the gradients of ||H x - b||^2.
+ * gx may share memory with x or r (which are then copied first), gU and gV with U
+ * and V, gD with D; the outputs share no other memory, with each other or with the
+ * inputs.
  * Stream-ordered scratch of O(k * (N / 256 * L + 2^(L+1))) floats is taken
  * from the CUDA memory pool of the stream's device and released in order.
  * Leaves too large for the per-leaf kernel's shared memory (about 37k points
@@ -546,15 +552,18 @@ hm_status hm_hodlr_factored_adjoint(const hm_tree* tree, int32_t k, const float*
  * residual and the adjoint above at it, in one call,
  *   y = H x,  r = y - b,  then gx, gU, gV, gD exactly as hm_hodlr_factored_adjoint
  *   with this r (scale = 2: the gradients of ||H x - b||^2).
- * The forward's projections V_j(I_b)^T x(I_b) are the ones the adjoint needs, so
- * they are computed once: every factor is read twice per call (U, V and D by
- * the forward and by the adjoint), where the two separate calls read V three
- * times.  b: device, length N.  y, r: device outputs of length N, or NULL (then
- * kept in scratch).  Gradient outputs as in hm_hodlr_factored_adjoint (any may
- * be NULL).  Scratch of O(k * (N / 256 * L + 2^(L+1)) + 2 N) floats is taken
- * from the stream's CUDA memory pool and released in order.  Results equal the
- * two separate calls up to the summation order of the node projections
- * (FP32 rounding).  Errors as hm_hodlr_factored_adjoint.
+ * The forward's projections V_j(I_b)^T x(I_b) are the ones the adjoint needs, and
+ * the forward's blocks also form the adjoint's U_j(I_a)^T r(I_a), D^T r and gD, so V
+ * is read twice per call, U and D once (the two separate calls read V three times,
+ * U and D twice).  b: device, length N.  y, r: device outputs of length N, or NULL
+ * (then kept in scratch).  Gradient outputs as in hm_hodlr_factored_adjoint (any may
+ * be NULL).  y, r and gx may share memory with x and b (which are then copied first),
+ * and gx with r (which it then overwrites); what is said of the gradient outputs
+ * above holds otherwise.  Scratch of O(k * (N / 256 * L + 2^(L+1)) + 2 N) floats, and
+ * (k L 2^L + N) for every tile of 32 rows (16 where L k > 797) that a leaf has, is
+ * taken from the stream's CUDA memory pool and released in order.  Results equal the
+ * two separate calls up to the summation order of the node projections (FP32
+ * rounding).  Errors as hm_hodlr_factored_adjoint.
  */
 hm_status hm_hodlr_factored_loss_grad(const hm_tree* tree, int32_t k, const float* U,
                                       const float* V, const float* D, const float* x,

@@ -267,9 +267,16 @@ hm_status hm_hodlr_factored_apply(const hm_tree* tree, int32_t k, const float* U
   cudaStream_t st = (cudaStream_t)stream;
   HM_TRY(factored_check(tree, false));
   HM_TRY(tree_device(const_cast<hm_tree*>(tree), st));
+  const int64_t n = tree->n;
+  const bool shifted = x != y && factored_overlap(x, n, y, n);
   float* scratch = nullptr;
   const size_t sbytes = factored_scratch_bytes(tree, k);
-  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes, st));
+  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes + (shifted ? n * sizeof(float) : 0), st));
+  if (shifted) {
+    float* own = (float*)((char*)scratch + sbytes);
+    launch_copy_cols<float>(x, n, own, n, n, 1, st);
+    x = own;
+  }
   launch_factored_apply(tree, k, U, V, D, trans, x, y, scratch, st);
   cudaFreeAsync(scratch, st);
   return check_launch("hm_hodlr_factored_apply");
@@ -318,15 +325,21 @@ hm_status hm_hodlr_factored_loss_grad(const hm_tree* tree, int32_t k, const floa
   HM_TRY(factored_check(tree, true));
   HM_TRY(tree_device(const_cast<hm_tree*>(tree), st));
   const int64_t n = tree->n;
-  const bool in_place =
-      (y && factored_overlap(y, n, x, n)) || (res && factored_overlap(res, n, x, n));
+  auto shares = [&](const float* out, const float* in) { return out && factored_overlap(out, n, in, n); };
+  const bool own_x = shares(y, x) || shares(res, x) || shares(gx, x);
+  const bool own_b = shares(y, b) || shares(res, b);
   float* scratch = nullptr;
   const size_t sbytes = factored_loss_grad_scratch_bytes(tree, k);
-  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes + (in_place ? n * sizeof(float) : 0), st));
-  if (in_place) {
-    float* own = (float*)((char*)scratch + sbytes);
+  HM_CUDA_TRY(cudaMallocAsync((void**)&scratch, sbytes + (own_x + own_b) * n * sizeof(float), st));
+  float* own = (float*)((char*)scratch + sbytes);
+  if (own_x) {
     launch_copy_cols<float>(x, n, own, n, n, 1, st);
     x = own;
+    own += n;
+  }
+  if (own_b) {
+    launch_copy_cols<float>(b, n, own, n, n, 1, st);
+    b = own;
   }
   launch_factored_loss_grad(tree, k, U, V, D, x, b, scale, y, res, gx, gU, gV, gD, scratch, st);
   cudaFreeAsync(scratch, st);

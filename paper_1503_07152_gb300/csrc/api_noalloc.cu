@@ -40,7 +40,10 @@ extern "C" hm_status hm_hodlr_factored_apply_noalloc(const hm_tree* tree, int32_
   // (hm_tree_create builds the chunk list, so n_fchunks is exact here)
   const size_t nodes = (size_t)1 << (tree->L + 1);
   const size_t chunks = (size_t)tree->n_fchunks;
-  const size_t need = sizeof(float) * (chunks * (size_t)k + nodes * (size_t)k);
+  // (and a copy of x where y shares part of its memory)
+  const size_t work = chunks * (size_t)k + nodes * (size_t)k;
+  const bool shifted = x != y && factored_overlap(x, tree->n, y, tree->n);
+  const size_t need = sizeof(float) * (work + (shifted ? (size_t)tree->n : 0));
   if (need > kNoallocScratchBytes) {
     set_error("hm_hodlr_factored_apply_noalloc: this tree and k need " + std::to_string(need) +
               " bytes of scratch; the static buffer holds " +
@@ -81,6 +84,11 @@ extern "C" hm_status hm_hodlr_factored_apply_noalloc(const hm_tree* tree, int32_
       g_addr[dev] = p;
     }
     scratch = g_addr[dev];
+  }
+  if (shifted) {
+    float* own = (float*)scratch + work;
+    launch_copy_cols<float>(x, tree->n, own, tree->n, tree->n, 1, (cudaStream_t)stream);
+    x = own;
   }
   launch_factored_apply(tree, k, U, V, D, trans, x, y, (float*)scratch, (cudaStream_t)stream);
   return check_launch("hm_hodlr_factored_apply_noalloc");

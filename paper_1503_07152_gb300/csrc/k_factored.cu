@@ -200,10 +200,11 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
 // come from HBM (leaf_form): N = 262144, k = 32, 604 MB: 100 us, the tiles 113-128 (shorter
 // runs of each column); N = 65536, k = 16, leaves of 128 (71 MB, in L2): 36 us, the tiles
 // 24-32.
-// x and y may be one buffer: a block reads its leaf of x before its first barrier, writes
-// its leaf of y after, and touches no other.  Plain loops over qualified pointers: the
-// whole apply 181 us at k = 32; 189 with batches of eight conditional loads, 235 with the
-// same loops unqualified.
+// IN_PLACE: x is y (the same address) and is read through y: a block reads its leaf before
+// its first barrier, writes it after, and touches no other.  Plain loops over qualified
+// pointers: the whole apply 181 us at k = 32; 189 with batches of eight conditional loads,
+// 235 with the same loops unqualified.
+template <bool IN_PLACE>
 __global__ __launch_bounds__(256) void k_fact_expand_leaf(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
     int nmax, const float* __restrict__ Uex, const float* __restrict__ coef,
@@ -219,7 +220,7 @@ __global__ __launch_bounds__(256) void k_fact_expand_leaf(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int e = tid; e < ncol; e += 256)
     cs[e] = coef[(int64_t)((leaf >> (L - 1 - e / k)) ^ 1) * k + e % k];
-  for (int m = tid; m < ns; m += 256) xs[m] = x[s0 + m];
+  for (int m = tid; m < ns; m += 256) xs[m] = (IN_PLACE ? y : x)[s0 + m];
   __syncthreads();
   const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
   if (trans) {
@@ -573,10 +574,17 @@ static size_t adjoint_smem(const hm_tree* t, int k, int rt) {
 }
 static size_t dsize(const hm_tree* t) { return ((size_t)1 << t->L) * t->nmax * t->nmax; }
 
-// An output in an input's place: the tiles of a leaf read its whole slices of x, res and
-// D while others write, so such calls take a copy or a form of their own.
+// An output that shares memory with an input: the tiles of a leaf read its whole slices of
+// x, res and D while others write, and the kernels' pointers are qualified as disjoint, so
+// such calls take a copy or launches of their own.
 bool factored_overlap(const float* a, size_t na, const float* b, size_t nb) {
   return a < b + nb && b < a + na;
+}
+
+// V is read for gx by the launch that writes gU and gV.  (U is not.)
+static bool v_in_place(const hm_tree* t, int k, const float* V, const float* gU, const float* gV) {
+  const size_t m = (size_t)t->n * t->L * k;
+  return (gU && factored_overlap(gU, m, V, m)) || (gV && factored_overlap(gV, m, V, m));
 }
 
 static dim3 leaf_grid(const hm_tree* t, int rt) {
@@ -594,9 +602,10 @@ hm_status factored_check(const hm_tree* t, bool adjoint) {
               " bytes of shared memory per block; the device allows " + std::to_string(optin));
     return HM_EINVAL;
   }
-  static std::atomic<uint32_t> done_e{0}, done_i{0}, done_a{0}, done_l{0};
+  static std::atomic<uint32_t> done_e{0}, done_i{0}, done_p{0}, done_a{0}, done_l{0};
   raise_smem_limit((const void*)k_fact_expand, done_e);
-  raise_smem_limit((const void*)k_fact_expand_leaf, done_i);
+  raise_smem_limit((const void*)k_fact_expand_leaf<false>, done_i);
+  raise_smem_limit((const void*)k_fact_expand_leaf<true>, done_p);
   if (adjoint) {
     raise_smem_limit((const void*)k_fact_adjoint, done_a);
     raise_smem_limit((const void*)k_fact_adjoint_leaf, done_l);
@@ -609,6 +618,7 @@ size_t factored_scratch_bytes(const hm_tree* t, int k) {
   return sizeof(float) * ((size_t)t->n_fchunks * 2 * k + nodes * 2 * k) + 256;
 }
 
+// x and y: one vector (x == y) or disjoint ones (other overlaps: the callers copy x).
 void launch_factored_apply(const hm_tree* t, int k, const float* U, const float* V,
                            const float* D, int trans, const float* x, float* y, float* scratch,
                            cudaStream_t st) {
@@ -621,14 +631,19 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
   k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
                                                nullptr, partial);
   k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
-  if (leaf_form(t, k, trans ? 128 : 256) || factored_overlap(x, t->n, y, t->n))
-    k_fact_expand_leaf<<<1u << L, 256, sizeof(float) * ((size_t)L * k + 2 * t->nmax), st>>>(
+  const size_t leaf_smem = sizeof(float) * ((size_t)L * k + 2 * t->nmax);
+  if (x == y)
+    k_fact_expand_leaf<true><<<1u << L, 256, leaf_smem, st>>>(
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, nullptr, y);
+  else if (leaf_form(t, k, trans ? 128 : 256))
+    k_fact_expand_leaf<false><<<1u << L, 256, leaf_smem, st>>>(
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, x, y);
   else
     k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
 }
 
+// gU and gV may share memory with U and V, gD with D; gx shares none with the inputs.
 void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const float* V,
                              const float* D, const float* x, const float* res, float scale,
                              float* gx, float* gU, float* gV, float* gD, float* scratch,
@@ -652,8 +667,17 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
           t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
           scale, nullptr, 0, ox, oU, oV, oD);
   };
-  run(gx, gU, gV, d_in_place ? nullptr : gD);
-  if (d_in_place) run(nullptr, nullptr, nullptr, gD);  // once every tile has read D
+  if (gx && v_in_place(t, k, V, gU, gV)) {
+    run(gx, nullptr, nullptr, d_in_place ? nullptr : gD);
+    count_launches(1);
+    run(nullptr, gU, gV, nullptr);  // once every row of V has been read
+  } else {
+    run(gx, gU, gV, d_in_place ? nullptr : gD);
+  }
+  if (d_in_place) {  // once every tile has read D
+    count_launches(1);
+    run(nullptr, nullptr, nullptr, gD);
+  }
 }
 
 size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
@@ -666,7 +690,9 @@ size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
 // y = H x, res = y - b and the adjoint at res: the forward's projections t = V^T x are
 // the adjoint's too, the forward's blocks also form s = U^T res (per tile of rows;
 // reduced per node), D^T res and the gradient of D, and the adjoint's pass reads V once
-// more and writes gx, gU, gV.  N = 262144, k = 32 (2.2 GB instead of 2.8): 557 -> 502 us.
+// more and writes gx, gU, gV.  y and res share no memory with x and b, gx none with x; gU
+// and gV may with U and V, gD with D, gx with res.  N = 262144, k = 32 (2.2 GB instead of
+// 2.8): 557 -> 502 us.
 void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const float* V,
                                const float* D, const float* x, const float* b, float scale,
                                float* y, float* res, float* gx, float* gU, float* gV, float* gD,
@@ -709,14 +735,28 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
     default: forward(k_fact_forward<0, 4>, done[7]); break;
   }
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
-  if (d_in_place)  // once every tile has read D
+  if (d_in_place) {  // once every tile has read D
+    count_launches(1);
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
         t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, nullptr,
         0, nullptr, nullptr, nullptr, gD);
-  if (gx || gU || gV)
+  }
+  if (res && gx && factored_overlap(gx, t->n, res, t->n)) {
+    launch_copy_cols<float>(res, t->n, tmp + t->n, t->n, t->n, 1, st);
+    rr = tmp + t->n;
+  }
+  auto adjoint = [&](float* ox, float* oU, float* oV) {
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
         t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
-        tiles, gx, gU, gV, nullptr);
+        tiles, ox, oU, oV, nullptr);
+  };
+  if (gx && v_in_place(t, k, V, gU, gV)) {
+    adjoint(gx, nullptr, nullptr);
+    count_launches(1);
+    adjoint(nullptr, gU, gV);  // once every row of V has been read
+  } else if (gx || gU || gV) {
+    adjoint(gx, gU, gV);
+  }
 }
 
 }  // namespace hm
