@@ -318,7 +318,9 @@ hm_status hm_tune_batched(int32_t nops, const hm_operator* ops, hm_tree* const* 
  * HODLR product of Sec. 2.8 (block diagonal plus every sibling block), or the
  * HBS / HBS-ID product of Fig. "Application of A^(m) in the HBS framework"
  * with m = L plus the leaf blocks.  X, Y: device, column-major, n x ncols,
- * element type of the handle's precision.  X and Y must not overlap.
+ * element type of the handle's precision.  Y may be X, or columns beside X's in
+ * one buffer; where the two share elements in any other way X is copied first (the
+ * copy is taken from the stream's memory pool).
  */
 hm_status hm_apply(const hm_handle* h, int trans, int64_t ncols, const void* X, int64_t ldx,
                    void* Y, int64_t ldy, void* stream);
@@ -404,7 +406,8 @@ hm_status hm_hodlr_factorize(hm_handle* h, void* stream);
 
 /*
  * X = A_c^{-1} B (trans = 0) or A_c^{-T} B (trans = 1) for a factorized HODLR
- * handle; B, X device, column-major, n x ncols, the handle's element type.
+ * handle; B, X device, column-major, n x ncols, the handle's element type (X may
+ * share B's memory, as in hm_apply).
  * O(k N log N) per column.  HM_EINVAL if the handle is not factorized.
  */
 hm_status hm_solve(const hm_handle* h, int trans, int64_t ncols, const void* B, int64_t ldb,

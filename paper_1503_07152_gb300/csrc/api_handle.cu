@@ -26,11 +26,12 @@ static hm_status apply_any(const hm_handle* h, int trans, int64_t ncols, const T
     if (h->format == HM_FORMAT_HODLR) return hodlr_apply_t<T>(h, trans, w, Xb, ld, Yb, ldy, st);
     return hbs_apply_t<T>(h, trans, w, Xb, ld, Yb, ldy, st);
   };
-  // the products read X while they write Y: where the two share memory (one buffer, or
-  // alternating columns of one), from a copy of X, 128 columns at a time
-  if (X + (ncols - 1) * ldx + h->n <= Y || Y + (ncols - 1) * ldy + h->n <= X)
-    return run(ncols, X, ldx, Y);
-  const int64_t cbw = 128, N = h->n;
+  // the products read X while they write Y: where the two share memory, from a copy of X
+  // (Y in X's place: 128 columns at a time; else a block's columns may be columns of X
+  // that come later: all of X)
+  const Share share = block_share(X, ldx, Y, ldy, h->n, ncols);
+  if (share == Share::kNone) return run(ncols, X, ldx, Y);
+  const int64_t cbw = share == Share::kSame ? 128 : ncols, N = h->n;
   T* Xc = nullptr;
   HM_CUDA_TRY(cudaMallocAsync((void**)&Xc, sizeof(T) * N * std::min(cbw, ncols), st));
   hm_status s = HM_OK;

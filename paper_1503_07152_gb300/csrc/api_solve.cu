@@ -232,8 +232,12 @@ hm_status solve_t(const hm_handle* h, int trans, int64_t ncols, const T* B, int6
   c.W = (T*)h->solv + h->solv_w;
   c.M = (T*)h->solv + h->solv_m;
   c.items_cap = 4 * (size_t)nleaf + 16;
-  T *Yc = nullptr, *Bc = nullptr;
+  // X may share B's memory: each block of B is copied before X's is written, and all of B
+  // where a block of X may hold columns of B that come later
+  const bool whole = block_share(B, ldb, X, ldx, N, ncols) == Share::kOther;
+  T *Yc = nullptr, *Bc = nullptr, *Ball = nullptr;
   auto layout = [&](Arena& a) {
+    if (whole) Ball = a.take<T>((size_t)N * ncols);
     Yc = a.take<T>((size_t)N * cbw);
     Bc = a.take<T>((size_t)N * cbw);
     c.q = a.take<T>((size_t)nleaf * r * cbw);
@@ -249,6 +253,11 @@ hm_status solve_t(const hm_handle* h, int trans, int64_t ncols, const T* B, int6
   a.base = (unsigned char*)blk;
   a.cap = m.off + 256;
   layout(a);
+  if (whole) {
+    launch_copy_cols<T>(B, ldb, Ball, N, N, ncols, st);
+    B = Ball;
+    ldb = N;
+  }
   hm_status s = HM_OK;
   for (int64_t cb = 0; cb < ncols && s == HM_OK; cb += cbw) {
     const int w = (int)std::min<int64_t>(cbw, ncols - cb);

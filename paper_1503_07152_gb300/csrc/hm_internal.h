@@ -75,6 +75,22 @@ __device__ __forceinline__ void with_count(int n, F&& f) {
 }
 #endif
 
+// How two column-major blocks of n rows lie to each other: no element in common (apart, or
+// columns of one buffer side by side), the same block, or anything else.
+enum class Share { kNone, kSame, kOther };
+template <typename T>
+Share block_share(const T* X, int64_t ldx, const T* Y, int64_t ldy, int64_t n, int64_t ncols) {
+  const intptr_t x = (intptr_t)X, y = (intptr_t)Y, es = (intptr_t)sizeof(T);
+  if (x + es * ((ncols - 1) * ldx + n) <= y || y + es * ((ncols - 1) * ldy + n) <= x)
+    return Share::kNone;
+  if (x == y && (ldx == ldy || ncols == 1)) return Share::kSame;
+  if (ldx == ldy && ncols > 1 && (y - x) % es == 0) {
+    const int64_t m = (((y - x) / es) % ldx + ldx) % ldx;  // Y's columns, m rows below X's
+    if (m >= n && m + n <= ldx) return Share::kNone;
+  }
+  return Share::kOther;
+}
+
 // Row chunk of one tree node: rows [r0, r1) of node `node`.
 struct Chunk {
   int32_t node;

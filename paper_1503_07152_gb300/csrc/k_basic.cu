@@ -6,6 +6,8 @@
 //  - block-diagonal products with the leaf blocks D_tau,
 //  - tile kernels of the Frobenius error (Sec. 5), the log-kernel workload
 //    generator, and a NaN/Inf detector.
+#include <algorithm>
+
 #include <cuda_bf16.h>
 
 #include "hm_internal.h"
@@ -345,10 +347,12 @@ void launch_blockdiag_apply(const T* D, int nmax, int trans, const T* X, int64_t
 template <typename T>
 void launch_copy_cols(const T* src, int64_t lds, T* dst, int64_t ldd, int64_t rows, int64_t cols,
                       cudaStream_t st) {
-  if (rows <= 0 || cols <= 0) return;
-  count_launches(1);
-  dim3 grid(blocks_for(rows, 256), (unsigned)cols);
-  k_copy_cols<T><<<grid, 256, 0, st>>>(src, lds, dst, ldd, rows);
+  if (rows <= 0) return;
+  for (int64_t c = 0; c < cols; c += 65535) {  // (the grid's second dimension)
+    count_launches(1);
+    dim3 grid(blocks_for(rows, 256), (unsigned)std::min<int64_t>(65535, cols - c));
+    k_copy_cols<T><<<grid, 256, 0, st>>>(src + c * lds, lds, dst + c * ldd, ldd, rows);
+  }
 }
 
 template <typename T>

@@ -1,8 +1,10 @@
-"""Outputs that share memory with inputs: the factored layer's calls where the header
-allows it, at shifts that make a block's output another block's input, give what they
-give with buffers of their own."""
+"""Outputs that share memory with inputs: the factored layer's calls and the handles' where
+the header allows it, at shifts that make a block's output another block's input, give
+what they give with buffers of their own."""
 import pytest
 import torch
+
+import workloads as W
 
 pytestmark = pytest.mark.gpu
 hm = pytest.importorskip("paper_1503_07152_gb300")
@@ -114,3 +116,42 @@ def test_gradients_over_inputs(n, m, k):
     out = [new()[0], Vi, *new()[2:]]
     step(x, b, ny, nr, out, U, Vi, D)
     assert same([ny, nr, *out], [y, r, *want])
+
+
+def handle(kind, n):
+    A = torch.from_numpy(W.log_kernel(n)).to(DEV, torch.float32 if kind == "mixed" else torch.float64)
+    A += float(n) * torch.eye(n, device=DEV, dtype=A.dtype)
+    op, t = hm.hm_dense_operator_create(A), hm.Tree(n, 65)
+    if kind == "hbsid":
+        return hm.hm_compress_hbs(op, t, tol=1e-6, r=24, seed=2, prec=hm.HM_FP64)
+    return hm.hm_compress_hodlr(op, t, k=16, p=4, seed=2, prec=hm.HM_MIXED if kind == "mixed" else hm.HM_FP64)
+
+
+@pytest.mark.parametrize("kind", ["fp64", "mixed", "hbsid"])
+@pytest.mark.parametrize("c", [1, 3, 128, 129, 300])
+def test_blocks_that_share_memory(kind, c):
+    """hm_apply and hm_solve with Y (X) at shifts by rows and columns over X (B), at other
+    leading dimensions and in X's place, past the 128 columns that go together."""
+    n = 515
+    h = handle(kind, n)
+    dt = torch.float32 if kind == "mixed" else torch.float64
+    X = torch.randn((c, n), device=DEV, dtype=dt, generator=torch.Generator(DEV).manual_seed(c))
+    calls = [hm.hm_apply]
+    if kind != "hbsid":
+        hm.hm_hodlr_factorize(h)
+        calls.append(hm.hm_solve)
+    for call in calls:
+        for trans in (0, 1):
+            want = torch.full_like(X, float("nan"))
+            call(h, trans, X, want)
+            for ldx, ldy, off in ((n, n, 0), (n + 7, n, 0), (n, n + 7, 0), (n, n, n), (n, n, -n), (n, n, 1),
+                                  (n, n + 1, -5), (2 * n, 2 * n, n), (2 * n, 2 * n, n - 1), (n, 2 * n, n),
+                                  (n, n, (c // 2) * n)):
+                buf = torch.full(((c + 1) * 2 * n + abs(off) + 8 * c,), float("nan"), device=DEV, dtype=dt)
+                x0 = max(0, -off)
+                a = torch.as_strided(buf, (c, n), (ldx, 1), x0)
+                y = torch.as_strided(buf, (c, n), (ldy, 1), x0 + off)
+                a.copy_(X)
+                call(h, trans, a, y)
+                torch.cuda.synchronize()
+                assert torch.equal(y, want), (call.__name__, trans, ldx, ldy, off)
