@@ -103,7 +103,9 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial(
 // outputs of a chunk are dealt out flat, M to a thread and 128 M to a block (a
 // grid of output tiles would idle lanes at every edge, and one block per chunk
 // left most of the chip idle: 64 chunks x 60 x 37 at N = 16384 took 278 us, this
-// 81).
+// 81).  Products are summed over SUM64 rows and those sums added up: the rounding error
+// of a 256-row chain is 2.7 times that, for one FP64 add in 17 less.
+constexpr int SUM64 = 16;  // terms of a chain in the FP64 sums
 template <int M>
 __global__ __launch_bounds__(128) void k_seg_tn_partial64(
     const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
@@ -137,10 +139,16 @@ __global__ __launch_bounds__(128) void k_seg_tn_partial64(
         Bs[rr * pb + c] = B[r0 + rr + (int64_t)(boff + jlo + c) * ldb];
     }
     __syncthreads();
+    for (int q0 = 0; q0 < rows; q0 += SUM64) {
+      const int q1 = min(rows, q0 + SUM64);
+      double t[M] = {};
 #pragma unroll 4
-    for (int q = 0; q < rows; ++q)
+      for (int q = q0; q < q1; ++q)
 #pragma unroll
-      for (int m = 0; m < M; ++m) acc[m] = fma(As[q * pa + ia[m]], Bs[q * pb + jb[m]], acc[m]);
+        for (int m = 0; m < M; ++m) t[m] = fma(As[q * pa + ia[m]], Bs[q * pb + jb[m]], t[m]);
+#pragma unroll
+      for (int m = 0; m < M; ++m) acc[m] += t[m];
+    }
     __syncthreads();
   }
   double* out = partial + (int64_t)blockIdx.x * mtot;  // output (i, j) at i + j ka
@@ -151,17 +159,18 @@ __global__ __launch_bounds__(128) void k_seg_tn_partial64(
   }
 }
 
-// The same for few chunks (a small operator): 32 outputs a block, the chunk's rows split
-// over its eight warps, whose sums are added in warp order.  One thread per output
-// would be a chain of 256 dependent FMAs (10 us) behind eight exposed rounds of loads
-// (12 us); here all rows are staged at once and a chain is 32 long.  4 chunks x 20 x 40
-// (N = 1024): 23 -> 10 us (164 with one block per chunk).
+// The same for few chunks (a small operator): 32 outputs a block, the chunk's groups of
+// SUM64 rows dealt out to its eight warps, the groups' sums added in row order as above
+// (the same bits: a column's result does not depend on how many go along).  One thread per
+// output would be a chain of 256 dependent FMAs (10 us) behind eight exposed rounds of
+// loads (12 us); here all rows are staged at once and a chain is 16 long.  4 chunks x
+// 20 x 40 (N = 1024): 23 -> 10 us (164 with one block per chunk).
 __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
     const Chunk* __restrict__ chunks, const double* __restrict__ A, int64_t lda, int aoff_e,
     int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
     int kb, double* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[8][32];
+  __shared__ double red[256 / SUM64][32];
   const Chunk ch = chunks[blockIdx.x];
   const int rows = (int)(ch.r1 - ch.r0);  // <= 256
   const int aoff = (ch.node & 1) ? aoff_o : aoff_e;
@@ -183,15 +192,18 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
   __syncthreads();
   const int jb = lane < ne ? (e0 + lane) / ka - jlo : 0;
   const int c = lane < ne ? lane : 0;
-  const int per = (rows + 7) / 8, q0 = min(rows, w * per), q1 = min(rows, q0 + per);
-  double acc = 0.0;
+  const int groups = (rows + SUM64 - 1) / SUM64;
+  for (int g = w; g < groups; g += 8) {
+    const int q1 = min(rows, (g + 1) * SUM64);
+    double t = 0.0;
 #pragma unroll 4
-  for (int q = q0; q < q1; ++q) acc = fma(As[q * 33 + c], Bs[q * pb + jb], acc);
-  red[w][lane] = acc;
+    for (int q = g * SUM64; q < q1; ++q) t = fma(As[q * 33 + c], Bs[q * pb + jb], t);
+    red[g][lane] = t;
+  }
   __syncthreads();
   if (w == 0 && lane < ne) {
-    double v = red[0][lane];
-    for (int q = 1; q < 8; ++q) v += red[q][lane];
+    double v = 0.0;
+    for (int g = 0; g < groups; ++g) v += red[g][lane];
     partial[(int64_t)blockIdx.x * mtot + e0 + lane] = v;
   }
 }
@@ -418,11 +430,17 @@ __global__ __launch_bounds__(128) void k_seg_nn64(
     double acc[CT / 2] = {};
     if (nj > 0)
       with_count<CT / 2>(nj, [&](auto cols) {
+        for (int k0 = 0; k0 < kin; k0 += SUM64) {
+          const int k1 = min(kin, k0 + SUM64);
+          double t[cols] = {};
 #pragma unroll 4
-        for (int k = 0; k < kin; ++k) {
-          const double a = Ps[k * NN_ROWS + rr];
+          for (int k = k0; k < k1; ++k) {
+            const double a = Ps[k * NN_ROWS + rr];
 #pragma unroll
-          for (int j = 0; j < cols; ++j) acc[j] = fma(a, Cs[(g + ng * j) * kin + k], acc[j]);
+            for (int j = 0; j < cols; ++j) t[j] = fma(a, Cs[(g + ng * j) * kin + k], t[j]);
+          }
+#pragma unroll
+          for (int j = 0; j < cols; ++j) acc[j] += t[j];
         }
       });
 #pragma unroll
