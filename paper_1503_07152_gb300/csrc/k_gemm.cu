@@ -134,9 +134,16 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
 // on every scheduler and none for padding: a block of four warps takes 32 rows
 // (lanes) x 32 columns (warp w: columns w, w + 4, ..), only columns that exist are
 // multiplied, and where the row blocks alone would not fill the chip a cluster of S
-// blocks shares a tile's active K tiles (dealt out in turn) and sums its shares over
-// distributed shared memory in rank order (deterministic, no workspace).  N = 1024,
-// 20 columns, half of K active: 1175 us as 8 blocks of 128 x 64 outputs, 39 us so.
+// blocks shares a tile's K tiles and sums its shares over distributed shared memory in
+// rank order (deterministic, no workspace).  N = 1024, 20 columns, half of K active:
+// 1175 us as 8 blocks of 128 x 64 outputs, 41 us so.
+//
+// K tile t belongs to block t mod 2S, or its mirror image 2S - 1 - t mod 2S where that
+// is not below S: half-active patterns of any period then spread over the blocks, and
+// neither the other columns nor their zeros decide which sums a column's terms go to.
+// Products are summed 16 at a time and those sums added up (a chain over all of K
+// rounds 3 times as much at N = 8192, for one FP64 add in 17 less: N = 4096, 5 columns
+// 329 us, 340 so).
 template <typename TA, int TRANS>
 __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, int64_t lda,
                                                       int64_t n, int64_t ncols,
@@ -154,12 +161,10 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
   const int nq = w < nc ? (nc - w + 3) / 4 : 0;  // this warp's columns
   double acc[8] = {};
   const int nkt = (int)((n + BK - 1) / BK);
-  int turn = 0;
   for (int kt = 0; kt < nkt; ++kt) {
-    if (flags && !flags[(int64_t)kt * nct + ct]) continue;  // uniform over the cluster
-    const bool mine = turn == part;
-    turn = turn + 1 == S ? 0 : turn + 1;
-    if (!mine) continue;
+    if (flags && !flags[(int64_t)kt * nct + ct]) continue;  // uniform over the block
+    const int q = kt & (2 * S - 1);  // (S is a power of two)
+    if ((q < S ? q : 2 * S - 1 - q) != part) continue;
     const int64_t k0 = (int64_t)kt * BK;
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
@@ -174,11 +179,17 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
     __syncthreads();
     if (nq > 0)
       with_count<8>(nq, [&](auto cols) {
-#pragma unroll 4
-        for (int k = 0; k < BK; ++k) {
-          const double a = TRANS ? As[k][lane] : As[lane][k];
 #pragma unroll
-          for (int q = 0; q < cols; ++q) acc[q] = fma(a, Xs[w + 4 * q][k], acc[q]);
+        for (int k0 = 0; k0 < BK; k0 += 16) {
+          double t[cols] = {};
+#pragma unroll 4
+          for (int k = k0; k < k0 + 16; ++k) {
+            const double a = TRANS ? As[k][lane] : As[lane][k];
+#pragma unroll
+            for (int q = 0; q < cols; ++q) t[q] = fma(a, Xs[w + 4 * q][k], t[q]);
+          }
+#pragma unroll
+          for (int q = 0; q < cols; ++q) acc[q] += t[q];
         }
       });
     __syncthreads();
@@ -204,9 +215,10 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
 
 }  // namespace
 
-// The FP64 GEMM with its cluster size: doubled while the blocks are fewer than three
-// per SM (152 SMs) and there is a K tile for each (N = 1024 x 20: 8 blocks a tile;
-// from N ~ 15000 on: 1).
+// The FP64 GEMM with its cluster size: doubled while one column tile's blocks are fewer
+// than three per SM (152 SMs) and there is a K tile for each (N = 1024: 8 blocks a tile;
+// from N ~ 15000 on: 1).  The number of columns plays no part: it would decide how a
+// column's terms are grouped.
 template <typename TA>
 static void dense_gemm64(const TA* A, int64_t lda, int trans, int64_t n, int64_t ncols,
                          const double* X, int64_t ldx, double* Y, int64_t ldy, uint8_t* flags,
@@ -216,7 +228,7 @@ static void dense_gemm64(const TA* A, int64_t lda, int trans, int64_t n, int64_t
   if (flags) k_tile_flags<double, 32><<<dim3(nkt, nct), 256, 0, st>>>(X, ldx, n, ncols, flags, nct);
   const int64_t rows = (n + 31) / 32;
   int S = 1;
-  while (S < 8 && rows * nct * S < 456 && 2 * S <= nkt) S *= 2;
+  while (S < 8 && rows * S < 456 && 2 * S <= nkt) S *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)rows, (unsigned)S, (unsigned)nct);
   cfg.blockDim = dim3(128);
