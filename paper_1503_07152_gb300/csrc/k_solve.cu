@@ -10,23 +10,6 @@
 namespace hm {
 namespace {
 
-// 1 / x to within an ulp: in FP64 three Newton steps r <- r + r (1 - x r) from the FP32
-// reciprocal of the fraction (a chain of six FMAs; the division is ~20 instructions of
-// 76 cycles each).  Zeros, infinities, NaN and subnormals take the division.
-__device__ __forceinline__ float reciprocal(float x) { return 1.f / x; }
-__device__ __forceinline__ double reciprocal(double x) {
-  const int e = (int)((__double2hiint(x) >> 20) & 0x7ff);
-  if (e < 2 || e > 2044) return 1.0 / x;
-  // x = m 2^(e - 1023), 1 <= |m| < 2
-  const double m = __hiloint2double((__double2hiint(x) & (int)0x800fffff) | 0x3ff00000,
-                                    __double2loint(x));
-  double r = (double)(1.f / (float)m);
-  r = fma(r, fma(-m, r, 1.0), r);
-  r = fma(r, fma(-m, r, 1.0), r);
-  r = fma(r, fma(-m, r, 1.0), r);
-  return r * __hiloint2double((2046 - e) << 20, 0);
-}
-
 // |x| as an integer of the same order (the bits of a non-negative number), NaN below all:
 // a comparison on the integer pipe instead of one on the FP64 pipe.
 __device__ __forceinline__ long long magnitude_key(double x) {
@@ -52,9 +35,10 @@ __device__ __forceinline__ long long magnitude_key(float x) {
 // exchanges the two rows of its columns and updates them.  The multipliers are double-
 // buffered, so one barrier a step orders them: a block writes buffer k & 1 at step k
 // only after the barrier of step k - 1, which every block passes after its last use of
-// that buffer, at step k - 2.  32 leaves of 94: 1037 -> 218 us (one block a matrix, the
-// augmented n x 2n form in L2); 36 x 36 Woodbury blocks: 188 -> 67 us (of these 486 and
-// 136 before the pivot search left the FP64 pipe: its comparisons held every scheduler).
+// that buffer, at step k - 2.  32 leaves of 94: 1037 -> 204 us (one block a matrix, the
+// augmented n x 2n form in L2); 36 x 36 Woodbury blocks: 188 -> 62 us (486 and 136 before
+// the pivot search left the FP64 pipe: its comparisons held every scheduler; 218 and 68
+// with three Newton steps from the FP32 reciprocal in the division's place).
 template <typename T>
 __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, int n,
                                                       T* __restrict__ out,
@@ -104,7 +88,7 @@ __global__ __launch_bounds__(256) void k_gauss_jordan(const T* __restrict__ W, i
       }
       if (warp == 0) {  // (one warp: an FP64 division is a long chain on the FP64 pipe)
         const T pv = col[p];
-        const T iv = (pv != (T)0) ? reciprocal(pv) : (T)0;
+        const T iv = (pv != (T)0) ? (T)1 / pv : (T)0;
         if (lane < S) {
           (S > 1 ? cl.map_shared_rank(&prow[buf], lane) : &prow[buf])[0] = p;
           (S > 1 ? cl.map_shared_rank(&pinv[buf], lane) : &pinv[buf])[0] = iv;
