@@ -552,16 +552,15 @@ static int leaf_rows(const hm_tree* t) {
   return leaves * ((t->nmax + 63) / 64) >= 304 ? 64 : 32;
 }
 // The fused forward keeps its tile's L k columns of U and, where two blocks an SM then
-// still fit, its rows of D in shared memory: 32 rows, fewer where L k is large.
+// still fit, its rows of D in shared memory: 32 rows, 16 where L k is above 797 (13 levels
+// at k = 64; at the most, L = 24 and k = 64, one block an SM).
 static size_t forward_smem(const hm_tree* t, int k, int rt, bool ds) {
   const size_t ncol = (size_t)t->L * k, nmax = (size_t)t->nmax;
   return sizeof(float) * (ncol * (rt + 2) + LEAF_T + rt + (ds ? nmax * (rt + 2) : LEAF_X));
 }
 constexpr size_t kForwardSmem = 112 * 1024;
 static int forward_rows(const hm_tree* t, int k) {
-  int rt = 32;
-  while (rt > 4 && forward_smem(t, k, rt, false) > kForwardSmem) rt /= 2;
-  return rt;
+  return forward_smem(t, k, 32, false) <= kForwardSmem ? 32 : 16;
 }
 static bool forward_ds(const hm_tree* t, int k) {
   return forward_smem(t, k, forward_rows(t, k), true) <= kForwardSmem;
@@ -723,17 +722,9 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
                                                          coef_t, D, x, yy, b, rr, scale, sp, dtr,
                                                          d_in_place ? nullptr : gD);
   };
-  static std::atomic<uint32_t> done[8] = {{0}, {0}, {0}, {0}, {0}, {0}, {0}, {0}};
-  switch (2 * rf + ds) {
-    case 65: forward(k_fact_forward<1, 32>, done[0]); break;
-    case 64: forward(k_fact_forward<0, 32>, done[1]); break;
-    case 33: forward(k_fact_forward<1, 16>, done[2]); break;
-    case 32: forward(k_fact_forward<0, 16>, done[3]); break;
-    case 17: forward(k_fact_forward<1, 8>, done[4]); break;
-    case 16: forward(k_fact_forward<0, 8>, done[5]); break;
-    case 9: forward(k_fact_forward<1, 4>, done[6]); break;
-    default: forward(k_fact_forward<0, 4>, done[7]); break;
-  }
+  static std::atomic<uint32_t> done[4] = {{0}, {0}, {0}, {0}};
+  if (rf == 32) ds ? forward(k_fact_forward<1, 32>, done[0]) : forward(k_fact_forward<0, 32>, done[1]);
+  else ds ? forward(k_fact_forward<1, 16>, done[2]) : forward(k_fact_forward<0, 16>, done[3]);
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
   if (d_in_place) {  // once every tile has read D
     count_launches(1);
