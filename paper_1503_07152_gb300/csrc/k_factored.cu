@@ -143,7 +143,7 @@ __device__ __forceinline__ float warp_total(float v) {
 // rows.
 __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
-    int nmax, int rt, const float* __restrict__ Uex, const float* __restrict__ coef,
+    int nmax, int rt, int tiles, const float* __restrict__ Uex, const float* __restrict__ coef,
     const float* __restrict__ D, int trans, const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ float sm[];
   const int ncol = L * k;          // column e of level 1 + e / k starts at Uex + e n
@@ -151,10 +151,10 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
   float* xs = cs + ncol;           // LEAF_X entries of the leaf's x
   float* part = xs + LEAF_X;       // the groups' row sums
   float* rs = part + LEAF_T;       // rt rows of D^T x (trans)
-  const int leaf = (1 << L) + blockIdx.x;
+  const int li = blockIdx.x / tiles, leaf = (1 << L) + li;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int i0 = blockIdx.y * rt;
+  const int i0 = (blockIdx.x - li * tiles) * rt;
   if (i0 >= ns) return;  // uniform over the block
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
@@ -163,7 +163,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
     const int anc = leaf >> (L - j);
     cs[e] = coef[(int64_t)(anc ^ 1) * k + col];
   }
-  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+  const float* Dl = D + (int64_t)li * nmax * nmax;
   if (trans)
     for (int q = warp; q < rt; q += LEAF_T / 32) {
       float v = 0.f;
@@ -264,7 +264,7 @@ __device__ __forceinline__ void copy_async4(float* dst, const float* src) {
 template <int DS, int rt>
 __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
-    int nmax, const float* __restrict__ U, const float* __restrict__ coef,
+    int nmax, int tiles, const float* __restrict__ U, const float* __restrict__ coef,
     const float* __restrict__ D, const float* __restrict__ x, float* __restrict__ y,
     const float* __restrict__ b, float* __restrict__ res, float scale, float* __restrict__ sp,
     float* __restrict__ dtr, float* __restrict__ gD) {
@@ -277,14 +277,14 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
   float* rs = part + LEAF_T;       // rt rows of res
   float* us = rs + rt;             // the tile's rows of U, [ncol][pt]
   float* ds = us + ncol * pt;      // DS: its rows of D, [nmax][pt]
-  const int leaf = (1 << L) + blockIdx.x;
+  const int li = blockIdx.x / tiles, tile = blockIdx.x - li * tiles, leaf = (1 << L) + li;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int i0 = blockIdx.y * rt;
+  const int i0 = tile * rt;
   const int tid = threadIdx.x;
   const int g = tid / rt, ti = tid & (rt - 1), i = i0 + ti;
   const bool live = i < ns;
-  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+  const float* Dl = D + (int64_t)li * nmax * nmax;
   if (live) {
     const float* u = U + s0 + i + (int64_t)g * n;
     float* d = us + g * pt + ti;
@@ -340,8 +340,8 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
   }
   __syncthreads();
   // a thread a column: D^T res, then U^T res over the tile's rows
-  float* spt = sp + ((int64_t)blockIdx.x * gridDim.y + blockIdx.y) * ncol;
-  float* dt = dtr + (int64_t)blockIdx.y * n + s0;
+  float* spt = sp + (int64_t)blockIdx.x * ncol;
+  float* dt = dtr + (int64_t)tile * n + s0;
   const int nd = DS ? ns : 0;
   for (int e = tid; e < nd + ncol; e += LEAF_T) {
     const float* c = e < nd ? ds + e * pt : us + (e - nd) * pt;
@@ -363,7 +363,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
   if (gD && i < nmax) {
     // (zero past the leaf's size, in rows and columns)
     const float sr = scale * rs[ti];
-    float* o = gD + (int64_t)blockIdx.x * nmax * nmax + i + (int64_t)g * nmax;
+    float* o = gD + (int64_t)li * nmax * nmax + i + (int64_t)g * nmax;
 #pragma unroll 4
     for (int m = g; m < nmax; m += G, o += G * nmax)
       __stcs(o, live && m < ns ? sr * (DS ? xs[m] : x[s0 + m]) : 0.f);
@@ -375,7 +375,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
 // tiles' shares of D^T res where the forward has formed them (and written gD), else null.
 __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
-    int nmax, int rt, const float* __restrict__ V, const float* __restrict__ D,
+    int nmax, int rt, int tiles, const float* __restrict__ V, const float* __restrict__ D,
     const float* __restrict__ coef_t, const float* __restrict__ coef_s, int cw,
     const float* __restrict__ x, const float* __restrict__ res, float scale,
     const float* __restrict__ dtr, int dtiles, float* __restrict__ gx, float* __restrict__ gU,
@@ -386,10 +386,10 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
   float* ss = ts + ncol;           // s of the sibling per level
   float* part = ss + ncol;         // the groups' row sums
   float* dt = part + LEAF_T;       // D^T res of the tile's rows
-  const int leaf = (1 << L) + blockIdx.x;
+  const int li = blockIdx.x / tiles, leaf = (1 << L) + li;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int i0 = blockIdx.y * rt;
+  const int i0 = (blockIdx.x - li * tiles) * rt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
   for (int e = tid; e < ncol; e += LEAF_T) {
@@ -399,7 +399,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
     ss[e] = coef_s[(int64_t)sib * cw + col];
   }
   if (gx && !dtr) {
-    const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
+    const float* Dl = D + (int64_t)li * nmax * nmax;
     for (int q = warp; q < rt; q += LEAF_T / 32) {
       float v = 0.f;
       if (i0 + q < ns)
@@ -448,7 +448,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
   }
   if (gD && !dtr && i < nmax) {
     // (zero past the leaf's size, in rows and columns)
-    float* gDl = gD + (int64_t)blockIdx.x * nmax * nmax + i;
+    float* gDl = gD + (int64_t)li * nmax * nmax + i;
     const float sr = scale * ri;
 #pragma unroll 4
     for (int m = g; m < nmax; m += G)
@@ -586,8 +586,14 @@ static bool v_in_place(const hm_tree* t, int k, const float* V, const float* gU,
   return (gU && factored_overlap(gU, m, V, m)) || (gV && factored_overlap(gV, m, V, m));
 }
 
-static dim3 leaf_grid(const hm_tree* t, int rt) {
-  return dim3(1u << t->L, (unsigned)((t->nmax + rt - 1) / rt));
+// Tiles of rt rows that a leaf has, and the grid: a leaf's tiles are neighbours in it, so
+// that the memory sectors that two of them share (rows may start anywhere) meet in L2.
+// With all leaves' first tiles before their second the two parts of a gradient's sector
+// went to HBM apart: fused step, k = 32, N = 262144 525 us (513 so), N = 262143 763 (571),
+// N = 200001 666 (467).
+static int leaf_tiles(const hm_tree* t, int rt) { return (int)((t->nmax + rt - 1) / rt); }
+static unsigned leaf_grid(const hm_tree* t, int rt) {
+  return (1u << t->L) * (unsigned)leaf_tiles(t, rt);
 }
 
 hm_status factored_check(const hm_tree* t, bool adjoint) {
@@ -639,7 +645,8 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, x, y);
   else
     k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, leaf_tiles(t, rt), trans ? V : U, coef,
+        D, trans, x, y);
 }
 
 // gU and gV may share memory with U and V, gD with D; gx shares none with the inputs.
@@ -663,8 +670,8 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
           oD);
     else
       k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, V, D, coef, coef + k, 2 * k, x, res,
-          scale, nullptr, 0, ox, oU, oV, oD);
+          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, leaf_tiles(t, rt), V, D, coef, coef + k,
+          2 * k, x, res, scale, nullptr, 0, ox, oU, oV, oD);
   };
   if (gx && v_in_place(t, k, V, gU, gV)) {
     run(gx, nullptr, nullptr, d_in_place ? nullptr : gD);
@@ -681,7 +688,7 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
 
 size_t factored_loss_grad_scratch_bytes(const hm_tree* t, int k) {
   const size_t nodes = (size_t)1 << (t->L + 1);
-  const size_t tiles = leaf_grid(t, forward_rows(t, k)).y;
+  const size_t tiles = leaf_tiles(t, forward_rows(t, k));
   return sizeof(float) * ((size_t)t->n_fchunks * k + (nodes / 2) * tiles * t->L * k +
                           2 * nodes * k + (2 + tiles) * (size_t)t->n) + 512;
 }
@@ -701,8 +708,7 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   const int nodes = 1 << (L + 1);
   const int nmax = (int)t->nmax;
   const int rf = forward_rows(t, k), rt = leaf_rows(t);
-  const dim3 gf = leaf_grid(t, rf);
-  const int tiles = (int)gf.y;
+  const int tiles = leaf_tiles(t, rf), atiles = leaf_tiles(t, rt);
   float* partial = scratch;
   float* sp = partial + (size_t)t->n_fchunks * k;
   float* coef_t = sp + (size_t)(nodes / 2) * tiles * L * k;
@@ -718,9 +724,9 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
     raise_smem_limit((const void*)kern, done);
-    kern<<<gf, LEAF_T, forward_smem(t, k, rf, ds), st>>>(t->d_start, t->d_size, L, t->n, k, nmax, U,
-                                                         coef_t, D, x, yy, b, rr, scale, sp, dtr,
-                                                         d_in_place ? nullptr : gD);
+    kern<<<leaf_grid(t, rf), LEAF_T, forward_smem(t, k, rf, ds), st>>>(
+        t->d_start, t->d_size, L, t->n, k, nmax, tiles, U, coef_t, D, x, yy, b, rr, scale, sp, dtr,
+        d_in_place ? nullptr : gD);
   };
   static std::atomic<uint32_t> done[4] = {{0}, {0}, {0}, {0}};
   if (rf == 32) ds ? forward(k_fact_forward<1, 32>, done[0]) : forward(k_fact_forward<0, 32>, done[1]);
@@ -729,7 +735,7 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   if (d_in_place) {  // once every tile has read D
     count_launches(1);
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, nullptr,
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, atiles, V, D, coef_t, coef_s, k, x, rr, scale, nullptr,
         0, nullptr, nullptr, nullptr, gD);
   }
   if (res && gx && factored_overlap(gx, t->n, res, t->n)) {
@@ -738,7 +744,7 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   }
   auto adjoint = [&](float* ox, float* oU, float* oV) {
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, nmax, rt, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, atiles, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
         tiles, ox, oU, oV, nullptr);
   };
   if (gx && v_in_place(t, k, V, gU, gV)) {
