@@ -71,9 +71,10 @@ __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restric
 // out[node][e] = sum over the node's chunks (heap ids 2 .. 2^(L+1)-1): chunks
 // begin[node] .. begin[node + 1] at partial[chunk * stride + e], or, without `begin`,
 // the row tiles (`tiles` a leaf) of the node's leaves (L rows of k per tile).  The
-// threads (RED_T over row tiles, RED_C over chunks) form blockDim / width groups; group q sums chunks q, q + groups, ... and the
-// group sums are added in group order (deterministic).  width <= 128.  (A node of level
-// 1 has thousands of row tiles: the chain of its loads is what takes the time.)
+// threads (RED_T over row tiles, RED_C over chunks) form blockDim / width groups; group q
+// sums chunks q, q + groups, ... and the group sums are added in group order
+// (deterministic).  width <= 128.  (A node of level 1 has thousands of row tiles: the
+// chain of its loads is what takes the time.)
 constexpr int RED_T = 1024, RED_C = 256;
 __global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__ partial,
                                                      const int32_t* __restrict__ fbegin,
@@ -114,6 +115,14 @@ __global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__
 // groups' row sums meet in shared memory.  The leaf's x is staged LEAF_X at a time.
 constexpr int LEAF_T = 512, LEAF_X = 1024;
 
+// Leaf and tile of a block (see tile_order): a leaf's tiles next to each other, or (tiles
+// negative) every leaf's first tile before any second one.
+__device__ __forceinline__ int2 leaf_tile(int L, int tiles) {
+  const int b = blockIdx.x;
+  if (tiles < 0) return make_int2(b & ((1 << L) - 1), b >> L);
+  return make_int2(b / tiles, b % tiles);
+}
+
 // acc + sum over columns e = g, g + G, .. < m of a[e * ld] c[e]
 constexpr int ROWB = 8;
 __device__ __forceinline__ float row_dot(const float* a, int64_t ld, const float* c, int g, int G,
@@ -143,7 +152,7 @@ __device__ __forceinline__ float warp_total(float v) {
 // rows.
 __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
-    int nmax, int rt, int tiles, const float* __restrict__ Uex, const float* __restrict__ coef,
+    int nmax, int rt, const float* __restrict__ Uex, const float* __restrict__ coef,
     const float* __restrict__ D, int trans, const float* __restrict__ x, float* __restrict__ y) {
   extern __shared__ float sm[];
   const int ncol = L * k;          // column e of level 1 + e / k starts at Uex + e n
@@ -151,10 +160,10 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
   float* xs = cs + ncol;           // LEAF_X entries of the leaf's x
   float* part = xs + LEAF_X;       // the groups' row sums
   float* rs = part + LEAF_T;       // rt rows of D^T x (trans)
-  const int li = blockIdx.x / tiles, leaf = (1 << L) + li;
+  const int leaf = (1 << L) + blockIdx.x;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int i0 = (blockIdx.x - li * tiles) * rt;
+  const int i0 = blockIdx.y * rt;
   if (i0 >= ns) return;  // uniform over the block
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
@@ -163,7 +172,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
     const int anc = leaf >> (L - j);
     cs[e] = coef[(int64_t)(anc ^ 1) * k + col];
   }
-  const float* Dl = D + (int64_t)li * nmax * nmax;
+  const float* Dl = D + (int64_t)blockIdx.x * nmax * nmax;
   if (trans)
     for (int q = warp; q < rt; q += LEAF_T / 32) {
       float v = 0.f;
@@ -197,13 +206,14 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_expand(
 // The same by whole leaves: a block of 256 threads holds the leaf's x (and D^T x) in shared
 // memory, a thread takes a row.  For y in x's place (the tiles above read x over the whole
 // leaf while other tiles write), and where the leaves alone fill the chip and the factors
-// come from HBM (leaf_form): N = 262144, k = 32, 604 MB: 100 us, the tiles 113-128 (shorter
-// runs of each column); N = 65536, k = 16, leaves of 128 (71 MB, in L2): 36 us, the tiles
-// 24-32.
+// come from HBM (leaf_form_apply): N = 262144, k = 32, 604 MB: 100 us, the tiles 113-128
+// (shorter runs of each column).
 // IN_PLACE: x is y (the same address) and is read through y: a block reads its leaf before
 // its first barrier, writes it after, and touches no other.  Plain loops over qualified
-// pointers: the whole apply 181 us at k = 32; 189 with batches of eight conditional loads,
-// 235 with the same loops unqualified.
+// pointers (the whole apply 181 us at k = 32; 189 with batches of eight conditional loads,
+// 235 with the same loops unqualified; more loads in flight cost up to 1.6 times, N = 65536,
+// k = 8 or 180001, k = 32: a block's warps then leave the column that they share).  Sums by
+// level and by 32 columns of D: one chain over all of them rounds 2.5 times as much.
 template <bool IN_PLACE>
 __global__ __launch_bounds__(256) void k_fact_expand_leaf(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
@@ -235,12 +245,20 @@ __global__ __launch_bounds__(256) void k_fact_expand_leaf(
   for (int i = tid; i < ns; i += 256) {
     const float* u = Uex + s0 + i;
     float acc = 0.f;
-    for (int j = 0; j < L; ++j)
-      for (int c = 0; c < k; ++c) acc = fmaf(u[(int64_t)(j * k + c) * n], cs[j * k + c], acc);
+    for (int j = 0; j < L; ++j) {
+      float t = 0.f;
+      for (int c = 0; c < k; ++c) t = fmaf(u[(int64_t)(j * k + c) * n], cs[j * k + c], t);
+      acc += t;
+    }
     if (trans) {
       acc += dt[i];
     } else {
-      for (int m = 0; m < ns; ++m) acc = fmaf(Dl[i + (int64_t)m * nmax], xs[m], acc);
+      float t = 0.f;
+      for (int m = 0; m < ns; ++m) {
+        t = fmaf(Dl[i + (int64_t)m * nmax], xs[m], t);
+        if ((m & 31) == 31) { acc += t; t = 0.f; }
+      }
+      acc += t;
     }
     y[s0 + i] = acc;
   }
@@ -277,7 +295,8 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
   float* rs = part + LEAF_T;       // rt rows of res
   float* us = rs + rt;             // the tile's rows of U, [ncol][pt]
   float* ds = us + ncol * pt;      // DS: its rows of D, [nmax][pt]
-  const int li = blockIdx.x / tiles, tile = blockIdx.x - li * tiles, leaf = (1 << L) + li;
+  const int2 lt = leaf_tile(L, tiles);
+  const int li = lt.x, tile = lt.y, leaf = (1 << L) + li;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
   const int i0 = tile * rt;
@@ -340,7 +359,7 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_forward(
   }
   __syncthreads();
   // a thread a column: D^T res, then U^T res over the tile's rows
-  float* spt = sp + (int64_t)blockIdx.x * ncol;
+  float* spt = sp + ((int64_t)li * abs(tiles) + tile) * ncol;
   float* dt = dtr + (int64_t)tile * n + s0;
   const int nd = DS ? ns : 0;
   for (int e = tid; e < nd + ncol; e += LEAF_T) {
@@ -386,10 +405,11 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
   float* ss = ts + ncol;           // s of the sibling per level
   float* part = ss + ncol;         // the groups' row sums
   float* dt = part + LEAF_T;       // D^T res of the tile's rows
-  const int li = blockIdx.x / tiles, leaf = (1 << L) + li;
+  const int2 lt = leaf_tile(L, tiles);
+  const int li = lt.x, leaf = (1 << L) + li;
   const int64_t s0 = start[leaf];
   const int ns = (int)size[leaf];
-  const int i0 = (blockIdx.x - li * tiles) * rt;
+  const int i0 = lt.y * rt;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int G = LEAF_T / rt, g = tid / rt, i = i0 + (tid & (rt - 1));
   for (int e = tid; e < ncol; e += LEAF_T) {
@@ -456,9 +476,11 @@ __global__ __launch_bounds__(LEAF_T) void k_fact_adjoint(
   }
 }
 
-// The same by whole leaves (leaf_form), coefficients of t and s in one array: a thread a
-// row of the leaf, x, res and D^T res in shared memory.  N = 262144, leaves of 256: 276 us
-// at k = 32 (the tiles 301); the whole adjoint at k = 8 208 us (231).
+// The same by whole leaves (leaf_form_adjoint), coefficients of t and s in one array: a
+// thread a row of the leaf, x, res and D^T res in shared memory.  N = 262144, leaves of 256:
+// 276 us at k = 32 (the tiles 301); the whole adjoint at k = 8 208 us (231).  A thread's sum
+// over all columns is compensated (its own rounding would be 1.8 times the tiles'); sums by
+// groups of columns cost up to a fifth of the time.
 __global__ __launch_bounds__(256) void k_fact_adjoint_leaf(
     const int64_t* __restrict__ start, const int64_t* __restrict__ size, int L, int64_t n, int k,
     int nmax, const float* __restrict__ V, const float* __restrict__ D,
@@ -500,14 +522,18 @@ __global__ __launch_bounds__(256) void k_fact_adjoint_leaf(
   for (int i = tid; i < ns; i += 256) {
     const int64_t row = s0 + i;
     const float xr = xs[i], rr = rs[i];
-    float acc = 0.f;
+    float acc = 0.f, err = 0.f;
     for (int e = 0; e < ncol; ++e) {
       const int64_t off = row + (int64_t)e * n;
-      if (gx) acc = fmaf(V[off], ss[e], acc);
+      if (gx) {
+        const float v = V[off], s = fmaf(v, ss[e], acc);
+        err += fmaf(v, ss[e], acc - s);  // what the sum has just lost
+        acc = s;
+      }
       if (gU) gU[off] = scale * rr * ts[e];
       if (gV) gV[off] = scale * xr * ss[e];
     }
-    if (gx) gx[row] = scale * (acc + dt[i]);
+    if (gx) gx[row] = scale * (acc + err + dt[i]);
     if (gD)
       for (int m = 0; m < nmax; ++m) gDl[i + (int64_t)m * nmax] = m < ns ? scale * rr * xs[m] : 0.f;
   }
@@ -536,14 +562,27 @@ static size_t fact_partial_smem(int k) {
   return sizeof(float) * 256 * (size_t)(k + 1);
 }
 
-// Whole leaves where they fill the chip (four blocks an SM) and the factors exceed L2
-// twice over (once for the transposed product): then long runs of each column count, not
-// the number of blocks.  N = 131072, k = 32, leaves of 128 (235 MB), the apply's three
-// kernels: 115 us by leaves and 109 by tiles, transposed 119 and 124.
-static bool leaf_form(const hm_tree* t, int k, int mib = 256) {
-  const size_t leaves = (size_t)1 << t->L;
-  return leaves >= 608 &&
-         sizeof(float) * (size_t)t->n * ((size_t)t->L * k + t->nmax) >= (size_t)mib << 20;
+// Whole leaves where they fill the chip and long runs of each column count more than the
+// number of blocks: leaves enough, and few columns beside a leaf's own (its D is most of
+// what is read), or a large n.  Measured on 400 trees of 512 to 262144 points, us by
+// leaves / by tiles: apply N = 70000, leaves of 137, k = 8 24 / 40, N = 200001, 196, 32
+// 137 / 179, N = 50000, 196, 4 (256 leaves) 21 / 27; the other side N = 65536, 128, 64
+// 113 / 95, N = 131072, 64, 32 131 / 113, N = 65536, 512, 4 101 / 51.  (The transposed
+// product's tiles read D along its columns and hold out longer: N = 131072, 256, 4 74 / 65.)
+static bool leaf_form_apply(const hm_tree* t, int k, int trans) {
+  const int64_t leaves = (int64_t)1 << t->L, ncol = (int64_t)t->L * k;
+  if (!trans && leaves >= 256 && ncol <= 96) return true;
+  if (leaves >= 608 && 4 * t->n * (ncol + t->nmax) >= (trans ? 128ll : 256ll) << 20) return true;
+  if (trans && (t->n < 57000 || (leaves < 1024 && t->nmax > 200))) return false;
+  return leaves >= 512 &&
+         (ncol <= std::max<int64_t>(t->nmax, 160) || (t->n >= 100000 && t->nmax >= 70));
+}
+// The adjoint writes as much as it reads: N = 131072, leaves of 256, k = 8 102 / 128,
+// N = 262144, 256, 32 420 / 433; the other side N = 262144, 128, 32 514 / 432, N = 30001, 15,
+// 64 488 / 244.
+static bool leaf_form_adjoint(const hm_tree* t, int k) {
+  const int64_t leaves = (int64_t)1 << t->L, ncol = (int64_t)t->L * k;
+  return leaves >= 512 && 2 * ncol <= 3 * t->nmax && (t->nmax >= 100 || 5 * ncol <= 3 * t->nmax);
 }
 // Rows of a block's tile: 64, or 32 where 64 would leave SMs without two blocks
 // (N = 4096 in leaves of 256: 64 blocks of 64 rows, 128 of 32).
@@ -586,14 +625,20 @@ static bool v_in_place(const hm_tree* t, int k, const float* V, const float* gU,
   return (gU && factored_overlap(gU, m, V, m)) || (gV && factored_overlap(gV, m, V, m));
 }
 
-// Tiles of rt rows that a leaf has, and the grid: a leaf's tiles are neighbours in it, so
-// that the memory sectors that two of them share (rows may start anywhere) meet in L2.
-// With all leaves' first tiles before their second the two parts of a gradient's sector
-// went to HBM apart: fused step, k = 32, N = 262144 525 us (513 so), N = 262143 763 (571),
-// N = 200001 666 (467).
 static int leaf_tiles(const hm_tree* t, int rt) { return (int)((t->nmax + rt - 1) / rt); }
 static unsigned leaf_grid(const hm_tree* t, int rt) {
   return (1u << t->L) * (unsigned)leaf_tiles(t, rt);
+}
+// The order of the tiles in the kernels that write gradients.  Two tiles of a leaf share
+// memory sectors (rows may start anywhere).  With every leaf's first tile before any second
+// one the two parts of a gradient's sector went to HBM apart: fused step, k = 32, N = 262143
+// 763 us (571 with a leaf's tiles next to each other; N = 262144 525 and 513), N = 200001
+// 666 (467).  While the gradients fit L2 they meet there in any order, and the leaves' last
+// tiles, which may be short, are better last (adjoint, N = 20000, leaves of 157, k = 64: 69
+// us, 74 by neighbours); so they are in the apply, which writes no columns.
+static int tile_order(const hm_tree* t, int k, int rt) {
+  const int64_t written = 4 * t->n * (2 * (int64_t)t->L * k + t->nmax);
+  return written < (96ll << 20) ? -leaf_tiles(t, rt) : leaf_tiles(t, rt);
 }
 
 hm_status factored_check(const hm_tree* t, bool adjoint) {
@@ -633,20 +678,19 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * k;
   // t_node = Proj(I_node)^T x with Proj = V (H x) or U (H^T x)
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, trans ? U : V, x, nullptr,
-                                               nullptr, partial);
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(
+      t->d_fchunks, t->n, k, trans ? U : V, x, nullptr, nullptr, partial);
   k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
   const size_t leaf_smem = sizeof(float) * ((size_t)L * k + 2 * t->nmax);
   if (x == y)
     k_fact_expand_leaf<true><<<1u << L, 256, leaf_smem, st>>>(
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, nullptr, y);
-  else if (leaf_form(t, k, trans ? 128 : 256))
+  else if (leaf_form_apply(t, k, trans))
     k_fact_expand_leaf<false><<<1u << L, 256, leaf_smem, st>>>(
         t->d_start, t->d_size, L, t->n, k, (int)t->nmax, trans ? V : U, coef, D, trans, x, y);
   else
-    k_fact_expand<<<leaf_grid(t, rt), LEAF_T, expand_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, leaf_tiles(t, rt), trans ? V : U, coef,
-        D, trans, x, y);
+    k_fact_expand<<<dim3(1u << L, leaf_tiles(t, rt)), LEAF_T, expand_smem(t, k, rt), st>>>(
+        t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, trans ? V : U, coef, D, trans, x, y);
 }
 
 // gU and gV may share memory with U and V, gD with D; gx shares none with the inputs.
@@ -659,19 +703,19 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
   const int nodes = 1 << (L + 1), rt = leaf_rows(t);
   float* partial = scratch;
   float* coef = scratch + (size_t)t->n_fchunks * 2 * k;
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, U, res,
-                                                        partial);
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, U,
+                                                                  res, partial);
   k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto run = [&](float* ox, float* oU, float* oV, float* oD) {
-    if (leaf_form(t, k))
+    if (leaf_form_adjoint(t, k))
       k_fact_adjoint_leaf<<<1u << L, 256, sizeof(float) * (2 * (size_t)L * k + 3 * t->nmax), st>>>(
           t->d_start, t->d_size, L, t->n, k, (int)t->nmax, V, D, coef, x, res, scale, ox, oU, oV,
           oD);
     else
       k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, leaf_tiles(t, rt), V, D, coef, coef + k,
-          2 * k, x, res, scale, nullptr, 0, ox, oU, oV, oD);
+          t->d_start, t->d_size, L, t->n, k, (int)t->nmax, rt, tile_order(t, k, rt), V, D, coef,
+          coef + k, 2 * k, x, res, scale, nullptr, 0, ox, oU, oV, oD);
   };
   if (gx && v_in_place(t, k, V, gU, gV)) {
     run(gx, nullptr, nullptr, d_in_place ? nullptr : gD);
@@ -708,7 +752,7 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   const int nodes = 1 << (L + 1);
   const int nmax = (int)t->nmax;
   const int rf = forward_rows(t, k), rt = leaf_rows(t);
-  const int tiles = leaf_tiles(t, rf), atiles = leaf_tiles(t, rt);
+  const int tiles = leaf_tiles(t, rf), order = tile_order(t, k, rt);
   float* partial = scratch;
   float* sp = partial + (size_t)t->n_fchunks * k;
   float* coef_t = sp + (size_t)(nodes / 2) * tiles * L * k;
@@ -717,26 +761,28 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   float* yy = y ? y : tmp;
   float* rr = res ? res : tmp + t->n;
   float* dtr = tmp + 2 * t->n;
-  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, nullptr, nullptr,
-                                               partial);
+  k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x,
+                                                                  nullptr, nullptr, partial);
   k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
   const bool ds = forward_ds(t, k);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
     raise_smem_limit((const void*)kern, done);
     kern<<<leaf_grid(t, rf), LEAF_T, forward_smem(t, k, rf, ds), st>>>(
-        t->d_start, t->d_size, L, t->n, k, nmax, tiles, U, coef_t, D, x, yy, b, rr, scale, sp, dtr,
-        d_in_place ? nullptr : gD);
+        t->d_start, t->d_size, L, t->n, k, nmax, tile_order(t, k, rf), U, coef_t, D, x, yy, b, rr,
+        scale, sp, dtr, d_in_place ? nullptr : gD);
   };
   static std::atomic<uint32_t> done[4] = {{0}, {0}, {0}, {0}};
-  if (rf == 32) ds ? forward(k_fact_forward<1, 32>, done[0]) : forward(k_fact_forward<0, 32>, done[1]);
-  else ds ? forward(k_fact_forward<1, 16>, done[2]) : forward(k_fact_forward<0, 16>, done[3]);
+  if (rf == 32 && ds) forward(k_fact_forward<1, 32>, done[0]);
+  else if (rf == 32) forward(k_fact_forward<0, 32>, done[1]);
+  else if (ds) forward(k_fact_forward<1, 16>, done[2]);
+  else forward(k_fact_forward<0, 16>, done[3]);
   k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
   if (d_in_place) {  // once every tile has read D
     count_launches(1);
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, nmax, rt, atiles, V, D, coef_t, coef_s, k, x, rr, scale, nullptr,
-        0, nullptr, nullptr, nullptr, gD);
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, order, V, D, coef_t, coef_s, k, x, rr, scale,
+        nullptr, 0, nullptr, nullptr, nullptr, gD);
   }
   if (res && gx && factored_overlap(gx, t->n, res, t->n)) {
     launch_copy_cols<float>(res, t->n, tmp + t->n, t->n, t->n, 1, st);
@@ -744,8 +790,8 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   }
   auto adjoint = [&](float* ox, float* oU, float* oV) {
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
-        t->d_start, t->d_size, L, t->n, k, nmax, rt, atiles, V, D, coef_t, coef_s, k, x, rr, scale, dtr,
-        tiles, ox, oU, oV, nullptr);
+        t->d_start, t->d_size, L, t->n, k, nmax, rt, order, V, D, coef_t, coef_s, k, x, rr, scale,
+        dtr, tiles, ox, oU, oV, nullptr);
   };
   if (gx && v_in_place(t, k, V, gU, gV)) {
     adjoint(gx, nullptr, nullptr);

@@ -1,6 +1,6 @@
-"""The factored layer's forms that only large trees take, with uneven leaves: whole leaves
-(608 leaves and 256 MiB of factors or more), and the fused step's forward with D outside
-shared memory and with tiles of 16 rows."""
+"""The factored layer's forms that only large trees take, with uneven leaves: whole leaves,
+gradients in both orders of the tiles, and the fused step's forward with D outside shared
+memory and with tiles of 16 rows."""
 import numpy as np
 import pytest
 import torch
@@ -61,7 +61,9 @@ class Reference:
         return self.apply(r, True), gU, gV, torch.bmm(self.leaves(x), self.leaves(r).transpose(1, 2))
 
 
-@pytest.mark.parametrize("n,m,k", [(200001, 256, 32),   # whole leaves of 195 and 196
+@pytest.mark.parametrize("n,m,k", [(200001, 256, 32),   # apply by whole leaves of 195 and 196
+                                   (70001, 256, 8),     # apply and adjoint, of 136 and 137
+                                   (50001, 256, 4),     # apply, not transposed, 256 leaves
                                    (130001, 256, 64),   # 576 columns of U beside 254 of D do not fit
                                    (20000, 2, 64)])     # 896 columns of U: tiles of 16 rows
 def test_forms_against_fp64(n, m, k):

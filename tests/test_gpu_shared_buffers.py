@@ -30,8 +30,8 @@ def pair(x, d):
     return a, c
 
 
-# the last one takes the whole-leaf kernels (608 leaves and 256 MiB of factors or more)
-SIZES = [(515, 33, 9), (4096, 256, 32), (5003, 64, 5), (200001, 256, 32)]
+# the last two take the whole-leaf kernels (the adjoint's: the last)
+SIZES = [(515, 33, 9), (4096, 256, 32), (5003, 64, 5), (200001, 256, 32), (70001, 256, 8)]
 
 
 @pytest.mark.parametrize("n,m,k", SIZES)
