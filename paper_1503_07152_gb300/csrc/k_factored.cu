@@ -69,37 +69,22 @@ __global__ __launch_bounds__(256) void k_fact_partial(const FactChunk* __restric
 }
 
 // out[node][e] = sum over the node's chunks (heap ids 2 .. 2^(L+1)-1): chunks
-// begin[node] .. begin[node + 1] at partial[chunk * stride + e], or, without `begin`,
-// the row tiles (`tiles` a leaf) of the node's leaves (L rows of k per tile).  The
-// threads (RED_T over row tiles, RED_C over chunks) form blockDim / width groups; group q
-// sums chunks q, q + groups, ... and the group sums are added in group order
-// (deterministic).  width <= 128.  (A node of level 1 has thousands of row tiles: the
-// chain of its loads is what takes the time.)
+// begin[node] .. begin[node + 1] at partial[chunk * width + e].  The threads form
+// RED_C / width groups; group q sums chunks q, q + groups, ... and the group sums are
+// added in group order (deterministic).  width <= 128.
 constexpr int RED_T = 1024, RED_C = 256;
-__global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__ partial,
-                                                     const int32_t* __restrict__ fbegin,
-                                                     int width, int L, int tiles,
-                                                     float* __restrict__ out) {
-  __shared__ float sred[RED_T];
+__global__ __launch_bounds__(RED_C) void k_fact_reduce(const float* __restrict__ partial,
+                                                       const int32_t* __restrict__ fbegin,
+                                                       int width, float* __restrict__ out) {
+  __shared__ float sred[RED_C];
   const int node = 2 + blockIdx.x;
-  int c0, c1;
-  int64_t stride = width, off = 0;
-  if (fbegin) {
-    c0 = fbegin[node];
-    c1 = fbegin[node + 1];
-  } else {
-    const int j = 31 - __clz(node);  // the node's level
-    c0 = ((node << (L - j)) - (1 << L)) * tiles;
-    c1 = (((node + 1) << (L - j)) - (1 << L)) * tiles;
-    stride = (int64_t)L * width;
-    off = (int64_t)(j - 1) * width;
-  }
-  const int groups = blockDim.x / width;
+  const int c0 = fbegin[node], c1 = fbegin[node + 1];
+  const int groups = RED_C / width;
   const int t = threadIdx.x, e = t % width, q = t / width;
   float s = 0.f;
   if (q < groups) {
 #pragma unroll 8
-    for (int c = c0 + q; c < c1; c += groups) s += partial[c * stride + off + e];
+    for (int c = c0 + q; c < c1; c += groups) s += partial[(int64_t)c * width + e];
   }
   sred[t] = s;
   __syncthreads();
@@ -107,6 +92,52 @@ __global__ __launch_bounds__(RED_T) void k_fact_reduce(const float* __restrict__
     float tot = 0.f;
     for (int g = 0; g < groups; ++g) tot += sred[g * width + t];
     out[(int64_t)node * width + t] = tot;
+  }
+}
+
+// The same over the row tiles (`tiles` a leaf, L rows of k per tile) of a node's leaves:
+// thousands for a node of level 1, where the chain of a thread's loads takes the time, one
+// or two for most nodes, where the blocks do.  A block's RED_T / k groups are dealt out to
+// as many nodes of one level as they serve with two tiles each.  N = 262144, k = 32: 16 us
+// with a block a node, 14 so; the fused step at N = 70000, leaves of 69, k = 4: 90 and 75,
+// at N = 131073, leaves of 9, k = 4: 702 and 440.
+struct TileReduce {
+  int k, L, tiles, blocks;
+  int first[32], gpn[32];  // of a level: its first block, a node's groups
+  TileReduce(int k_, int L_, int tiles_) : k(k_), L(L_), tiles(tiles_), blocks(0) {
+    const int groups = RED_T / k;
+    for (int j = 1; j <= L; ++j) {
+      first[j] = blocks;
+      gpn[j] = (int)std::min<int64_t>(groups, (((int64_t)tiles << (L - j)) + 1) / 2);
+      const int npb = groups / gpn[j];
+      blocks += ((1 << j) + npb - 1) / npb;
+    }
+  }
+};
+__global__ __launch_bounds__(RED_T, 2) void k_fact_reduce_tiles(const __grid_constant__ TileReduce r,
+                                                             const float* __restrict__ partial,
+                                                             float* __restrict__ out) {
+  __shared__ float sred[RED_T];
+  int j = 1;
+  while (j < r.L && (int)blockIdx.x >= r.first[j + 1]) ++j;
+  const int k = r.k, gpn = r.gpn[j], npb = RED_T / k / gpn;
+  const int t = threadIdx.x, e = t % k, q = t / k, local = q / gpn, p = q - local * gpn;
+  const int64_t x = (int64_t)(blockIdx.x - r.first[j]) * npb + local;  // node of the level
+  const bool on = local < npb && x < (1 << j);
+  float s = 0.f;
+  if (on) {
+    const int T = r.tiles << (r.L - j);
+    const int64_t step = (int64_t)gpn * r.L * k;
+    const float* a = partial + ((x * T + p) * r.L + j - 1) * k + e;
+#pragma unroll 8
+    for (int c = p; c < T; c += gpn, a += step) s += *a;
+  }
+  sred[t] = s;
+  __syncthreads();
+  if (on && p == 0) {
+    float tot = 0.f;
+    for (int g = 0; g < gpn; ++g) tot += sred[t + g * k];
+    out[((1 << j) + x) * k + e] = tot;
   }
 }
 
@@ -680,7 +711,7 @@ void launch_factored_apply(const hm_tree* t, int k, const float* U, const float*
   // t_node = Proj(I_node)^T x with Proj = V (H x) or U (H^T x)
   k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(
       t->d_fchunks, t->n, k, trans ? U : V, x, nullptr, nullptr, partial);
-  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef);
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, coef);
   const size_t leaf_smem = sizeof(float) * ((size_t)L * k + 2 * t->nmax);
   if (x == y)
     k_fact_expand_leaf<true><<<1u << L, 256, leaf_smem, st>>>(
@@ -705,7 +736,7 @@ void launch_factored_adjoint(const hm_tree* t, int k, const float* U, const floa
   float* coef = scratch + (size_t)t->n_fchunks * 2 * k;
   k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x, U,
                                                                   res, partial);
-  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, 2 * k, L, 1, coef);
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, 2 * k, coef);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto run = [&](float* ox, float* oU, float* oV, float* oD) {
     if (leaf_form_adjoint(t, k))
@@ -763,7 +794,7 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   float* dtr = tmp + 2 * t->n;
   k_fact_partial<<<t->n_fchunks, 256, fact_partial_smem(k), st>>>(t->d_fchunks, t->n, k, V, x,
                                                                   nullptr, nullptr, partial);
-  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, L, 1, coef_t);
+  k_fact_reduce<<<nodes - 2, RED_C, 0, st>>>(partial, t->d_fbegin, k, coef_t);
   const bool ds = forward_ds(t, k);
   const bool d_in_place = gD && factored_overlap(gD, dsize(t), D, dsize(t));
   auto forward = [&](auto kern, std::atomic<uint32_t>& done) {
@@ -777,7 +808,8 @@ void launch_factored_loss_grad(const hm_tree* t, int k, const float* U, const fl
   else if (rf == 32) forward(k_fact_forward<0, 32>, done[1]);
   else if (ds) forward(k_fact_forward<1, 16>, done[2]);
   else forward(k_fact_forward<0, 16>, done[3]);
-  k_fact_reduce<<<nodes - 2, RED_T, 0, st>>>(sp, nullptr, k, L, tiles, coef_s);
+  const TileReduce tr(k, L, tiles);
+  k_fact_reduce_tiles<<<tr.blocks, RED_T, 0, st>>>(tr, sp, coef_s);
   if (d_in_place) {  // once every tile has read D
     count_launches(1);
     k_fact_adjoint<<<leaf_grid(t, rt), LEAF_T, adjoint_smem(t, k, rt), st>>>(
