@@ -170,7 +170,6 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
     int aoff_o, int ka, const double* __restrict__ B, int64_t ldb, int boff_e, int boff_o,
     int kb, double* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[256 / SUM64][32];
   const Chunk ch = chunks[blockIdx.x];
   const int rows = (int)(ch.r1 - ch.r0);  // <= 256
   const int aoff = (ch.node & 1) ? aoff_o : aoff_e;
@@ -190,20 +189,21 @@ __global__ __launch_bounds__(256) void k_seg_tn_partial64_split(
     for (int c = 0; c < nb; ++c) Bs[row * pb + c] = bp[(int64_t)c * ldb];
   }
   __syncthreads();
-  const int jb = lane < ne ? (e0 + lane) / ka - jlo : 0;
-  const int c = lane < ne ? lane : 0;
   const int groups = (rows + SUM64 - 1) / SUM64;
-  for (int g = w; g < groups; g += 8) {
-    const int q1 = min(rows, (g + 1) * SUM64);
-    double t = 0.0;
+  if (lane < ne) {
+    const int jb = (e0 + lane) / ka - jlo;
+    for (int g = w; g < groups; g += 8) {
+      const int q1 = min(rows, (g + 1) * SUM64);
+      double t = 0.0;
 #pragma unroll 4
-    for (int q = g * SUM64; q < q1; ++q) t = fma(As[q * 33 + c], Bs[q * pb + jb], t);
-    red[g][lane] = t;
+      for (int q = g * SUM64; q < q1; ++q) t = fma(As[q * 33 + lane], Bs[q * pb + jb], t);
+      As[g * SUM64 * 33 + lane] = t;  // over an entry that this lane alone reads
+    }
   }
   __syncthreads();
   if (w == 0 && lane < ne) {
     double v = 0.0;
-    for (int g = 0; g < groups; ++g) v += red[g][lane];
+    for (int g = 0; g < groups; ++g) v += As[g * SUM64 * 33 + lane];
     partial[(int64_t)blockIdx.x * mtot + e0 + lane] = v;
   }
 }
