@@ -234,7 +234,9 @@ hm_status hm_set_wait_limit(int64_t polls);
 /*
  * The sampling GEMM behind the dense operator, callable directly:
  * Y = op(A) X for the row-major dense A above.  Same argument rules as
- * hm_apply_fn.  Returns HM_OK or an error status.
+ * hm_apply_fn.  Returns HM_OK or an error status.  With dtypes 0 and 2 a column's
+ * result does not depend on the others to the bit; with dtype 4 the grouping of its
+ * sum may (a split over K, chosen by the shape).
  */
 hm_status hm_dense_apply(const hm_operator* op, int trans, int64_t ncols, const void* X,
                          int64_t ldx, void* Y, int64_t ldy, void* stream);
@@ -320,7 +322,8 @@ hm_status hm_tune_batched(int32_t nops, const hm_operator* ops, hm_tree* const* 
  * with m = L plus the leaf blocks.  X, Y: device, column-major, n x ncols,
  * element type of the handle's precision.  Y may be X, or columns beside X's in
  * one buffer; where the two share elements in any other way X is copied first (the
- * copy is taken from the stream's memory pool).
+ * copy is taken from the stream's memory pool).  A column's result does not depend,
+ * to the bit, on the columns that go along with it.
  */
 hm_status hm_apply(const hm_handle* h, int trans, int64_t ncols, const void* X, int64_t ldx,
                    void* Y, int64_t ldy, void* stream);
@@ -407,7 +410,8 @@ hm_status hm_hodlr_factorize(hm_handle* h, void* stream);
 /*
  * X = A_c^{-1} B (trans = 0) or A_c^{-T} B (trans = 1) for a factorized HODLR
  * handle; B, X device, column-major, n x ncols, the handle's element type (X may
- * share B's memory, as in hm_apply).
+ * share B's memory, and a column's result does not depend on the others, as in
+ * hm_apply).
  * O(k N log N) per column.  HM_EINVAL if the handle is not factorized.
  */
 hm_status hm_solve(const hm_handle* h, int trans, int64_t ncols, const void* B, int64_t ldb,

@@ -148,7 +148,7 @@ __global__ void k_extract_diag(const T* __restrict__ Y, int64_t ldy, T* __restri
 // their sums are added in warp order, so that the warps' work is equal whatever the
 // column count and the leaf size.  D is read straight from global memory along its
 // contiguous index (transposed: through a 32 x 33 tile of the warp's own).  In FP64 it
-// is bound by the FP64 pipe (76 cycles a warp FMA): N = 65536, leaves of 256, 10 columns
+// is bound by the FP64 pipe (64 cycles a warp FMA): N = 65536, leaves of 256, 10 columns
 // 285 us (transposed 565) with a block per leaf and column, 283 (325) now, near the floor.
 constexpr int BD_COLS = 8;
 template <typename T, int TRANS>

@@ -787,7 +787,7 @@ __device__ __forceinline__ void hh_axpy(const float2* v, int qa, int qb, int gl,
   }
 }
 
-// |x|^2 of v[first .. last] (at most 160 entries), one warp: each lane's entries of
+// |x|^2 of v[first .. last] (at most 128 entries), one warp: each lane's entries of
 // every 32-row piece summed over the warp, the pieces in order
 __device__ __forceinline__ void hh_norm2(const float2* v, int first, int last, int lane, float& th,
                                          float& tl) {
