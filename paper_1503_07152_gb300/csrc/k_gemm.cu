@@ -141,9 +141,10 @@ __global__ __launch_bounds__(256) void k_dense_gemm(const T* __restrict__ A, int
 // K tile t belongs to block t mod 2S, or its mirror image 2S - 1 - t mod 2S where that
 // is not below S: half-active patterns of any period then spread over the blocks, and
 // neither the other columns nor their zeros decide which sums a column's terms go to.
-// Products are summed 16 at a time and those sums added up (a chain over all of K
-// rounds 3 times as much at N = 8192, for one FP64 add in 17 less: N = 4096, 5 columns
-// 329 us, 340 so).
+// Products are summed 32 at a time, 16 below N = 1024, and those sums added up: with m
+// terms to a block the rounding grows as the root of 32 + m / 32 or 16 + m / 16, so that
+// neither is above that of 16 at a time and no split over K.  A chain over all of K rounds
+// 3 times as much at N = 8192 for one FP64 add in 33 less.
 template <typename TA, int TRANS>
 __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, int64_t lda,
                                                       int64_t n, int64_t ncols,
@@ -159,6 +160,7 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
   const int nc = (int)min((int64_t)32, ncols - c0);
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   const int nq = w < nc ? (nc - w + 3) / 4 : 0;  // this warp's columns
+  const bool halves = n < 1024;                  // sums of 16 (of 32)
   double acc[8] = {};
   const int nkt = (int)((n + BK - 1) / BK);
   for (int kt = 0; kt < nkt; ++kt) {
@@ -179,17 +181,21 @@ __global__ __launch_bounds__(128) void k_dense_gemm64(const TA* __restrict__ A, 
     __syncthreads();
     if (nq > 0)
       with_count<8>(nq, [&](auto cols) {
+        double t[cols] = {};
 #pragma unroll
         for (int k0 = 0; k0 < BK; k0 += 16) {
-          double t[cols] = {};
 #pragma unroll 4
           for (int k = k0; k < k0 + 16; ++k) {
             const double a = TRANS ? As[k][lane] : As[lane][k];
 #pragma unroll
             for (int q = 0; q < cols; ++q) t[q] = fma(a, Xs[w + 4 * q][k], t[q]);
           }
+          if (k0 > 0 || halves)
 #pragma unroll
-          for (int q = 0; q < cols; ++q) acc[q] += t[q];
+            for (int q = 0; q < cols; ++q) {
+              acc[q] += t[q];
+              t[q] = 0.0;
+            }
         }
       });
     __syncthreads();
