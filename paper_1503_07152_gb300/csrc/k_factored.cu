@@ -564,7 +564,8 @@ __global__ __launch_bounds__(256) void k_fact_adjoint_leaf(
       if (gU) gU[off] = scale * rr * ts[e];
       if (gV) gV[off] = scale * xr * ss[e];
     }
-    if (gx) gx[row] = scale * (acc + err + dt[i]);
+    // (a sum that overflowed has lost NaN; it stays infinite)
+    if (gx) gx[row] = scale * (acc + (isnan(err) ? 0.f : err) + dt[i]);
     if (gD)
       for (int m = 0; m < nmax; ++m) gDl[i + (int64_t)m * nmax] = m < ns ? scale * rr * xs[m] : 0.f;
   }

@@ -131,3 +131,29 @@ def test_sixteen_rows_with_d_outside_shared_memory():
         d, rms = (a - c).double(), float(c.double().square().mean().sqrt())
         assert float(d.square().mean().sqrt()) <= 2e-5 * rms
         assert float(d.abs().max()) <= 1e-3 * rms
+
+
+@pytest.mark.parametrize("n,m,k", [(70001, 256, 8), (20000, 100, 16)])  # whole leaves, tiles
+def test_infinite_factors_stay_infinite(n, m, k):
+    """An infinite entry of V, and sums past FP32's range, make their rows of gx infinite (of
+    the sign that FP64 gives them), not NaN, and leave the others as they are."""
+    t, U, V, D, x, r = layer(n, m, k)
+    gx = torch.full_like(x, float("nan"))
+    hm.hm_hodlr_factored_adjoint(t, k, U, V, D, x, r, 1.0, gx)
+    L = t.levels
+    ref = Reference(n, m, U, V, D)
+    s = torch.stack([ref.project(U, r, j)[:, c] for j in range(1, L + 1) for c in range(k)])  # U^T r
+    Vi, rows = V.clone(), torch.tensor([5, 100, n // 2, n - 1], device=DEV)
+    Vi[0, 1, rows[:2]] = float("inf")
+    Vi[L - 1, k - 1, rows[2]] = float("-inf")
+    Vi[0, 0, rows[3]] = 3e38
+    Vi[0, 1, rows[3]] = 3e38 * torch.sign(s[0, rows[3]] * s[1, rows[3]]).float()
+    gi = torch.full_like(x, float("nan"))
+    hm.hm_hodlr_factored_adjoint(t, k, U, Vi, D, x, r, 1.0, gi)
+    torch.cuda.synchronize()
+    sign = torch.stack([s[1, 5].sign(), s[1, 100].sign(), -s[-1, n // 2].sign(), s[0, n - 1].sign()])
+    assert bool((s[:2, n - 1].abs().sum() * 3e38 > 3.5e38))  # the last row's sum is past the range
+    assert torch.equal(gi[rows].double(), sign * float("inf"))
+    keep = torch.ones(n, dtype=torch.bool, device=DEV)
+    keep[rows] = False
+    assert torch.equal(gi[keep], gx[keep])
